@@ -142,6 +142,25 @@ __device__ __forceinline__ uint32_t bucket_of(uint32_t d, uint32_t nb)
     return nb <= 1 ? 0u : (uint32_t)(((unsigned long long)hash32(d) * nb) >> 32);
 }
 
+// ceil(num / den) as the 64-bit division gives it, den > 0, without that
+// division (the 64-bit pipe is a few lanes wide).  For num < 2^24 every k *
+// den with k < 2^24 is exact in 64 bits, and no quotient above an integer k
+// is so close to it that its 64-bit rounding is k, so the answer is the
+// smallest k with k * den >= num; fmaf rounds k * den - num once, which keeps
+// its sign.  The 32-bit estimate is within 4 * 2^-24 of the quotient, so k is
+// the ceiling of its lower bound or one more.
+__device__ __forceinline__ uint32_t ceil_ratio(uint32_t num, float den)
+{
+    const float x = (float)num, q = x * (1.f / den);
+    if (num < (1u << 24) && q < 262144.f) {
+        float k = ceilf(q * (1.f - 1e-6f));
+        if (fmaf(k, den, -x) < 0.f)
+            k += 1.f;
+        return (uint32_t)k;
+    }
+    return (uint32_t)ceil((double)num / (double)den);
+}
+
 __device__ __forceinline__ unsigned long long pack_pair(uint32_t key, uint32_t w)
 {
     return ((unsigned long long)w << 32) | key;

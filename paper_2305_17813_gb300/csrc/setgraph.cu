@@ -25,7 +25,10 @@
 using namespace mk;
 
 // Kernels of other translation units, launched here unchanged.
-__global__ void k_degree(const uint32_t *src, uint64_t n, uint32_t V, uint32_t *deg, int *bad);
+constexpr uint32_t kDegBlock = 512;
+__global__ void __launch_bounds__(kDegBlock) k_degree(const uint32_t *__restrict__ src, uint64_t n, uint32_t V,
+                                                      uint32_t *deg, int *bad);
+uint32_t degree_grid(uint64_t n);
 __global__ void k_rule(uint32_t *deg, uint32_t V, float per_bucket);
 __global__ void k_init_bitmap(uint32_t *bitmap, uint32_t words, uint32_t P);
 __global__ void k_fill_buckets(uint32_t *b, uint32_t V, uint32_t nb, const uint32_t *user, int *bad);
@@ -65,11 +68,23 @@ __global__ void k_set_init_lists(const uint64_t *off, const uint32_t *buckets, u
                                  uint32_t *owner, uint64_t H, uint64_t total)
 {
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    for (uint64_t v = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; v < V; v += stride) {
-        const uint32_t first = (uint32_t)off[v], nb = buckets[v];
-        vinfo[v] = make_uint2(first, nb);
-        for (uint32_t b = 0; b < nb; ++b)
-            owner[first + b] = (uint32_t)v;
+    const uint32_t lane = lane_id();
+    for (uint64_t vb = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) & ~31ull; vb < V; vb += stride) {
+        const uint32_t v = (uint32_t)vb + lane;
+        const uint32_t first = v < V ? (uint32_t)off[v] : 0, nb = v < V ? buckets[v] : 0;
+        if (v < V)
+            vinfo[v] = make_uint2(first, nb);
+        if (nb <= 8)
+            for (uint32_t b = 0; b < nb; ++b)
+                owner[first + b] = v;
+        // a hub's lists are written by its whole warp
+        for (uint32_t big = __ballot_sync(kFull, nb > 8); big; big &= big - 1) {
+            const uint32_t l = __ffs(big) - 1;
+            const uint32_t f = __shfl_sync(kFull, first, l), m = __shfl_sync(kFull, nb, l);
+            const uint32_t own = __shfl_sync(kFull, v, l);
+            for (uint32_t b = lane; b < m; b += 32)
+                owner[f + b] = own;
+        }
     }
     for (uint64_t s = H + blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; s < total; s += stride)
         owner[s] = kNil;
@@ -702,7 +717,7 @@ mk_status mk_set_bucket_rule(uint32_t V, const uint32_t *d_src, uint64_t n, floa
     MK_CUDA(cudaMemsetAsync(d_bad, 0, sizeof(int), s));
     MK_CUDA(cudaMemsetAsync(d_buckets, 0, (size_t)V * 4, s));
     if (n)
-        k_degree<<<std::min<uint64_t>(grid_for(n, 256), 4096), 256, 0, s>>>(d_src, n, V, d_buckets, d_bad);
+        k_degree<<<degree_grid(n), kDegBlock, 0, s>>>(d_src, n, V, d_buckets, d_bad);
     k_rule<<<grid_for(V, 256), 256, 0, s>>>(d_buckets, V, load_factor * (float)kSetKeys);
     int bad = 0;
     MK_CUDA(cudaMemcpyAsync(&bad, d_bad, sizeof(int), cudaMemcpyDeviceToHost, s));
