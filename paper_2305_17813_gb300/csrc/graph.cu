@@ -36,34 +36,6 @@ void device_free(mk_graph *g, void *p, size_t bytes)
     }
 }
 
-// Grows the staging buffers to hold n batch entries (keys, indices and the
-// radix-sort workspace for the widest key).
-mk_status ensure_scratch(mk_graph *g, uint64_t n, cudaStream_t s)
-{
-    if (n <= g->scratch_cap)
-        return MK_OK;
-    uint64_t cap = std::max<uint64_t>(n, 1024);
-    cap = std::max<uint64_t>(cap, g->scratch_cap + g->scratch_cap / 2);
-    uint64_t table = 1;
-    while (table < 2 * cap)
-        table <<= 1;
-    MK_CUDA(cudaStreamSynchronize(s));
-    device_free(g, g->d_tpos, g->table_size * 4);
-    device_free(g, g->d_slot, g->scratch_cap * 4);
-    device_free(g, g->d_cand, g->scratch_cap * 4);
-    device_free(g, g->d_iflags, g->scratch_cap);
-    g->d_tpos = g->d_slot = g->d_cand = nullptr;
-    g->d_iflags = nullptr;
-    g->scratch_cap = g->table_size = 0;
-    MK_TRY(device_alloc(g, (void **)&g->d_tpos, table * 4));
-    MK_TRY(device_alloc(g, (void **)&g->d_slot, cap * 4));
-    MK_TRY(device_alloc(g, (void **)&g->d_cand, cap * 4));
-    MK_TRY(device_alloc(g, (void **)&g->d_iflags, cap));
-    g->table_size = table;
-    g->scratch_cap = cap;
-    return MK_OK;
-}
-
 } // namespace mk
 
 // ------------------------------------------------------------------ kernels
@@ -367,9 +339,7 @@ __global__ void k_decode_export(const uint64_t *keys, const uint32_t *wts, uint6
 
 __global__ void k_clear_logs(DevState *st)
 {
-    st->dlog_count = 0;
     st->ulog_count = 0;
-    st->ilog_count = 0;
 }
 
 // ---------------------------------------------------------------- host API
@@ -565,10 +535,7 @@ mk_status mk_graph_destroy(mk_graph *g)
     cudaFree(v.ulog);
     cudaFree(v.owner);
     cudaFree(g->d_state);
-    cudaFree(g->d_tpos);
-    cudaFree(g->d_slot);
-    cudaFree(g->d_cand);
-    cudaFree(g->d_iflags);
+    group_release(g->group, &g->bytes);
     cudaFree(g->d_dlog);
     cudaFree(g->d_ilog);
     if (g->h_pinned)

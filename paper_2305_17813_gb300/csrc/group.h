@@ -1,0 +1,95 @@
+// Grouping of a batch's edges by slab list (group.cu), shared by the two
+// stores' inserts and deletes.
+#pragma once
+
+#include "mk_device.cuh"
+
+namespace mk {
+
+// Most edges of one list that a 4-lane group applies by itself.
+constexpr uint32_t kGroupMax = 32;
+// Marks a hash-set index in GroupView::lst (an edge of a list with more); no
+// list has it (2^31 head slabs are 275 GB).
+constexpr uint32_t kSlotBit = 0x80000000u;
+
+// What the kernels that apply a grouped batch read.  The edges of list L sit
+// at ent[slot[L].y .. + slot[L].x) as <dst, batch position>, in no order, when
+// they are at most kGroupMax; otherwise that range holds a hash set of their
+// batch positions (2 * slot[L].x words, kNil free) as k_dedup keeps one for a
+// whole batch, lst[i] of each of them is its word's index with kSlotBit, and their batch
+// positions are the ctr[kGroupMany] words at many[ctr[kGroupActive]].
+struct GroupView {
+    uint2 *slot;           // per list <edges of this batch, their offset>; the count is 0 between calls
+    const uint2 *ent;
+    const uint32_t *lst;
+    const uint32_t *many;
+    const uint32_t *alist; // lists with edges, or null when every list is to be looked at
+    const uint32_t *ctr;
+};
+enum { kGroupActive = 0, kGroupCursor = 1, kGroupMany = 2, kGroupWords = 4 };
+
+// Staging arrays of one store, grown on demand: two allocations, at ent (the
+// per-edge arrays) and at slot (the lists' counts, then ctr).
+struct GroupScratch {
+    uint64_t cap = 0;
+    uint32_t lists = 0;
+    uint32_t *lst = nullptr, *alist = nullptr, *ctr = nullptr;
+    uint8_t *rank = nullptr;
+    uint2 *ent = nullptr, *slot = nullptr;
+};
+
+// Most edges of one grouping (indexes into a hash set, two words an edge,
+// have to tell from none).
+constexpr uint64_t kGroupEdges = (1ull << 30) - 1;
+
+// Whether every list is looked at (and the ranges of the entries follow the
+// lists, so that the slabs are streamed in address order), or the lists with
+// edges are collected first.
+inline bool group_dense(uint32_t H, uint64_t n) { return n >= 4 * (uint64_t)H; }
+
+// Grows the arrays to n edges over H lists (synchronises s when it does);
+// *bytes follows what is held.  cudaErrorMemoryAllocation when it cannot.
+cudaError_t group_reserve(GroupScratch &gs, uint64_t n, uint32_t H, cudaStream_t s, uint64_t *bytes);
+void group_release(GroupScratch &gs, uint64_t *bytes);
+
+// Validates and groups n edges (w nullable, a weight of 0 is invalid) and
+// fills *gv for the kernels launched after it on s.  An invalid edge sets the
+// graph's status.  *launches counts the kernels.  The kernel that applies the
+// batch must set every active list's count back to 0.
+cudaError_t group_batch(const GView &g, GroupScratch &gs, const uint32_t *src, const uint32_t *dst, const uint32_t *w,
+                        uint64_t n, cudaStream_t s, GroupView *gv, int *launches);
+
+// Hash of a destination among the 2c words of a list's hash set.
+__device__ __forceinline__ uint32_t group_hash(uint32_t d, uint32_t words)
+{
+    return (uint32_t)(((unsigned long long)hash32(d ^ 0x85ebca6bu) * words) >> 32);
+}
+
+// Lists a 256-thread block applies at a time (one a 4-lane group).
+constexpr uint32_t kGroupLists = 64;
+
+// Entries of the group's list in its shared-memory row, and which of them
+// are the first of their destination in batch order, as a mask over entries
+// (the same on the group's four lanes).  Every lane of the warp calls it.
+__device__ __forceinline__ uint32_t group_first(const GroupView &gv, uint32_t c, uint32_t off, uint2 *row)
+{
+    const uint32_t s4 = lane_id() & 3u;
+    for (uint32_t e = s4; e < c; e += 4)
+        row[e] = __ldcs(&gv.ent[off + e]);
+    __syncwarp();
+    uint32_t first = 0;
+    for (uint32_t e = s4; e < c; e += 4) {
+        const uint2 me = row[e];
+        bool is = true;
+        for (uint32_t j = 0; j < c; ++j) {
+            const uint2 o = row[j];
+            is = is && !(o.x == me.x && o.y < me.y);
+        }
+        first |= (is ? 1u : 0u) << e;
+    }
+    first |= __shfl_xor_sync(kFull, first, 1);
+    first |= __shfl_xor_sync(kFull, first, 2);
+    return first;
+}
+
+} // namespace mk

@@ -80,9 +80,7 @@ constexpr uint32_t kSlots = 64;
 // Mutable device-side state of one graph (one allocation).
 struct DevState {
     int status;                    // sticky error word
-    uint32_t dlog_count;           // entries in the delete log
     uint32_t ulog_count;           // entries in the updated-list log
-    uint32_t ilog_count;           // entries in the inserted-edge log
     long long pool_used[kSlots];   // pool slabs allocated minus freed (kept with the bitmap), per slot
     unsigned long long ctr[kNumCounters][kSlots];
 };
@@ -208,13 +206,16 @@ __device__ __forceinline__ bool block_enqueue(T *arr, uint32_t *count, uint32_t 
 // update in the epoch, which puts L in the updated-list log: later passes
 // over the updated lists (UpdateIterator consumers, UpdateSlabPointers) read
 // the log instead of testing every list's flag.
-__device__ __forceinline__ bool flag_updated(const GView &g, uint32_t L)
+__device__ __forceinline__ bool set_updated(const GView &g, uint32_t L)
 {
-    if (*(volatile const uint8_t *)&g.lupd[L])
-        return false;
     uint32_t *word = reinterpret_cast<uint32_t *>(g.lupd + (L & ~3u));
     const uint32_t bit = 1u << ((L & 3u) * 8);
     return !(atomicOr(word, bit) & bit);
+}
+
+__device__ __forceinline__ bool flag_updated(const GView &g, uint32_t L)
+{
+    return !*(volatile const uint8_t *)&g.lupd[L] && set_updated(g, L);
 }
 
 // Adds a per-warp count to a work counter (lane 0 only; v must be

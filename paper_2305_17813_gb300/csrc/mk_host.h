@@ -3,6 +3,7 @@
 #pragma once
 
 #include "meerkat.h"
+#include "group.h"
 #include "mk_device.cuh"
 
 #include <cuda_runtime.h>
@@ -69,14 +70,7 @@ struct mk_graph {
     uint32_t vbits = 1;          // bits of a vertex id in a sort key
     mk::DevState *d_state = nullptr;
     uint64_t bytes = 0;          // device bytes held
-    // staging scratch, grown on demand: the batch's hash set of (src, dst)
-    // pairs as batch positions (table_size entries, a power of two >= 2 *
-    // scratch_cap), each edge's entry, and the updated-list nominations of
-    // an insert
-    uint64_t scratch_cap = 0;
-    uint64_t table_size = 0;
-    uint32_t *d_tpos = nullptr, *d_slot = nullptr, *d_cand = nullptr;
-    uint8_t *d_iflags = nullptr;  // an insert's per-edge stored flags when the caller asks for none
+    mk::GroupScratch group;      // staging arrays of inserts and deletes, grown on demand
     // change log of the current epoch: deleted (src << 32 | dst)
     unsigned long long *d_dlog = nullptr;
     uint64_t dlog_cap = 0, dlog_bound = 0;
@@ -189,7 +183,6 @@ inline uint32_t grid_for(uint64_t threads, uint32_t block)
     return (uint32_t)(b == 0 ? 1 : b);
 }
 
-mk_status ensure_scratch(mk_graph *g, uint64_t n, cudaStream_t s);
 int rounds_grid(int units);
 int rounds_block(int units);
 int rounds_max_blocks_per_sm();

@@ -1,4 +1,4 @@
-// mk_insert_batch_noalloc: the batched insert of update.cu with its staging
+// mk_insert_batch_noalloc: the batched insert by tiles of update.cu with its staging
 // scratch (the batch's hash set of (src, dst) pairs, each edge's entry and
 // the updated-list nominations) taken from one fixed device array declared
 // in this file instead of buffers grown with cudaMalloc.  The graph itself
@@ -28,11 +28,10 @@ __global__ void __launch_bounds__(256, 6) k_insert(GView g, const uint32_t *__re
                                                    const uint32_t *__restrict__ dst, const uint32_t *__restrict__ w_in,
                                                    uint64_t n, const uint32_t *__restrict__ tpos,
                                                    const uint32_t *__restrict__ slot, uint8_t *__restrict__ flags,
-                                                   uint32_t max_hops, uint32_t *__restrict__ cand);
-__global__ void __launch_bounds__(256) k_log_updated(GView g, const uint32_t *__restrict__ cand, uint64_t n,
-                                                     const uint8_t *__restrict__ stored, const uint32_t *__restrict__ src,
-                                                     const uint32_t *__restrict__ dst, const uint32_t *__restrict__ w,
-                                                     uint4 *ilog, uint32_t ilog_cap);
+                                                   uint32_t max_hops, uint32_t *__restrict__ cand,
+                                                   const uint32_t *order, const uint32_t *group_ctr, uint2 *lists,
+                                                   uint4 *ilog);
+__global__ void __launch_bounds__(256) k_log_updated(GView g, const uint32_t *__restrict__ cand, uint64_t n);
 
 namespace {
 
@@ -150,11 +149,12 @@ extern "C" mk_status mk_insert_batch_noalloc(mk_graph *g, const uint32_t *d_src,
                                              g->d_state);
     g->ulog_bound = std::min<uint64_t>(g->v.H, g->ulog_bound + n);
     const uint32_t max_hops = g->v.P + 2;
-    k_insert<<<grid_for(n, 256), 256, 0, s>>>(g->v, d_src, d_dst, d_w, n, tpos, slot, d_inserted, max_hops, cand);
+    k_insert<<<grid_for(n, 256), 256, 0, s>>>(g->v, d_src, d_dst, d_w, n, tpos, slot, d_inserted, max_hops, cand, nullptr,
+                                              nullptr, nullptr, nullptr);
     // no inserted-edge log (growing it could allocate): this epoch's
     // incremental prologues walk the updated lists instead
     g->ilog_ok = false;
-    k_log_updated<<<grid_for(n, 256), 256, 0, s>>>(g->v, cand, n, nullptr, nullptr, nullptr, nullptr, nullptr, 0);
+    k_log_updated<<<grid_for(n, 256), 256, 0, s>>>(g->v, cand, n);
     g->launches += 3;
     MK_CUDA(cudaGetLastError());
     return MK_OK;

@@ -546,16 +546,13 @@ __global__ void k_sssp_init(unsigned long long *D, uint32_t V, uint32_t source, 
 
 // Decremental seeds: a deleted edge (u, v) that is v's tree edge invalidates
 // v (its tree node becomes <INF, INVALID> and its bit is set in `inv`).
-__global__ void k_invalidate(const unsigned long long *dlog, const DevState *st, RoundArgs a)
+__global__ void k_invalidate(const unsigned long long *dlog, uint64_t n, RoundArgs a)
 {
-    const uint32_t n = st->dlog_count;
-    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if ((i & ~31u) >= n)
-        return;
+    const uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
     bool hit = false;
     uint32_t v = 0;
-    if (i < n) {
-        const unsigned long long e = dlog[i];
+    const unsigned long long e = i < n ? __ldcs(&dlog[i]) : ~0ull; // all-ones: nothing was removed
+    if (e != ~0ull) {
         const uint32_t u = (uint32_t)(e >> 32);
         v = (uint32_t)e;
         const unsigned long long dv = __ldcg(&a.D[v]);
@@ -866,11 +863,10 @@ __global__ void __launch_bounds__(256, 5) k_relax_updated(RoundArgs a)
 // stamps), and enqueues the lists of each vertex it lowered first in this
 // round.  Two dependent gathers per edge instead of the walk's five loads
 // per updated list (log entry, list source, marker, source node, slab).
-__global__ void __launch_bounds__(256) k_relax_inserted(RoundArgs a, const uint4 *__restrict__ ilog, uint32_t cap)
+__global__ void __launch_bounds__(256) k_relax_inserted(RoundArgs a, const uint4 *__restrict__ ilog, uint64_t n)
 {
     __shared__ BlockFrontier bq;
     bq_init(bq);
-    const uint32_t n = min(__ldg(&a.g.st->ilog_count), cap);
     const uint32_t round = __ldg(a.ctr + kRid) + 1;
     int *overflow = (int *)(a.ctr + kOverflow);
     unsigned long long entries = 0, edges = 0, improved = 0;
@@ -883,11 +879,11 @@ __global__ void __launch_bounds__(256) k_relax_inserted(RoundArgs a, const uint4
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             const uint64_t i = wb + lane4 + k;
-            const uint4 e = i < n ? __ldcs(&ilog[i]) : make_uint4(0, 0, 0, 0);
+            const uint4 e = i < n ? __ldcs(&ilog[i]) : make_uint4(kNil, 0, 0, 0); // kNil: nothing was stored
             x[k] = e.x;
             y[k] = e.y;
             nd[k] = e.z;
-            up[k] = i < n;
+            up[k] = e.x != kNil;
         }
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
@@ -1396,7 +1392,7 @@ mk_status run_sssp(mk_graph *g, int kind, uint32_t source, uint32_t *d_dist, uin
             MK_CUDA(cudaMemsetAsync(c->inv, 0, (size_t)(V + 31) / 32 * 4, s));
             MK_TRY(timed(g, "sssp_invalidate", s, 1, [&]() {
                 k_invalidate<<<grid_for(std::max<uint64_t>(g->dlog_bound, 1), 256), 256, 0, s>>>(g->d_dlog,
-                                                                                                 g->d_state, a);
+                                                                                                 g->dlog_bound, a);
                 return cudaSuccess;
             }));
             MK_TRY(timed(g, "sssp_invalidate_walk", s, 1, [&]() {
@@ -1421,7 +1417,7 @@ mk_status run_sssp(mk_graph *g, int kind, uint32_t source, uint32_t *d_dist, uin
             MK_TRY(timed(g, "sssp_relax_updated", s, 1, [&]() {
                 const uint64_t threads = (g->ilog_bound + 3) / 4;
                 k_relax_inserted<<<std::min<uint32_t>(grid_for(threads, 256), num_sms() * 8), 256, 0, s>>>(
-                    a, g->d_ilog, (uint32_t)g->ilog_cap);
+                    a, g->d_ilog, g->ilog_bound);
                 return cudaSuccess;
             }));
         } else if (g->ulog_bound) {
@@ -1495,7 +1491,7 @@ mk_status run_multi(mk_graph *g, const mk_algo_req *reqs, uint32_t n, cudaStream
         const RoundArgs &a = dec.c[j];
         MK_CUDA(cudaMemsetAsync(a.inv, 0, (size_t)(V + 31) / 32 * 4, s));
         MK_TRY(timed(g, "sssp_invalidate", s, 1, [&]() {
-            k_invalidate<<<grid_for(std::max<uint64_t>(g->dlog_bound, 1), 256), 256, 0, s>>>(g->d_dlog, g->d_state,
+            k_invalidate<<<grid_for(std::max<uint64_t>(g->dlog_bound, 1), 256), 256, 0, s>>>(g->d_dlog, g->dlog_bound,
                                                                                              a);
             return cudaSuccess;
         }));

@@ -1,0 +1,128 @@
+"""Batches grouped by slab list, against the oracle: lists with just as many
+edges of a batch as one 4-lane group applies (32), one fewer, one more and many
+more; tails with room for some of them; repeats of a pair (the first one's
+weight is stored); sparse and dense batches of one graph (fewer and more edges
+than half its lists).  Everything is a whole number and has to be equal."""
+import numpy as np
+import pytest
+
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+PER_LIST = [1, 14, 15, 16, 30, 31, 32, 33, 47, 64, 200]
+
+
+def _pairs(rng, V, per_list, repeat):
+    """`n` edges of vertex 3 k for the k-th n of per_list, `repeat` of them again, shuffled."""
+    src, dst = [], []
+    for k, n in enumerate(per_list):
+        d = rng.choice(V, n - min(repeat, n - 1), replace=False)
+        d = np.concatenate([d, rng.choice(d, n - len(d))])
+        src.append(np.full(n, 3 * k))
+        dst.append(d)
+    src, dst = np.concatenate(src), np.concatenate(dst)
+    p = rng.permutation(len(src))
+    return src[p].astype(np.uint32), dst[p].astype(np.uint32)
+
+
+@pytest.mark.parametrize("store", ["map", "set"])
+@pytest.mark.parametrize("repeat", [0, 3])
+@pytest.mark.parametrize("V", [300, 5000])  # dense, sparse
+@pytest.mark.parametrize("per_list", [PER_LIST, [n for n in PER_LIST if n <= 32]])
+def test_edges_per_list(cuda_lib, store, repeat, V, per_list):
+    import paper_2305_17813_gb300 as mk
+
+    rng = np.random.default_rng(len(per_list) * 10 + repeat + V)
+    make = mk.Graph if store == "map" else mk.SetGraph
+    g, o = make(V, edge_capacity_hint=1 << 14, buckets=1), oracle.OracleGraph(V)
+    live = []
+    for step in range(4):
+        s, d = _pairs(rng, V, per_list, repeat)
+        w = rng.integers(1, 1000, len(s)).astype(np.uint32)
+        f = g.insert(s, d, w) if store == "map" else g.insert(s, d)
+        assert np.array_equal(f.cpu().numpy(), o.insert(s, d, w))
+        live.append((s, d))
+        s, d = live[rng.integers(len(live))]
+        take = rng.permutation(np.arange(len(s)).repeat(1 + (repeat > 0)))[: len(s)]
+        f = g.delete(s[take], d[take])
+        assert np.array_equal(f.cpu().numpy(), o.delete(s[take], d[take]))
+        s, d = (np.concatenate(x) for x in zip(*live))
+        q, ow = o.query(s, d)
+        if store == "map":
+            bm, gw = g.query(s, d)
+            assert np.array_equal(mk.to_numpy_u32(gw), ow)
+            for a, b in zip(g.export(), o.export()):
+                assert np.array_equal(mk.to_numpy_u32(a), b)
+        else:
+            bm = g.query(s, d)
+        assert np.array_equal(mk.to_numpy_u32(bm), q)
+    if store == "map":
+        assert g.last_error() == mk.MK_OK
+        dist, par = g.sssp(0)
+        od, op = o.sssp(0)
+        assert np.array_equal(mk.to_numpy_u32(dist), od) and np.array_equal(mk.to_numpy_u32(par), op)
+    g.close()
+
+
+def test_rejected_batch_leaves_the_grouping_clean(cuda_lib):
+    """A batch with an invalid id changes nothing, and the batches after it
+    find every list's count at zero again."""
+    import paper_2305_17813_gb300 as mk
+
+    rng = np.random.default_rng(5)
+    V = 400
+    g, o = mk.Graph(V, edge_capacity_hint=1 << 13, buckets=2), oracle.OracleGraph(V)
+    for n in (40, 700):
+        s, d = (rng.integers(0, V, n).astype(np.uint32) for _ in range(2))
+        bad = d.copy()
+        bad[n // 2] = V
+        assert not g.insert(s, bad).any()
+        assert g.last_error() == mk.MK_ERR_INVALID_ARG
+        w = rng.integers(1, 50, n).astype(np.uint32)
+        assert np.array_equal(g.insert(s, d, w).cpu().numpy(), o.insert(s, d, w))
+        assert np.array_equal(g.delete(s[:9], d[:9]).cpu().numpy(), o.delete(s[:9], d[:9]))
+        assert g.last_error() == mk.MK_OK
+    for a, b in zip(g.export(), o.export()):
+        assert np.array_equal(mk.to_numpy_u32(a), b)
+    g.close()
+
+
+def test_states_made_between_unlogged_and_logged_inserts(cuda_lib):
+    """An insert is logged for the states that are current when it runs:
+    states first computed in the middle of an epoch, after inserts that nobody
+    logged, follow the later ones."""
+    import paper_2305_17813_gb300 as mk
+
+    rng = np.random.default_rng(6)
+    V = 500
+    g, o = mk.Graph(V, edge_capacity_hint=1 << 14, buckets=2), oracle.OracleGraph(V)
+
+    def insert(n):
+        s, d = (rng.integers(0, V, n).astype(np.uint32) for _ in range(2))
+        w = rng.integers(1, 50, n).astype(np.uint32)
+        assert np.array_equal(g.insert(s, d, w).cpu().numpy(), o.insert(s, d, w))
+
+    def same(source):
+        for (a, b), (x, y) in ((g.sssp(source), o.sssp(source)), (g.bfs(source), o.bfs(source))):
+            assert np.array_equal(mk.to_numpy_u32(a), x) and np.array_equal(mk.to_numpy_u32(b), y)
+        assert np.array_equal(mk.to_numpy_u32(g.wcc()), o.wcc())
+
+    insert(300)            # no state yet: not logged
+    same(0)                # from scratch
+    same(0)                # nothing new
+    insert(300)            # logged
+    same(0)
+    insert(300)
+    same(1)                # a second source joins in the middle of the epoch
+    same(0)
+    g.commit()
+    insert(300)
+    same(0)
+    g.commit()
+    insert(300)            # an epoch that no state follows
+    g.commit()
+    insert(300)            # no state is current: not logged
+    same(0)
+    assert g.last_error() == mk.MK_OK
+    g.close()
