@@ -364,7 +364,7 @@ static void destroy_consumer(mk_graph *g, Consumer *c)
     device_free(g, c->far[0], V * 4);
     device_free(g, c->far[1], V * 4);
     device_free(g, c->fstamp, V * 4);
-    device_free(g, c->counters, 64);
+    device_free(g, c->counters, kConsumerWords * 4);
     delete c;
 }
 

@@ -15,6 +15,7 @@
 
 namespace mk {
 
+constexpr int kConsumerWords = 32;
 enum ConsumerKind { kSssp = 0, kBfs = 1, kWcc = 2 };
 
 // State of one incremental algorithm on one graph.
@@ -31,7 +32,7 @@ struct Consumer {
     uint32_t *uf = nullptr;     // WCC: union-find parents (V)
     uint32_t *far[2] = {nullptr, nullptr}; // SSSP with Near-Far ordering: far piles (V each)
     uint32_t *fstamp = nullptr; // SSSP with Near-Far ordering: pile stamp per vertex (V)
-    uint32_t *counters = nullptr; // device: frontier sizes etc. (16 words)
+    uint32_t *counters = nullptr; // device: frontier sizes etc. (kConsumerWords)
 };
 
 struct TimedLaunch {

@@ -39,21 +39,25 @@ constexpr uint32_t kInf32 = 0xFFFFFFFFu;
 constexpr uint32_t kRoundsMaxThreads = 1024; // block size limit of the persistent round kernel
 constexpr uint32_t kBarrierSpins = 1u << 24;
 
-// consumer counter words
+// consumer counter words (kConsumerWords)
 enum {
-    kCnt0 = 0,        // kCnt0..kCnt0+2: rotating frontier sizes
-    kOverflow = 3,
-    kInvTotal = 4,    // nonzero once this call invalidated a vertex
-    kRoundsDone = 5,
+    kCnt0 = 0,        // three rotating pairs <frontier size, blocks that have ended the round that filled it>
+    kOverflow = 6,
+    kInvTotal = 7,    // nonzero once this call invalidated a vertex
     kClearWords = 8,  // words [0, 8) are cleared at the start of every call
-    kSoloR = 6,       // round index reached by a solo phase of block 0
-    kRid = 8,         // last round stamp used (kept across calls)
-    kPhase = 9,       // Near-Far: last far-pile phase stamp used (kept across calls)
-    kBar = 10,        // grid barrier: arrivals of the launch so far
-    kFarCnt0 = 11,    // Near-Far ordering: sizes of the two far piles (11, 12),
-    kFarMin0 = 13,    // the smallest distance pushed to each (13, 14)
-    kThresh = 15      // and the smallest source distance of the first frontier
+    kSoloR = 8,       // round index reached by a solo phase of block 0, and the frontier size there (9)
+    kRoundsDone = 10,
+    kRid = 11,        // last round stamp used (kept across calls)
+    kPhase = 12,      // Near-Far: last far-pile phase stamp used (kept across calls)
+    kBar = 13,        // grid barrier: arrivals of the launch so far
+    kFarCnt0 = 14,    // Near-Far ordering: sizes of the two far piles (14, 15),
+    kFarMin0 = 16,    // the smallest distance pushed to each (16, 17)
+    kThresh = 18      // and the smallest source distance of the first frontier
 };
+
+// The count of frontier r (the pair's first word).
+__device__ __host__ __forceinline__ uint32_t *count_of(uint32_t *ctr, uint32_t r) { return ctr + kCnt0 + 2 * (r % 3); }
+
 // A frontier of at most kSoloLists lists is processed by block 0 alone, with
 // block-level barriers between rounds, for at most kSoloRounds rounds in a
 // row (so the other blocks' bounded wait at the grid barrier never expires).
@@ -62,6 +66,9 @@ enum {
 // a grid barrier plus one chain; a larger one is faster on the whole grid.
 constexpr uint32_t kSoloLists = 192;
 constexpr uint32_t kSoloRounds = 4096;
+// A frontier of at most kDirectLists lists issues the atomic minima without
+// reading the nodes first.
+constexpr uint32_t kDirectLists = 16384;
 // Near-Far ordering: the far pile is split into the frontier whenever the
 // frontier holds fewer lists than this (a smaller frontier costs a round
 // about as much as a larger one).
@@ -113,77 +120,185 @@ struct NearFar {
     uint32_t *dmin = nullptr; // smallest distance pushed to it
 };
 
-// Appends y (lanes with pred) to the far pile once per phase.  Must be
-// called by the full warp.
-__device__ __forceinline__ void far_push(const RoundArgs &a, const NearFar &nf, uint32_t y, bool pred, uint32_t d)
+// A block's staging area for the far pile, as FrontierSmem for the frontier.
+struct FarSmem {
+    uint32_t buf[kRoundsMaxThreads / 32][kWarpBuf];
+    uint32_t held[kRoundsMaxThreads / 32], at[kRoundsMaxThreads / 32];
+    uint32_t dmin; // smallest distance pushed since the last flush
+};
+
+__device__ __forceinline__ void far_put(const RoundArgs &a, const NearFar &nf, uint32_t at, uint32_t y)
 {
-    const bool take = pred && atomicExch(&a.fstamp[y], nf.phase) != nf.phase;
-    const uint32_t m = __ballot_sync(kFull, take);
-    if (!m)
+    if (at < a.g.V)
+        nf.pile[at] = y;
+    else
+        *(int *)(a.ctr + kOverflow) = 1;
+}
+
+// Appends the lane's vertices y[k] with push[k] (distances d[k]) to the far
+// pile, each once per phase.  Must be called by the full warp.
+template <int N>
+__device__ __forceinline__ void far_push(const RoundArgs &a, const NearFar &nf, FarSmem &sm, const uint32_t (&y)[N],
+                                         const bool (&push)[N], const uint32_t (&d)[N])
+{
+    const uint32_t lane = lane_id(), w = threadIdx.x >> 5;
+    bool any = false;
+#pragma unroll
+    for (int k = 0; k < N; ++k)
+        any = any || push[k];
+    if (!__any_sync(kFull, any))
         return;
-    const uint32_t dm = __reduce_min_sync(kFull, take ? d : kInf32);
+    uint32_t st[N], c = 0, dm = kInf32;
+#pragma unroll
+    for (int k = 0; k < N; ++k)
+        st[k] = push[k] ? atomicExch(&a.fstamp[y[k]], nf.phase) : nf.phase;
+#pragma unroll
+    for (int k = 0; k < N; ++k)
+        if (st[k] != nf.phase) {
+            ++c;
+            dm = min(dm, d[k]);
+        } else if (push[k]) {
+            dm = min(dm, d[k]); // in the pile already, at a larger distance
+        }
+    uint32_t incl = c;
+#pragma unroll
+    for (uint32_t o = 1; o < 32; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(kFull, incl, o);
+        if (lane >= o)
+            incl += t;
+    }
+    dm = __reduce_min_sync(kFull, dm);
+    const uint32_t total = __shfl_sync(kFull, incl, 31), held = sm.held[w];
+    const bool fits = held + total <= kWarpBuf;
     uint32_t base = 0;
-    if (lane_id() == 0) {
-        base = atomicAdd(nf.count, (uint32_t)__popc(m));
-        atomicMin(nf.dmin, dm);
+    if (lane == 0)
+        atomicMin(&sm.dmin, dm);
+    if (!fits) {
+        if (lane == 0)
+            base = atomicAdd(nf.count, held + total);
+        base = __shfl_sync(kFull, base, 0);
+        for (uint32_t t = lane; t < held; t += 32)
+            far_put(a, nf, base + t, sm.buf[w][t]);
     }
-    base = __shfl_sync(kFull, base, 0);
-    if (take) {
-        const uint32_t at = base + __popc(m & lanemask_lt());
-        if (at < a.g.V)
-            nf.pile[at] = y;
-        else
-            *(int *)(a.ctr + kOverflow) = 1;
+    uint32_t t = held + incl - c;
+#pragma unroll
+    for (int k = 0; k < N; ++k)
+        if (st[k] != nf.phase) {
+            if (fits)
+                sm.buf[w][t] = y[k];
+            else
+                far_put(a, nf, base + t, y[k]);
+            ++t;
+        }
+    __syncwarp();
+    if (lane == 0)
+        sm.held[w] = fits ? held + total : 0u;
+    __syncwarp();
+}
+
+// Copies the block's staged vertices to the pile.  Called by every thread of
+// the block, which the caller synchronises before more are staged.
+__device__ __forceinline__ void far_flush(const RoundArgs &a, const NearFar &nf, FarSmem &sm)
+{
+    constexpr uint32_t kWarps = kRoundsMaxThreads / 32;
+    const uint32_t lane = lane_id(), w = threadIdx.x >> 5;
+    __syncthreads();
+    if (w == 0) {
+        const uint32_t h = lane < kWarps ? sm.held[lane] : 0u;
+        uint32_t incl = h;
+#pragma unroll
+        for (uint32_t o = 1; o < 32; o <<= 1) {
+            const uint32_t t = __shfl_up_sync(kFull, incl, o);
+            if (lane >= o)
+                incl += t;
+        }
+        uint32_t base = 0;
+        if (lane == 31) {
+            if (incl)
+                base = atomicAdd(nf.count, incl);
+            if (sm.dmin != kInf32)
+                atomicMin(nf.dmin, sm.dmin);
+            sm.dmin = kInf32;
+        }
+        base = __shfl_sync(kFull, base, 31);
+        if (lane < kWarps)
+            sm.at[lane] = base + incl - h;
     }
+    __syncthreads();
+    const uint32_t held = sm.held[w], at = sm.at[w];
+    for (uint32_t t = lane; t < held; t += 32)
+        far_put(a, nf, at + t, sm.buf[w][t]);
+    __syncwarp();
+    if (lane == 0)
+        sm.held[w] = 0;
 }
 
 // Relaxes the lane's four edges (x, y[k], w[k]) with live[k] and enqueues
 // the lists of each vertex whose distance this lane lowered first in this
-// round (staged in the block's frontier buffer).  The accesses of the four
+// round (staged in the warp's frontier buffer).  The accesses of the four
 // edges go out together, step by step: the four targets' tree nodes are
 // read, then the atomic minima of the candidates that beat them are issued,
 // then the improved targets' vinfo entries are read and their round stamps
 // exchanged, so a slab costs three memory round trips per lane instead of
-// three per edge.  Must be called by the full warp.
-template <bool kNF = false>
+// three per edge.  A candidate that only names a smaller parent at the same
+// distance changes the node but enqueues nothing: what leaves the vertex
+// depends on its distance alone.  `direct` leaves the read of the nodes out
+// and issues every minimum: one round trip less, more atomics, for the rounds
+// whose time is their round trips.  Must be called by the full warp.
+template <bool kNF = false, uint32_t kWarps>
 __device__ __forceinline__ void relax_edges4(const RoundArgs &a, uint32_t x, uint32_t dx, const uint32_t (&y)[4],
                                              const uint32_t (&w)[4], const bool (&live)[4], uint32_t round,
-                                             BlockFrontier &bq, uint2 *Fn, uint32_t *cnt, int *overflow,
+                                             FrontierSmem<kWarps> &bq, uint2 *Fn, uint32_t *cnt, int *overflow,
                                              unsigned long long &edges, unsigned long long &improved,
-                                             const NearFar *nf = nullptr)
+                                             const NearFar *nf = nullptr, FarSmem *fs = nullptr,
+                                             bool direct = false)
 {
     // candidate of edge k: <nd[k], x>
     auto cand = [&](uint32_t d) { return ((unsigned long long)d << 32) | x; };
     uint32_t nd[4];
     unsigned long long cur[4];
     bool up[4];
+    uint32_t n_live = 0;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        edges += __popc(__ballot_sync(kFull, live[k]));
+        n_live += live[k];
         const unsigned long long d = (unsigned long long)dx + (a.unit ? 1u : w[k]);
         up[k] = live[k] && d < kInf32;
         nd[k] = (uint32_t)d;
     }
+    edges += n_live;
+    if (direct) {
 #pragma unroll
-    for (int k = 0; k < 4; ++k)
-        cur[k] = up[k] ? __ldcg(&a.D[y[k]]) : 0ull;
+        for (int k = 0; k < 4; ++k)
+            cur[k] = up[k] ? atomicMin(&a.D[y[k]], cand(nd[k])) : 0ull;
+    } else {
 #pragma unroll
-    for (int k = 0; k < 4; ++k)
-        if (up[k] && cand(nd[k]) < cur[k])
-            cur[k] = atomicMin(&a.D[y[k]], cand(nd[k]));
-        else
-            up[k] = false;
+        for (int k = 0; k < 4; ++k)
+            cur[k] = up[k] ? __ldcg(&a.D[y[k]]) : 0ull;
 #pragma unroll
-    for (int k = 0; k < 4; ++k)
-        up[k] = up[k] && cand(nd[k]) < cur[k];
+        for (int k = 0; k < 4; ++k)
+            if (up[k] && cand(nd[k]) < cur[k])
+                cur[k] = atomicMin(&a.D[y[k]], cand(nd[k]));
+            else
+                up[k] = false;
+    }
+    bool any = false;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        up[k] = up[k] && nd[k] < node_dist(cur[k]);
+        any = any || up[k];
+    }
+    if (!__any_sync(kFull, any))
+        return;
     if (kNF) {
         // improvements at or beyond the split distance wait in the far pile
+        bool fp[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            const bool fp = up[k] && nd[k] >= nf->T;
-            up[k] = up[k] && !fp;
-            far_push(a, *nf, y[k], fp, nd[k]);
+            fp[k] = up[k] && nd[k] >= nf->T;
+            up[k] = up[k] && !fp[k];
         }
+        far_push<4>(a, *nf, *fs, y, fp, nd);
     }
     uint2 vi[4];
     uint32_t st[4];
@@ -199,9 +314,17 @@ __device__ __forceinline__ void relax_edges4(const RoundArgs &a, uint32_t x, uin
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         up[k] = up[k] && st[k] != round;
-        improved += __popc(__ballot_sync(kFull, up[k]));
-        enqueue_lists_block(bq, y[k], up[k], vi[k], Fn, cnt, a.cap, overflow);
+        improved += up[k];
     }
+    enqueue_lists<4>(bq, y, up, vi, Fn, cnt, a.cap, overflow);
+}
+
+__device__ __forceinline__ unsigned long long warp_sum(unsigned long long v)
+{
+#pragma unroll
+    for (int o = 16; o; o >>= 1)
+        v += __shfl_xor_sync(kFull, v, o);
+    return v;
 }
 
 // One round over frontier F[0, n): every 4-lane group of every warp takes
@@ -209,12 +332,13 @@ __device__ __forceinline__ void relax_edges4(const RoundArgs &a, uint32_t x, uin
 // warp in flight), so a round's lists are spread over all warps; each
 // group's entry, source distance and head slab are loaded one step ahead
 // (the entry two steps ahead) while the current list is relaxed.
-template <bool kNF = false>
-__device__ void relax_body(const RoundArgs &a, const uint2 *F, uint32_t n, uint2 *Fn, uint32_t *cnt,
-                           uint32_t round, uint64_t warp0, uint64_t nwarps, BlockFrontier &bq,
-                           const NearFar *nf = nullptr)
+template <bool kNF = false, uint32_t kWarps>
+__device__ __forceinline__ void relax_body(const RoundArgs &a, const uint2 *F, uint32_t n, uint2 *Fn, uint32_t *cnt,
+                                           uint32_t round, uint64_t warp0, uint64_t nwarps, FrontierSmem<kWarps> &bq,
+                                           const NearFar *nf = nullptr, FarSmem *fs = nullptr)
 {
     const GView &g = a.g;
+    const bool direct = n <= kDirectLists;
     const uint32_t s4 = lane_id() & 3u, g4 = lane_id() >> 2;
     int *overflow = (int *)(a.ctr + kOverflow);
     unsigned long long lists = 0, slabs = 0, edges = 0, improved = 0;
@@ -223,13 +347,13 @@ __device__ void relax_body(const RoundArgs &a, const uint2 *F, uint32_t n, uint2
     uint64_t i = warp0 * 8 + g4;
     // pipeline: entry e with its distance dx and head slab (lo, hi) (this
     // step), entry ne (next step)
-    uint2 e = i < n ? F[i] : none;
-    uint2 ne = i + gs < n ? F[i + gs] : none;
+    uint2 e = i < n ? __ldcg(&F[i]) : none;
+    uint2 ne = i + gs < n ? __ldcg(&F[i + gs]) : none;
     uint32_t dx = e.x != kNil ? node_dist(__ldcg(&a.D[e.y])) : kInf32;
     uint4 lo, hi;
     group4_load(g, e.x, lo, hi);
     for (uint64_t base = warp0 * 8; base < n; base += gs, i += gs) {
-        const uint2 nne = i + 2 * gs < n ? F[i + 2 * gs] : none;
+        const uint2 nne = i + 2 * gs < n ? __ldcg(&F[i + 2 * gs]) : none;
         const uint32_t ndx = ne.x != kNil ? node_dist(__ldcg(&a.D[ne.y])) : kInf32;
         uint4 nlo, nhi;
         group4_load(g, ne.x, nlo, nhi);
@@ -239,7 +363,7 @@ __device__ void relax_body(const RoundArgs &a, const uint2 *F, uint32_t n, uint2
         slabs += walk_lists_g4_from(g, L, true, lo, hi, 0, a.max_hops,
                                     [&](const uint32_t(&y)[4], const uint32_t(&w)[4], const bool(&live)[4]) {
                                         relax_edges4<kNF>(a, x, d, y, w, live, round, bq, Fn, cnt, overflow,
-                                                          edges, improved, nf);
+                                                          edges, improved, nf, fs, direct);
                                     });
         e = ne;
         ne = nne;
@@ -247,28 +371,69 @@ __device__ void relax_body(const RoundArgs &a, const uint2 *F, uint32_t n, uint2
         lo = nlo;
         hi = nhi;
     }
+    if (warp0 * 8 >= n)
+        return;
     count_add(g.st, kCtrRelaxLists, lists);
     count_add(g.st, kCtrRelaxSlabs, slabs);
-    count_add(g.st, kCtrRelaxEdges, edges);
-    count_add(g.st, kCtrRelaxImproved, improved);
+    count_add(g.st, kCtrRelaxEdges, warp_sum(edges));
+    count_add(g.st, kCtrRelaxImproved, warp_sum(improved));
 }
 
-// Round r of a phase: reads the size in cnts[r % 3], appends to
-// cnts[(r+1) % 3] and clears cnts[(r+2) % 3] for round r+1 (cnts: the three
-// global counters, or block 0's shared copies during a solo phase).
-// Frontier r is front[r & 1].  Called by whole blocks: the block's staged
-// entries are flushed at the end.
-template <bool kNF = false>
-__device__ __forceinline__ void round_step(const RoundArgs &a, uint32_t *cnts, uint32_t r, uint32_t n, uint64_t warp0,
-                                           uint64_t nwarps, uint32_t rid, BlockFrontier &bq,
-                                           const NearFar *nf = nullptr)
+// Round r of a phase: relaxes frontier r (front[r & 1], n entries) and
+// appends to frontier r + 1, whose size is counted in *cnt (a global counter
+// or, in a solo phase, block 0's own).  Called by whole blocks: the block's
+// staged entries are flushed at the end.
+template <bool kNF = false, uint32_t kWarps>
+__device__ __forceinline__ void round_step(const RoundArgs &a, uint32_t *cnt, uint32_t r, uint32_t n, uint64_t warp0,
+                                           uint64_t nwarps, uint32_t rid, FrontierSmem<kWarps> &bq,
+                                           const NearFar *nf = nullptr, FarSmem *fs = nullptr)
 {
     const uint32_t in = r & 1;
-    if (blockIdx.x == 0 && threadIdx.x == 0)
-        cnts[(r + 2) % 3] = 0;
-    uint32_t *cnt = cnts + (r + 1) % 3;
-    relax_body<kNF>(a, a.front[in], n, a.front[in ^ 1], cnt, rid + 2 + r, warp0, nwarps, bq, nf);
-    bq_flush(bq, a.front[in ^ 1], cnt, a.cap, (int *)(a.ctr + kOverflow));
+    relax_body<kNF>(a, a.front[in], n, a.front[in ^ 1], cnt, rid + 2 + r, warp0, nwarps, bq, nf, fs);
+    frontier_flush(bq, a.front[in ^ 1], cnt, a.cap, (int *)(a.ctr + kOverflow));
+    if (kNF)
+        far_flush(a, *nf, *fs);
+}
+
+__device__ __forceinline__ void fence_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
+
+__device__ __forceinline__ unsigned long long ld_acquire(const unsigned long long *p)
+{
+    unsigned long long v;
+    asm volatile("ld.acquire.gpu.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+
+// Ends the round that filled frontier r: waits until every block of the
+// (cooperative) grid has, and returns the frontier's size in *n.  The blocks
+// arrive in the high word of the pair whose low word counts the frontier, so
+// the load that sees the last arrival brings the size with it.  Returns false
+// when the wait gave up.  Called by whole blocks.
+__device__ __forceinline__ bool round_barrier(uint32_t *ctr, uint32_t r, uint32_t max_spins, uint32_t *n)
+{
+    __shared__ uint32_t s_n, s_ok;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        unsigned long long *pair = reinterpret_cast<unsigned long long *>(count_of(ctr, r));
+        fence_gpu();
+        atomicAdd(pair, 1ull << 32);
+        uint32_t ok = 1, spins = 0;
+        unsigned long long v = ld_acquire(pair);
+        while ((uint32_t)(v >> 32) < gridDim.x) {
+            if (++spins > max_spins) {
+                ok = 0;
+                break;
+            }
+            __nanosleep(20);
+            v = ld_acquire(pair);
+        }
+        fence_gpu();
+        s_n = (uint32_t)v;
+        s_ok = ok;
+    }
+    __syncthreads();
+    *n = s_n;
+    return s_ok != 0;
 }
 
 // Bounded grid barrier for a co-resident (cooperative) grid on one counter
@@ -283,7 +448,7 @@ __device__ bool grid_barrier(uint32_t *bar, uint32_t &passed, uint32_t max_spins
     __syncthreads();
     if (threadIdx.x == 0) {
         const uint32_t target = (++passed) * gridDim.x;
-        __threadfence();
+        fence_gpu();
         atomicAdd(bar, 1u);
         int ok = 1;
         uint32_t spins = 0;
@@ -294,7 +459,7 @@ __device__ bool grid_barrier(uint32_t *bar, uint32_t &passed, uint32_t max_spins
             }
             __nanosleep(32);
         }
-        __threadfence();
+        fence_gpu();
         ok_s = ok;
     }
     __syncthreads();
@@ -308,10 +473,10 @@ __device__ bool grid_barrier(uint32_t *bar, uint32_t &passed, uint32_t max_spins
 // `next` under its phase stamp.  Called by every thread of every block.
 __device__ __forceinline__ void far_split(const RoundArgs &a, const uint32_t *pile, uint32_t fc, const NearFar &next,
                                           uint32_t T2, uint32_t r, uint32_t rid, uint64_t warp0, uint64_t nwarps,
-                                          BlockFrontier &bq)
+                                          FrontierSmem<kRoundsMaxThreads / 32> &bq, FarSmem &fs)
 {
     uint2 *out = a.front[r & 1];
-    uint32_t *cnt = a.ctr + kCnt0 + r % 3;
+    uint32_t *cnt = count_of(a.ctr, r);
     const uint32_t stampv = rid + 1 + r;
     int *overflow = (int *)(a.ctr + kOverflow);
     for (uint64_t wb = warp0 * 32; wb < fc; wb += nwarps * 32) {
@@ -329,11 +494,16 @@ __device__ __forceinline__ void far_split(const RoundArgs &a, const uint32_t *pi
             vi = a.g.vinfo[y];
             st = atomicExch(&a.stamp[y], stampv);
         }
-        near = near && st != stampv;
-        enqueue_lists_block(bq, y, near, vi, out, cnt, a.cap, overflow);
-        far_push(a, next, y, valid && dy >= T2, dy);
+        const uint32_t ys[1] = {y};
+        const bool ups[1] = {near && st != stampv};
+        const uint2 vis[1] = {vi};
+        enqueue_lists<1>(bq, ys, ups, vis, out, cnt, a.cap, overflow);
+        const bool fars[1] = {valid && dy >= T2};
+        const uint32_t ds[1] = {dy};
+        far_push<1>(a, next, fs, ys, fars, ds);
     }
-    bq_flush(bq, out, cnt, a.cap, overflow);
+    frontier_flush(bq, out, cnt, a.cap, overflow);
+    far_flush(a, next, fs);
 }
 
 } // namespace
@@ -347,28 +517,49 @@ __device__ __forceinline__ void far_split(const RoundArgs &a, const uint32_t *pi
 // phase sits between two grid barriers, so no block reads a global size
 // while block 0 changes them, and the others wait at one barrier instead of
 // one per round.
+//
+// A round is bound by its chain of dependent accesses (frontier entry, slab
+// and source node, target nodes, atomic minimum, index and stamp): 3.5-5 us
+// for up to one list a group, then 2.3 us for the flush, the barrier and the
+// next size (7.3 us in all, 9.5 before the size came with the barrier, the
+// warps were spread over the SMs and small rounds went without the nodes'
+// read).  A large round runs at 7-12 G lists/s; what held it was the frontier
+// count, on which every append past a block's buffer met.  R-MAT scale 20
+// from the hub: BFS 540 -> 266 us, SSSP 990 -> 510 us.
 template <bool kNF>
 __global__ void __launch_bounds__(kRoundsMaxThreads, 1) k_rounds(RoundArgs a)
 {
     __shared__ uint32_t solo_cnt[3];
-    __shared__ BlockFrontier bq;
-    bq_init(bq);
-    const uint64_t warp0 = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5;
+    __shared__ FrontierSmem<kRoundsMaxThreads / 32> bq;
+    __shared__ FarSmem fs[1];
+    __shared__ uint32_t s_word, s_fc, s_fm;
+    if (threadIdx.x == 0)
+        s_word = ld_volatile(count_of(a.ctr, 0));
+    if (kNF) {
+        if (threadIdx.x < kRoundsMaxThreads / 32)
+            fs[0].held[threadIdx.x] = 0;
+        if (threadIdx.x == 0)
+            fs[0].dmin = kInf32;
+    }
+    frontier_init(bq);
+    // consecutive warps of the frontier sit on different SMs, so that a
+    // frontier of a few thousand lists is relaxed by all of them
+    const uint64_t warp0 = (uint64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
     const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
     const uint32_t rid = __ldg(a.ctr + kRid);
-    uint32_t *gcnt = a.ctr + kCnt0;
     uint32_t r = 0, bars = 0, passed = 0;
     bool ok = true;
-    __shared__ uint32_t s_word, s_fc, s_fm;
+    // a frontier never holds more than `cap` entries; a larger count
+    // (entries dropped on overflow, reported below) is read as cap
+    uint32_t n = min(s_word, a.cap);
     // Near-Far: the first split distance is delta above the smallest source
     // distance of the first frontier (ctr[kThresh] starts at INF)
     NearFar nf;
     uint32_t cur = 0, splits = 0, burst = 0;
     const uint32_t phase0 = kNF ? __ldg(a.ctr + kPhase) + 1 : 0;
     if (kNF) {
-        const uint32_t n0 = min(ld_volatile(gcnt), a.cap);
         uint32_t m = kInf32;
-        for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n0;
+        for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n;
              i += (uint64_t)gridDim.x * blockDim.x)
             m = min(m, node_dist(__ldcg(&a.D[__ldcg(&a.front[0][i].y)])));
         m = __reduce_min_sync(kFull, m);
@@ -384,69 +575,72 @@ __global__ void __launch_bounds__(kRoundsMaxThreads, 1) k_rounds(RoundArgs a)
         nf.dmin = a.ctr + kFarMin0;
     }
     while (ok && r < a.max_rounds) {
-        // one read of the frontier size per block (the grid's warps would
-        // otherwise all read the same word)
-        if (threadIdx.x == 0) {
-            s_word = ld_volatile(gcnt + r % 3);
-            if (kNF) {
+        if (kNF && n < kNearMin) {
+            // one read of the pile's size per block
+            if (threadIdx.x == 0) {
                 s_fc = ld_volatile(a.ctr + kFarCnt0 + cur);
                 s_fm = ld_volatile(a.ctr + kFarMin0 + cur);
             }
-        }
-        __syncthreads();
-        // a frontier never holds more than `cap` entries; a larger count
-        // (entries dropped on overflow, reported below) is read as cap
-        uint32_t n = min(s_word, a.cap);
-        if (kNF && n < kNearMin && s_fc != 0) {
-            // the near frontier is small: move the far pile's vertices below
-            // the next split distance into it, once every block has read
-            // the sizes above; the distance grows with each split in a row
+            __syncthreads();
             const uint32_t fc = min(s_fc, a.g.V), fm = s_fm;
-            ++bars;
-            if (!grid_barrier(a.ctr + kBar, passed, a.barrier_spins)) {
-                ok = false;
-                break;
+            if (fc != 0) {
+                // the near frontier is small: move the far pile's vertices
+                // below the next split distance into it, once every block
+                // has read the sizes above; the distance grows with each
+                // split in a row
+                ++bars;
+                if (!grid_barrier(a.ctr + kBar, passed, a.barrier_spins)) {
+                    ok = false;
+                    break;
+                }
+                const uint32_t base = max(nf.T, fm);
+                const uint64_t width = (uint64_t)a.delta << min(burst, 16u);
+                NearFar next;
+                next.T = (uint64_t)base + width >= kInf32 ? kInf32 : (uint32_t)(base + width);
+                next.phase = phase0 + ++splits;
+                next.pile = a.far[cur ^ 1];
+                next.count = a.ctr + kFarCnt0 + (cur ^ 1);
+                next.dmin = a.ctr + kFarMin0 + (cur ^ 1);
+                far_split(a, nf.pile, fc, next, next.T, r, rid, warp0, nwarps, bq, fs[0]);
+                ++bars;
+                if (!grid_barrier(a.ctr + kBar, passed, a.barrier_spins)) {
+                    ok = false;
+                    break;
+                }
+                // the old pile is empty again; no block reads its words
+                // before the next split, two grid barriers on
+                if (threadIdx.x == 0) {
+                    if (blockIdx.x == 0) {
+                        a.ctr[kFarCnt0 + cur] = 0;
+                        a.ctr[kFarMin0 + cur] = kInf32;
+                    }
+                    s_word = ld_volatile(count_of(a.ctr, r));
+                }
+                __syncthreads();
+                n = min(s_word, a.cap);
+                cur ^= 1;
+                nf = next;
+                ++burst;
+                if (splits > a.max_rounds) {
+                    ok = false;
+                    break;
+                }
+                continue;
             }
-            const uint32_t base = max(nf.T, fm);
-            const uint64_t width = (uint64_t)a.delta << min(burst, 16u);
-            NearFar next;
-            next.T = (uint64_t)base + width >= kInf32 ? kInf32 : (uint32_t)(base + width);
-            next.phase = phase0 + ++splits;
-            next.pile = a.far[cur ^ 1];
-            next.count = a.ctr + kFarCnt0 + (cur ^ 1);
-            next.dmin = a.ctr + kFarMin0 + (cur ^ 1);
-            far_split(a, nf.pile, fc, next, next.T, r, rid, warp0, nwarps, bq);
-            ++bars;
-            if (!grid_barrier(a.ctr + kBar, passed, a.barrier_spins)) {
-                ok = false;
-                break;
-            }
-            // the old pile is empty again; no block reads its words before
-            // the next split, two grid barriers on
-            if (blockIdx.x == 0 && threadIdx.x == 0) {
-                a.ctr[kFarCnt0 + cur] = 0;
-                a.ctr[kFarMin0 + cur] = kInf32;
-            }
-            cur ^= 1;
-            nf = next;
-            ++burst;
-            if (splits > a.max_rounds) {
-                ok = false;
-                break;
-            }
-            continue;
         }
         burst = 0;
         if (n == 0)
             break;
         if (n > kSoloLists) {
-            round_step<kNF>(a, gcnt, r, n, warp0, nwarps, rid, bq, &nf);
+            // the pair of frontier r - 1, which every block has left, is
+            // that of frontier r + 2
+            if (blockIdx.x == 0 && threadIdx.x == 0)
+                *reinterpret_cast<unsigned long long *>(count_of(a.ctr, r + 2)) = 0;
+            round_step<kNF>(a, count_of(a.ctr, r + 1), r, n, warp0, nwarps, rid, bq, &nf, fs);
             ++bars;
-            if (!grid_barrier(a.ctr + kBar, passed, a.barrier_spins)) {
-                ok = false;
-                break;
-            }
             ++r;
+            ok = round_barrier(a.ctr, r, a.barrier_spins, &n);
+            n = min(n, a.cap);
             continue;
         }
         // every block has read n: block 0 may now change the global sizes
@@ -457,37 +651,40 @@ __global__ void __launch_bounds__(kRoundsMaxThreads, 1) k_rounds(RoundArgs a)
         }
         if (blockIdx.x == 0) {
             const uint64_t bw0 = threadIdx.x >> 5, bnw = blockDim.x >> 5;
-            if (threadIdx.x == 0) {
-                solo_cnt[r % 3] = n;
-                solo_cnt[(r + 1) % 3] = 0;
-                solo_cnt[(r + 2) % 3] = 0;
-            }
+            if (threadIdx.x < 3)
+                solo_cnt[threadIdx.x] = 0;
             __syncthreads();
             uint32_t steps = 0;
             do {
-                round_step<kNF>(a, solo_cnt, r, n, bw0, bnw, rid, bq, &nf);
+                round_step<kNF>(a, &solo_cnt[(r + 1) % 3], r, n, bw0, bnw, rid, bq, &nf, fs);
                 __syncthreads();
                 ++r;
                 ++steps;
-                n = *(volatile uint32_t *)&solo_cnt[r % 3];
-                __syncthreads();
+                n = min(*(volatile uint32_t *)&solo_cnt[r % 3], a.cap);
+                // written again two rounds on
+                if (threadIdx.x == 0)
+                    solo_cnt[(r + 2) % 3] = 0;
             } while (n > 0 && n <= kSoloLists && steps < kSoloRounds && r < a.max_rounds);
             if (threadIdx.x == 0) {
-                gcnt[r % 3] = n;
-                gcnt[(r + 1) % 3] = 0;
-                gcnt[(r + 2) % 3] = 0;
+                *count_of(a.ctr, r) = n;
+                for (uint32_t k = 1; k < 3; ++k)
+                    *reinterpret_cast<unsigned long long *>(count_of(a.ctr, r + k)) = 0;
                 a.ctr[kSoloR] = r;
+                a.ctr[kSoloR + 1] = n;
             }
         }
         if (!grid_barrier(a.ctr + kBar, passed, a.barrier_spins)) {
             ok = false;
             break;
         }
-        if (threadIdx.x == 0)
+        if (threadIdx.x == 0) {
             s_word = ld_volatile(a.ctr + kSoloR);
+            s_fc = ld_volatile(a.ctr + kSoloR + 1);
+        }
         __syncthreads();
         r = s_word;
-        __syncthreads(); // every thread has read s_word before thread 0 rewrites it
+        n = s_fc;
+        __syncthreads(); // every thread has read them before thread 0 rewrites them
     }
     // The phase is over: every block left the loop at the same round, after
     // the grid barrier that ended the last relaxation, so D is final.  The
@@ -521,13 +718,15 @@ __global__ void __launch_bounds__(kRoundsMaxThreads, 1) k_rounds(RoundArgs a)
 // One round, for the host-driven fallback.
 __global__ void __launch_bounds__(256) k_round_once(RoundArgs a, uint32_t r, uint32_t n)
 {
-    __shared__ BlockFrontier bq;
-    bq_init(bq);
+    __shared__ FrontierSmem<8> bq;
+    frontier_init(bq);
     const uint64_t warp0 = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5;
     const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
-    round_step(a, a.ctr + kCnt0, r, n, warp0, nwarps, __ldg(a.ctr + kRid), bq);
-    if (blockIdx.x == 0 && threadIdx.x == 0)
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        *count_of(a.ctr, r + 2) = 0;
         a.ctr[kRoundsDone] = r + 1;
+    }
+    round_step(a, count_of(a.ctr, r + 1), r, n, warp0, nwarps, __ldg(a.ctr + kRid), bq);
 }
 
 __global__ void k_sssp_init(unsigned long long *D, uint32_t V, uint32_t source, uint2 *front, uint32_t *count,
@@ -813,8 +1012,8 @@ __global__ void __launch_bounds__(256, 5) k_relax_updated(RoundArgs a)
     const uint32_t n = min(__ldg(&g.st->ulog_count), g.H);
     const uint64_t warp0 = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5;
     const uint64_t gs = (((uint64_t)gridDim.x * blockDim.x) >> 5) * 8; // 4-lane groups in the grid
-    __shared__ BlockFrontier bq;
-    bq_init(bq);
+    __shared__ FrontierSmem<8> bq;
+    frontier_init(bq);
     const uint32_t round = __ldg(a.ctr + kRid) + 1;
     int *overflow = (int *)(a.ctr + kOverflow);
     unsigned long long lists = 0, slabs = 0, edges = 0, improved = 0;
@@ -846,11 +1045,11 @@ __global__ void __launch_bounds__(256, 5) k_relax_updated(RoundArgs a)
         src = nsrc;
         mk = nmk;
     }
-    bq_flush(bq, a.front[0], a.ctr + kCnt0, a.cap, overflow);
+    frontier_flush(bq, a.front[0], a.ctr + kCnt0, a.cap, overflow);
     count_add(g.st, kCtrSeedLists, lists);
     count_add(g.st, kCtrSeedSlabs, slabs);
-    count_add(g.st, kCtrSeedEdges, edges);
-    count_add(g.st, kCtrSeedImproved, improved);
+    count_add(g.st, kCtrSeedEdges, warp_sum(edges));
+    count_add(g.st, kCtrSeedImproved, warp_sum(improved));
 }
 
 // Incremental seeds from the inserted-edge log (the paper's incremental
@@ -865,8 +1064,8 @@ __global__ void __launch_bounds__(256, 5) k_relax_updated(RoundArgs a)
 // per updated list (log entry, list source, marker, source node, slab).
 __global__ void __launch_bounds__(256) k_relax_inserted(RoundArgs a, const uint4 *__restrict__ ilog, uint64_t n)
 {
-    __shared__ BlockFrontier bq;
-    bq_init(bq);
+    __shared__ FrontierSmem<8> bq;
+    frontier_init(bq);
     const uint32_t round = __ldg(a.ctr + kRid) + 1;
     int *overflow = (int *)(a.ctr + kOverflow);
     unsigned long long entries = 0, edges = 0, improved = 0;
@@ -909,7 +1108,7 @@ __global__ void __launch_bounds__(256) k_relax_inserted(RoundArgs a, const uint4
         uint32_t st[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            up[k] = up[k] && cand(k) < cur[k];
+            up[k] = up[k] && nd[k] < node_dist(cur[k]);
             vi[k] = make_uint2(0, 0);
             st[k] = round;
             if (up[k]) {
@@ -921,10 +1120,10 @@ __global__ void __launch_bounds__(256) k_relax_inserted(RoundArgs a, const uint4
         for (int k = 0; k < 4; ++k) {
             up[k] = up[k] && st[k] != round;
             improved += __popc(__ballot_sync(kFull, up[k]));
-            enqueue_lists_block(bq, y[k], up[k], vi[k], a.front[0], a.ctr + kCnt0, a.cap, overflow);
         }
+        enqueue_lists<4>(bq, y, up, vi, a.front[0], a.ctr + kCnt0, a.cap, overflow);
     }
-    bq_flush(bq, a.front[0], a.ctr + kCnt0, a.cap, overflow);
+    frontier_flush(bq, a.front[0], a.ctr + kCnt0, a.cap, overflow);
     count_add(a.g.st, kCtrSeedLog, entries);
     count_add(a.g.st, kCtrSeedEdges, edges);
     count_add(a.g.st, kCtrSeedImproved, improved);
@@ -972,20 +1171,18 @@ struct MultiArgs {
 // The incremental prologue (k_relax_updated) for every state at once: each
 // logged list is walked once from its UpdateIterator start and every slab's
 // new edges are relaxed into each state whose copy of the list's source has
-// a finite distance.  Dynamic shared memory: one BlockFrontier per state.
+// a finite distance.  Dynamic shared memory: one staging area per state.
 __global__ void __launch_bounds__(256, 5) k_relax_updated_multi(MultiArgs m)
 {
     extern __shared__ unsigned char multi_smem[];
-    BlockFrontier *bqs = reinterpret_cast<BlockFrontier *>(multi_smem);
+    FrontierSmem<8> *bqs = reinterpret_cast<FrontierSmem<8> *>(multi_smem);
     const GView &g = m.c[0].g;
     const uint32_t s4 = lane_id() & 3u, g4 = lane_id() >> 2;
     const uint32_t n = min(__ldg(&g.st->ulog_count), g.H);
     const uint64_t warp0 = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5;
     const uint64_t gs = (((uint64_t)gridDim.x * blockDim.x) >> 5) * 8;
     for (uint32_t j = 0; j < m.k; ++j)
-        if (threadIdx.x == 0)
-            bqs[j].count = 0;
-    __syncthreads();
+        frontier_init(bqs[j]);
     uint32_t round[kMaxMulti];
 #pragma unroll
     for (uint32_t j = 0; j < kMaxMulti; ++j)
@@ -1030,11 +1227,11 @@ __global__ void __launch_bounds__(256, 5) k_relax_updated_multi(MultiArgs m)
         mk = nmk;
     }
     for (uint32_t j = 0; j < m.k; ++j)
-        bq_flush(bqs[j], m.c[j].front[0], m.c[j].ctr + kCnt0, m.c[j].cap, (int *)(m.c[j].ctr + kOverflow));
+        frontier_flush(bqs[j], m.c[j].front[0], m.c[j].ctr + kCnt0, m.c[j].cap, (int *)(m.c[j].ctr + kOverflow));
     count_add(g.st, kCtrSeedLists, lists);
     count_add(g.st, kCtrSeedSlabs, slabs);
-    count_add(g.st, kCtrSeedEdges, edges);
-    count_add(g.st, kCtrSeedImproved, improved);
+    count_add(g.st, kCtrSeedEdges, warp_sum(edges));
+    count_add(g.st, kCtrSeedImproved, warp_sum(improved));
 }
 
 // The decremental relax-into-invalid scan (k_relax_into_invalid_slabs) for
@@ -1133,17 +1330,15 @@ __global__ void __launch_bounds__(kScanWarps * 32) k_relax_into_invalid_multi(Mu
 // counter for round r + 2 every round, so a state whose frontier emptied
 // keeps reading zero.  No solo phase: rounds of a few lists cost a grid
 // barrier each.  Then every state's epilogue (dist/parent, round stamp).
-// Dynamic shared memory: one BlockFrontier per state.
+// Dynamic shared memory: one staging area per state.
 __global__ void __launch_bounds__(kRoundsMaxThreads, 1) k_rounds_multi(MultiArgs m)
 {
     extern __shared__ unsigned char multi_smem[];
-    BlockFrontier *bqs = reinterpret_cast<BlockFrontier *>(multi_smem);
+    auto *bqs = reinterpret_cast<FrontierSmem<kRoundsMaxThreads / 32> *>(multi_smem);
     __shared__ uint32_t s_n[kMaxMulti];
     for (uint32_t j = 0; j < m.k; ++j)
-        if (threadIdx.x == 0)
-            bqs[j].count = 0;
-    __syncthreads();
-    const uint64_t warp0 = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5;
+        frontier_init(bqs[j]);
+    const uint64_t warp0 = (uint64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x; // as in k_rounds
     const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
     const RoundArgs &a0 = m.c[0];
     uint32_t r = 0, bars = 0, passed = 0;
@@ -1151,7 +1346,7 @@ __global__ void __launch_bounds__(kRoundsMaxThreads, 1) k_rounds_multi(MultiArgs
     while (r < a0.max_rounds) {
         if (threadIdx.x == 0)
             for (uint32_t j = 0; j < m.k; ++j)
-                s_n[j] = min(ld_volatile(m.c[j].ctr + kCnt0 + r % 3), m.c[j].cap);
+                s_n[j] = min(ld_volatile(count_of(m.c[j].ctr, r)), m.c[j].cap);
         __syncthreads();
         uint32_t total = 0;
         for (uint32_t j = 0; j < m.k; ++j)
@@ -1160,16 +1355,16 @@ __global__ void __launch_bounds__(kRoundsMaxThreads, 1) k_rounds_multi(MultiArgs
             break;
         if (blockIdx.x == 0 && threadIdx.x == 0)
             for (uint32_t j = 0; j < m.k; ++j)
-                m.c[j].ctr[kCnt0 + (r + 2) % 3] = 0;
+                *count_of(m.c[j].ctr, r + 2) = 0;
         for (uint32_t j = 0; j < m.k; ++j) {
             const uint32_t n = s_n[j];
             if (n == 0)
                 continue;
             const RoundArgs &a = m.c[j];
             const uint32_t in = r & 1;
-            uint32_t *cnt = a.ctr + kCnt0 + (r + 1) % 3;
+            uint32_t *cnt = count_of(a.ctr, r + 1);
             relax_body(a, a.front[in], n, a.front[in ^ 1], cnt, __ldg(a.ctr + kRid) + 2 + r, warp0, nwarps, bqs[j]);
-            bq_flush(bqs[j], a.front[in ^ 1], cnt, a.cap, (int *)(a.ctr + kOverflow));
+            frontier_flush(bqs[j], a.front[in ^ 1], cnt, a.cap, (int *)(a.ctr + kOverflow));
         }
         ++bars;
         if (!grid_barrier(a0.ctr + kBar, passed, a0.barrier_spins)) {
@@ -1238,8 +1433,8 @@ mk_status get_consumer(mk_graph *g, int kind, uint32_t source, Consumer **out)
     if (st == MK_OK)
         st = device_alloc(g, (void **)&c->inv, (V + 31) / 32 * 4);
     if (st == MK_OK)
-        st = device_alloc(g, (void **)&c->counters, 64);
-    if (st == MK_OK && (cudaMemset(c->stamp, 0, V * 4) != cudaSuccess || cudaMemset(c->counters, 0, 64) != cudaSuccess))
+        st = device_alloc(g, (void **)&c->counters, kConsumerWords * 4);
+    if (st == MK_OK && (cudaMemset(c->stamp, 0, V * 4) != cudaSuccess || cudaMemset(c->counters, 0, kConsumerWords * 4) != cudaSuccess))
         st = MK_ERR_CUDA;
     if (st != MK_OK) {
         device_free(g, c->D, V * 8);
@@ -1247,7 +1442,7 @@ mk_status get_consumer(mk_graph *g, int kind, uint32_t source, Consumer **out)
         device_free(g, c->front[1], H * 8);
         device_free(g, c->stamp, V * 4);
         device_free(g, c->inv, (V + 31) / 32 * 4);
-        device_free(g, c->counters, 64);
+        device_free(g, c->counters, kConsumerWords * 4);
         delete c;
         return st;
     }
@@ -1308,7 +1503,7 @@ mk_status run_phase(mk_graph *g, RoundArgs a, const char *name, cudaStream_t s)
     for (uint32_t r = 0;; ++r) {
         if (r > a.max_rounds)
             return MK_ERR_TIMEOUT;
-        MK_CUDA(cudaMemcpyAsync(g->h_pinned, a.ctr + kCnt0 + r % 3, 4, cudaMemcpyDeviceToHost, s));
+        MK_CUDA(cudaMemcpyAsync(g->h_pinned, count_of(a.ctr, r), 4, cudaMemcpyDeviceToHost, s));
         MK_CUDA(cudaStreamSynchronize(s));
         const uint32_t n = std::min(g->h_pinned[0], a.cap);
         if (n == 0) {
@@ -1514,10 +1709,10 @@ mk_status run_multi(mk_graph *g, const mk_algo_req *reqs, uint32_t n, cudaStream
     }
     // incremental prologue: one walk over the updated lists for all states
     if (inc.k) {
-        const size_t smem = inc.k * sizeof(BlockFrontier);
+        const size_t smem = inc.k * sizeof(FrontierSmem<8>);
         // (a function attribute of the current device: set on every call)
         MK_CUDA(cudaFuncSetAttribute(k_relax_updated_multi, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)(kMaxMulti * sizeof(BlockFrontier))));
+                                     (int)(kMaxMulti * sizeof(FrontierSmem<8>))));
         MK_TRY(timed(g, "sssp_relax_updated", s, 1, [&]() {
             const uint64_t threads = g->ulog_bound * 4;
             k_relax_updated_multi<<<std::min<uint32_t>(grid_for(threads, 256), num_sms() * 10), 256, smem, s>>>(inc);
@@ -1527,9 +1722,9 @@ mk_status run_multi(mk_graph *g, const mk_algo_req *reqs, uint32_t n, cudaStream
     // rounds of every state together
     const int grid = rounds_grid(g->tune.rounds_blocks_per_sm);
     const int block = rounds_block(g->tune.rounds_blocks_per_sm);
-    const size_t smem = n * sizeof(BlockFrontier);
+    const size_t smem = n * sizeof(FrontierSmem<kRoundsMaxThreads / 32>);
     MK_CUDA(cudaFuncSetAttribute(k_rounds_multi, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)(kMaxMulti * sizeof(BlockFrontier))));
+                                 (int)(kMaxMulti * sizeof(FrontierSmem<kRoundsMaxThreads / 32>))));
     void *args[] = {&m};
     mk_status st = MK_ERR_CUDA;
     if (!g->dbg_host_rounds)

@@ -5,36 +5,52 @@
 
 namespace mk {
 
-// A block's staging area for frontier entries.  Warps reserve slots with
-// shared-memory atomics; the block copies the staged entries to the global
-// frontier with one global atomicAdd (bq_flush), instead of one atomic per
-// enqueuing warp on the single global frontier counter, where thousands of
-// warps a round would serialise.
-constexpr uint32_t kBlockBuf = 2048;
-struct BlockFrontier {
-    uint2 buf[kBlockBuf];
-    uint32_t count; // slots reserved; those at or past kBlockBuf went to the global frontier
-    uint32_t base;
+// A block's staging area for frontier entries: a buffer a warp, so that
+// nothing is shared while a round runs.  A full buffer goes to the global
+// frontier with one atomicAdd on its count (at least kWarpBuf / 2 entries at
+// a time); what is left at the end of a round with one a block
+// (frontier_flush).  Thousands of warps meet on that one count: with one
+// buffer a block, and an atomic for every later append of a warp, the static
+// BFS on R-MAT scale 20 waited for the count most of the time.
+constexpr uint32_t kWarpBuf = 64;
+template <uint32_t kWarps>
+struct FrontierSmem {
+    uint2 buf[kWarps][kWarpBuf];
+    uint32_t held[kWarps]; // entries in each warp's buffer
+    uint32_t at[kWarps];   // their places at a flush
 };
 
-// Appends the slab lists of vertex y (for every lane with pred; vi is y's
-// vinfo entry, loaded by the caller) to the list frontier as <list, y>
-// entries (the source travels with the list, so a consumer needs no list_src
-// lookup).  Lanes with few buckets write their entries through the block's
-// staging area: the warp's entries take slots [off, off + total) of the
-// block buffer and those that do not fit go to the global frontier directly.
-// A vertex with many buckets is written to the global frontier by the whole
-// warp.  Must be called by the full warp; sets *overflow for an entry that
-// would not fit in `cap`.
-__device__ __forceinline__ void enqueue_lists_block(BlockFrontier &bq, uint32_t y, bool pred, uint2 vi, uint2 *out,
-                                                    uint32_t *count, uint32_t cap, int *overflow)
+template <uint32_t kWarps>
+__device__ __forceinline__ void frontier_init(FrontierSmem<kWarps> &sm)
+{
+    if (threadIdx.x < kWarps)
+        sm.held[threadIdx.x] = 0;
+    __syncthreads();
+}
+
+// Appends the slab lists of the lane's vertices y[k] with up[k] (vi[k]: its
+// vinfo entry) to the frontier as <list, y> entries (the source travels with
+// the list, so a consumer needs no list_src lookup): one scan over the warp
+// and at most one reservation for all of them (one for each vertex with many
+// buckets made the round after a hub wait for 25 of them in a row).  Must be
+// called by the full warp; sets
+// *overflow for an entry that would not fit in `cap`.
+template <int N, uint32_t kWarps>
+__device__ __forceinline__ void enqueue_lists(FrontierSmem<kWarps> &sm, const uint32_t (&y)[N], const bool (&up)[N],
+                                              const uint2 (&vi)[N], uint2 *out, uint32_t *count, uint32_t cap,
+                                              int *overflow)
 {
     constexpr uint32_t kSmall = 8;
-    const uint32_t lane = lane_id();
-    if (!__any_sync(kFull, pred))
+    const uint32_t lane = lane_id(), w = threadIdx.x >> 5;
+    uint32_t c = 0;
+    bool big = false;
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        c += up[k] ? vi[k].y : 0u;
+        big = big || (up[k] && vi[k].y > kSmall);
+    }
+    if (!__any_sync(kFull, c != 0))
         return;
-    const bool small = pred && vi.y <= kSmall;
-    const uint32_t c = small ? vi.y : 0;
     uint32_t incl = c;
 #pragma unroll
     for (uint32_t o = 1; o < 32; o <<= 1) {
@@ -42,77 +58,86 @@ __device__ __forceinline__ void enqueue_lists_block(BlockFrontier &bq, uint32_t 
         if (lane >= o)
             incl += t;
     }
-    const uint32_t total = __shfl_sync(kFull, incl, 31);
-    if (total) {
-        uint32_t off = 0;
+    const uint32_t total = __shfl_sync(kFull, incl, 31), held = sm.held[w];
+    const bool any_big = __any_sync(kFull, big), fits = !any_big && held + total <= kWarpBuf;
+    auto put = [&](uint32_t at, uint2 ent) {
+        if (at < cap)
+            out[at] = ent;
+        else
+            *overflow = 1;
+    };
+    uint32_t base = 0;
+    if (!fits) {
         if (lane == 0)
-            off = atomicAdd(&bq.count, total);
-        off = __shfl_sync(kFull, off, 0);
-        const uint32_t room = off < kBlockBuf ? min(kBlockBuf - off, total) : 0u;
-        uint32_t gbase = 0;
-        if (room < total && lane == 0)
-            gbase = atomicAdd(count, total - room);
-        gbase = __shfl_sync(kFull, gbase, 0);
-        for (uint32_t k = 0; k < c; ++k) {
-            const uint32_t t = incl - c + k; // the warp's t-th entry
-            const uint2 ent = make_uint2(vi.x + k, y);
-            if (t < room)
-                bq.buf[off + t] = ent;
-            else if (gbase + (t - room) < cap)
-                out[gbase + (t - room)] = ent;
-            else
-                *overflow = 1;
-        }
-    }
-    uint32_t big = __ballot_sync(kFull, pred && !small);
-    while (big) {
-        const uint32_t l = __ffs(big) - 1;
-        big &= big - 1;
-        const uint32_t first = __shfl_sync(kFull, vi.x, l);
-        const uint32_t nb = __shfl_sync(kFull, vi.y, l);
-        const uint32_t yl = __shfl_sync(kFull, y, l);
-        uint32_t base = 0;
-        if (lane == 0)
-            base = atomicAdd(count, nb);
+            base = atomicAdd(count, held + total);
         base = __shfl_sync(kFull, base, 0);
-        for (uint32_t k = lane; k < nb; k += 32) {
-            if (base + k < cap)
-                out[base + k] = make_uint2(first + k, yl);
-            else
-                *overflow = 1;
-        }
+        for (uint32_t t = lane; t < held; t += 32)
+            put(base + t, sm.buf[w][t]);
     }
+    uint32_t t = held + incl - c;
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        const uint32_t nb = up[k] ? vi[k].y : 0u;
+        if (nb <= kSmall)
+            for (uint32_t b = 0; b < nb; ++b) {
+                if (fits)
+                    sm.buf[w][t + b] = make_uint2(vi[k].x + b, y[k]);
+                else
+                    put(base + t + b, make_uint2(vi[k].x + b, y[k]));
+            }
+        if (any_big)
+            for (uint32_t m = __ballot_sync(kFull, nb > kSmall); m; m &= m - 1) {
+                const uint32_t l = __ffs(m) - 1;
+                const uint32_t first = __shfl_sync(kFull, vi[k].x, l), n = __shfl_sync(kFull, nb, l);
+                const uint32_t yl = __shfl_sync(kFull, y[k], l), at = base + __shfl_sync(kFull, t, l);
+                for (uint32_t b = lane; b < n; b += 32)
+                    put(at + b, make_uint2(first + b, yl));
+            }
+        t += nb;
+    }
+    __syncwarp();
+    if (lane == 0)
+        sm.held[w] = fits ? held + total : 0u;
+    __syncwarp();
 }
 
 // Copies the block's staged entries to the global frontier and empties the
-// staging area.  Called by every thread of the block (it synchronises the
-// block).
-__device__ __forceinline__ void bq_flush(BlockFrontier &bq, uint2 *out, uint32_t *count, uint32_t cap, int *overflow)
+// staging area.  Called by every thread of the block; the caller synchronises
+// the block before the entries or the staging area are used again.
+template <uint32_t kWarps>
+__device__ __forceinline__ void frontier_flush(FrontierSmem<kWarps> &sm, uint2 *out, uint32_t *count, uint32_t cap,
+                                               int *overflow)
 {
+    const uint32_t lane = lane_id(), w = threadIdx.x >> 5;
     __syncthreads();
-    const uint32_t n = min(bq.count, kBlockBuf);
-    if (threadIdx.x == 0)
-        bq.base = n ? atomicAdd(count, n) : 0u;
+    if (w == 0) {
+        const uint32_t h = lane < kWarps ? sm.held[lane] : 0u;
+        uint32_t incl = h;
+#pragma unroll
+        for (uint32_t o = 1; o < 32; o <<= 1) {
+            const uint32_t t = __shfl_up_sync(kFull, incl, o);
+            if (lane >= o)
+                incl += t;
+        }
+        uint32_t base = 0;
+        if (lane == 31 && incl)
+            base = atomicAdd(count, incl);
+        base = __shfl_sync(kFull, base, 31);
+        if (lane < kWarps)
+            sm.at[lane] = base + incl - h;
+    }
     __syncthreads();
-    for (uint32_t t = threadIdx.x; t < n; t += blockDim.x) {
-        if (bq.base + t < cap)
-            out[bq.base + t] = bq.buf[t];
+    const uint32_t held = sm.held[w], at = sm.at[w];
+    for (uint32_t t = lane; t < held; t += 32) {
+        if (at + t < cap)
+            out[at + t] = sm.buf[w][t];
         else
             *overflow = 1;
     }
-    __syncthreads();
-    if (threadIdx.x == 0)
-        bq.count = 0;
-    __syncthreads();
+    __syncwarp();
+    if (lane == 0)
+        sm.held[w] = 0;
 }
-
-__device__ __forceinline__ void bq_init(BlockFrontier &bq)
-{
-    if (threadIdx.x == 0)
-        bq.count = 0;
-    __syncthreads();
-}
-
 
 } // namespace mk
 

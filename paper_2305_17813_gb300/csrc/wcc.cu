@@ -239,10 +239,10 @@ extern "C" mk_status mk_incr_wcc(mk_graph *g, uint32_t *d_label, void *stream)
         c->kind = kWcc;
         mk_status st = device_alloc(g, (void **)&c->uf, (size_t)V * 4);
         if (st == MK_OK)
-            st = device_alloc(g, (void **)&c->counters, 64);
+            st = device_alloc(g, (void **)&c->counters, kConsumerWords * 4);
         if (st != MK_OK) {
             device_free(g, c->uf, (size_t)V * 4);
-            device_free(g, c->counters, 64);
+            device_free(g, c->counters, kConsumerWords * 4);
             delete c;
             return st;
         }

@@ -218,3 +218,28 @@ def test_near_far_sssp_power_law_stream(cuda_lib, delta):
         g.commit()
         assert g.last_error() == mk.MK_OK
     g.close()
+
+
+@pytest.mark.parametrize("delta", [0, 40])
+def test_frontier_staging_limits(cuda_lib, delta):
+    """One round that improves every vertex: vertices with 1 to 20 lists (up
+    to 8 are staged a warp, more are written by the whole warp), far more
+    entries than the staging buffers hold, with and without far piles."""
+    mk = _mk()
+    rng = np.random.default_rng(31)
+    V = 6000
+    nb = rng.integers(1, 21, V).astype(np.uint32)
+    nb[0] = 64
+    g = mk.Graph(V, edge_capacity_hint=1 << 17, buckets=mk.to_device_u32(nb))
+    g.set_sssp_delta(delta, delta)
+    o = oracle.OracleGraph(V)
+    s = np.concatenate([np.zeros(V - 1), rng.integers(0, V, 30000)]).astype(np.uint32)
+    d = np.concatenate([np.arange(1, V), rng.integers(0, V, 30000)]).astype(np.uint32)
+    w = rng.integers(1, 200, len(s)).astype(np.uint32)
+    assert np.array_equal(g.insert(s, d, w).cpu().numpy(), o.insert(s, d, w))
+    check_algos(g, o, [0])
+    g.commit()
+    g.delete(s[: V // 2], d[: V // 2])
+    o.delete(s[: V // 2], d[: V // 2])
+    check_algos(g, o, [0])
+    g.close()
