@@ -27,7 +27,8 @@ struct Consumer {
     unsigned long long *D = nullptr; // BFS/SSSP: V packed <distance, parent>
     uint2 *front[2] = {nullptr, nullptr}; // BFS/SSSP list frontiers (H entries <list, source> each)
     uint32_t *stamp = nullptr;  // BFS/SSSP: round in which a vertex was last enqueued
-    uint32_t *inv = nullptr;    // BFS/SSSP: bitmap of vertices invalidated by this call's deletes
+    uint32_t *inv = nullptr;    // BFS/SSSP: bitmap of vertices invalidated by this call's deletes; WCC: of
+                                // the giant tree's vertices
     uint32_t round = 0;         // last stamp value used
     uint32_t *uf = nullptr;     // WCC: union-find parents (V)
     uint32_t *far[2] = {nullptr, nullptr}; // SSSP with Near-Far ordering: far piles (V each)

@@ -546,99 +546,6 @@ __global__ void k_set_bfs_init(GView g, uint32_t *dist, uint32_t *parent, uint32
     }
 }
 
-namespace {
-
-__device__ __forceinline__ uint32_t set_find(uint32_t *p, uint32_t x)
-{
-    for (;;) {
-        const uint32_t px = __ldcg(&p[x]);
-        if (px == x)
-            return x;
-        const uint32_t ppx = __ldcg(&p[px]);
-        if (ppx == px)
-            return px;
-        p[x] = ppx; // path halving: ppx is an ancestor of x
-        x = ppx;
-    }
-}
-
-} // namespace
-
-__global__ void k_set_uf_init(uint32_t *p, uint32_t V)
-{
-    const uint32_t v = blockIdx.x * blockDim.x + threadIdx.x;
-    if (v < V)
-        p[v] = v;
-}
-
-// Static WCC (Union-Async, the larger root hooked under the smaller, so each
-// root is its set's smallest vertex): a warp takes 32 consecutive slabs,
-// keeps those in use (owner set) and unites four slabs at a time, one per
-// 8-lane group, each lane holding four keys of the slab (one 16-byte load);
-// the group's last lane puts the slab's owner in place of the next index,
-// so the owner and the slab's 31 destinations are hooked under the
-// smallest of their roots in one group union.  The next step's slabs are
-// loaded a step ahead.
-__global__ void __launch_bounds__(256) k_set_wcc_hook(GView g, uint32_t *p, int *failed)
-{
-    __shared__ uint8_t comp[8][32];
-    const uint32_t lane = lane_id(), g8 = lane >> 3, s8 = lane & 7u, w = threadIdx.x >> 5;
-    const uint64_t total = (uint64_t)g.H + g.P;
-    const uint64_t warp0 = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5;
-    const uint64_t stride = (((uint64_t)gridDim.x * blockDim.x) >> 5) * 32;
-    const uint4 none = make_uint4(kEmptyKey, kEmptyKey, kEmptyKey, kEmptyKey);
-    auto part = [&](uint64_t s) {
-        return __ldcg(reinterpret_cast<const uint4 *>(slab_ptr(g, (uint32_t)s)) + s8);
-    };
-    unsigned long long slabs = 0, edges = 0;
-    uint64_t c = warp0 * 32;
-    uint32_t own_next = c + lane < total ? __ldcg(&g.owner[c + lane]) : kNil;
-    for (; c < total; c += stride) {
-        const uint32_t own_l = own_next;
-        own_next = c + stride + lane < total ? __ldcg(&g.owner[c + stride + lane]) : kNil;
-        const uint32_t live = __ballot_sync(kFull, own_l != kNil);
-        const uint32_t n = __popc(live);
-        if (own_l != kNil)
-            comp[w][__popc(live & lanemask_lt())] = (uint8_t)lane;
-        __syncwarp();
-        uint32_t it = g8 < n ? comp[w][g8] : 32u;
-        uint4 q = it < 32 ? part(c + it) : none;
-        for (uint32_t j = g8; j - g8 < n; j += 4) {
-            const uint32_t nit = j + 4 < n ? comp[w][j + 4] : 32u;
-            const uint4 nq = nit < 32 ? part(c + nit) : none;
-            const bool active = it < 32;
-            const uint32_t own = __shfl_sync(kFull, own_l, it & 31);
-            slabs += __popc(__ballot_sync(kFull, active && s8 == 0));
-            const bool last = s8 == 7u;
-            const uint32_t e[4] = {q.x, q.y, q.z, last ? own : q.w};
-            const bool act[4] = {active && q.x < kTombKey, active && q.y < kTombKey, active && q.z < kTombKey,
-                                 last ? active : (active && q.w < kTombKey)};
-            edges += __popc(__ballot_sync(kFull, act[0])) + __popc(__ballot_sync(kFull, act[1])) +
-                     __popc(__ballot_sync(kFull, act[2])) + __popc(__ballot_sync(kFull, act[3] && !last));
-            if (!group_union<8, 4>(p, e, act, 1u << 20) && lane == 0)
-                *failed = 1;
-            q = nq;
-            it = nit;
-        }
-        __syncwarp();
-    }
-    count_add(g.st, kCtrWccSlabs, slabs);
-    count_add(g.st, kCtrWccEdges, edges);
-}
-
-__global__ void k_set_wcc_label(uint32_t *p, uint32_t V, uint32_t *label)
-{
-    const uint32_t v = blockIdx.x * blockDim.x + threadIdx.x;
-    if (v < V)
-        label[v] = set_find(p, v);
-}
-
-__global__ void k_set_flag_status(const int *failed, DevState *st)
-{
-    if (*failed)
-        set_status(st, kErrTimeout);
-}
-
 __global__ void k_set_pool_used(const DevState *st, unsigned long long *out)
 {
     long long t = 0;
@@ -910,18 +817,17 @@ mk_status mk_set_wcc(mk_set_graph *g, uint32_t *d_label, void *stream)
         return MK_ERR_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)stream;
     const uint32_t V = g->v.V;
+    // the forest (and the labels), the giant tree's bitmap, its root and the
+    // failure flag in one block
+    const size_t words = (size_t)V + ((size_t)V + 31) / 32 + 2;
     uint32_t *p = nullptr;
-    int *failed = nullptr;
-    MK_CUDA(cudaMallocAsync((void **)&p, (size_t)V * 4, s));
-    MK_CUDA(cudaMallocAsync((void **)&failed, sizeof(int), s));
-    MK_CUDA(cudaMemsetAsync(failed, 0, sizeof(int), s));
-    k_set_uf_init<<<grid_for(V, 256), 256, 0, s>>>(p, V);
-    k_set_wcc_hook<<<resident_grid(k_set_wcc_hook, 256), 256, 0, s>>>(g->v, p, failed);
-    k_set_wcc_label<<<grid_for(V, 256), 256, 0, s>>>(p, V, d_label);
-    k_set_flag_status<<<1, 1, 0, s>>>(failed, g->v.st);
-    const cudaError_t e = cudaGetLastError();
+    MK_CUDA(cudaMallocAsync((void **)&p, words * 4, s));
+    uint32_t *bits = p + V, *ctr = p + words - 2;
+    int launches = 0;
+    cudaError_t e = cudaMemsetAsync(ctr, 0, 8, s);
+    if (e == cudaSuccess)
+        e = static_components(g->v, true, p, d_label, bits, ctr, (int *)(ctr + 1), s, &launches);
     cudaFreeAsync(p, s);
-    cudaFreeAsync(failed, s);
     return e == cudaSuccess ? MK_OK : MK_ERR_CUDA;
 }
 

@@ -142,4 +142,12 @@ __device__ __forceinline__ bool group_union(uint32_t *p, const uint32_t (&e)[N],
     return false;
 }
 
+// Components of every live edge of a store (wcc.cu; `set`: the set layout's
+// slabs), from scratch: p (V words) becomes the forest with every vertex under
+// its root, the smallest vertex of its component, and label (nullable) a copy.
+// bits: V bits, giant: one word, *failed: 0 at the call.
+constexpr uint32_t kCcSampleLists = 8192;
+cudaError_t static_components(const GView &g, bool set, uint32_t *p, uint32_t *label, uint32_t *bits, uint32_t *giant,
+                              int *failed, cudaStream_t s, int *launches);
+
 } // namespace mk

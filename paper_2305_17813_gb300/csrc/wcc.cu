@@ -10,9 +10,11 @@
 // hooked under the smallest of their roots (one parallel round of finds and
 // CASes per slab instead of one union per edge on the same source root), and
 // a warp walks eight lists at a time (incremental pass) or eight slabs (static
-// pass).
+// pass; four of the set layout).
 //
-// Static pass: every live edge of every list.  Incremental pass (insert-only
+// Static pass: every live edge of every list, most of them settled by a
+// sampled forest (below; the set layout's components run here too).
+// Incremental pass (insert-only
 // epochs): only the entries written since the last commit, read with the
 // UpdateIterator from each updated list's marker (the paper's
 // ApplyUnionUpdate, which skips lanes before the first updated lane).
@@ -139,78 +141,106 @@ __global__ void __launch_bounds__(256) k_uf_hook_log(DevState *st, const uint4 *
     count_add(st, kCtrWccUpdEdges, entries);
 }
 
-// Static pass as a streaming scan over the whole slab array instead of chain
-// walks.  A warp takes 32 consecutive slabs at a time: one coalesced load of
-// their owners (per-slab source, kNil for an unused pool slab; read a chunk
-// ahead), the slabs in use compacted in shared memory, then eight slabs per
-// step, one per 4-lane group (lane s4 holds words 8*s4 .. 8*s4+7, i.e. pairs
-// 4*s4 .. 4*s4+3, as two 16-byte loads), the next step's slabs loaded before
-// this step's finds.  Each slab's owner (in the last lane's fourth slot: the
-// unused lane and the next lane) and its live destinations are united with
-// one group_union (four elements per lane, found in lockstep).  The scan
-// keeps the slabs in registers rather than staging them in shared memory:
-// the finds' parent loads depend on L1, which shared-memory buffers would
-// take away.
-__global__ void __launch_bounds__(256) k_uf_hook_slabs(GView g, uint32_t *p, int *failed)
+// ------------------------------------------------------------- static pass
+//
+// Most edges of most graphs lie inside one component, and finding that out
+// edge by edge is what the pass cost: two finds each, ending in the same few
+// roots, and hooks that lose to one another there (168-194 us on an R-MAT
+// graph of scale 18 whose slabs are read in 12).  So the pass first builds a
+// forest from a sample -- the pairs in the first 32 bytes of every vertex's
+// first slab, at most 4 (8 keys of the set layout): every vertex points to its
+// smallest sampled neighbour below it, the trees are compressed, the roots
+// that sampled edges connect are hooked with plain atomic minima, and the
+// trees are compressed again.  The tree that holds most of 1,024 sampled
+// vertices is the giant one; a bitmap names its vertices.  The scan over all
+// slabs then tests both ends of an edge in the bitmap, which it keeps in
+// shared memory where it fits, and only slabs with an edge that is not inside
+// the giant tree unite anything.  Kernel boundaries in between also drop the
+// parents that the SMs' L1 caches still hold from before the hooks.
+// Sampled hooks may lose a link (a minimum replaces a root's earlier one):
+// the forest stays one of connected vertices with parents below their
+// children, and the scan looks at every edge again.
+
+namespace {
+
+// One slab is read by eight lanes, 16 bytes each, so that a load covers whole
+// sectors: a lane has two keys of the map layout, four of the set's.  The last
+// lane's last place is no key (the map's unused lane, the set's next index).
+constexpr uint32_t kLanes = 8;
+
+template <bool kSet>
+__device__ __forceinline__ void keys_of(const uint4 &q, uint32_t (&e)[kSet ? 4 : 2])
 {
-    __shared__ uint8_t comp[8][32];
-    const uint32_t lane = lane_id(), g4 = lane >> 2, s4 = lane & 3u, w = threadIdx.x >> 5;
-    const uint64_t total = (uint64_t)g.H + g.P;
-    const uint64_t warp0 = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5;
-    const uint64_t stride = (((uint64_t)gridDim.x * blockDim.x) >> 5) * 32;
-    const uint4 none = make_uint4(kEmptyKey, kFull, kFull, kFull);
-    auto part = [&](uint64_t s, int h) {
-        return __ldcg(reinterpret_cast<const uint4 *>(slab_ptr(g, (uint32_t)s) + s4 * 8 + h * 4));
-    };
-    unsigned long long slabs = 0, edges = 0;
-    uint64_t c = warp0 * 32;
-    uint32_t own_next = c + lane < total ? __ldcg(&g.owner[c + lane]) : kNil;
-    for (; c < total; c += stride) {
-        const uint32_t own_l = own_next;
-        own_next = c + stride + lane < total ? __ldcg(&g.owner[c + stride + lane]) : kNil;
-        const uint32_t live = __ballot_sync(kFull, own_l != kNil);
-        const uint32_t n = __popc(live);
-        if (own_l != kNil)
-            comp[w][__popc(live & ((1u << lane) - 1))] = (uint8_t)lane;
-        __syncwarp();
-        uint32_t it = g4 < n ? comp[w][g4] : 32u;
-        uint4 lo = none, hi = none;
-        if (it < 32) {
-            lo = part(c + it, 0);
-            hi = part(c + it, 1);
-        }
-        for (uint32_t j = g4; j - g4 < n; j += 8) {
-            // the next step's slabs
-            const uint32_t nit = j + 8 < n ? comp[w][j + 8] : 32u;
-            uint4 nlo = none, nhi = none;
-            if (nit < 32) {
-                nlo = part(c + nit, 0);
-                nhi = part(c + nit, 1);
-            }
-            const bool active = it < 32;
-            const uint32_t own = __shfl_sync(kFull, own_l, it & 31);
-            slabs += __popc(__ballot_sync(kFull, active && s4 == 0));
-            const bool last = s4 == 3u;
-            const uint32_t e[4] = {lo.x, lo.z, hi.x, last ? own : hi.z};
-            const bool act[4] = {active && lo.x < kTombKey, active && lo.z < kTombKey, active && hi.x < kTombKey,
-                                 last ? active : (active && hi.z < kTombKey)};
-            edges += __popc(__ballot_sync(kFull, act[0])) + __popc(__ballot_sync(kFull, act[1])) +
-                     __popc(__ballot_sync(kFull, act[2])) + __popc(__ballot_sync(kFull, act[3] && !last));
-            if (!group_union<4, 4>(p, e, act, 1u << 20) && lane == 0)
-                *failed = 1;
-            lo = nlo;
-            hi = nhi;
-            it = nit;
-        }
-        __syncwarp();
+    if constexpr (kSet) {
+        e[0] = q.x, e[1] = q.y, e[2] = q.z, e[3] = q.w;
+    } else {
+        e[0] = q.x, e[1] = q.z;
     }
-    count_add(g.st, kCtrWccSlabs, slabs);
-    count_add(g.st, kCtrWccEdges, edges);
 }
 
-__global__ void k_uf_compress(uint32_t *p, uint32_t V, uint32_t *label)
+// The sampled neighbours of v: keys of the first 32 bytes of its first slab
+// (kNil where there is none; the next index is past them).
+template <bool kSet>
+__device__ __forceinline__ void sample_of(const GView &g, uint32_t v, uint32_t (&d)[8])
+{
+    const uint4 *p = reinterpret_cast<const uint4 *>(slab_ptr(g, __ldg(&g.vinfo[v]).x));
+    const uint4 a = __ldcg(p), b = __ldcg(p + 1);
+    const uint32_t w[8] = {a.x, kSet ? a.y : kNil, a.z, kSet ? a.w : kNil, b.x, kSet ? b.y : kNil, b.z, kSet ? b.w : kNil};
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+        d[k] = w[k] < kTombKey ? w[k] : kNil;
+}
+
+} // namespace
+
+template <bool kSet>
+__global__ void __launch_bounds__(256) k_cc_sample(GView g, uint32_t *p)
 {
     const uint32_t v = blockIdx.x * blockDim.x + threadIdx.x;
+    if (v >= g.V)
+        return;
+    uint32_t d[8], m = v;
+    sample_of<kSet>(g, v, d);
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+        m = min(m, d[k]);
+    p[v] = m;
+}
+
+// Every kLinkStep-th vertex: enough to hook nearly every root (what is left
+// is united in the scan), and few enough at a time that the hooks of the
+// larger trees' roots do not queue up on a few words.
+constexpr uint32_t kLinkStep = 8;
+
+template <bool kSet>
+__global__ void __launch_bounds__(256) k_cc_link(GView g, uint32_t *p)
+{
+    const uint64_t at = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) * kLinkStep;
+    if (at >= g.V)
+        return;
+    const uint32_t v = (uint32_t)at;
+    uint32_t d[8], r[8];
+    sample_of<kSet>(g, v, d);
+    const uint32_t rv = __ldcg(&p[v]);
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+        r[k] = d[k] != kNil ? __ldcg(&p[d[k]]) : rv;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        const uint32_t hi = max(r[k], rv), lo = min(r[k], rv);
+        if (hi != lo && __ldcg(&p[hi]) > lo)
+            atomicMin(&p[hi], lo);
+    }
+}
+
+// p[v] = v's root for every vertex, and into label where that is given.  Ends
+// a pass when `failed` is given: a hook that gave up sets the status.
+__global__ void __launch_bounds__(256) k_uf_compress(uint32_t *p, uint32_t V, uint32_t *label, const int *failed,
+                                                     DevState *st)
+{
+    const uint32_t v = blockIdx.x * blockDim.x + threadIdx.x;
+    if (failed && v == 0 && *failed)
+        set_status(st, kErrTimeout);
     if (v >= V)
         return;
     const uint32_t r = uf_find(p, v);
@@ -219,18 +249,238 @@ __global__ void k_uf_compress(uint32_t *p, uint32_t V, uint32_t *label)
         label[v] = r;
 }
 
-__global__ void k_uf_failed(const int *failed, DevState *st)
+// *giant = the root that most of 1,024 vertices spread over the range have.
+__global__ void __launch_bounds__(1024) k_cc_giant(const uint32_t *p, uint32_t V, uint32_t *giant)
 {
-    if (*failed)
-        set_status(st, kErrTimeout);
+    __shared__ uint32_t key[2048], cnt[2048], best;
+    const uint32_t t = threadIdx.x;
+    for (uint32_t i = t; i < 2048; i += 1024) {
+        key[i] = kNil;
+        cnt[i] = 0;
+    }
+    if (t == 0)
+        best = 0;
+    __syncthreads();
+    const uint32_t r = __ldcg(&p[(uint32_t)((uint64_t)V * t >> 10)]);
+    uint32_t h = hash32(r) & 2047u;
+    for (;;) { // at most half full
+        const uint32_t own = atomicCAS(&key[h], kNil, r);
+        if (own == kNil || own == r)
+            break;
+        h = (h + 1) & 2047u;
+    }
+    const uint32_t mine = atomicAdd(&cnt[h], 1u) + 1; // the last of a root counts them all
+    atomicMax(&best, mine);
+    __syncthreads();
+    if (mine == best)
+        *giant = r; // of equals, any
 }
+
+__global__ void __launch_bounds__(256) k_cc_bits(const uint32_t *p, uint32_t V, const uint32_t *giant, uint32_t *bits)
+{
+    const uint32_t v = blockIdx.x * blockDim.x + threadIdx.x;
+    const uint32_t m = __ballot_sync(kFull, v < V && p[v] == __ldg(giant));
+    if (lane_id() == 0 && v < V)
+        bits[v >> 5] = m;
+}
+
+namespace {
+
+// Edges waiting to be united, a buffer a warp.
+constexpr uint32_t kPairBuf = 192; // 63 of the steps before and 128 of this one
+
+// Unites the warp's first min(n, 64) pairs of buf, two a lane, their finds in
+// lockstep; a hook that loses is done again one pair at a time.
+__device__ __forceinline__ bool unite_pairs(uint32_t *p, const uint2 *buf, uint32_t n)
+{
+    const uint32_t lane = lane_id();
+    uint32_t x[4];
+    bool lost[2];
+#pragma unroll
+    for (uint32_t i = 0; i < 2; ++i) {
+        const uint32_t at = lane + 32 * i;
+        const uint2 e = at < n ? buf[at] : make_uint2(kNil, kNil);
+        x[2 * i] = e.x;
+        x[2 * i + 1] = e.y;
+    }
+    uf_find_n<4, true>(p, x);
+#pragma unroll
+    for (uint32_t i = 0; i < 2; ++i) {
+        const uint32_t hi = max(x[2 * i], x[2 * i + 1]), lo = min(x[2 * i], x[2 * i + 1]);
+        lost[i] = hi != lo && atomicCAS(&p[hi], hi, lo) != hi;
+    }
+    bool ok = true;
+#pragma unroll
+    for (uint32_t i = 0; i < 2; ++i)
+        if (__any_sync(kFull, lost[i])) {
+            const uint32_t e[2] = {x[2 * i], x[2 * i + 1]};
+            const bool act[2] = {lost[i], lost[i]};
+            ok = group_union<1, 2>(p, e, act, 1u << 20) && ok;
+        }
+    __syncwarp();
+    return ok;
+}
+
+} // namespace
+
+// The scan: a warp takes 32 consecutive slabs at a time, one a group of
+// kLanes lanes: their owners in one load (read a chunk ahead; kNil for an
+// unused pool slab), then all of their parts at once.  kBits: 0 unites every
+// slab, 1 tests the bitmap in shared memory, 2 in global memory; an edge that
+// is not inside the giant tree then waits in a buffer until 64 are there, so
+// that the scan does not stop for the round trips of every few.  Bound by
+// instructions (R-MAT scale 20: 0.8 % of the edges are united; 91 us for
+// 300 MB of slabs).
+constexpr uint32_t kScanThreads = 1024;
+
+template <bool kSet, int kBits>
+__global__ void __launch_bounds__(kScanThreads, 1) k_cc_scan(GView g, uint32_t *p, const uint32_t *__restrict__ bits,
+                                                             const uint32_t *giant, int *failed)
+{
+    constexpr uint32_t kGroups = 32 / kLanes, kSteps = 32 / kGroups;
+    constexpr int kKeys = kSet ? 4 : 2;
+    extern __shared__ uint32_t s_bits[];
+    __shared__ uint2 pairs[kBits ? kScanThreads / 32 : 1][kBits ? kPairBuf : 1];
+    const uint32_t lane = lane_id(), gr = lane / kLanes, sub = lane % kLanes, w = threadIdx.x >> 5;
+    const bool last = sub == kLanes - 1;
+    const uint32_t root = kBits ? __ldg(giant) : 0u;
+    if (kBits == 1) {
+        for (uint32_t i = threadIdx.x; i < (g.V + 31) / 32; i += kScanThreads)
+            s_bits[i] = __ldg(&bits[i]);
+        __syncthreads();
+    }
+    auto inside = [&](uint32_t v) -> uint32_t {
+        return ((kBits == 1 ? s_bits[v >> 5] : __ldg(&bits[v >> 5])) >> (v & 31u)) & 1u;
+    };
+    const uint64_t total = (uint64_t)g.H + g.P;
+    const uint64_t stride = (((uint64_t)gridDim.x * kScanThreads) >> 5) * 32;
+    uint32_t slabs = 0, edges = 0; // of this warp, of this lane
+    uint32_t held = 0;             // pairs in the warp's buffer
+    bool ok = true;
+    uint64_t c = ((blockIdx.x * (uint64_t)kScanThreads + threadIdx.x) >> 5) * 32;
+    uint32_t own_next = c + lane < total ? __ldcg(&g.owner[c + lane]) : kNil;
+    for (; c < total; c += stride) {
+        const uint32_t own_l = own_next;
+        own_next = c + stride + lane < total ? __ldcg(&g.owner[c + stride + lane]) : kNil;
+        const uint32_t live = __ballot_sync(kFull, own_l != kNil);
+        if (!live)
+            continue;
+        uint4 part[kSteps];
+        const uint4 *at = reinterpret_cast<const uint4 *>(slab_ptr(g, (uint32_t)c + gr)) + sub;
+#pragma unroll
+        for (uint32_t j = 0; j < kSteps; ++j)
+            part[j] = (live >> (j * kGroups + gr)) & 1u ? __ldcg(at + j * kGroups * 8)
+                                                        : make_uint4(kEmptyKey, kEmptyKey, kEmptyKey, kEmptyKey);
+        const uint32_t in = kBits ? __ballot_sync(kFull, own_l != kNil && inside(own_l)) : 0u;
+        slabs += __popc(live);
+#pragma unroll
+        for (uint32_t j = 0; j < kSteps; ++j) {
+            const uint32_t it = j * kGroups + gr;
+            uint32_t e[kKeys], keys = 0, out = 0; // bit k: e[k] is a key; and it is outside the giant tree
+            keys_of<kSet>(part[j], e);
+#pragma unroll
+            for (int k = 0; k < kKeys; ++k)
+                if (e[k] < kTombKey && !(last && k == kKeys - 1)) {
+                    keys |= 1u << k;
+                    if (kBits)
+                        out |= (inside(e[k]) ^ 1u) << k;
+                }
+            edges += __popc(keys);
+            if (kBits) {
+                const bool u_in = (in >> it) & 1u;
+                const uint32_t need = u_in ? out : keys;
+                if (!__any_sync(kFull, need))
+                    continue;
+                const uint32_t own = __shfl_sync(kFull, own_l, it), a = u_in ? root : own;
+#pragma unroll
+                for (int k = 0; k < kKeys; ++k) {
+                    const uint32_t m = __ballot_sync(kFull, (need >> k) & 1u);
+                    if ((need >> k) & 1u)
+                        pairs[w][held + __popc(m & lanemask_lt())] = make_uint2(a, (out >> k) & 1u ? e[k] : root);
+                    held += __popc(m);
+                }
+                __syncwarp();
+                while (held >= 64) {
+                    held -= 64;
+                    ok = unite_pairs(p, &pairs[w][held], 64) && ok;
+                }
+            } else {
+                const uint32_t own = __shfl_sync(kFull, own_l, it);
+                bool act[kKeys];
+#pragma unroll
+                for (int k = 0; k < kKeys; ++k)
+                    act[k] = (keys >> k) & 1u;
+                if (last) {
+                    e[kKeys - 1] = own;
+                    act[kKeys - 1] = (live >> it) & 1u;
+                }
+                ok = group_union<kLanes, kKeys>(p, e, act, 1u << 20) && ok;
+            }
+        }
+    }
+    if (kBits && held)
+        ok = unite_pairs(p, pairs[w], held) && ok;
+    if (!ok)
+        *failed = 1;
+    count_add(g.st, kCtrWccSlabs, slabs);
+    count_add(g.st, kCtrWccEdges, __reduce_add_sync(kFull, edges));
+}
+
+namespace mk {
+
+template <bool kSet>
+static cudaError_t launch_static(const GView &g, uint32_t *p, uint32_t *label, uint32_t *bits, uint32_t *giant,
+                                 int *failed, cudaStream_t s, int *launches)
+{
+    const uint32_t vgrid = grid_for(g.V, 256);
+    const size_t bytes = ((size_t)g.V + 31) / 32 * 4;
+    // largest bitmap in shared memory, beside 50 KB of pairs
+    constexpr size_t kCcBitBytes = 160 << 10;
+    // A graph of few slabs is scanned in less time than the sample takes to
+    // launch.
+    if (g.H < kCcSampleLists) {
+        k_uf_init<<<vgrid, 256, 0, s>>>(p, g.V);
+        static const uint32_t grid = resident_grid(k_cc_scan<kSet, 0>, kScanThreads);
+        k_cc_scan<kSet, 0><<<grid, kScanThreads, 0, s>>>(g, p, nullptr, nullptr, failed);
+        *launches += 2;
+    } else {
+        k_cc_sample<kSet><<<vgrid, 256, 0, s>>>(g, p);
+        k_uf_compress<<<vgrid, 256, 0, s>>>(p, g.V, nullptr, nullptr, g.st);
+        k_cc_link<kSet><<<grid_for(g.V / kLinkStep + 1, 256), 256, 0, s>>>(g, p);
+        k_uf_compress<<<vgrid, 256, 0, s>>>(p, g.V, nullptr, nullptr, g.st);
+        k_cc_giant<<<1, 1024, 0, s>>>(p, g.V, giant);
+        k_cc_bits<<<vgrid, 256, 0, s>>>(p, g.V, giant, bits);
+        if (bytes <= kCcBitBytes) {
+            auto k = k_cc_scan<kSet, 1>;
+            cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+            if (e != cudaSuccess)
+                return e;
+            k<<<num_sms(), kScanThreads, bytes, s>>>(g, p, bits, giant, failed);
+        } else {
+            k_cc_scan<kSet, 2><<<num_sms(), kScanThreads, 0, s>>>(g, p, bits, giant, failed);
+        }
+        *launches += 7;
+    }
+    k_uf_compress<<<vgrid, 256, 0, s>>>(p, g.V, label, failed, g.st);
+    *launches += 1;
+    return cudaGetLastError();
+}
+
+cudaError_t static_components(const GView &g, bool set, uint32_t *p, uint32_t *label, uint32_t *bits, uint32_t *giant,
+                              int *failed, cudaStream_t s, int *launches)
+{
+    return set ? launch_static<true>(g, p, label, bits, giant, failed, s, launches)
+               : launch_static<false>(g, p, label, bits, giant, failed, s, launches);
+}
+
+} // namespace mk
 
 extern "C" mk_status mk_incr_wcc(mk_graph *g, uint32_t *d_label, void *stream)
 {
     if (!g)
         return MK_ERR_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)stream;
-    const uint32_t V = g->v.V, H = g->v.H;
+    const uint32_t V = g->v.V;
     auto key = std::make_pair((int)kWcc, 0u);
     Consumer *c = nullptr;
     auto it = g->consumers.find(key);
@@ -239,9 +489,12 @@ extern "C" mk_status mk_incr_wcc(mk_graph *g, uint32_t *d_label, void *stream)
         c->kind = kWcc;
         mk_status st = device_alloc(g, (void **)&c->uf, (size_t)V * 4);
         if (st == MK_OK)
+            st = device_alloc(g, (void **)&c->inv, ((size_t)V + 31) / 32 * 4);
+        if (st == MK_OK)
             st = device_alloc(g, (void **)&c->counters, kConsumerWords * 4);
         if (st != MK_OK) {
             device_free(g, c->uf, (size_t)V * 4);
+            device_free(g, c->inv, ((size_t)V + 31) / 32 * 4);
             device_free(g, c->counters, kConsumerWords * 4);
             delete c;
             return st;
@@ -256,38 +509,30 @@ extern "C" mk_status mk_incr_wcc(mk_graph *g, uint32_t *d_label, void *stream)
     int *failed = (int *)c->counters;
     MK_CUDA(cudaMemsetAsync(c->counters, 0, 64, s));
     if (!incremental) {
-        MK_TRY(timed(g, "wcc_init", s, 1, [&]() {
-            k_uf_init<<<grid_for(V, 256), 256, 0, s>>>(c->uf, V);
-            return cudaSuccess;
+        int launches = 0;
+        MK_TRY(timed(g, "wcc_static", s, 0, [&]() {
+            return static_components(g->v, false, c->uf, d_label, c->inv, c->counters + 1, failed, s, &launches);
         }));
-    }
-    if (incremental && g->ilog_ok && g->d_ilog) {
-        MK_TRY(timed(g, "wcc_hook_updated", s, 1, [&]() {
-            const uint64_t threads = std::max<uint64_t>(g->ilog_bound, 1);
-            k_uf_hook_log<<<std::min<uint32_t>(grid_for(threads, 256), num_sms() * 8), 256, 0, s>>>(
-                g->d_state, g->d_ilog, g->ilog_bound, c->uf, failed);
-            return cudaSuccess;
-        }));
-    } else if (incremental) {
-        MK_TRY(timed(g, "wcc_hook_updated", s, 1, [&]() {
-            // one 4-lane group per logged list
-            const uint64_t threads = std::max<uint64_t>(g->ulog_bound, 1) * 4;
-            k_uf_hook<<<std::min<uint32_t>(grid_for(threads, 256), num_sms() * 12), 256, 0, s>>>(g->v, c->uf, max_hops,
-                                                                                               failed);
-            return cudaSuccess;
-        }));
+        g->launches += (uint64_t)launches;
     } else {
-        MK_TRY(timed(g, "wcc_hook_all", s, 1, [&]() {
-            static const uint32_t grid = resident_grid(k_uf_hook_slabs, 256);
-            k_uf_hook_slabs<<<grid, 256, 0, s>>>(g->v, c->uf, failed);
+        MK_TRY(timed(g, "wcc_hook_updated", s, 1, [&]() {
+            if (g->ilog_ok && g->d_ilog) {
+                const uint64_t threads = std::max<uint64_t>(g->ilog_bound, 1);
+                k_uf_hook_log<<<std::min<uint32_t>(grid_for(threads, 256), num_sms() * 8), 256, 0, s>>>(
+                    g->d_state, g->d_ilog, g->ilog_bound, c->uf, failed);
+            } else {
+                // one 4-lane group per logged list
+                const uint64_t threads = std::max<uint64_t>(g->ulog_bound, 1) * 4;
+                k_uf_hook<<<std::min<uint32_t>(grid_for(threads, 256), num_sms() * 12), 256, 0, s>>>(
+                    g->v, c->uf, max_hops, failed);
+            }
+            return cudaSuccess;
+        }));
+        MK_TRY(timed(g, "wcc_compress", s, 1, [&]() {
+            k_uf_compress<<<grid_for(V, 256), 256, 0, s>>>(c->uf, V, d_label, failed, g->d_state);
             return cudaSuccess;
         }));
     }
-    MK_TRY(timed(g, "wcc_compress", s, 2, [&]() {
-        k_uf_compress<<<grid_for(V, 256), 256, 0, s>>>(c->uf, V, d_label);
-        k_uf_failed<<<1, 1, 0, s>>>(failed, g->d_state);
-        return cudaSuccess;
-    }));
     c->epoch = g->epoch;
     c->seq = g->change_seq;
     return MK_OK;

@@ -243,3 +243,35 @@ def test_frontier_staging_limits(cuda_lib, delta):
     o.delete(s[: V // 2], d[: V // 2])
     check_algos(g, o, [0])
     g.close()
+
+
+@pytest.mark.parametrize("store", ["map", "set"])
+@pytest.mark.parametrize("V", [600, 20000, 1500000])  # no sample; bitmap in shared memory; in global memory
+@pytest.mark.parametrize("shape", ["giant", "many", "path"])
+def test_static_components(cuda_lib, store, V, shape):
+    """Static components with one giant tree, with many small ones, and along
+    a path, ids in no order, then after deletes."""
+    mk = _mk()
+    rng = np.random.default_rng(V + len(shape))
+    name = rng.permutation(V).astype(np.uint32)
+    if shape == "path":
+        s, d = np.arange(V - 1), np.arange(1, V)
+    else:
+        n = V if shape == "giant" else V // 3
+        s, d = rng.integers(0, V, n), rng.integers(0, V, n)
+    s, d = name[s], name[d]
+    o = oracle.OracleGraph(V)
+    o.insert(s, d, np.ones(len(s), np.uint32))
+    if store == "map":
+        g = mk.Graph(V, edge_capacity_hint=2 * len(s), buckets=1)
+        g.insert(s, d, np.ones(len(s), np.uint32))
+    else:
+        g = mk.SetGraph(V, edge_capacity_hint=2 * len(s), buckets=1)
+        g.insert(s, d)
+    assert np.array_equal(mk.to_numpy_u32(g.wcc()), o.wcc())
+    cut = rng.permutation(len(s))[: len(s) // 4]
+    g.delete(s[cut], d[cut])
+    o.delete(s[cut], d[cut])
+    assert np.array_equal(mk.to_numpy_u32(g.wcc()), o.wcc())
+    assert g.last_error() == mk.MK_OK
+    g.close()
