@@ -164,36 +164,59 @@ __global__ void k_pr_out(const unsigned long long *pr, uint32_t V, float *out)
 
 namespace {
 
-// Whether edge (u, w) is in g: the lane walks the chain of w's bucket among
-// u's buckets, eight 16-byte loads per slab issued together.
-__device__ __forceinline__ bool lane_has_edge(const GView &g, uint32_t u, uint32_t w, uint32_t max_hops)
+// How many of the warp's n keys (in shared memory) are neighbours of a vertex
+// with index entry vi in g: the groups' tally, one count a found key on one
+// lane of its group.  Each 4-lane group walks the chain of one key's bucket,
+// 32 bytes of a slab a lane, two keys in flight; a lane reading whole slabs by
+// itself touched four times as many lines a load (the load pipe 57 % busy).
+__device__ __forceinline__ uint32_t count_neighbours(const GView &g, uint2 vi, const uint32_t *keys, uint32_t n,
+                                                     uint32_t max_hops)
 {
-    const uint2 vi = __ldg(&g.vinfo[u]);
-    uint32_t slab = vi.x + bucket_of(w, vi.y);
-    for (uint32_t hop = 0; hop < max_hops && slab != kNil; ++hop) {
-        const uint4 *p = reinterpret_cast<const uint4 *>(slab_ptr(g, slab));
-        uint4 x[8];
+    const uint32_t lane = lane_id(), gi = lane >> 2, s4 = lane & 3u, gbase = lane & ~3u;
+    uint32_t count = 0;
+    for (uint32_t base = 0; base < n; base += 16) {
+        uint32_t key[2], slab[2];
 #pragma unroll
-        for (int q = 0; q < 8; ++q)
-            x[q] = __ldcg(p + q);
-        bool hit = false;
+        for (uint32_t h = 0; h < 2; ++h) {
+            const uint32_t k = base + 8 * h + gi;
+            key[h] = k < n ? keys[k] : kNil;
+            slab[h] = k < n ? vi.x + bucket_of(key[h], vi.y) : kNil;
+        }
+        for (uint32_t hop = 0; __any_sync(kFull, slab[0] != kNil || slab[1] != kNil); ++hop) {
+            uint4 lo[2], hi[2];
 #pragma unroll
-        for (int q = 0; q < 8; ++q)
-            hit |= x[q].x == w || (q < 7 && x[q].z == w);
-        if (hit)
-            return true;
-        slab = x[7].w;
+            for (uint32_t h = 0; h < 2; ++h) {
+                lo[h] = make_uint4(kEmptyKey, 0u, kEmptyKey, 0u);
+                hi[h] = make_uint4(kEmptyKey, 0u, kEmptyKey, kNil);
+                if (slab[h] != kNil) {
+                    const uint4 *p = reinterpret_cast<const uint4 *>(slab_ptr(g, slab[h]) + s4 * 8);
+                    lo[h] = __ldcg(p);
+                    hi[h] = __ldcg(p + 1);
+                }
+            }
+#pragma unroll
+            for (uint32_t h = 0; h < 2; ++h) {
+                const bool hit = slab[h] != kNil && (lo[h].x == key[h] || lo[h].z == key[h] || hi[h].x == key[h] ||
+                                                     (s4 != 3u && hi[h].z == key[h]));
+                count += hit;
+                const bool found = (__ballot_sync(kFull, hit) >> gbase) & 0xFu;
+                const uint32_t nxt = __shfl_sync(kFull, hi[h].w, gbase + 3);
+                slab[h] = found || hop + 1 >= max_hops ? kNil : slab[h] != kNil ? nxt : kNil;
+            }
+        }
     }
-    return false;
+    return count;
 }
 
 // |N_g1(u) ∩ N_g2(v)| spread over the warp's lanes (each lane returns its
 // share; the full warp calls it with warp-uniform u, v).  The side with
-// fewer buckets is walked (one list: slab by slab, a word a lane; several:
-// eight lists at a time in 4-lane groups) and each key lane searches the
-// other side for its neighbour.
+// fewer buckets is walked, eight lists at a time in 4-lane groups (one list,
+// slab by slab, by the first group alone), its keys collected in `keys`
+// (kTcKeys words of the warp), and looked up in the other side.
+constexpr uint32_t kTcKeys = 8 * kPairs;
+
 __device__ __forceinline__ uint32_t warp_edge_count(const GView &g1, const GView &g2, uint32_t u, uint32_t v,
-                                                    uint32_t mh1, uint32_t mh2, unsigned long long &slabs)
+                                                    uint32_t mh1, uint32_t mh2, uint32_t *keys)
 {
     const uint32_t lane = lane_id();
     const uint2 vu = __ldg(&g1.vinfo[u]), vv = __ldg(&g2.vinfo[v]);
@@ -201,50 +224,33 @@ __device__ __forceinline__ uint32_t warp_edge_count(const GView &g1, const GView
     const bool walk_u = vu.y < vv.y;
     const GView &gw = walk_u ? g1 : g2;
     const GView &gs = walk_u ? g2 : g1;
-    const uint2 vw = walk_u ? vu : vv;
-    const uint32_t probe = walk_u ? v : u;
+    const uint2 vw = walk_u ? vu : vv, vs = walk_u ? __ldg(&g2.vinfo[v]) : __ldg(&g1.vinfo[u]);
     const uint32_t mh = walk_u ? mh1 : mh2, mhs = walk_u ? mh2 : mh1;
-    uint32_t count = 0;
-    if (vw.y == 1) {
-        // one list: the warp reads it slab by slab, one word a lane
-        uint32_t slab = vw.x;
-        for (uint32_t hop = 0; hop < mh && slab != kNil; ++hop) {
-            const uint32_t word = __ldcg(slab_ptr(gw, slab) + lane);
-            ++slabs;
-            if (is_key_lane(lane) && word < kTombKey)
-                count += lane_has_edge(gs, probe, word, mhs) ? 1u : 0u;
-            slab = __shfl_sync(kFull, word, kNextLane);
-        }
-        return count;
-    }
-    // several lists: eight at a time, one per 4-lane group (bucket b by
-    // group b % 8), each lane holding 32 bytes of the slab (four pairs; the
-    // group's last lane three and the unused and next words)
     const uint32_t g4 = lane >> 2, s4 = lane & 3u, gbase = lane & ~3u;
+    uint32_t count = 0;
     for (uint32_t b0 = 0; b0 < vw.y; b0 += 8) {
         uint32_t slab = b0 + g4 < vw.y ? vw.x + b0 + g4 : kNil;
-        bool active = slab != kNil;
-        for (uint32_t hop = 0; __any_sync(kFull, active); ++hop) {
-            uint4 lo = make_uint4(kEmptyKey, 0u, kEmptyKey, 0u), hi = lo;
-            if (active) {
+        for (uint32_t hop = 0; __any_sync(kFull, slab != kNil); ++hop) {
+            uint4 lo = make_uint4(kEmptyKey, 0u, kEmptyKey, 0u), hi = make_uint4(kEmptyKey, 0u, kEmptyKey, kNil);
+            if (slab != kNil) {
                 const uint4 *q = reinterpret_cast<const uint4 *>(slab_ptr(gw, slab) + s4 * 8);
                 lo = __ldcg(q);
                 hi = __ldcg(q + 1);
-                if (s4 == 0)
-                    ++slabs;
             }
             const uint32_t key[4] = {lo.x, lo.z, hi.x, s4 == 3u ? kEmptyKey : hi.z};
+            uint32_t n = 0;
 #pragma unroll
-            for (int k = 0; k < 4; ++k)
-                if (active && key[k] < kTombKey)
-                    count += lane_has_edge(gs, probe, key[k], mhs) ? 1u : 0u;
-            const uint32_t nxt = __shfl_sync(kFull, hi.w, gbase + 3);
-            if (active) {
-                if (nxt == kNil || hop + 1 >= mh)
-                    active = false;
-                else
-                    slab = nxt;
+            for (int k = 0; k < 4; ++k) {
+                const uint32_t m = __ballot_sync(kFull, key[k] < kTombKey);
+                if (key[k] < kTombKey)
+                    keys[n + __popc(m & lanemask_lt())] = key[k];
+                n += __popc(m);
             }
+            __syncwarp();
+            count += count_neighbours(gs, vs, keys, n, mhs);
+            __syncwarp();
+            const uint32_t nxt = __shfl_sync(kFull, hi.w, gbase + 3);
+            slab = slab == kNil || hop + 1 >= mh ? kNil : nxt;
         }
     }
     return count;
@@ -261,8 +267,9 @@ __global__ void __launch_bounds__(256) k_tc_count(GView g1, GView g2, const uint
                                                   uint32_t mh2, unsigned long long *total,
                                                   unsigned long long *next)
 {
+    __shared__ uint32_t keys[8][kTcKeys];
     const uint32_t lane = lane_id();
-    unsigned long long count = 0, slabs = 0;
+    unsigned long long count = 0;
     for (;;) {
         unsigned long long e = 0;
         if (lane == 0)
@@ -276,7 +283,7 @@ __global__ void __launch_bounds__(256) k_tc_count(GView g1, GView g2, const uint
                 set_status(g1.st, kErrInvalid);
             continue;
         }
-        count += warp_edge_count(g1, g2, u, v, mh1, mh2, slabs);
+        count += warp_edge_count(g1, g2, u, v, mh1, mh2, keys[threadIdx.x >> 5]);
     }
     warp_add_u64(total, count);
 }
@@ -294,48 +301,286 @@ __device__ __forceinline__ unsigned long long tc_rank(uint32_t buckets, uint32_t
 } // namespace
 
 // Static count, each triangle once: with the vertices ranked by tc_rank, a
-// triangle a < b < c is counted on its edge (a, b) as the common neighbour
-// c.  One warp per slab in use (address order, owner u); each live edge
-// (u, v) with rank(u) < rank(v) walks N(u) (u ranks lower, so it has no
-// more buckets than v) slab by slab, and a key lane w with rank(w) > rank(v)
-// looks (v, w) up.  Needs both directions of every edge stored.
-__global__ void __launch_bounds__(256) k_tc_static(GView g, uint32_t mh, unsigned long long *total)
+// triangle a < b < c is counted on its edge (a, b) as the common neighbour c.
+// The edges u -> v with rank(u) < rank(v) are first copied out of the slabs
+// into one array, vertex by vertex (N+(u)); then, for every u, N+(u) becomes a
+// hash set in shared memory, and N+(v) of each v in it is streamed past that
+// set: sum over u and v in N+(u) of |N+(u) and N+(v)|.  A test of a streamed
+// neighbour moves 4 bytes and looks at one or two words of shared memory; a
+// search of v's slab chain for it moved 128 bytes from L2 (R-MAT scale 17,
+// 1.9 M undirected edges, 251 M tests: 7.7 ms, 0.6 so).
+
+namespace {
+
+constexpr uint32_t kTcWarp = 32;         // N+(u) of at most this many: one warp, else one block
+constexpr uint32_t kTcWarpBits = 8;      // a warp's set: 2^8 words, an eighth full at most
+constexpr uint32_t kTcBlockKeys = 1024;  // neighbours of one pass of a block
+constexpr uint32_t kTcBlockBits = 13;    // a block's set: up to 2^13 words, an eighth full at most
+constexpr uint32_t kTcThreads = 256;
+
+struct TcArrays {
+    uint32_t *cnt;             // |N+(u)|
+    uint32_t *fill;            // neighbours written so far
+    ulonglong2 *list;          // N+(u) at adj[list[u].x], list[u].y of them
+    uint32_t *large;           // vertices with more than kTcWarp
+    unsigned long long *ctr;   // neighbours in all, vertices in `large`, taken from it, triangles
+    uint32_t *adj;
+};
+enum { kTcTotal = 0, kTcLarge = 1, kTcNext = 2, kTcTriangles = 3, kTcWords = 4 };
+
+__device__ __forceinline__ uint32_t tc_hash(uint32_t x) { return x * 0x9E3779B1u; }
+
+// Enters x in the set of 2^bits words (free words kNil).
+__device__ __forceinline__ void tc_enter(uint32_t *set, uint32_t bits, uint32_t x)
 {
-    const uint32_t lane = lane_id();
-    const uint64_t all = (uint64_t)g.H + g.P;
-    const uint64_t stride = ((uint64_t)gridDim.x * blockDim.x) >> 5;
-    unsigned long long count = 0;
-    for (uint64_t s = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5; s < all; s += stride) {
-        const uint32_t u = __ldg(&g.owner[s]);
-        if (u == kNil)
-            continue;
-        const uint2 vu = __ldg(&g.vinfo[u]);
-        const unsigned long long ru = tc_rank(vu.y, u);
-        const uint32_t word = __ldcg(slab_ptr(g, (uint32_t)s) + lane);
-        bool up = false;
-        unsigned long long rv = 0;
-        if (is_key_lane(lane) && word < kTombKey) {
-            rv = tc_rank(__ldg(&g.vinfo[word]).y, word);
-            up = rv > ru;
+    uint32_t h = tc_hash(x) >> (32 - bits);
+    while (atomicCAS(&set[h], kNil, x) != kNil)
+        h = (h + 1) & ((1u << bits) - 1);
+}
+
+// Streams N+(v) of the vertices v = row[j], j = first, first + step, ... below
+// c, past `lanes` lanes of which the caller is `sub`: test(x) is called with
+// the lane's next four neighbours (kNil past a list's end).  A list's place is
+// read while the list before it is streamed.
+template <typename Test>
+__device__ __forceinline__ void tc_stream(const TcArrays &t, const uint32_t *row, uint32_t first, uint32_t c,
+                                          uint32_t step, uint32_t sub, uint32_t lanes, Test &&test)
+{
+    uint32_t j = first;
+    ulonglong2 next = j < c ? __ldg(&t.list[row[j]]) : make_ulonglong2(0, 0);
+    for (; j < c; j += step) {
+        const uint32_t *list = t.adj + next.x;
+        const uint32_t n = (uint32_t)next.y;
+        if (j + step < c)
+            next = __ldg(&t.list[row[j + step]]);
+        for (uint32_t i = sub; i < n; i += 4 * lanes) {
+            uint32_t x[4];
+#pragma unroll
+            for (uint32_t k = 0; k < 4; ++k)
+                x[k] = i + k * lanes < n ? __ldg(list + i + k * lanes) : kNil;
+            test(x);
         }
-        uint32_t todo = __ballot_sync(kFull, up);
-        while (todo) {
-            const uint32_t j = __ffs(todo) - 1;
-            todo &= todo - 1;
-            const uint32_t v = __shfl_sync(kFull, word, j);
-            const unsigned long long rvj = __shfl_sync(kFull, rv, j);
-            for (uint32_t b = 0; b < vu.y; ++b) {
-                uint32_t slab = vu.x + b;
-                for (uint32_t hop = 0; hop < mh && slab != kNil; ++hop) {
-                    const uint32_t w = __ldcg(slab_ptr(g, slab) + lane);
-                    if (is_key_lane(lane) && w < kTombKey && tc_rank(__ldg(&g.vinfo[w]).y, w) > rvj)
-                        count += lane_has_edge(g, v, w, mh) ? 1u : 0u;
-                    slab = __shfl_sync(kFull, w, kNextLane);
+    }
+}
+
+// Bit of vertex x in a bitmap over 2^bits vertices, as <word, bit>: an odd
+// multiple modulo 2^bits and a fold, both one to one.  The vertices tested
+// most are a power-law graph's hubs, whose ids share most of their bits; by id
+// a load of 32 words met 8.8 of them in one bank.
+__device__ __forceinline__ uint2 tc_bit(uint32_t x, uint32_t bits)
+{
+    const uint32_t y = (x * 0x9E3779B1u) & (uint32_t)((1ull << bits) - 1), word = y >> 5;
+    return make_uint2(word ^ (word >> 5), y & 31u);
+}
+
+// How many of x are in the hash set: four first probes in flight; the few
+// that meet another key there go on one by one.
+__device__ __forceinline__ uint32_t tc_probe(const uint32_t *set, uint32_t bits, const uint32_t (&x)[4])
+{
+    const uint32_t mask = (1u << bits) - 1, shift = 32 - bits;
+    uint32_t k[4], more = 0, count = 0;
+#pragma unroll
+    for (uint32_t j = 0; j < 4; ++j)
+        k[j] = set[tc_hash(x[j]) >> shift];
+#pragma unroll
+    for (uint32_t j = 0; j < 4; ++j) {
+        count += k[j] == x[j] && x[j] != kNil;
+        more |= (k[j] != x[j] && k[j] != kNil && x[j] != kNil ? 1u : 0u) << j;
+    }
+    while (more) {
+        const uint32_t j = __ffs(more) - 1;
+        more &= more - 1;
+        const uint32_t y = j == 0 ? x[0] : j == 1 ? x[1] : j == 2 ? x[2] : x[3];
+        uint32_t h = ((tc_hash(y) >> shift) + 1) & mask, key = set[h];
+        while (key != y && key != kNil) {
+            h = (h + 1) & mask;
+            key = set[h];
+        }
+        count += key == y;
+    }
+    return count;
+}
+
+} // namespace
+
+// One pass over the slabs in use, eight lanes a slab (16 bytes a lane):
+// counts the neighbours that rank above their slab's owner, or (kFill) writes
+// them to N+(owner), one atomic a slab.
+template <bool kFill>
+__global__ void __launch_bounds__(kTcThreads) k_tc_orient(GView g, TcArrays t)
+{
+    const uint64_t all = (uint64_t)g.H + g.P, stride = ((uint64_t)gridDim.x * kTcThreads) >> 3;
+    const uint32_t lane = lane_id(), part = lane & 7u, first = lane & ~7u;
+    const uint64_t s0 = (blockIdx.x * (uint64_t)kTcThreads + threadIdx.x) >> 3;
+    for (uint64_t sb = s0 & ~3ull; sb < all; sb += stride) { // the warp's four slabs
+        const uint64_t s = sb + (lane >> 3);
+        const uint32_t u = s < all ? __ldg(&g.owner[s]) : kNil;
+        uint4 q = make_uint4(kEmptyKey, 0u, kEmptyKey, 0u);
+        unsigned long long ru = ~0ull;
+        if (u != kNil) {
+            q = __ldcg(reinterpret_cast<const uint4 *>(slab_ptr(g, (uint32_t)s)) + part);
+            ru = tc_rank(__ldg(&g.vinfo[u]).y, u);
+        }
+        const bool up0 = q.x < kTombKey && tc_rank(__ldg(&g.vinfo[q.x]).y, q.x) > ru;
+        const bool up1 = part != 7u && q.z < kTombKey && tc_rank(__ldg(&g.vinfo[q.z]).y, q.z) > ru;
+        const uint32_t m0 = (__ballot_sync(kFull, up0) >> first) & 0xFFu;
+        const uint32_t m1 = (__ballot_sync(kFull, up1) >> first) & 0xFFu;
+        const uint32_t n0 = __popc(m0), n = n0 + __popc(m1);
+        if (!kFill) {
+            if (part == 0 && n)
+                atomicAdd(&t.cnt[u], n);
+            continue;
+        }
+        uint32_t base = 0;
+        if (part == 0 && n)
+            base = atomicAdd(&t.fill[u], n);
+        base = __shfl_sync(kFull, base, first);
+        if (n) {
+            uint32_t *to = t.adj + t.list[u].x + base;
+            const uint32_t lt = (1u << part) - 1;
+            if (up0)
+                to[__popc(m0 & lt)] = q.x;
+            if (up1)
+                to[n0 + __popc(m1 & lt)] = q.z;
+        }
+    }
+}
+
+// The vertices' places in adj, in blocks of vertices, and the large ones.
+__global__ void __launch_bounds__(kTcThreads) k_tc_place(TcArrays t, uint32_t V)
+{
+    __shared__ uint32_t s_warp[kTcThreads / 32];
+    __shared__ unsigned long long s_base;
+    const uint32_t v = blockIdx.x * kTcThreads + threadIdx.x, lane = lane_id();
+    const uint32_t c = v < V ? t.cnt[v] : 0u;
+    uint32_t incl = c;
+#pragma unroll
+    for (uint32_t o = 1; o < 32; o <<= 1) {
+        const uint32_t x = __shfl_up_sync(kFull, incl, o);
+        if (lane >= o)
+            incl += x;
+    }
+    if (lane == 31)
+        s_warp[threadIdx.x >> 5] = incl;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        uint32_t sum = 0;
+        for (uint32_t k = 0; k < kTcThreads / 32; ++k) {
+            const uint32_t x = s_warp[k];
+            s_warp[k] = sum;
+            sum += x;
+        }
+        s_base = sum ? atomicAdd(&t.ctr[kTcTotal], (unsigned long long)sum) : 0ull;
+    }
+    __syncthreads();
+    if (v < V)
+        t.list[v] = make_ulonglong2(s_base + s_warp[threadIdx.x >> 5] + incl - c, c);
+    const uint32_t m = __ballot_sync(kFull, c > kTcWarp);
+    unsigned long long base = 0;
+    if (m && lane == 0)
+        base = atomicAdd(&t.ctr[kTcLarge], (unsigned long long)__popc(m));
+    base = __shfl_sync(kFull, base, 0);
+    if (c > kTcWarp)
+        t.large[base + __popc(m & lanemask_lt())] = v;
+}
+
+// Vertices with 2 to kTcWarp neighbours above them, one a warp, four of the
+// streamed lists at a time.
+__global__ void __launch_bounds__(kTcThreads) k_tc_small(TcArrays t, uint32_t V)
+{
+    __shared__ uint32_t sets[kTcThreads / 32][1u << kTcWarpBits], rows[kTcThreads / 32][kTcWarp];
+    static_assert(8 * kTcWarp <= 1u << kTcWarpBits, "an eighth full");
+    const uint32_t lane = lane_id(), w = threadIdx.x >> 5, sub = lane & 7u;
+    uint32_t *set = sets[w], *row = rows[w];
+    unsigned long long count = 0;
+    const uint32_t stride = (gridDim.x * kTcThreads) >> 5;
+    for (uint64_t u = (blockIdx.x * kTcThreads + threadIdx.x) >> 5; u < V; u += stride) {
+        const ulonglong2 mine = __ldg(&t.list[u]);
+        const uint32_t c = (uint32_t)mine.y;
+        if (c < 2 || c > kTcWarp)
+            continue;
+#pragma unroll
+        for (uint32_t i = 0; i < 1u << kTcWarpBits; i += 32)
+            set[i + lane] = kNil;
+        __syncwarp();
+        if (lane < c) {
+            row[lane] = __ldg(t.adj + mine.x + lane);
+            tc_enter(set, kTcWarpBits, row[lane]);
+        }
+        __syncwarp();
+        tc_stream(t, row, lane >> 3, c, 4, sub, 8,
+                  [&](const uint32_t(&x)[4]) { count += tc_probe(set, kTcWarpBits, x); });
+        __syncwarp();
+    }
+    warp_add_u64(&t.ctr[kTcTriangles], count);
+}
+
+// The vertices with more, one a block at a time (taken from a counter: their
+// work differs), the streamed lists one a warp.  With kMap the set is a bitmap
+// over all vertices (dynamic shared memory): a test is one load and a shift,
+// 10 instructions where the hash set takes 54 and is bound by them (R-MAT
+// scale 17: 329 -> 224 us).
+template <bool kMap>
+__global__ void __launch_bounds__(1024) k_tc_large(TcArrays t, uint32_t vbits)
+{
+    extern __shared__ uint32_t set[]; // kMap: 2^vbits bits, else 2^kTcBlockBits words
+    static_assert(8 * kTcBlockKeys <= 1u << kTcBlockBits, "an eighth full");
+    __shared__ unsigned long long s_next;
+    const uint32_t lane = lane_id(), w = threadIdx.x >> 5, warps = blockDim.x >> 5;
+    const unsigned long long n = t.ctr[kTcLarge];
+    unsigned long long count = 0;
+    if (kMap)
+        for (uint32_t i = threadIdx.x; i < (1u << vbits) / 32; i += blockDim.x)
+            set[i] = 0;
+    for (;;) {
+        __syncthreads();
+        if (threadIdx.x == 0)
+            s_next = atomicAdd(&t.ctr[kTcNext], 1ull);
+        __syncthreads();
+        if (s_next >= n)
+            break;
+        const ulonglong2 list = __ldg(&t.list[t.large[s_next]]);
+        const uint32_t c = (uint32_t)list.y, *mine = t.adj + list.x;
+        const uint32_t pass = kMap ? c : kTcBlockKeys;
+        for (uint32_t at = 0; at < c; at += pass) {
+            const uint32_t m = min(c - at, pass);
+            const uint32_t bits = 32 - __clz(8 * m - 1);
+            if (!kMap) {
+                __syncthreads();
+                for (uint32_t i = threadIdx.x; i < 1u << bits; i += blockDim.x)
+                    set[i] = kNil;
+                __syncthreads();
+            }
+            for (uint32_t i = threadIdx.x; i < m; i += blockDim.x) {
+                const uint32_t x = __ldg(mine + at + i);
+                const uint2 b = tc_bit(x, vbits);
+                if (kMap)
+                    atomicOr(&set[b.x], 1u << b.y);
+                else
+                    tc_enter(set, bits, x);
+            }
+            __syncthreads();
+            uint32_t found = 0;
+            tc_stream(t, mine, w, c, warps, lane, 32, [&](const uint32_t(&x)[4]) {
+                if (!kMap) {
+                    found += tc_probe(set, bits, x);
+                    return;
                 }
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const uint2 at = tc_bit(x[k], vbits);
+                    found += x[k] != kNil ? (set[at.x] >> at.y) & 1u : 0u;
+                }
+            });
+            count += found;
+            if (kMap) {
+                __syncthreads();
+                for (uint32_t i = threadIdx.x; i < m; i += blockDim.x)
+                    set[tc_bit(__ldg(mine + i), vbits).x] = 0;
             }
         }
     }
-    warp_add_u64(total, count);
+    warp_add_u64(&t.ctr[kTcTriangles], count);
 }
 
 // ---------------------------------------------------------------- host side
@@ -437,18 +682,72 @@ mk_status mk_tc_static(mk_graph *g, uint64_t *h_triangles, void *stream)
     if (!g || !h_triangles)
         return MK_ERR_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)stream;
-    unsigned long long *d = nullptr;
-    MK_CUDA(cudaMallocAsync((void **)&d, 8, s));
-    MK_CUDA(cudaMemsetAsync(d, 0, 8, s));
-    mk_status st = timed(g, "tc_static", s, 1, [&]() {
-        k_tc_static<<<resident_grid(k_tc_static, 256), 256, 0, s>>>(g->v, g->v.P + 2, d);
-        return cudaSuccess;
-    });
+    const uint64_t V = g->v.V;
+    // the per-vertex arrays in one block, the neighbours (as many as there
+    // are, read back first) in another
+    unsigned char *block = nullptr;
+    const size_t bytes = V * (16 + 4 + 4 + 4) + kTcWords * 8;
+    MK_CUDA(cudaMallocAsync((void **)&block, bytes, s));
+    TcArrays t{};
+    t.list = (ulonglong2 *)block;
+    t.ctr = (unsigned long long *)(t.list + V);
+    t.cnt = (uint32_t *)(t.ctr + kTcWords);
+    t.fill = t.cnt + V;
+    t.large = t.fill + V;
+    const uint32_t slab_grid = resident_grid(k_tc_orient<false>, kTcThreads);
     unsigned long long total = 0;
-    if (st == MK_OK && (cudaMemcpyAsync(&total, d, 8, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-                        cudaStreamSynchronize(s) != cudaSuccess))
-        st = MK_ERR_CUDA;
-    cudaFreeAsync(d, s);
+    mk_status st = MK_OK;
+    auto cuda = [&](cudaError_t e) {
+        if (st == MK_OK && e != cudaSuccess)
+            st = e == cudaErrorMemoryAllocation ? MK_ERR_NO_MEMORY : MK_ERR_CUDA;
+        return st == MK_OK;
+    };
+    if (cuda(cudaMemsetAsync(t.ctr, 0, kTcWords * 8 + V * 8, s)))
+        st = timed(g, "tc_orient", s, 2, [&]() {
+            k_tc_orient<false><<<slab_grid, kTcThreads, 0, s>>>(g->v, t);
+            k_tc_place<<<grid_for(V, kTcThreads), kTcThreads, 0, s>>>(t, (uint32_t)V);
+            return cudaSuccess;
+        });
+    if (st == MK_OK)
+        cuda(cudaMemcpyAsync(&total, t.ctr + kTcTotal, 8, cudaMemcpyDeviceToHost, s));
+    if (st == MK_OK)
+        cuda(cudaStreamSynchronize(s));
+    if (st == MK_OK && total) {
+        if (cuda(cudaMallocAsync((void **)&t.adj, total * 4, s)))
+            st = timed(g, "tc_static", s, 3, [&]() {
+                k_tc_orient<true><<<slab_grid, kTcThreads, 0, s>>>(g->v, t);
+                // a bitmap of up to 128 KB (2^20 vertices), with blocks large
+                // enough that those an SM holds fill it
+                uint32_t vbits = 5;
+                while (vbits < 32 && (1ull << vbits) < V)
+                    ++vbits;
+                const size_t map = (1ull << vbits) / 8;
+                const bool use_map = map <= 128u << 10;
+                const size_t smem = use_map ? map : sizeof(uint32_t) << kTcBlockBits;
+                const int threads = smem <= 24u << 10 ? 256 : smem <= 48u << 10 ? 512 : 1024;
+                const void *k = use_map ? (const void *)k_tc_large<true> : (const void *)k_tc_large<false>;
+                int per = 0;
+                cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                if (e == cudaSuccess)
+                    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, threads, smem);
+                if (e != cudaSuccess)
+                    return e;
+                void *args[] = {&t, &vbits};
+                e = cudaLaunchKernel(k, dim3(num_sms() * std::max(per, 1)), dim3(threads), args, smem, s);
+                if (e != cudaSuccess)
+                    return e;
+                k_tc_small<<<resident_grid(k_tc_small, kTcThreads), kTcThreads, 0, s>>>(t, (uint32_t)V);
+                return cudaSuccess;
+            });
+        total = 0;
+        if (st == MK_OK)
+            cuda(cudaMemcpyAsync(&total, t.ctr + kTcTriangles, 8, cudaMemcpyDeviceToHost, s));
+        if (st == MK_OK)
+            cuda(cudaStreamSynchronize(s));
+        if (t.adj)
+            cudaFreeAsync(t.adj, s);
+    }
+    cudaFreeAsync(block, s);
     *h_triangles = total;
     return st;
 }

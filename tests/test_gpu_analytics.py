@@ -142,3 +142,28 @@ def test_analytics_degenerate_graphs(cuda_lib):
     assert grid.last_error() == mk.MK_OK
     upd.close()
     grid.close()
+
+
+@pytest.mark.parametrize("V", [5000, (1 << 20) + 9])  # bitmaps, hash sets
+@pytest.mark.parametrize("buckets", [1, "rule"])
+def test_triangles_neighbourhood_sizes(cuda_lib, V, buckets):
+    """Vertices with 2 to 1,500 neighbours ranked above them (one warp up to
+    32, then one block, which takes hash sets 1,024 at a time): a clique of 90,
+    a hub joined to 1,500 vertices, sparse edges among those."""
+    mk = _mk()
+    rng = np.random.default_rng(V)
+    name = np.sort(rng.choice(V, 1600, replace=False)).astype(np.uint32)
+    i, j = np.triu_indices(90, 1)
+    a = [i, np.zeros(1500, np.int64), rng.integers(0, 1600, 6000)]
+    b = [j, np.arange(1, 1501), rng.integers(0, 1600, 6000)]
+    pairs = np.unique(np.sort(np.stack([np.concatenate(a), np.concatenate(b)], 1), 1), axis=0)
+    s, d = _undirected(name[pairs[:, 0]], name[pairs[:, 1]])
+    o = oracle.OracleGraph(V)
+    o.insert(s, d, np.ones(len(s), np.uint32))
+    nb = 1 if buckets == 1 else mk.bucket_rule(V, s, 0.7)
+    g = mk.Graph(V, edge_capacity_hint=2 * len(s), buckets=nb)
+    g.insert(s, d)
+    g.commit()
+    assert g.triangles() == o.triangles()
+    assert g.last_error() == mk.MK_OK
+    g.close()
