@@ -5,16 +5,19 @@
 // the Count kernel).
 //
 // PageRank.  The paper's Compute kernel pulls over a graph object that
-// stores in-edges; this store keeps out-edges, so each super-step pushes
-// instead: every live edge u -> v adds u's contribution PR[u] / out[u] to
-// v's accumulator, reading the slab array in address order (the per-slab
-// owner names u), which keeps every slab read coalesced.  To make the pushes
-// order-independent the ranks, contributions and accumulators are 64-bit
-// fixed-point numbers (value * 2^48) added with integer atomics, so a
-// result does not depend on the order in which the atomics land; the L1
-// delta of a super-step is summed the same way.  The teleport term for
-// zero-out-degree vertices is added as in the paper (FindTeleportProb).
-// The host reads the delta after every super-step, as in the paper's loop.
+// stores in-edges; this store keeps out-edges.  A call first copies its live
+// edges out of the slabs into bins by destination, so that each super-step
+// reads them in order and adds u's contribution PR[u] / out[u] up in shared
+// memory for every edge u -> v of a bin.  Graphs and calls for which the copy
+// does not pay (more than 2^24 vertices, fewer than four super-steps, no
+// memory for it) push along the slabs instead, in address order.  Ranks,
+// contributions and sums are 64-bit fixed-point numbers (value * 2^48) added
+// as integers, so a result does not depend on the order of the additions, nor
+// on which of the two forms runs; the L1 delta of a super-step is summed the
+// same way.  The teleport term for zero-out-degree vertices is added as in
+// the paper (FindTeleportProb).  The super-steps test the delta themselves;
+// the host, which reads it after every one in the paper's loop, reads those of
+// four at a time.
 //
 // Triangle counting.  Count(G1, G2, edges) adds, for every edge (u, v), the
 // size of the intersection of u's neighbours in G1 and v's neighbours in
@@ -50,107 +53,339 @@ __device__ __forceinline__ void warp_add_u64(unsigned long long *dst, unsigned l
 
 // ----------------------------------------------------------------- PageRank
 
-// out[u] += live pairs of every slab in use owned by u (one warp per slab,
-// grid-stride; one atomic per slab).
-__global__ void __launch_bounds__(256) k_pr_outdeg(GView g, uint32_t *out)
+namespace {
+
+// Words of a call's counters: rings over the super-steps, so that several go
+// out before the host reads anything.  Step i adds the rank without out-edges
+// that step i + 1 hands out to dangling[i + 1], its L1 change to delta[i], and
+// clears the words of step i + 2.
+constexpr uint32_t kRing = 8, kAhead = 4; // steps launched for each read of the deltas
+struct PrCtr {
+    unsigned long long dangling[kRing], pad[8]; // a line each
+    unsigned long long delta[kRing], pad2[8];
+    unsigned long long chunks; // of the binned edges
+};
+
+// Whether a step before this one met eps: its change is in the ring, and the
+// steps after it, which do nothing, leave theirs at zero.  One thread of the
+// block reads (a load a warp on that one word took 30 us of a step); *tele
+// receives the teleport share of this step.  Called by the whole block.
+__device__ __forceinline__ bool pr_done(const PrCtr *ctr, uint32_t step, double eps, uint32_t V = 1,
+                                        unsigned long long *tele = nullptr)
 {
-    const uint64_t total = (uint64_t)g.H + g.P;
-    const uint64_t stride = ((uint64_t)gridDim.x * blockDim.x) >> 5;
-    const uint32_t lane = lane_id();
-    for (uint64_t s = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5; s < total; s += stride) {
-        const uint32_t own = __ldg(&g.owner[s]);
-        if (own == kNil)
-            continue;
-        const uint32_t word = __ldcg(slab_ptr(g, (uint32_t)s) + lane);
-        const uint32_t live = __ballot_sync(kFull, is_key_lane(lane) && word < kTombKey);
-        if (lane == 0 && live)
-            atomicAdd(&out[own], (uint32_t)__popc(live));
+    __shared__ unsigned long long s_tele;
+    bool done = false;
+    if (threadIdx.x == 0) {
+        done = step && (double)__ldcg(&ctr->delta[(step - 1) % kRing]) * kInvFix <= eps;
+        if (tele)
+            s_tele = __ldcg(&ctr->dangling[step % kRing]) / V;
     }
+    done = __syncthreads_or(done);
+    if (tele)
+        *tele = s_tele;
+    return done;
+}
+
+// Adds a and b of every thread to *da and *db, one atomic a block each (one a
+// warp made 32,768 of them wait for one word: 57 us a step at 2^20 vertices).
+__device__ __forceinline__ void block_add2_u64(unsigned long long *da, unsigned long long a, unsigned long long *db,
+                                               unsigned long long b)
+{
+    __shared__ unsigned long long sa[8], sb[8];
+    for (int o = 16; o; o >>= 1) {
+        a += __shfl_xor_sync(kFull, a, o);
+        b += __shfl_xor_sync(kFull, b, o);
+    }
+    if (lane_id() == 0) {
+        sa[threadIdx.x >> 5] = a;
+        sb[threadIdx.x >> 5] = b;
+    }
+    __syncthreads();
+    if (threadIdx.x < 2) {
+        unsigned long long t = 0;
+        for (int k = 0; k < 8; ++k)
+            t += threadIdx.x ? sb[k] : sa[k];
+        if (t)
+            atomicAdd(threadIdx.x ? db : da, t);
+    }
+}
+
+// A vertex's out-degree with floor((2^64 - 1) / it), which turns the division
+// of a super-step into a multiplication and one correction: for p < 2^63 the
+// high product is the quotient or one less.
+struct OutDegree {
+    unsigned long long inv;
+    uint32_t n, pad;
+};
+
+// FindContributionPerVertex: contrib[u] = PR[u] / out[u]; the rank of a vertex
+// without out-edges is returned for the teleport sum instead.
+__device__ __forceinline__ unsigned long long contribution(unsigned long long p, const OutDegree &o,
+                                                           unsigned long long *contrib)
+{
+    unsigned long long q = __umul64hi(p, o.inv);
+    q += p - q * o.n >= o.n;
+    *contrib = o.n ? q : 0ull;
+    return o.n ? 0ull : p;
+}
+
+// One block's slabs of a pass over all of them (a contiguous range).
+struct SlabRange {
+    uint64_t first, last;
+};
+__device__ __forceinline__ SlabRange block_slabs(const GView &g)
+{
+    const uint64_t all = (uint64_t)g.H + g.P, per = ((all + gridDim.x - 1) / gridDim.x + 3) & ~3ull;
+    const uint64_t a = blockIdx.x * per;
+    return {a < all ? a : all, a + per < all ? a + per : all};
+}
+
+// The lane's 16 bytes of its slab (eight lanes a slab, four slabs a warp):
+// two keys, kEmptyKey where there is none; *own is the slab's owner.
+__device__ __forceinline__ void slab_keys(const GView &g, uint64_t s, uint64_t last, uint32_t (&key)[2], uint32_t *own)
+{
+    const uint32_t part = lane_id() & 7u;
+    *own = s < last ? __ldg(&g.owner[s]) : kNil;
+    key[0] = key[1] = kEmptyKey;
+    if (*own != kNil) { // an unused pool slab holds stale keys
+        const uint4 q = __ldcg(reinterpret_cast<const uint4 *>(slab_ptr(g, (uint32_t)s)) + part);
+        key[0] = q.x;
+        key[1] = part != 7u ? q.z : kEmptyKey;
+    }
+}
+
+constexpr uint32_t kBinThreads = 1024, kMaxBins = 1024;
+
+} // namespace
+
+// out[u] += live pairs of every slab in use owned by u (one atomic a slab),
+// and, with bins, the block's edges into each bin of 2^shift vertices
+// (hist[bin * gridDim.x + block]).
+template <bool kBins>
+__global__ void __launch_bounds__(kBinThreads) k_pr_outdeg(GView g, uint32_t *out, uint32_t shift, uint32_t bins,
+                                                           uint32_t *hist)
+{
+    __shared__ uint32_t h[kMaxBins];
+    const uint32_t lane = lane_id(), first = lane & ~7u;
+    if (kBins) {
+        for (uint32_t i = threadIdx.x; i < bins; i += kBinThreads)
+            h[i] = 0;
+        __syncthreads();
+    }
+    const SlabRange r = block_slabs(g);
+    for (uint64_t sb = r.first + (threadIdx.x >> 5) * 4; sb < r.last; sb += kBinThreads / 8) {
+        uint32_t key[2], own;
+        slab_keys(g, sb + (lane >> 3), r.last, key, &own);
+        const bool live0 = key[0] < kTombKey, live1 = key[1] < kTombKey;
+        const uint32_t n = __popc((__ballot_sync(kFull, live0) >> first) & 0xFFu) +
+                           __popc((__ballot_sync(kFull, live1) >> first) & 0xFFu);
+        if (lane == first && n)
+            atomicAdd(&out[own], n);
+        if (kBins) {
+            if (live0)
+                atomicAdd(&h[key[0] >> shift], 1u);
+            if (live1)
+                atomicAdd(&h[key[1] >> shift], 1u);
+        }
+    }
+    if (kBins) {
+        __syncthreads();
+        for (uint32_t i = threadIdx.x; i < bins; i += kBinThreads)
+            hist[(uint64_t)i * gridDim.x + blockIdx.x] = h[i];
+    }
+}
+
+// Writes the block's edges to its places in their destinations' bins, as
+// <source, destination> (T = uint2) or, where both fit one word, as the
+// source above the destination's place in the bin (T = uint32_t).
+template <typename T>
+__global__ void __launch_bounds__(kBinThreads) k_pr_bin(GView g, uint32_t shift, uint32_t bins,
+                                                        const uint64_t *__restrict__ off, T *edges)
+{
+    __shared__ uint64_t base[kMaxBins];
+    __shared__ uint32_t used[kMaxBins];
+    for (uint32_t i = threadIdx.x; i < bins; i += kBinThreads) {
+        base[i] = off[(uint64_t)i * gridDim.x + blockIdx.x];
+        used[i] = 0;
+    }
+    __syncthreads();
+    const SlabRange r = block_slabs(g);
+    for (uint64_t sb = r.first + (threadIdx.x >> 5) * 4; sb < r.last; sb += kBinThreads / 8) {
+        uint32_t key[2], own;
+        slab_keys(g, sb + (lane_id() >> 3), r.last, key, &own);
+#pragma unroll
+        for (int k = 0; k < 2; ++k)
+            if (key[k] < kTombKey) {
+                const uint32_t b = key[k] >> shift;
+                T *to = edges + base[b] + atomicAdd(&used[b], 1u);
+                if constexpr (sizeof(T) == 8)
+                    *to = make_uint2(own, key[k]);
+                else
+                    *to = own << shift | (key[k] & ((1u << shift) - 1));
+            }
+    }
+}
+
+// The bins in chunks of at most kChunk edges: chunk[i] = <bin, first edge>.
+constexpr uint32_t kChunk = 16384;
+
+__global__ void __launch_bounds__(kMaxBins) k_pr_chunks(const uint64_t *__restrict__ off, uint32_t bins,
+                                                        uint32_t blocks, ulonglong2 *chunk, PrCtr *ctr)
+{
+    const uint32_t b = threadIdx.x;
+    const uint64_t from = b < bins ? off[(uint64_t)b * blocks] : 0, to = b < bins ? off[(uint64_t)(b + 1) * blocks] : 0;
+    const uint64_t n = (to - from + kChunk - 1) / kChunk;
+    uint64_t at = n ? atomicAdd(&ctr->chunks, n) : 0;
+    for (uint64_t e = from; e < to; e += kChunk)
+        chunk[at++] = make_ulonglong2(b, e);
 }
 
 // Start vector: 1 / V for every vertex (static), or the caller's ranks
-// (incremental / decremental: the ranks before the batch).
-__global__ void k_pr_init(unsigned long long *pr, const float *init, uint32_t V)
+// (incremental / decremental: the ranks before the batch); and what the first
+// super-step reads.
+__global__ void __launch_bounds__(256) k_pr_start(const float *init, const uint32_t *out, uint32_t V,
+                                                  unsigned long long *pr, unsigned long long *contrib,
+                                                  unsigned long long *acc, OutDegree *deg, PrCtr *ctr)
 {
-    const uint32_t v = blockIdx.x * blockDim.x + threadIdx.x;
-    if (v < V)
-        pr[v] = init ? __double2ull_rn((double)fmaxf(init[v], 0.f) * kFix) : __double2ull_rn(kFix / (double)V);
-}
-
-// FindContributionPerVertex: contrib[u] = PR[u] / out[u] (0 for a vertex
-// without out-edges, whose rank goes to the teleport sum); clears the
-// accumulators.  ctr[0] receives the teleport sum of this super-step.
-__global__ void k_pr_contrib(const unsigned long long *pr, const uint32_t *out, uint32_t V,
-                             unsigned long long *contrib, unsigned long long *acc, unsigned long long *ctr)
-{
-    const uint32_t v = blockIdx.x * blockDim.x + threadIdx.x;
     unsigned long long dangling = 0;
-    if (v < V) {
-        const unsigned long long p = pr[v];
-        const uint32_t o = out[v];
-        contrib[v] = o ? p / o : 0ull;
-        dangling = o ? 0ull : p;
+    for (uint64_t v = blockIdx.x * 256ull + threadIdx.x; v < V; v += gridDim.x * 256ull) {
+        const unsigned long long p =
+            init ? __double2ull_rn((double)fmaxf(init[v], 0.f) * kFix) : __double2ull_rn(kFix / (double)V);
+        pr[v] = p;
+        const uint32_t n = out[v];
+        deg[v] = {n ? ~0ull / n : 0ull, n, 0u};
+        dangling += contribution(p, deg[v], &contrib[v]);
         acc[v] = 0;
     }
-    warp_add_u64(ctr, dangling);
+    block_add2_u64(&ctr->dangling[0], dangling, &ctr->delta[0], 0ull);
 }
 
-// Pushes contrib[u] along every live edge u -> v.  A warp takes
-// 4 * kPushHalves consecutive slabs a step, four at a time: eight lanes a
-// slab, each lane one 16-byte block (two pairs; the last lane of a slab one
-// pair and the unused and next words); the owners, slab parts and
-// contributions of every group of four are loaded before any atomic, so
-// kPushHalves independent load chains are in flight per lane.
+// Adds contrib[u] of a chunk's edges u -> v up in shared memory (64-bit sums
+// as two words with a carry) and the sums to acc.  A bin's vertices take
+// 8 << shift bytes; the edges are read in order and the contributions gathered
+// from L2 (8 bytes an edge, 266 G/s at most).  Pushing along the slabs instead
+// put one 64-bit atomic an edge on the accumulators in L2, where a power-law
+// graph's hubs share a few lines: its slices 50 % busy at most and 13 % on
+// average, 339 us a step on R-MAT scale 20 against 48 so, after 310 us
+// once a call for the bins.
+template <typename T>
+__global__ void __launch_bounds__(512) k_pr_pull(const T *__restrict__ edges, const uint64_t *__restrict__ off,
+                                                 const ulonglong2 *__restrict__ chunk, uint32_t shift,
+                                                 uint32_t blocks, const unsigned long long *__restrict__ contrib,
+                                                 unsigned long long *acc, uint32_t V, const PrCtr *ctr, uint32_t step,
+                                                 double eps)
+{
+    extern __shared__ uint32_t sums[]; // low words, then high words
+    if (pr_done(ctr, step, eps))
+        return;
+    const uint32_t width = 1u << shift, mask = width - 1;
+    uint32_t *lo = sums, *hi = sums + width;
+    const unsigned long long n = __ldg(&ctr->chunks);
+    for (unsigned long long c = blockIdx.x; c < n; c += gridDim.x) {
+        for (uint32_t i = threadIdx.x; i < 2 * width; i += 512)
+            sums[i] = 0;
+        const ulonglong2 me = chunk[c];
+        const uint64_t end = off[(me.x + 1) * blocks], last = me.y + kChunk < end ? me.y + kChunk : end;
+        __syncthreads();
+        for (uint64_t i = me.y + threadIdx.x; i < last; i += 4 * 512) {
+            uint32_t v[4];
+            unsigned long long x[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const bool in = i + k * 512 < last;
+                uint32_t u = kNil;
+                v[k] = 0;
+                if (in) {
+                    const T e = __ldcs(&edges[i + k * 512]);
+                    if constexpr (sizeof(T) == 8) {
+                        u = e.x;
+                        v[k] = e.y & mask;
+                    } else {
+                        u = e >> shift;
+                        v[k] = e & mask;
+                    }
+                }
+                x[k] = in ? __ldg(&contrib[u]) : 0ull;
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const uint32_t l = (uint32_t)x[k];
+                uint32_t h = (uint32_t)(x[k] >> 32);
+                if (l)
+                    h += atomicAdd(&lo[v[k]], l) + l < l; // the carry
+                if (h)
+                    atomicAdd(&hi[v[k]], h);
+            }
+        }
+        __syncthreads();
+        for (uint32_t i = threadIdx.x; i < width; i += 512) {
+            const unsigned long long sum = (unsigned long long)hi[i] << 32 | lo[i];
+            if (sum)
+                atomicAdd(&acc[(me.x << shift) + i], sum);
+        }
+        __syncthreads();
+    }
+}
+
+// Pushes contrib[u] along every live edge u -> v, where the edges are not
+// binned.  A warp takes 4 * kPushHalves consecutive slabs a step, four at a
+// time: eight lanes a slab, each lane one 16-byte block; the owners, slab
+// parts and contributions of every group of four are loaded before any
+// atomic, so kPushHalves independent load chains are in flight per lane.
 constexpr int kPushHalves = 2;
 
 __global__ void __launch_bounds__(256) k_pr_push(GView g, const unsigned long long *__restrict__ contrib,
-                                                 unsigned long long *acc)
+                                                 unsigned long long *acc, const PrCtr *ctr, uint32_t step, double eps)
 {
+    if (pr_done(ctr, step, eps))
+        return;
     const uint64_t nslab = (uint64_t)g.H + g.P;
-    const uint32_t lane = lane_id(), part = lane & 7u, sub = lane >> 3;
     const uint64_t warp = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5;
     const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
     for (uint64_t s0 = warp * (4 * kPushHalves); s0 < nslab; s0 += nwarps * (4 * kPushHalves)) {
-        uint32_t own[kPushHalves];
-        uint4 q[kPushHalves];
+        uint32_t own[kPushHalves], key[kPushHalves][2];
 #pragma unroll
-        for (int h = 0; h < kPushHalves; ++h) {
-            const uint64_t s = s0 + h * 4 + sub;
-            own[h] = s < nslab ? __ldg(&g.owner[s]) : kNil;
-            q[h] = s < nslab ? __ldcg(reinterpret_cast<const uint4 *>(slab_ptr(g, (uint32_t)s)) + part)
-                             : make_uint4(kEmptyKey, 0u, kEmptyKey, 0u);
-        }
+        for (int h = 0; h < kPushHalves; ++h)
+            slab_keys(g, s0 + h * 4 + (lane_id() >> 3), nslab, key[h], &own[h]);
         unsigned long long c[kPushHalves];
 #pragma unroll
         for (int h = 0; h < kPushHalves; ++h)
-            c[h] = own[h] != kNil ? __ldg(&contrib[own[h]]) : 0ull; // an unused pool slab holds stale keys
+            c[h] = own[h] != kNil ? __ldg(&contrib[own[h]]) : 0ull;
 #pragma unroll
         for (int h = 0; h < kPushHalves; ++h) {
             if (!c[h])
                 continue;
-            if (q[h].x < kTombKey)
-                atomicAdd(&acc[q[h].x], c[h]);
-            if (part != 7u && q[h].z < kTombKey)
-                atomicAdd(&acc[q[h].z], c[h]);
+            if (key[h][0] < kTombKey)
+                atomicAdd(&acc[key[h][0]], c[h]);
+            if (key[h][1] < kTombKey)
+                atomicAdd(&acc[key[h][1]], c[h]);
         }
     }
 }
 
 // Compute + teleport (Eq. 1): PR[v] = (1 - d) / V + d * (acc[v] + teleport
-// / V); ctr[1] receives the L1 delta of the super-step.
-__global__ void k_pr_finish(unsigned long long *pr, const unsigned long long *acc, uint32_t V, double d,
-                            unsigned long long base, unsigned long long *ctr)
+// / V), the L1 delta of the super-step, and what the next one reads.
+__global__ void __launch_bounds__(256) k_pr_finish(unsigned long long *pr, unsigned long long *acc,
+                                                   const OutDegree *__restrict__ deg, unsigned long long *contrib,
+                                                   uint32_t V, double d, unsigned long long base, PrCtr *ctr, uint32_t step, double eps)
 {
-    const uint32_t v = blockIdx.x * blockDim.x + threadIdx.x;
-    unsigned long long diff = 0;
-    if (v < V) {
-        const unsigned long long tele = __ldcg(&ctr[0]) / V;
+    unsigned long long tele;
+    if (pr_done(ctr, step, eps, V, &tele))
+        return;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        ctr->dangling[(step + 2) % kRing] = 0;
+        ctr->delta[(step + 2) % kRing] = 0;
+    }
+    unsigned long long diff = 0, dangling = 0;
+    for (uint64_t v = blockIdx.x * 256ull + threadIdx.x; v < V; v += gridDim.x * 256ull) {
         const unsigned long long nv = base + __double2ull_rn(d * (double)(acc[v] + tele));
         const unsigned long long ov = pr[v];
-        diff = nv > ov ? nv - ov : ov - nv;
+        diff += nv > ov ? nv - ov : ov - nv;
         pr[v] = nv;
+        acc[v] = 0;
+        dangling += contribution(nv, deg[v], &contrib[v]);
     }
-    warp_add_u64(&ctr[1], diff);
+    block_add2_u64(&ctr->delta[step % kRing], diff, &ctr->dangling[(step + 1) % kRing], dangling);
 }
 
 __global__ void k_pr_out(const unsigned long long *pr, uint32_t V, float *out)
@@ -594,62 +829,141 @@ mk_status mk_pagerank(mk_graph *g, float *d_pr, int warm_start, float damping, f
         return MK_ERR_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)stream;
     const uint32_t V = g->v.V;
-    const uint64_t words = ((uint64_t)g->v.H + g->v.P) * 32;
-    unsigned long long *pr = nullptr, *acc = nullptr, *contrib = nullptr, *ctr = nullptr;
-    uint32_t *out = nullptr;
-    MK_CUDA(cudaMallocAsync((void **)&pr, (size_t)V * 8, s));
-    MK_CUDA(cudaMallocAsync((void **)&acc, (size_t)V * 8, s));
-    MK_CUDA(cudaMallocAsync((void **)&contrib, (size_t)V * 8, s));
-    MK_CUDA(cudaMallocAsync((void **)&out, (size_t)V * 4, s));
-    MK_CUDA(cudaMallocAsync((void **)&ctr, 16, s));
-    MK_CUDA(cudaMemsetAsync(out, 0, (size_t)V * 4, s));
-    mk_status st = timed(g, "pr_outdeg", s, 2, [&]() {
-        k_pr_outdeg<<<resident_grid(k_pr_outdeg, 256), 256, 0, s>>>(g->v, out);
-        k_pr_init<<<grid_for(V, 256), 256, 0, s>>>(pr, warm_start ? d_pr : nullptr, V);
-        return cudaSuccess;
-    });
-    const double d = damping;
+    const double d = damping, stop = eps;
     const unsigned long long base = (unsigned long long)std::llround((1.0 - d) / (double)V * kFix);
-    uint32_t it = 0;
-    double delta = 0;
-    // 4 * kPushHalves slabs per warp step
-    const uint32_t push_grid = std::min<uint64_t>(grid_for(words / (4 * kPushHalves), 256),
-                                                  (uint64_t)resident_grid(k_pr_push, 256) * 4);
-    while (st == MK_OK && it < max_iter) {
-        if (cudaMemsetAsync(ctr, 0, 16, s) != cudaSuccess) {
-            st = MK_ERR_CUDA;
-            break;
+    mk_status st = MK_OK;
+    auto cuda = [&](cudaError_t e) {
+        if (st == MK_OK && e != cudaSuccess)
+            st = e == cudaErrorMemoryAllocation ? MK_ERR_NO_MEMORY : MK_ERR_CUDA;
+        return st == MK_OK;
+    };
+    // Bins of 2^shift destinations, at most kMaxBins of them: 2^10 vertices
+    // (8 KB of sums) up to 2^20 vertices, 2^14 (128 KB) at 2^24.
+    uint32_t vbits = 1, shift = 10;
+    while (vbits < 32 && (1ull << vbits) < V)
+        ++vbits;
+    shift = std::max(shift, vbits > 10 ? vbits - 10 : 0u);
+    const uint32_t bins = (uint32_t)(((uint64_t)V + (1ull << shift) - 1) >> shift);
+    const uint32_t blocks = num_sms() * 2;
+    bool binned = shift <= 14 && max_iter >= 4;
+    const bool packed = vbits + shift <= 32;
+    // per-vertex arrays and counters in one block; the bins' counts and
+    // places, and the edges, in another
+    unsigned char *vert = nullptr, *bin = nullptr;
+    MK_CUDA(cudaMallocAsync((void **)&vert, (size_t)V * (16 + 3 * 8 + 4) + sizeof(PrCtr), s));
+    OutDegree *deg = (OutDegree *)vert;
+    unsigned long long *pr = (unsigned long long *)(deg + V), *acc = pr + V, *contrib = acc + V;
+    PrCtr *ctr = (PrCtr *)(contrib + V);
+    uint32_t *out = (uint32_t *)(ctr + 1);
+    const uint64_t cells = (uint64_t)bins * blocks + 1;
+    const size_t scan_bytes = exclusive_scan_scratch_bytes(cells);
+    uint32_t *hist = nullptr;
+    uint64_t *off = nullptr, edges_n = 0;
+    ulonglong2 *chunk = nullptr;
+    void *edges = nullptr;
+    cuda(cudaMemsetAsync(ctr, 0, sizeof(PrCtr) + (size_t)V * 4, s));
+    if (st == MK_OK && binned) {
+        if (cudaMallocAsync((void **)&bin, cells * 12 + 8 + scan_bytes, s) != cudaSuccess) {
+            cudaGetLastError();
+            bin = nullptr;
+            binned = false;
         }
-        st = timed(g, "pr_step", s, 3, [&]() {
-            k_pr_contrib<<<grid_for(V, 256), 256, 0, s>>>(pr, out, V, contrib, acc, ctr);
-            k_pr_push<<<push_grid, 256, 0, s>>>(g->v, contrib, acc);
-            k_pr_finish<<<grid_for(V, 256), 256, 0, s>>>(pr, acc, V, d, base, ctr);
+    }
+    if (st == MK_OK && binned) {
+        off = (uint64_t *)bin;
+        void *scratch = off + cells;
+        hist = (uint32_t *)((unsigned char *)scratch + scan_bytes);
+        int scans = 0;
+        cuda(cudaMemsetAsync(hist + cells - 1, 0, 4, s));
+        if (st == MK_OK)
+            st = timed(g, "pr_outdeg", s, 1, [&]() {
+                k_pr_outdeg<true><<<blocks, kBinThreads, 0, s>>>(g->v, out, shift, bins, hist);
+                return exclusive_scan_u32_u64(hist, off, cells, scratch, s, &scans);
+            });
+        g->launches += (uint64_t)scans;
+        if (st == MK_OK)
+            cuda(cudaMemcpyAsync(g->h_pinned, off + cells - 1, 8, cudaMemcpyDeviceToHost, s));
+        if (st == MK_OK && cuda(cudaStreamSynchronize(s))) {
+            std::memcpy(&edges_n, g->h_pinned, 8);
+            const size_t rec = packed ? 4 : 8, chunks = bins + edges_n / kChunk;
+            if (cudaMallocAsync((void **)&chunk, chunks * 16 + edges_n * rec, s) != cudaSuccess) {
+                cudaGetLastError();
+                chunk = nullptr;
+                binned = false;
+            } else {
+                edges = chunk + chunks;
+                st = timed(g, "pr_bin", s, 2, [&]() {
+                    k_pr_chunks<<<1, kMaxBins, 0, s>>>(off, bins, blocks, chunk, ctr);
+                    if (packed)
+                        k_pr_bin<uint32_t><<<blocks, kBinThreads, 0, s>>>(g->v, shift, bins, off, (uint32_t *)edges);
+                    else
+                        k_pr_bin<uint2><<<blocks, kBinThreads, 0, s>>>(g->v, shift, bins, off, (uint2 *)edges);
+                    return cudaSuccess;
+                });
+            }
+        }
+    } else if (st == MK_OK) {
+        st = timed(g, "pr_outdeg", s, 1, [&]() {
+            k_pr_outdeg<false><<<blocks, kBinThreads, 0, s>>>(g->v, out, 0, 0, nullptr);
             return cudaSuccess;
         });
-        if (st != MK_OK)
-            break;
-        ++it;
-        unsigned long long dfx = 0;
-        if (cudaMemcpyAsync(g->h_pinned, ctr + 1, 8, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-            cudaStreamSynchronize(s) != cudaSuccess) {
-            st = MK_ERR_CUDA;
-            break;
+    }
+    const uint32_t vgrid = std::min<uint32_t>(grid_for(V, 256), num_sms() * 8);
+    if (st == MK_OK)
+        st = timed(g, "pr_start", s, 1, [&]() {
+            k_pr_start<<<vgrid, 256, 0, s>>>(warm_start ? d_pr : nullptr, out, V, pr, contrib, acc, deg, ctr);
+            return cudaSuccess;
+        });
+    const size_t sums = (size_t)8 << shift;
+    const void *pull = packed ? (const void *)k_pr_pull<uint32_t> : (const void *)k_pr_pull<uint2>;
+    int per = 1;
+    if (st == MK_OK && binned && cuda(cudaFuncSetAttribute(pull, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sums)))
+        cuda(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, pull, 512, sums));
+    const uint32_t pull_grid = (uint32_t)std::min<uint64_t>((uint64_t)num_sms() * std::max(per, 1), bins + edges_n / kChunk);
+    // 4 * kPushHalves slabs per warp step
+    const uint32_t push_grid = std::min<uint64_t>(grid_for(((uint64_t)g->v.H + g->v.P) * 32 / (4 * kPushHalves), 256),
+                                                  (uint64_t)resident_grid(k_pr_push, 256) * 4);
+    uint32_t it = 0;
+    double delta = 0;
+    for (bool met = false; st == MK_OK && !met && it < max_iter;) {
+        const uint32_t n = std::min(kAhead, max_iter - it);
+        for (uint32_t k = 0; k < n && st == MK_OK; ++k) {
+            uint32_t step = it + k;
+            st = timed(g, "pr_step", s, 2, [&]() {
+                if (binned) {
+                    void *args[] = {&edges, &off, &chunk, &shift, (void *)&blocks, &contrib, &acc, (void *)&V, &ctr,
+                                    &step, (void *)&stop};
+                    const cudaError_t e = cudaLaunchKernel(pull, dim3(pull_grid), dim3(512), args, sums, s);
+                    if (e != cudaSuccess)
+                        return e;
+                } else {
+                    k_pr_push<<<push_grid, 256, 0, s>>>(g->v, contrib, acc, ctr, step, stop);
+                }
+                k_pr_finish<<<vgrid, 256, 0, s>>>(pr, acc, deg, contrib, V, d, base, ctr, step, stop);
+                return cudaSuccess;
+            });
         }
-        std::memcpy(&dfx, g->h_pinned, 8);
-        delta = (double)dfx * kInvFix;
-        if (delta <= eps)
-            break;
+        if (st == MK_OK)
+            cuda(cudaMemcpyAsync(g->h_pinned, ctr->delta, sizeof ctr->delta, cudaMemcpyDeviceToHost, s));
+        if (st == MK_OK)
+            cuda(cudaStreamSynchronize(s));
+        for (uint32_t k = 0; k < n && st == MK_OK && !met; ++k, ++it) {
+            unsigned long long dfx = 0;
+            std::memcpy(&dfx, g->h_pinned + 2 * (it % kRing), 8);
+            delta = (double)dfx * kInvFix;
+            met = delta <= stop;
+        }
     }
     if (st == MK_OK)
         st = timed(g, "pr_out", s, 1, [&]() {
             k_pr_out<<<grid_for(V, 256), 256, 0, s>>>(pr, V, d_pr);
             return cudaSuccess;
         });
-    cudaFreeAsync(pr, s);
-    cudaFreeAsync(acc, s);
-    cudaFreeAsync(contrib, s);
-    cudaFreeAsync(out, s);
-    cudaFreeAsync(ctr, s);
+    cudaFreeAsync(vert, s);
+    if (bin)
+        cudaFreeAsync(bin, s);
+    if (chunk)
+        cudaFreeAsync(chunk, s);
     if (h_iters)
         *h_iters = it;
     if (h_delta)

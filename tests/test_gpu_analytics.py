@@ -167,3 +167,42 @@ def test_triangles_neighbourhood_sizes(cuda_lib, V, buckets):
     assert g.triangles() == o.triangles()
     assert g.last_error() == mk.MK_OK
     g.close()
+
+
+@pytest.mark.parametrize("V", [700, 70000, 3000000])  # one bin; bins of packed edges; of wide ones
+def test_pagerank_binned_and_pushed(cuda_lib, V):
+    """A call of three super-steps at most pushes, one of more bins its edges:
+    both against double precision within the float32 rounding of the ranks
+    (2^-24 of each) and 2^-48 for each of the in-degree + 3 terms of a step,
+    and stopping after the same step with the same delta."""
+    mk = _mk()
+    rng = np.random.default_rng(V)
+    n = min(8 * V, 400000)
+    s = rng.integers(0, V, n).astype(np.uint32)
+    d = (rng.integers(0, V, n) * rng.random(n) ** 3).astype(np.uint32)  # some vertices with many in-edges
+    g = mk.Graph(V, edge_capacity_hint=2 * n, buckets=mk.bucket_rule(V, s, 0.7))
+    g.insert(s, d)
+    g.commit()
+    pushed, it, _ = g.pagerank(eps=1e-30, max_iter=3)
+    binned, it4, _ = g.pagerank(eps=1e-30, max_iter=4)
+    assert (it, it4) == (3, 4)
+    # the oracle's steps in double precision
+    k = np.unique(s.astype(np.int64) * V + d)
+    us, ud = k // V, k % V
+    out = np.bincount(us, minlength=V)
+    pr, damp = np.full(V, 1.0 / V), float(np.float32(0.85))
+    for step in range(4):
+        share = np.where(out > 0, pr / np.maximum(out, 1), 0.0)
+        pr = (1 - damp) / V + damp * (np.bincount(ud, share[us], minlength=V) + pr[out == 0].sum() / V)
+        if step == 2:
+            three = pr.copy()
+    term = (np.bincount(ud, minlength=V) + 3) * 4 * 2.0 ** -48
+    for got, want in ((pushed, three), (binned, pr)):
+        err = np.abs(got.cpu().numpy().astype(np.float64) - want)
+        assert (err <= want * 2.0 ** -24 + term.max() + term).all()
+    # the stop after the same step with both forms
+    _, i3, d3 = g.pagerank(eps=0.5, max_iter=3)
+    _, i9, d9 = g.pagerank(eps=0.5, max_iter=9)
+    assert i3 == i9 and d3 == d9
+    assert g.last_error() == mk.MK_OK
+    g.close()
