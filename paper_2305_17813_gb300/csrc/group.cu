@@ -96,9 +96,9 @@ __global__ void __launch_bounds__(kBlock) k_group_count(GView g, const uint32_t 
 
 // Ranges of the entry array, one atomic a block on the cursor, so that the
 // ranges follow the order of the lists up to the order of the blocks.  The
-// range of a list with more than kGroupMax edges starts as a free hash set.
+// range of a list with more than `most` edges starts as a free hash set.
 __global__ void __launch_bounds__(kBlock) k_group_place(const uint32_t *__restrict__ alist, uint32_t H, uint2 *slot,
-                                                        uint2 *ent, uint32_t *ctr)
+                                                        uint2 *ent, uint32_t most, uint32_t *ctr)
 {
     __shared__ uint32_t s_warp[kBlock / 32], s_base;
     const uint32_t n = alist ? __ldcg(&ctr[kGroupActive]) : H;
@@ -129,7 +129,7 @@ __global__ void __launch_bounds__(kBlock) k_group_place(const uint32_t *__restri
         const uint32_t off = s_base + s_warp[threadIdx.x >> 5] + incl - c;
         if (c)
             slot[L].y = off;
-        for (uint32_t big = __ballot_sync(kFull, c > kGroupMax); big; big &= big - 1) {
+        for (uint32_t big = __ballot_sync(kFull, c > most); big; big &= big - 1) {
             const uint32_t l = __ffs(big) - 1;
             const uint32_t o = __shfl_sync(kFull, off, l), m = __shfl_sync(kFull, c, l);
             for (uint32_t e = lane_id(); e < m; e += 32)
@@ -143,7 +143,7 @@ __global__ void __launch_bounds__(kBlock) k_group_place(const uint32_t *__restri
 __global__ void __launch_bounds__(kBlock) k_group_scatter(const uint32_t *__restrict__ dst, uint64_t n,
                                                           const uint2 *__restrict__ slot, uint32_t *lst,
                                                           const uint8_t *__restrict__ rank, uint2 *ent, uint32_t lo,
-                                                          uint32_t hi, uint32_t *many, uint32_t *ctr)
+                                                          uint32_t hi, uint32_t most, uint32_t *many, uint32_t *ctr)
 {
     const uint64_t i0 = blockIdx.x * (uint64_t)(kBlock * kPer) + threadIdx.x;
     uint32_t L[kPer];
@@ -164,7 +164,7 @@ __global__ void __launch_bounds__(kBlock) k_group_scatter(const uint32_t *__rest
         if (L[k] == kNil)
             continue;
         const uint32_t d = __ldg(dst + i), c = sl[k].x;
-        if (c <= kGroupMax) {
+        if (c <= most) {
             ent[sl[k].y + rank[i]] = make_uint2(d, (uint32_t)i);
             continue;
         }
@@ -243,7 +243,7 @@ cudaError_t group_reserve(GroupScratch &gs, uint64_t n, uint32_t H, cudaStream_t
 }
 
 cudaError_t group_batch(const GView &g, GroupScratch &gs, const uint32_t *src, const uint32_t *dst, const uint32_t *w,
-                        uint64_t n, cudaStream_t s, GroupView *gv, int *launches)
+                        uint64_t n, uint32_t most, cudaStream_t s, GroupView *gv, int *launches)
 {
     const bool dense = group_dense(g.H, n);
     uint32_t *alist = dense ? nullptr : gs.alist;
@@ -254,7 +254,7 @@ cudaError_t group_batch(const GView &g, GroupScratch &gs, const uint32_t *src, c
     k_group_count<<<grid, kBlock, 0, s>>>(g, src, dst, w, n, gs.slot, gs.lst, gs.rank, alist, gs.ctr);
     const uint64_t lists = dense ? g.H : n;
     k_group_place<<<std::min<uint32_t>(grid_for(lists, kBlock), num_sms() * 64), kBlock, 0, s>>>(alist, g.H, gs.slot,
-                                                                                             gs.ent, gs.ctr);
+                                                                                             gs.ent, most, gs.ctr);
     // One pass for each 64 MB of entries: the range of lists a pass writes
     // stays in L2, where its 8-byte stores run at 190 G/s; over an array
     // beyond L2 they run at 33 G/s.
@@ -262,9 +262,9 @@ cudaError_t group_batch(const GView &g, GroupScratch &gs, const uint32_t *src, c
     for (uint32_t p = 0; p < passes; ++p)
         k_group_scatter<<<grid, kBlock, 0, s>>>(dst, n, gs.slot, gs.lst, gs.rank, gs.ent,
                                                 (uint32_t)((uint64_t)g.H * p / passes),
-                                                (uint32_t)((uint64_t)g.H * (p + 1) / passes), gs.alist, gs.ctr);
+                                                (uint32_t)((uint64_t)g.H * (p + 1) / passes), most, gs.alist, gs.ctr);
     *launches += 2 + (int)passes;
-    *gv = {gs.slot, gs.ent, gs.lst, gs.alist, alist, gs.ctr};
+    *gv = {gs.slot, gs.ent, gs.lst, gs.alist, alist, gs.ctr, most};
     return cudaGetLastError();
 }
 

@@ -6,15 +6,17 @@
 
 namespace mk {
 
-// Most edges of one list that a 4-lane group applies by itself.
-constexpr uint32_t kGroupMax = 32;
+// Most edges of one list that a 4-lane group applies by itself: about twice
+// the load-factor rule's mean for a list (10 edges of the map layout, 22 of the
+// set's).
+constexpr uint32_t kGroupMax = 32, kSetGroupMax = 64;
 // Marks a hash-set index in GroupView::lst (an edge of a list with more); no
 // list has it (2^31 head slabs are 275 GB).
 constexpr uint32_t kSlotBit = 0x80000000u;
 
 // What the kernels that apply a grouped batch read.  The edges of list L sit
 // at ent[slot[L].y .. + slot[L].x) as <dst, batch position>, in no order, when
-// they are at most kGroupMax; otherwise that range holds a hash set of their
+// they are at most `most`; otherwise that range holds a hash set of their
 // batch positions (2 * slot[L].x words, kNil free) as k_dedup keeps one for a
 // whole batch, lst[i] of each of them is its word's index with kSlotBit, and their batch
 // positions are the ctr[kGroupMany] words at many[ctr[kGroupActive]].
@@ -25,6 +27,7 @@ struct GroupView {
     const uint32_t *many;
     const uint32_t *alist; // lists with edges, or null when every list is to be looked at
     const uint32_t *ctr;
+    uint32_t most;
 };
 enum { kGroupActive = 0, kGroupCursor = 1, kGroupMany = 2, kGroupWords = 4 };
 
@@ -52,12 +55,12 @@ inline bool group_dense(uint32_t H, uint64_t n) { return n >= 4 * (uint64_t)H; }
 cudaError_t group_reserve(GroupScratch &gs, uint64_t n, uint32_t H, cudaStream_t s, uint64_t *bytes);
 void group_release(GroupScratch &gs, uint64_t *bytes);
 
-// Validates and groups n edges (w nullable, a weight of 0 is invalid) and
-// fills *gv for the kernels launched after it on s.  An invalid edge sets the
+// Validates and groups n edges (w nullable, a weight of 0 is invalid), lists of
+// up to `most` edges apart from the others, and fills *gv for the kernels launched after it on s.  An invalid edge sets the
 // graph's status.  *launches counts the kernels.  The kernel that applies the
 // batch must set every active list's count back to 0.
 cudaError_t group_batch(const GView &g, GroupScratch &gs, const uint32_t *src, const uint32_t *dst, const uint32_t *w,
-                        uint64_t n, cudaStream_t s, GroupView *gv, int *launches);
+                        uint64_t n, uint32_t most, cudaStream_t s, GroupView *gv, int *launches);
 
 // Hash of a destination among the 2c words of a list's hash set.
 __device__ __forceinline__ uint32_t group_hash(uint32_t d, uint32_t words)
@@ -68,16 +71,68 @@ __device__ __forceinline__ uint32_t group_hash(uint32_t d, uint32_t words)
 // Lists a 256-thread block applies at a time (one a 4-lane group).
 constexpr uint32_t kGroupLists = 64;
 
+// The lists of an apply kernel's steps, one a group and step: the list is
+// read two steps ahead, its count and range one step ahead.
+struct ListCursor {
+    uint64_t at, step;
+    uint32_t n, L, L1;
+    uint2 sl;
+};
+
+__device__ __forceinline__ uint32_t list_at(const GroupView &gv, uint64_t k, uint32_t n)
+{
+    return k < n ? (gv.alist ? __ldg(&gv.alist[k]) : (uint32_t)k) : kNil;
+}
+
+__device__ __forceinline__ ListCursor first_lists(const GView &g, const GroupView &gv)
+{
+    ListCursor c;
+    c.n = gv.alist ? __ldg(&gv.ctr[kGroupActive]) : g.H;
+    c.at = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 2;
+    c.step = ((uint64_t)gridDim.x * blockDim.x) >> 2;
+    c.L = list_at(gv, c.at, c.n);
+    c.L1 = list_at(gv, c.at + c.step, c.n);
+    c.sl = c.L != kNil ? gv.slot[c.L] : make_uint2(0, 0);
+    return c;
+}
+
+// <list, edges, offset> of the calling lane's group, kNil and 0 without work;
+// the list's count is set back.  Called by the full warp.
+__device__ __forceinline__ uint3 next_list(const GroupView &gv, ListCursor &c, bool dead)
+{
+    const uint32_t L = c.L;
+    const uint2 sl = c.sl;
+    c.at += c.step;
+    c.L = c.L1;
+    c.L1 = list_at(gv, c.at + c.step, c.n);
+    c.sl = c.L != kNil ? gv.slot[c.L] : make_uint2(0, 0);
+    __syncwarp();
+    if (sl.x && (lane_id() & 3u) == 0)
+        gv.slot[L].x = 0;
+    const bool mine = sl.x != 0 && sl.x <= gv.most && !dead;
+    return make_uint3(mine ? L : kNil, mine ? sl.x : 0u, sl.y);
+}
+
+// Bits of the four lanes of a group together.
+template <typename M>
+__device__ __forceinline__ M group_or(M m)
+{
+    m |= __shfl_xor_sync(kFull, m, 1);
+    return m | __shfl_xor_sync(kFull, m, 2);
+}
+
 // Entries of the group's list in its shared-memory row, and which of them
 // are the first of their destination in batch order, as a mask over entries
-// (the same on the group's four lanes).  Every lane of the warp calls it.
-__device__ __forceinline__ uint32_t group_first(const GroupView &gv, uint32_t c, uint32_t off, uint2 *row)
+// (the same on the group's four lanes; a bit for each of gv.most).  Every lane
+// of the warp calls it.
+template <typename M>
+__device__ __forceinline__ M group_first(const GroupView &gv, uint32_t c, uint32_t off, uint2 *row)
 {
     const uint32_t s4 = lane_id() & 3u;
     for (uint32_t e = s4; e < c; e += 4)
         row[e] = __ldcs(&gv.ent[off + e]);
     __syncwarp();
-    uint32_t first = 0;
+    M first = 0;
     for (uint32_t e = s4; e < c; e += 4) {
         const uint2 me = row[e];
         bool is = true;
@@ -85,11 +140,9 @@ __device__ __forceinline__ uint32_t group_first(const GroupView &gv, uint32_t c,
             const uint2 o = row[j];
             is = is && !(o.x == me.x && o.y < me.y);
         }
-        first |= (is ? 1u : 0u) << e;
+        first |= (M)is << e;
     }
-    first |= __shfl_xor_sync(kFull, first, 1);
-    first |= __shfl_xor_sync(kFull, first, 2);
-    return first;
+    return group_or(first);
 }
 
 } // namespace mk

@@ -10,12 +10,12 @@
 // counts, overflow slabs claimed from a bitmap pool, EMPTY and TOMBSTONE
 // keys, deleted keys never reused (so free keys exist only in a chain's last
 // slab), set semantics with the first occurrence of a repeated pair applied
-// (the batch is deduplicated by the map store's staging kernel).  Inserts,
-// deletes and queries walk eight chains per warp in 4-lane groups, each
-// lane reading 32 bytes of a slab (the whole group one 128-byte slab).  BFS
-// (hop counts, with the smallest-id tight parent) and WCC (smallest-id
+// (a batch is grouped by slab list, as the map store's batches are: group.cu).
+// Inserts, deletes and queries walk eight chains per warp in 4-lane groups,
+// each lane reading 32 bytes of a slab (the whole group one 128-byte slab).
+// BFS (hop counts, with the smallest-id tight parent) and WCC (smallest-id
 // labels) run statically: BFS level by level over a frontier of lists, WCC
-// as one union-find pass over the slab array.
+// as the map store's static pass (wcc.cu).
 #include "mk_host.h"
 #include "uf.cuh"
 
@@ -32,23 +32,20 @@ uint32_t degree_grid(uint64_t n);
 __global__ void k_rule(uint32_t *deg, uint32_t V, float per_bucket);
 __global__ void k_init_bitmap(uint32_t *bitmap, uint32_t words, uint32_t P);
 __global__ void k_fill_buckets(uint32_t *b, uint32_t V, uint32_t nb, const uint32_t *user, int *bad);
-__global__ void k_dedup(const uint32_t *__restrict__ src, const uint32_t *__restrict__ dst,
-                        const uint32_t *__restrict__ w, uint64_t n, uint32_t V, uint32_t *tpos, uint32_t mask,
-                        uint32_t *__restrict__ slot, DevState *st);
+__global__ void __launch_bounds__(256) k_check_edges(const uint32_t *__restrict__ src, const uint32_t *__restrict__ dst,
+                                                     const uint32_t *__restrict__ w, uint64_t n, uint32_t V,
+                                                     DevState *st);
 
 namespace {
 
 constexpr uint32_t kSetKeys = 31; // key lanes 0..30, lane 31 = next
-
-__device__ __forceinline__ bool is_set_key_lane(uint32_t lane) { return lane < kSetKeys; }
 
 } // namespace
 
 struct mk_set_graph {
     GView v{};                 // V, H, P, pool_words, vinfo, slabs, bitmap, owner, st (the rest unused)
     uint64_t bytes = 0;
-    uint64_t cap = 0, table = 0; // staging: batch hash set (table entries) and per-edge slots (cap)
-    uint32_t *d_tpos = nullptr, *d_slot = nullptr;
+    GroupScratch group;        // staging of inserts and deletes
     uint32_t *h_pinned = nullptr;
 };
 
@@ -253,27 +250,28 @@ __device__ __forceinline__ int group_set_delete(const GView &g, bool go, uint32_
 
 } // namespace
 
-// One warp per chunk of 32 edges: eight 4-lane groups take the chunk's first
-// occurrences eight at a time (edge it * 8 + group in step it), so eight
-// chains are walked at once.
-__global__ void __launch_bounds__(256) k_set_insert(GView g, const uint32_t *__restrict__ src,
-                                                    const uint32_t *__restrict__ dst, uint64_t n,
-                                                    const uint32_t *__restrict__ tpos,
-                                                    const uint32_t *__restrict__ slot, uint8_t *__restrict__ flags,
+// The lists with many edges in the batch (grouping.many), 32 edges a warp:
+// eight 4-lane groups take the first occurrences among them eight at a time,
+// so eight chains are walked at once.
+template <bool kInsert>
+__global__ void __launch_bounds__(256) k_set_update(GView g, GroupView gv, const uint32_t *__restrict__ src,
+                                                    const uint32_t *__restrict__ dst, uint8_t *__restrict__ flags,
                                                     uint32_t max_hops)
 {
     const uint32_t lane = lane_id(), gi = lane >> 2;
     const uint64_t warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
+    const uint32_t n = __ldg(&gv.ctr[kGroupMany]);
+    const uint32_t *order = gv.many + __ldg(&gv.ctr[kGroupActive]);
+    const uint32_t *tpos = reinterpret_cast<const uint32_t *>(gv.ent);
     unsigned long long loads = 0, linked = 0;
     for (uint64_t q0 = ((blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5) * 32; q0 < n; q0 += warps * 32) {
         if (__any_sync(kFull, status_hint(g.st) != 0))
             break;
-        const uint64_t i = q0 + lane;
         bool first = false;
-        uint32_t s = 0, d = 0;
-        if (i < n) {
-            const uint32_t sl = slot[i];
-            first = sl != kNil && __ldcg(&tpos[sl]) == (uint32_t)i;
+        uint32_t i = 0, s = 0, d = 0;
+        if (q0 + lane < n) {
+            i = order[q0 + lane];
+            first = __ldcg(&tpos[gv.lst[i] & ~kSlotBit]) == i;
             s = src[i];
             d = dst[i];
         }
@@ -282,8 +280,9 @@ __global__ void __launch_bounds__(256) k_set_insert(GView g, const uint32_t *__r
         for (uint32_t it = 0; it < 4; ++it) {
             const uint32_t who = it * 8 + gi;
             const bool go = __shfl_sync(kFull, first, who);
-            const int r = group_set_insert(g, go, __shfl_sync(kFull, s, who), __shfl_sync(kFull, d, who), max_hops,
-                                           loads, linked);
+            const uint32_t ws = __shfl_sync(kFull, s, who), wd = __shfl_sync(kFull, d, who);
+            const int r = kInsert ? group_set_insert(g, go, ws, wd, max_hops, loads, linked)
+                                  : group_set_delete(g, go, ws, wd, max_hops, loads);
             if (r < 0 && (lane & 3u) == 0)
                 set_status(g.st, r);
             // lane L's edge was taken by group L % 8 in step L / 8
@@ -291,48 +290,183 @@ __global__ void __launch_bounds__(256) k_set_insert(GView g, const uint32_t *__r
             if (lane / 8 == it)
                 mine = rl > 0 ? 1 : 0;
         }
-        if (flags && i < n)
-            flags[i] = mine;
+        if (flags && mine)
+            flags[i] = 1;
+    }
+    count_add(g.st, kInsert ? kCtrInsertSlabs : kCtrDeleteSlabs, loads);
+    count_add(g.st, kCtrInsertNewSlabs, linked);
+}
+
+namespace {
+
+// Bit q: the lane's key q of a slab is k (the last lane's eighth word is the
+// next index).
+__device__ __forceinline__ uint32_t set_keys_with(const uint4 &lo, const uint4 &hi, uint32_t k)
+{
+    return (lo.x == k ? 1u : 0u) | (lo.y == k ? 2u : 0u) | (lo.z == k ? 4u : 0u) | (lo.w == k ? 8u : 0u) |
+           (hi.x == k ? 16u : 0u) | (hi.y == k ? 32u : 0u) | (hi.z == k ? 64u : 0u) |
+           ((lane_id() & 3u) != 3u && hi.w == k ? 128u : 0u);
+}
+
+using SetMask = unsigned long long; // over a list's edges
+static_assert(kSetGroupMax <= 64, "a bit an edge");
+
+} // namespace
+
+// Applies the grouped inserts, one list a 4-lane group, eight a warp, as the
+// weighted store's k_apply_insert does (no weights, no logs): the list's
+// repeats found among its edges, its chain walked once, its free keys filled
+// and pool slabs linked with plain stores.  R-MAT scale 19 load, 8.4 M edges
+// into 0.9 M lists, staging included: 720 us with a batch hash set and a CAS
+// an edge, 470 so.
+__global__ void __launch_bounds__(256, 4) k_set_apply_insert(GView g, GroupView gv, uint8_t *__restrict__ flags,
+                                                             uint32_t max_hops)
+{
+    __shared__ uint2 rows[kGroupLists][kSetGroupMax + 1];    // each list's edges (an odd stride: the lists of a
+    __shared__ uint32_t fresh[kGroupLists][kSetGroupMax + 1]; // warp differ in their banks), and its new keys
+    const uint32_t lane = lane_id(), s4 = lane & 3u, gbase = lane & ~3u;
+    uint2 *row = rows[threadIdx.x >> 2];
+    uint32_t *add = fresh[threadIdx.x >> 2];
+    const bool dead = read_status(g.st) != 0;
+    ListCursor cur = first_lists(g, gv);
+    unsigned long long loads = 0, linked = 0;
+    while (__any_sync(kFull, cur.at < cur.n)) {
+        const uint3 my = next_list(gv, cur, dead);
+        const uint32_t L = my.x, c = my.y;
+        if (!__any_sync(kFull, c))
+            continue;
+        uint4 lo = make_uint4(kEmptyKey, kEmptyKey, kEmptyKey, kEmptyKey), hi = lo;
+        if (c)
+            set_group_load(g, L, lo, hi);
+        SetMask news = group_first<SetMask>(gv, c, my.z, row), have = 0;
+        uint32_t slab = L, frees = 0;
+        bool active = c != 0;
+        int err = 0;
+        for (uint32_t hop = 0; __any_sync(kFull, active); ++hop) {
+            if (active && hop)
+                set_group_load(g, slab, lo, hi);
+            loads += __popc(__ballot_sync(kFull, active && s4 == 0));
+            const bool empty = __shfl_sync(kFull, lo.x, gbase) == kEmptyKey; // keys fill in order
+            if (active && !empty)
+                for (uint32_t e = 0; e < c; ++e)
+                    have |= (SetMask)(set_keys_with(lo, hi, row[e].x) != 0) << e;
+            const uint32_t f = group_or(set_keys_with(lo, hi, kEmptyKey) << (8 * s4));
+            const uint32_t nxt = __shfl_sync(kFull, hi.w, gbase + 3);
+            if (active) {
+                frees = f;
+                if (f || nxt == kNil) {
+                    active = false; // the tail: free keys exist only in the last slab
+                } else if (hop + 1 >= max_hops) {
+                    err = kErrTimeout;
+                    active = false;
+                } else {
+                    slab = nxt;
+                }
+            }
+        }
+        news = err ? 0ull : news & ~group_or(have);
+        const uint32_t k = __popcll(news), room = __popc(frees);
+        for (uint32_t e = s4; e < c; e += 4)
+            if ((news >> e) & 1u)
+                add[__popcll(news & ((1ull << e) - 1))] = row[e].x;
+        __syncwarp();
+#pragma unroll
+        for (uint32_t q = 0; q < 8; ++q) {
+            const uint32_t p = 8 * s4 + q, r = __popc(frees & ((1u << p) - 1));
+            if (((frees >> p) & 1u) && r < k)
+                slab_ptr(g, slab)[p] = add[r];
+        }
+        uint32_t stored = min(k, room), prev = slab;
+        for (uint32_t t = 0; __any_sync(kFull, !err && stored < k); ++t) {
+            const bool grow = !err && stored < k;
+            uint32_t ns = kNil;
+            if (grow && s4 == 0)
+                ns = alloc_slab_one(g, L * 0x9E3779B9u ^ (t << 24));
+            ns = __shfl_sync(kFull, ns, gbase);
+            linked += __popc(__ballot_sync(kFull, grow && ns != kNil && s4 == 0));
+            if (grow && ns == kNil)
+                err = kErrPool;
+            if (grow && ns != kNil) {
+                uint32_t w[8];
+#pragma unroll
+                for (uint32_t q = 0; q < 8; ++q) {
+                    const uint32_t r = stored + 8 * s4 + q;
+                    w[q] = r < k && 8 * s4 + q < kSetKeys ? add[r] : kEmptyKey;
+                }
+                if (s4 == 3u)
+                    w[7] = kNil;
+                uint4 *to = reinterpret_cast<uint4 *>(slab_ptr(g, ns) + s4 * 8);
+                __stcg(to, make_uint4(w[0], w[1], w[2], w[3]));
+                __stcg(to + 1, make_uint4(w[4], w[5], w[6], w[7]));
+                if (s4 == 3u) // lane 3 holds the next words, so it links what it wrote before
+                    slab_ptr(g, prev)[kNextLane] = ns;
+                if (s4 == 0)
+                    g.owner[ns] = __ldg(&g.owner[L]);
+                prev = ns;
+                stored = min(k, stored + kSetKeys);
+            }
+        }
+        if (err && s4 == 0)
+            set_status(g.st, err);
+        if (flags)
+            for (uint32_t e = s4; e < c; e += 4)
+                if (((news >> e) & 1u) && (uint32_t)__popcll(news & ((1ull << e) - 1)) < stored)
+                    flags[row[e].y] = 1;
     }
     count_add(g.st, kCtrInsertSlabs, loads);
     count_add(g.st, kCtrInsertNewSlabs, linked);
 }
 
-// Deletes, in the same chunks and groups.
-__global__ void __launch_bounds__(256) k_set_delete(GView g, const uint32_t *__restrict__ src,
-                                                    const uint32_t *__restrict__ dst, uint64_t n,
-                                                    const uint32_t *__restrict__ tpos,
-                                                    const uint32_t *__restrict__ slot, uint8_t *__restrict__ flags,
-                                                    uint32_t max_hops)
+// Applies the grouped deletes in the same way.
+__global__ void __launch_bounds__(256, 5) k_set_apply_delete(GView g, GroupView gv, uint8_t *__restrict__ flags,
+                                                             uint32_t max_hops)
 {
-    const uint32_t lane = lane_id(), gi = lane >> 2;
-    const uint64_t warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
+    __shared__ uint2 rows[kGroupLists][kSetGroupMax + 1];
+    const uint32_t lane = lane_id(), s4 = lane & 3u, gbase = lane & ~3u;
+    uint2 *row = rows[threadIdx.x >> 2];
+    const bool dead = read_status(g.st) != 0;
+    ListCursor cur = first_lists(g, gv);
     unsigned long long loads = 0;
-    for (uint64_t q0 = ((blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5) * 32; q0 < n; q0 += warps * 32) {
-        if (__any_sync(kFull, status_hint(g.st) != 0))
-            break;
-        const uint64_t i = q0 + lane;
-        bool first = false;
-        uint32_t s = 0, d = 0;
-        if (i < n) {
-            const uint32_t sl = slot[i];
-            first = sl != kNil && __ldcg(&tpos[sl]) == (uint32_t)i;
-            s = src[i];
-            d = dst[i];
+    while (__any_sync(kFull, cur.at < cur.n)) {
+        const uint3 my = next_list(gv, cur, dead);
+        const uint32_t L = my.x, c = my.y;
+        if (!__any_sync(kFull, c))
+            continue;
+        uint4 lo = make_uint4(kEmptyKey, kEmptyKey, kEmptyKey, kEmptyKey), hi = lo;
+        if (c)
+            set_group_load(g, L, lo, hi);
+        SetMask todo = group_first<SetMask>(gv, c, my.z, row), gone = 0;
+        uint32_t slab = L;
+        bool active = c != 0;
+        for (uint32_t hop = 0; __any_sync(kFull, active); ++hop) {
+            if (active && hop)
+                set_group_load(g, slab, lo, hi);
+            loads += __popc(__ballot_sync(kFull, active && s4 == 0));
+            SetMask hit = 0;
+            if (active)
+                for (SetMask left = todo; left; left &= left - 1) {
+                    const uint32_t e = __ffsll((long long)left) - 1, at = set_keys_with(lo, hi, row[e].x);
+                    if (at) {
+                        hit |= 1ull << e;
+                        slab_ptr(g, slab)[8 * s4 + __ffs(at) - 1] = kTombKey;
+                    }
+                }
+            hit = group_or(hit);
+            const uint32_t f = group_or(set_keys_with(lo, hi, kEmptyKey));
+            const uint32_t nxt = __shfl_sync(kFull, hi.w, gbase + 3);
+            todo &= ~hit;
+            gone |= hit;
+            if (active) {
+                if (!todo || f || nxt == kNil || hop + 1 >= max_hops)
+                    active = false;
+                else
+                    slab = nxt;
+            }
         }
-        uint8_t mine = 0;
-#pragma unroll 1
-        for (uint32_t it = 0; it < 4; ++it) {
-            const uint32_t who = it * 8 + gi;
-            const bool go = __shfl_sync(kFull, first, who);
-            const int r = group_set_delete(g, go, __shfl_sync(kFull, s, who), __shfl_sync(kFull, d, who), max_hops,
-                                           loads);
-            const int rl = __shfl_sync(kFull, r, (lane & 7u) * 4);
-            if (lane / 8 == it)
-                mine = rl > 0 ? 1 : 0;
-        }
-        if (flags && i < n)
-            flags[i] = mine;
+        if (flags)
+            for (uint32_t e = s4; e < c; e += 4)
+                if ((gone >> e) & 1u)
+                    flags[row[e].y] = 1;
     }
     count_add(g.st, kCtrDeleteSlabs, loads);
 }
@@ -573,41 +707,42 @@ mk_status set_alloc(mk_set_graph *g, void **p, size_t bytes)
     return MK_OK;
 }
 
-void set_free(mk_set_graph *g, void *p, size_t bytes)
-{
-    if (p) {
-        cudaFree(p);
-        g->bytes -= bytes;
-    }
-}
-
-mk_status set_stage(mk_set_graph *g, const uint32_t *src, const uint32_t *dst, uint64_t n, cudaStream_t s)
-{
-    if (n > g->cap) {
-        uint64_t cap = std::max<uint64_t>(n, std::max<uint64_t>(1024, g->cap + g->cap / 2)), table = 1;
-        while (table < 2 * cap)
-            table <<= 1;
-        MK_CUDA(cudaStreamSynchronize(s));
-        set_free(g, g->d_tpos, g->table * 4);
-        set_free(g, g->d_slot, g->cap * 4);
-        g->d_tpos = g->d_slot = nullptr;
-        g->cap = g->table = 0;
-        MK_TRY(set_alloc(g, (void **)&g->d_tpos, table * 4));
-        MK_TRY(set_alloc(g, (void **)&g->d_slot, cap * 4));
-        g->cap = cap;
-        g->table = table;
-    }
-    MK_CUDA(cudaMemsetAsync(g->d_tpos, 0xFF, g->table * 4, s));
-    k_dedup<<<grid_for(n, 256), 256, 0, s>>>(src, dst, nullptr, n, g->v.V, g->d_tpos, (uint32_t)(g->table - 1),
-                                             g->d_slot, g->v.st);
-    MK_CUDA(cudaGetLastError());
-    return MK_OK;
-}
-
 uint32_t set_grid(uint64_t items_per_warp32)
 {
     return std::min<uint32_t>(grid_for(std::max<uint64_t>(items_per_warp32, 1) * 32, 256), num_sms() * 32);
 }
+
+// Inserts or deletes n edges, in parts of at most kGroupEdges (a batch of more
+// is checked whole first, so that it is still rejected whole).
+template <bool kInsert>
+mk_status set_apply(mk_set_graph *g, const uint32_t *d_src, const uint32_t *d_dst, uint64_t n, uint8_t *d_flags,
+                    cudaStream_t s)
+{
+    if (d_flags)
+        MK_CUDA(cudaMemsetAsync(d_flags, 0, n, s));
+    if (n > kGroupEdges)
+        k_check_edges<<<grid_for(n, 256), 256, 0, s>>>(d_src, d_dst, nullptr, n, g->v.V, g->v.st);
+    for (uint64_t at = 0; at < n; at += kGroupEdges) {
+        const uint64_t m = std::min(kGroupEdges, n - at);
+        const uint32_t *src = d_src + at, *dst = d_dst + at;
+        uint8_t *fl = d_flags ? d_flags + at : nullptr;
+        GroupView gv{};
+        int launches = 0;
+        MK_CUDA(group_reserve(g->group, m, g->v.H, s, &g->bytes));
+        MK_CUDA(group_batch(g->v, g->group, src, dst, nullptr, m, kSetGroupMax, s, &gv, &launches));
+        k_set_update<kInsert><<<set_grid((m + 31) / 32), 256, 0, s>>>(g->v, gv, src, dst, fl, g->v.P + 2);
+        const uint64_t lists = group_dense(g->v.H, m) ? g->v.H : m;
+        const uint32_t grid = (uint32_t)std::min<uint64_t>((lists + kGroupLists - 1) / kGroupLists,
+                                                           (uint64_t)num_sms() * (kInsert ? 4 : 5));
+        if (kInsert)
+            k_set_apply_insert<<<grid, 256, 0, s>>>(g->v, gv, fl, g->v.P + 2);
+        else
+            k_set_apply_delete<<<grid, 256, 0, s>>>(g->v, gv, fl, g->v.P + 2);
+        MK_CUDA(cudaGetLastError());
+    }
+    return MK_OK;
+}
+
 
 } // namespace
 
@@ -643,8 +778,7 @@ mk_status mk_set_destroy(mk_set_graph *g)
     cudaFree(g->v.bitmap);
     cudaFree(g->v.owner);
     cudaFree(g->v.st);
-    cudaFree(g->d_tpos);
-    cudaFree(g->d_slot);
+    group_release(g->group, &g->bytes);
     if (g->h_pinned)
         cudaFreeHost(g->h_pinned);
     delete g;
@@ -733,14 +867,7 @@ mk_status mk_set_insert_batch(mk_set_graph *g, const uint32_t *d_src, const uint
         return MK_ERR_INVALID_ARG;
     if (!n)
         return MK_OK;
-    cudaStream_t s = (cudaStream_t)stream;
-    if (d_inserted)
-        MK_CUDA(cudaMemsetAsync(d_inserted, 0, n, s));
-    MK_TRY(set_stage(g, d_src, d_dst, n, s));
-    k_set_insert<<<set_grid((n + 31) / 32), 256, 0, s>>>(g->v, d_src, d_dst, n, g->d_tpos, g->d_slot, d_inserted,
-                                                        g->v.P + 2);
-    MK_CUDA(cudaGetLastError());
-    return MK_OK;
+    return set_apply<true>(g, d_src, d_dst, n, d_inserted, (cudaStream_t)stream);
 }
 
 mk_status mk_set_delete_batch(mk_set_graph *g, const uint32_t *d_src, const uint32_t *d_dst, uint64_t n,
@@ -750,14 +877,7 @@ mk_status mk_set_delete_batch(mk_set_graph *g, const uint32_t *d_src, const uint
         return MK_ERR_INVALID_ARG;
     if (!n)
         return MK_OK;
-    cudaStream_t s = (cudaStream_t)stream;
-    if (d_deleted)
-        MK_CUDA(cudaMemsetAsync(d_deleted, 0, n, s));
-    MK_TRY(set_stage(g, d_src, d_dst, n, s));
-    k_set_delete<<<set_grid((n + 31) / 32), 256, 0, s>>>(g->v, d_src, d_dst, n, g->d_tpos, g->d_slot, d_deleted,
-                                                        g->v.P + 2);
-    MK_CUDA(cudaGetLastError());
-    return MK_OK;
+    return set_apply<false>(g, d_src, d_dst, n, d_deleted, (cudaStream_t)stream);
 }
 
 mk_status mk_set_query_batch(mk_set_graph *g, const uint32_t *d_src, const uint32_t *d_dst, uint64_t n,

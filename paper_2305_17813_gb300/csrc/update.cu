@@ -675,48 +675,6 @@ __device__ __forceinline__ void log_lists(const GView &g, uint32_t *buf, uint32_
     __syncwarp();
 }
 
-// The lists of an apply kernel's steps, one a group and step: the list is
-// read two steps ahead, its count and range one step ahead.
-struct ListCursor {
-    uint64_t at, step;
-    uint32_t n, L, L1;
-    uint2 sl;
-};
-
-__device__ __forceinline__ uint32_t list_at(const GroupView &gv, uint64_t k, uint32_t n)
-{
-    return k < n ? (gv.alist ? __ldg(&gv.alist[k]) : (uint32_t)k) : kNil;
-}
-
-__device__ __forceinline__ ListCursor first_lists(const GView &g, const GroupView &gv)
-{
-    ListCursor c;
-    c.n = gv.alist ? __ldg(&gv.ctr[kGroupActive]) : g.H;
-    c.at = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 2;
-    c.step = ((uint64_t)gridDim.x * blockDim.x) >> 2;
-    c.L = list_at(gv, c.at, c.n);
-    c.L1 = list_at(gv, c.at + c.step, c.n);
-    c.sl = c.L != kNil ? gv.slot[c.L] : make_uint2(0, 0);
-    return c;
-}
-
-// <list, edges, offset> of the calling lane's group, kNil and 0 without work;
-// the list's count is set back.  Called by the full warp.
-__device__ __forceinline__ uint3 next_list(const GroupView &gv, ListCursor &c, bool dead)
-{
-    const uint32_t L = c.L;
-    const uint2 sl = c.sl;
-    c.at += c.step;
-    c.L = c.L1;
-    c.L1 = list_at(gv, c.at + c.step, c.n);
-    c.sl = c.L != kNil ? gv.slot[c.L] : make_uint2(0, 0);
-    __syncwarp();
-    if (sl.x && (lane_id() & 3u) == 0)
-        gv.slot[L].x = 0;
-    const bool mine = sl.x != 0 && sl.x <= kGroupMax && !dead;
-    return make_uint3(mine ? L : kNil, mine ? sl.x : 0u, sl.y);
-}
-
 // Bit q: the lane's pair q of a slab is free (layout of first_pair_with).
 __device__ __forceinline__ uint32_t free_pairs(const uint4 &lo, const uint4 &hi)
 {
@@ -727,12 +685,6 @@ __device__ __forceinline__ uint32_t free_pairs(const uint4 &lo, const uint4 &hi)
 __device__ __forceinline__ bool lane_has(const uint4 &lo, const uint4 &hi, uint32_t d)
 {
     return lo.x == d || lo.z == d || hi.x == d || ((lane_id() & 3u) != 3u && hi.z == d);
-}
-
-__device__ __forceinline__ uint32_t group_or(uint32_t m)
-{
-    m |= __shfl_xor_sync(kFull, m, 1);
-    return m | __shfl_xor_sync(kFull, m, 2);
 }
 
 } // namespace
@@ -770,7 +722,7 @@ __global__ void __launch_bounds__(256, 5) k_apply_insert(GView g, GroupView gv, 
                 src = __ldg(&g.list_src[L]);
                 seen = *(volatile const uint8_t *)&g.lupd[L];
             }
-            uint32_t news = group_first(gv, c, my.z, row);
+            uint32_t news = group_first<uint32_t>(gv, c, my.z, row);
             // walk the whole chain: a present destination is a duplicate
             uint32_t slab = L, have = 0, nxt = kNil, frees = 0;
             bool active = c != 0;
@@ -779,7 +731,8 @@ __global__ void __launch_bounds__(256, 5) k_apply_insert(GView g, GroupView gv, 
                 if (active && hop)
                     group_load(g, slab, lo, hi);
                 loads += __popc(__ballot_sync(kFull, active && s4 == 0));
-                if (active)
+                const bool empty = __shfl_sync(kFull, lo.x, gbase) == kEmptyKey; // pairs fill in order
+                if (active && !empty)
                     for (uint32_t e = 0; e < c; ++e)
                         have |= (lane_has(lo, hi, row[e].x) ? 1u : 0u) << e;
                 const uint32_t f = group_or(free_pairs(lo, hi) << (4 * s4));
@@ -886,7 +839,7 @@ __global__ void __launch_bounds__(256, 6) k_apply_delete(GView g, GroupView gv, 
                 group_load(g, L, lo, hi);
                 src = __ldg(&g.list_src[L]);
             }
-            uint32_t todo = group_first(gv, c, my.z, row), slab = L;
+            uint32_t todo = group_first<uint32_t>(gv, c, my.z, row), slab = L;
             bool active = c != 0;
             for (uint32_t hop = 0; __any_sync(kFull, active); ++hop) {
                 if (active && hop)
@@ -951,7 +904,7 @@ mk_status stage(mk_graph *g, const uint32_t *src, const uint32_t *dst, const uin
     int launches = 0;
     MK_CUDA(group_reserve(g->group, n, g->v.H, s, &g->bytes));
     const mk_status st = timed(g, "stage_group", s, 0, [&]() {
-        return group_batch(g->v, g->group, src, dst, w, n, s, gv, &launches);
+        return group_batch(g->v, g->group, src, dst, w, n, kGroupMax, s, gv, &launches);
     });
     g->launches += (uint64_t)launches;
     return st;
