@@ -112,8 +112,17 @@ mk_status mk_graph_create_ex(const mk_config *cfg, void *stream, mk_graph **out)
 mk_status mk_graph_create(uint32_t V, uint64_t edge_capacity_hint, uint32_t buckets,
                           const uint32_t *d_bucket_per_vertex, void *stream, mk_graph **out);
 
-/* Frees every device buffer of the graph after synchronising the device. */
+/* Frees every device buffer of the graph after synchronising the device.
+ * Device memory comes from a memory pool of the library (one a device, apart
+ * from the process's default pool), which keeps up to 2 GiB that nothing uses
+ * for the next graph or call; see mk_trim. */
 mk_status mk_graph_destroy(mk_graph *g);
+
+/* Gives the memory that the library's pool of the current device holds and
+ * nothing uses back to the device (the paper has no counterpart: this is a
+ * service of this library).  The pool does so by itself beyond 2 GiB, and when
+ * one of the library's own allocations would fail.  Synchronises the device. */
+mk_status mk_trim(void);
 
 /* ---------------------------------------------------------------- updates */
 

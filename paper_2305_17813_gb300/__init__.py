@@ -21,7 +21,7 @@ from ._native import (MK_ERR_CUDA, MK_ERR_INTERNAL, MK_ERR_INVALID_ARG, MK_ERR_N
 
 __all__ = [
     "Graph", "load", "MkError", "MK_OK", "MK_ERR_INVALID_ARG", "MK_ERR_POOL_EXHAUSTED", "MK_ERR_TIMEOUT",
-    "MK_ERR_CUDA", "MK_ERR_NO_MEMORY", "MK_ERR_INTERNAL", "MK_NONE", "MK_INVALID_LANE", "bucket_rule",
+    "MK_ERR_CUDA", "MK_ERR_NO_MEMORY", "MK_ERR_INTERNAL", "MK_NONE", "MK_INVALID_LANE", "bucket_rule", "trim",
     "to_device_u32", "to_numpy_u32", "Batcher", "Server", "SetGraph", "set_bucket_rule", "MK_L2_NONE", "MK_L2_VINFO", "MK_L2_HEADS", "MK_L2_POOL",
 ]
 
@@ -72,6 +72,12 @@ def bucket_rule(V: int, src, load_factor: float = 0.7, stream=None):
     out = torch.empty(V, dtype=torch.int32, device=s.device)
     check(lib.mk_bucket_rule(V, _ptr(s), s.numel(), load_factor, _ptr(out), _stream(stream)), "mk_bucket_rule")
     return out
+
+
+def trim():
+    """Give device memory that the library keeps for later graphs back
+    (mk_trim)."""
+    check(load().mk_trim(), "mk_trim")
 
 
 class Graph:

@@ -124,6 +124,7 @@ SIGNATURES = {
     "mk_graph_create_ex": (_INT, [ctypes.POINTER(mk_config), _P, ctypes.POINTER(_P)]),
     "mk_graph_create": (_INT, [_U32, _U64, _U32, _P, _P, ctypes.POINTER(_P)]),
     "mk_graph_destroy": (_INT, [_P]),
+    "mk_trim": (_INT, []),
     "mk_insert_batch": (_INT, [_P, _P, _P, _P, _U64, _P, _P]),
     "mk_insert_batch_noalloc": (_INT, [_P, _P, _P, _P, _U64, _P, _P]),
     "mk_delete_batch": (_INT, [_P, _P, _P, _U64, _P, _P]),

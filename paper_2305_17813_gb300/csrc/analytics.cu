@@ -850,7 +850,7 @@ mk_status mk_pagerank(mk_graph *g, float *d_pr, int warm_start, float damping, f
     // per-vertex arrays and counters in one block; the bins' counts and
     // places, and the edges, in another
     unsigned char *vert = nullptr, *bin = nullptr;
-    MK_CUDA(cudaMallocAsync((void **)&vert, (size_t)V * (16 + 3 * 8 + 4) + sizeof(PrCtr), s));
+    MK_CUDA(pool_alloc((void **)&vert, (size_t)V * (16 + 3 * 8 + 4) + sizeof(PrCtr), s));
     OutDegree *deg = (OutDegree *)vert;
     unsigned long long *pr = (unsigned long long *)(deg + V), *acc = pr + V, *contrib = acc + V;
     PrCtr *ctr = (PrCtr *)(contrib + V);
@@ -863,7 +863,7 @@ mk_status mk_pagerank(mk_graph *g, float *d_pr, int warm_start, float damping, f
     void *edges = nullptr;
     cuda(cudaMemsetAsync(ctr, 0, sizeof(PrCtr) + (size_t)V * 4, s));
     if (st == MK_OK && binned) {
-        if (cudaMallocAsync((void **)&bin, cells * 12 + 8 + scan_bytes, s) != cudaSuccess) {
+        if (pool_alloc((void **)&bin, cells * 12 + 8 + scan_bytes, s) != cudaSuccess) {
             cudaGetLastError();
             bin = nullptr;
             binned = false;
@@ -886,7 +886,7 @@ mk_status mk_pagerank(mk_graph *g, float *d_pr, int warm_start, float damping, f
         if (st == MK_OK && cuda(cudaStreamSynchronize(s))) {
             std::memcpy(&edges_n, g->h_pinned, 8);
             const size_t rec = packed ? 4 : 8, chunks = bins + edges_n / kChunk;
-            if (cudaMallocAsync((void **)&chunk, chunks * 16 + edges_n * rec, s) != cudaSuccess) {
+            if (pool_alloc((void **)&chunk, chunks * 16 + edges_n * rec, s) != cudaSuccess) {
                 cudaGetLastError();
                 chunk = nullptr;
                 binned = false;
@@ -981,7 +981,7 @@ mk_status mk_tc_count(mk_graph *g1, mk_graph *g2, const uint32_t *d_src, const u
     cudaStream_t s = (cudaStream_t)stream;
     const uint32_t grid = std::min<uint64_t>(grid_for(n * 32, 256), (uint64_t)resident_grid(k_tc_count, 256));
     unsigned long long *next = nullptr;
-    MK_CUDA(cudaMallocAsync((void **)&next, 8, s));
+    MK_CUDA(pool_alloc((void **)&next, 8, s));
     MK_CUDA(cudaMemsetAsync(next, 0, 8, s));
     const mk_status st = timed(g1, "tc_count", s, 1, [&]() {
         k_tc_count<<<grid, 256, 0, s>>>(g1->v, g2->v, d_src, d_dst, n, g1->v.P + 2, g2->v.P + 2, d_total, next);
@@ -1001,7 +1001,7 @@ mk_status mk_tc_static(mk_graph *g, uint64_t *h_triangles, void *stream)
     // are, read back first) in another
     unsigned char *block = nullptr;
     const size_t bytes = V * (16 + 4 + 4 + 4) + kTcWords * 8;
-    MK_CUDA(cudaMallocAsync((void **)&block, bytes, s));
+    MK_CUDA(pool_alloc((void **)&block, bytes, s));
     TcArrays t{};
     t.list = (ulonglong2 *)block;
     t.ctr = (unsigned long long *)(t.list + V);
@@ -1027,7 +1027,7 @@ mk_status mk_tc_static(mk_graph *g, uint64_t *h_triangles, void *stream)
     if (st == MK_OK)
         cuda(cudaStreamSynchronize(s));
     if (st == MK_OK && total) {
-        if (cuda(cudaMallocAsync((void **)&t.adj, total * 4, s)))
+        if (cuda(pool_alloc((void **)&t.adj, total * 4, s)))
             st = timed(g, "tc_static", s, 3, [&]() {
                 k_tc_orient<true><<<slab_grid, kTcThreads, 0, s>>>(g->v, t);
                 // a bitmap of up to 128 KB (2^20 vertices), with blocks large
@@ -1073,7 +1073,7 @@ mk_status mk_tc_update(mk_graph *g_post, mk_graph *g_upd, const uint32_t *d_src,
         return MK_ERR_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)stream;
     unsigned long long *d = nullptr;
-    MK_CUDA(cudaMallocAsync((void **)&d, 24, s));
+    MK_CUDA(pool_alloc((void **)&d, 24, s));
     MK_CUDA(cudaMemsetAsync(d, 0, 24, s));
     mk_status st = mk_tc_count(g_post, g_post, d_src, d_dst, n, d + 0, stream);
     if (st == MK_OK)

@@ -99,7 +99,7 @@ mk_status mk_query_multi(mk_graph *g, const mk_query_req *h_reqs, uint32_t nreq,
     if (!total)
         return MK_OK;
     unsigned char *d = nullptr;
-    MK_CUDA(cudaMallocAsync((void **)&d, img.size(), s));
+    MK_CUDA(pool_alloc((void **)&d, img.size(), s));
     MK_CUDA(cudaMemcpyAsync(d, img.data(), img.size(), cudaMemcpyHostToDevice, s));
     const QueryReq *reqs = reinterpret_cast<const QueryReq *>(d);
     const uint64_t *prefix = reinterpret_cast<const uint64_t *>(d + nreq * sizeof(QueryReq));

@@ -11,26 +11,23 @@ using namespace mk;
 
 namespace mk {
 
-mk_status device_alloc(mk_graph *g, void **p, size_t bytes)
+mk_status device_alloc(mk_graph *g, void **p, size_t bytes, cudaStream_t s)
 {
     *p = nullptr;
     if (bytes == 0)
         return MK_OK;
-    cudaError_t e = cudaMalloc(p, bytes);
-    if (e != cudaSuccess) {
-        cudaGetLastError();
-        *p = nullptr;
+    const cudaError_t e = pool_alloc_kept(p, bytes, s);
+    if (e != cudaSuccess)
         return e == cudaErrorMemoryAllocation ? MK_ERR_NO_MEMORY : MK_ERR_CUDA;
-    }
     if (g)
         g->bytes += bytes;
     return MK_OK;
 }
 
-void device_free(mk_graph *g, void *p, size_t bytes)
+void device_free(mk_graph *g, void *p, size_t bytes, cudaStream_t s)
 {
     if (p) {
-        cudaFree(p);
+        pool_free(p, s);
         if (g)
             g->bytes -= bytes;
     }
@@ -355,16 +352,16 @@ static uint32_t bits_for(uint32_t V)
 static void destroy_consumer(mk_graph *g, Consumer *c)
 {
     const size_t V = g->v.V, H = g->v.H;
-    device_free(g, c->D, V * 8);
-    device_free(g, c->front[0], H * 8);
-    device_free(g, c->front[1], H * 8);
-    device_free(g, c->stamp, V * 4);
-    device_free(g, c->inv, (V + 31) / 32 * 4);
-    device_free(g, c->uf, V * 4);
-    device_free(g, c->far[0], V * 4);
-    device_free(g, c->far[1], V * 4);
-    device_free(g, c->fstamp, V * 4);
-    device_free(g, c->counters, kConsumerWords * 4);
+    device_free(g, c->D, V * 8, nullptr);
+    device_free(g, c->front[0], H * 8, nullptr);
+    device_free(g, c->front[1], H * 8, nullptr);
+    device_free(g, c->stamp, V * 4, nullptr);
+    device_free(g, c->inv, (V + 31) / 32 * 4, nullptr);
+    device_free(g, c->uf, V * 4, nullptr);
+    device_free(g, c->far[0], V * 4, nullptr);
+    device_free(g, c->far[1], V * 4, nullptr);
+    device_free(g, c->fstamp, V * 4, nullptr);
+    device_free(g, c->counters, kConsumerWords * 4, nullptr);
     delete c;
 }
 
@@ -381,7 +378,7 @@ mk_status mk_bucket_rule(uint32_t V, const uint32_t *d_src, uint64_t n, float lo
         return MK_ERR_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)stream;
     int *d_bad = nullptr;
-    MK_CUDA(cudaMallocAsync((void **)&d_bad, sizeof(int), s));
+    MK_CUDA(pool_alloc((void **)&d_bad, sizeof(int), s));
     MK_CUDA(cudaMemsetAsync(d_bad, 0, sizeof(int), s));
     MK_CUDA(cudaMemsetAsync(d_buckets, 0, (size_t)V * 4, s));
     if (n)
@@ -411,21 +408,21 @@ mk_status mk_graph_create_ex(const mk_config *cfg, void *stream, mk_graph **out)
     uint64_t *d_off = nullptr;
     int *d_bad = nullptr;
     mk_status st = MK_OK;
-    st = device_alloc(nullptr, (void **)&d_b, (size_t)V * 4);
+    st = device_alloc(nullptr, (void **)&d_b, (size_t)V * 4, s);
     if (st == MK_OK)
-        st = device_alloc(nullptr, (void **)&d_off, (size_t)V * 8);
+        st = device_alloc(nullptr, (void **)&d_off, (size_t)V * 8, s);
     if (st == MK_OK)
-        st = device_alloc(nullptr, (void **)&d_bad, sizeof(int));
+        st = device_alloc(nullptr, (void **)&d_bad, sizeof(int), s);
     if (st != MK_OK) {
-        device_free(nullptr, d_b, 0);
-        device_free(nullptr, d_off, 0);
-        device_free(nullptr, d_bad, 0);
+        device_free(nullptr, d_b, 0, s);
+        device_free(nullptr, d_off, 0, s);
+        device_free(nullptr, d_bad, 0, s);
         return fail(st);
     }
     auto cleanup_tmp = [&]() {
-        device_free(nullptr, d_b, 0);
-        device_free(nullptr, d_off, 0);
-        device_free(nullptr, d_bad, 0);
+        device_free(nullptr, d_b, 0, s);
+        device_free(nullptr, d_off, 0, s);
+        device_free(nullptr, d_bad, 0, s);
         d_b = nullptr;
     };
     cudaMemsetAsync(d_bad, 0, sizeof(int), s);
@@ -434,9 +431,9 @@ mk_status mk_graph_create_ex(const mk_config *cfg, void *stream, mk_graph **out)
     // exclusive scan of bucket counts -> head offsets (one allocation for
     // every head slab; paper, Sec. "Memory Management in Meerkat")
     void *d_tmp = nullptr;
-    if (cudaMalloc(&d_tmp, exclusive_scan_scratch_bytes(V)) != cudaSuccess ||
+    if (pool_alloc(&d_tmp, exclusive_scan_scratch_bytes(V), s) != cudaSuccess ||
         exclusive_scan_u32_u64(d_b, d_off, V, d_tmp, s, nullptr) != cudaSuccess) {
-        cudaFree(d_tmp);
+        pool_free(d_tmp, s);
         cleanup_tmp();
         return fail(MK_ERR_CUDA);
     }
@@ -447,11 +444,11 @@ mk_status mk_graph_create_ex(const mk_config *cfg, void *stream, mk_graph **out)
     cudaMemcpyAsync(&last_b, d_b + (V - 1), 4, cudaMemcpyDeviceToHost, s);
     cudaMemcpyAsync(&bad, d_bad, 4, cudaMemcpyDeviceToHost, s);
     if (cudaStreamSynchronize(s) != cudaSuccess) {
-        cudaFree(d_tmp);
+        pool_free(d_tmp, s);
         cleanup_tmp();
         return fail(MK_ERR_CUDA);
     }
-    cudaFree(d_tmp);
+    pool_free(d_tmp, s);
     const uint64_t H = last_off + last_b;
     uint64_t P = cfg->pool_slabs;
     if (P == 0)
@@ -466,23 +463,23 @@ mk_status mk_graph_create_ex(const mk_config *cfg, void *stream, mk_graph **out)
     v.H = (uint32_t)H;
     v.P = (uint32_t)P;
     v.pool_words = (uint32_t)(P / 32);
-    st = device_alloc(g, (void **)&v.vinfo, (size_t)V * 8);
+    st = device_alloc(g, (void **)&v.vinfo, (size_t)V * 8, s);
     if (st == MK_OK)
-        st = device_alloc(g, (void **)&v.slabs, (size_t)(H + P) * 128);
+        st = device_alloc(g, (void **)&v.slabs, (size_t)(H + P) * 128, s);
     if (st == MK_OK)
-        st = device_alloc(g, (void **)&v.bitmap, (size_t)v.pool_words * 4 + 4);
+        st = device_alloc(g, (void **)&v.bitmap, (size_t)v.pool_words * 4 + 4, s);
     if (st == MK_OK)
-        st = device_alloc(g, (void **)&v.list_src, (size_t)H * 4);
+        st = device_alloc(g, (void **)&v.list_src, (size_t)H * 4, s);
     if (st == MK_OK)
-        st = device_alloc(g, (void **)&v.lmark, (size_t)H * 8);
+        st = device_alloc(g, (void **)&v.lmark, (size_t)H * 8, s);
     if (st == MK_OK)
-        st = device_alloc(g, (void **)&v.lupd, ((size_t)H + 3) & ~(size_t)3);
+        st = device_alloc(g, (void **)&v.lupd, ((size_t)H + 3) & ~(size_t)3, s);
     if (st == MK_OK)
-        st = device_alloc(g, (void **)&v.ulog, (size_t)H * 4);
+        st = device_alloc(g, (void **)&v.ulog, (size_t)H * 4, s);
     if (st == MK_OK)
-        st = device_alloc(g, (void **)&v.owner, (size_t)(H + P) * 4);
+        st = device_alloc(g, (void **)&v.owner, (size_t)(H + P) * 4, s);
     if (st == MK_OK)
-        st = device_alloc(g, (void **)&g->d_state, sizeof(DevState));
+        st = device_alloc(g, (void **)&g->d_state, sizeof(DevState), s);
     if (st == MK_OK && cudaMallocHost((void **)&g->h_pinned, 64) != cudaSuccess)
         st = MK_ERR_NO_MEMORY;
     if (st != MK_OK) {
@@ -526,18 +523,18 @@ mk_status mk_graph_destroy(mk_graph *g)
         destroy_consumer(g, kv.second);
     g->consumers.clear();
     GView &v = g->v;
-    cudaFree((void *)v.vinfo);
-    cudaFree(v.slabs);
-    cudaFree(v.bitmap);
-    cudaFree((void *)v.list_src);
-    cudaFree(v.lmark);
-    cudaFree(v.lupd);
-    cudaFree(v.ulog);
-    cudaFree(v.owner);
-    cudaFree(g->d_state);
-    group_release(g->group, &g->bytes);
-    cudaFree(g->d_dlog);
-    cudaFree(g->d_ilog);
+    pool_free((void *)v.vinfo, nullptr);
+    pool_free((void *)v.slabs, nullptr);
+    pool_free((void *)v.bitmap, nullptr);
+    pool_free((void *)v.list_src, nullptr);
+    pool_free((void *)v.lmark, nullptr);
+    pool_free((void *)v.lupd, nullptr);
+    pool_free((void *)v.ulog, nullptr);
+    pool_free((void *)v.owner, nullptr);
+    pool_free((void *)g->d_state, nullptr);
+    group_release(g->group, &g->bytes, nullptr);
+    pool_free((void *)g->d_dlog, nullptr);
+    pool_free((void *)g->d_ilog, nullptr);
     if (g->h_pinned)
         cudaFreeHost(g->h_pinned);
     for (auto &t : g->timed) {
@@ -546,6 +543,7 @@ mk_status mk_graph_destroy(mk_graph *g)
     }
     for (auto e : g->spare_events)
         cudaEventDestroy(e);
+    pool_settle();
     delete g;
     return MK_OK;
 }
@@ -588,13 +586,13 @@ mk_status mk_graph_export(mk_graph *g, uint64_t cap, uint32_t *d_src, uint32_t *
     const uint32_t max_hops = g->v.P + 2;
     uint32_t *d_cnt = nullptr;
     uint64_t *d_off = nullptr;
-    MK_CUDA(cudaMallocAsync((void **)&d_cnt, (H + 1) * 4, s));
-    MK_CUDA(cudaMallocAsync((void **)&d_off, (H + 1) * 8, s));
+    MK_CUDA(pool_alloc((void **)&d_cnt, (H + 1) * 4, s));
+    MK_CUDA(pool_alloc((void **)&d_off, (H + 1) * 8, s));
     MK_CUDA(cudaMemsetAsync(d_cnt + H, 0, 4, s));
     k_count_live<<<grid_for(H * 32, 256), 256, 0, s>>>(g->v, d_cnt, max_hops);
     void *d_tmp = nullptr;
     int scan_launches = 0;
-    MK_CUDA(cudaMallocAsync(&d_tmp, exclusive_scan_scratch_bytes(H + 1), s));
+    MK_CUDA(pool_alloc(&d_tmp, exclusive_scan_scratch_bytes(H + 1), s));
     MK_CUDA(exclusive_scan_u32_u64(d_cnt, d_off, H + 1, d_tmp, s, &scan_launches));
     uint64_t m = 0;
     MK_CUDA(cudaMemcpyAsync(&m, d_off + H, 8, cudaMemcpyDeviceToHost, s));
@@ -602,15 +600,15 @@ mk_status mk_graph_export(mk_graph *g, uint64_t cap, uint32_t *d_src, uint32_t *
     uint64_t *k0 = nullptr, *k1 = nullptr;
     uint32_t *w0 = nullptr, *w1 = nullptr;
     const uint64_t mm = std::max<uint64_t>(m, 1);
-    MK_CUDA(cudaMallocAsync((void **)&k0, mm * 8, s));
-    MK_CUDA(cudaMallocAsync((void **)&k1, mm * 8, s));
-    MK_CUDA(cudaMallocAsync((void **)&w0, mm * 4, s));
-    MK_CUDA(cudaMallocAsync((void **)&w1, mm * 4, s));
+    MK_CUDA(pool_alloc((void **)&k0, mm * 8, s));
+    MK_CUDA(pool_alloc((void **)&k1, mm * 8, s));
+    MK_CUDA(pool_alloc((void **)&w0, mm * 4, s));
+    MK_CUDA(pool_alloc((void **)&w1, mm * 4, s));
     k_write_live<<<grid_for(H * 32, 256), 256, 0, s>>>(g->v, d_off, k0, w0, g->vbits, max_hops);
     size_t tb2 = 0;
     MK_CUDA(sort_pairs_u64_u32(nullptr, tb2, k0, k1, w0, w1, m, 2 * g->vbits, s));
     void *d_tmp2 = nullptr;
-    MK_CUDA(cudaMallocAsync(&d_tmp2, std::max<size_t>(tb2, 1), s));
+    MK_CUDA(pool_alloc(&d_tmp2, std::max<size_t>(tb2, 1), s));
     if (m)
         MK_CUDA(sort_pairs_u64_u32(d_tmp2, tb2, k0, k1, w0, w1, m, 2 * g->vbits, s));
     k_decode_export<<<grid_for(mm, 256), 256, 0, s>>>(k1, w1, m, cap, g->vbits, d_src, d_dst, d_w, d_count);
@@ -634,8 +632,8 @@ mk_status mk_graph_stats(mk_graph *g, mk_stats *out, void *stream)
     cudaStream_t s = (cudaStream_t)stream;
     ChainStats *d_cs = nullptr;
     unsigned long long *d_pop = nullptr;
-    MK_CUDA(cudaMallocAsync((void **)&d_cs, sizeof(ChainStats), s));
-    MK_CUDA(cudaMallocAsync((void **)&d_pop, 8, s));
+    MK_CUDA(pool_alloc((void **)&d_cs, sizeof(ChainStats), s));
+    MK_CUDA(pool_alloc((void **)&d_pop, 8, s));
     MK_CUDA(cudaMemsetAsync(d_cs, 0, sizeof(ChainStats), s));
     MK_CUDA(cudaMemsetAsync(d_pop, 0, 8, s));
     k_chain_stats<<<grid_for((uint64_t)g->v.H * 32, 256), 256, 0, s>>>(g->v, d_cs, g->v.P + 2);

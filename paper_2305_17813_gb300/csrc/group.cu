@@ -196,10 +196,10 @@ uint64_t edge_bytes(uint64_t cap) { return cap * kEdgeBytes + (cap / 32 + 16) * 
 
 namespace mk {
 
-void group_release(GroupScratch &gs, uint64_t *bytes)
+void group_release(GroupScratch &gs, uint64_t *bytes, cudaStream_t s)
 {
-    cudaFree(gs.ent);
-    cudaFree(gs.slot);
+    pool_free(gs.ent, s);
+    pool_free(gs.slot, s);
     *bytes -= (gs.cap ? edge_bytes(gs.cap) : 0) + (gs.slot ? (uint64_t)gs.lists * 8 + kGroupWords * 4 : 0);
     gs = GroupScratch{};
 }
@@ -209,11 +209,8 @@ cudaError_t group_reserve(GroupScratch &gs, uint64_t n, uint32_t H, cudaStream_t
     cudaError_t e = cudaSuccess;
     if (!gs.slot) {
         const uint64_t size = (uint64_t)H * 8 + kGroupWords * 4;
-        if ((e = cudaMalloc((void **)&gs.slot, size)) != cudaSuccess) {
-            cudaGetLastError();
-            gs.slot = nullptr;
+        if ((e = pool_alloc_kept((void **)&gs.slot, size, s)) != cudaSuccess)
             return e;
-        }
         gs.lists = H;
         gs.ctr = reinterpret_cast<uint32_t *>(gs.slot + H);
         *bytes += size;
@@ -225,15 +222,12 @@ cudaError_t group_reserve(GroupScratch &gs, uint64_t n, uint32_t H, cudaStream_t
     const uint64_t old = gs.cap, cap = (std::max<uint64_t>({n, 1024, old + old / 2}) + 15) & ~15ull;
     if ((e = cudaStreamSynchronize(s)) != cudaSuccess)
         return e;
-    cudaFree(gs.ent);
+    pool_free(gs.ent, s);
     *bytes -= old ? edge_bytes(old) : 0;
     gs.ent = nullptr;
     gs.cap = 0;
-    if ((e = cudaMalloc((void **)&gs.ent, edge_bytes(cap))) != cudaSuccess) {
-        cudaGetLastError();
-        gs.ent = nullptr;
+    if ((e = pool_alloc_kept((void **)&gs.ent, edge_bytes(cap), s)) != cudaSuccess)
         return e;
-    }
     *bytes += edge_bytes(cap);
     gs.cap = cap;
     gs.lst = reinterpret_cast<uint32_t *>(gs.ent + cap);

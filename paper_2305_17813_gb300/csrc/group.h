@@ -53,7 +53,7 @@ inline bool group_dense(uint32_t H, uint64_t n) { return n >= 4 * (uint64_t)H; }
 // Grows the arrays to n edges over H lists (synchronises s when it does);
 // *bytes follows what is held.  cudaErrorMemoryAllocation when it cannot.
 cudaError_t group_reserve(GroupScratch &gs, uint64_t n, uint32_t H, cudaStream_t s, uint64_t *bytes);
-void group_release(GroupScratch &gs, uint64_t *bytes);
+void group_release(GroupScratch &gs, uint64_t *bytes, cudaStream_t s);
 
 // Validates and groups n edges (w nullable, a weight of 0 is invalid), lists of
 // up to `most` edges apart from the others, and fills *gv for the kernels launched after it on s.  An invalid edge sets the

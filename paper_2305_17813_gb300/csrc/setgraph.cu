@@ -692,17 +692,14 @@ __global__ void k_set_pool_used(const DevState *st, unsigned long long *out)
 
 namespace {
 
-mk_status set_alloc(mk_set_graph *g, void **p, size_t bytes)
+mk_status set_alloc(mk_set_graph *g, void **p, size_t bytes, cudaStream_t s)
 {
     *p = nullptr;
     if (!bytes)
         return MK_OK;
-    const cudaError_t e = cudaMalloc(p, bytes);
-    if (e != cudaSuccess) {
-        cudaGetLastError();
-        *p = nullptr;
+    const cudaError_t e = pool_alloc_kept(p, bytes, s);
+    if (e != cudaSuccess)
         return e == cudaErrorMemoryAllocation ? MK_ERR_NO_MEMORY : MK_ERR_CUDA;
-    }
     g->bytes += bytes;
     return MK_OK;
 }
@@ -755,7 +752,7 @@ mk_status mk_set_bucket_rule(uint32_t V, const uint32_t *d_src, uint64_t n, floa
         return MK_ERR_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)stream;
     int *d_bad = nullptr;
-    MK_CUDA(cudaMallocAsync((void **)&d_bad, sizeof(int), s));
+    MK_CUDA(pool_alloc((void **)&d_bad, sizeof(int), s));
     MK_CUDA(cudaMemsetAsync(d_bad, 0, sizeof(int), s));
     MK_CUDA(cudaMemsetAsync(d_buckets, 0, (size_t)V * 4, s));
     if (n)
@@ -773,14 +770,15 @@ mk_status mk_set_destroy(mk_set_graph *g)
     if (!g)
         return MK_ERR_INVALID_ARG;
     cudaDeviceSynchronize();
-    cudaFree((void *)g->v.vinfo);
-    cudaFree(g->v.slabs);
-    cudaFree(g->v.bitmap);
-    cudaFree(g->v.owner);
-    cudaFree(g->v.st);
-    group_release(g->group, &g->bytes);
+    pool_free((void *)g->v.vinfo, nullptr);
+    pool_free((void *)g->v.slabs, nullptr);
+    pool_free((void *)g->v.bitmap, nullptr);
+    pool_free((void *)g->v.owner, nullptr);
+    pool_free((void *)g->v.st, nullptr);
+    group_release(g->group, &g->bytes, nullptr);
     if (g->h_pinned)
         cudaFreeHost(g->h_pinned);
+    pool_settle();
     delete g;
     return MK_OK;
 }
@@ -800,17 +798,17 @@ mk_status mk_set_create(uint32_t V, uint64_t edge_capacity_hint, uint32_t bucket
     int *d_bad = nullptr;
     mk_status st = MK_OK;
     auto fail = [&](mk_status code) {
-        cudaFree(d_b);
-        cudaFree(d_off);
-        cudaFree(d_tmp);
-        cudaFree(d_bad);
+        pool_free(d_b, s);
+        pool_free(d_off, s);
+        pool_free(d_tmp, s);
+        pool_free(d_bad, s);
         mk_set_destroy(g);
         return code;
     };
-    if (cudaMalloc((void **)&d_b, (size_t)V * 4) != cudaSuccess ||
-        cudaMalloc((void **)&d_off, ((size_t)V + 1) * 8) != cudaSuccess ||
-        cudaMalloc((void **)&d_bad, sizeof(int)) != cudaSuccess ||
-        cudaMalloc(&d_tmp, exclusive_scan_scratch_bytes(V + 1)) != cudaSuccess)
+    if (pool_alloc((void **)&d_b, (size_t)V * 4, s) != cudaSuccess ||
+        pool_alloc((void **)&d_off, ((size_t)V + 1) * 8, s) != cudaSuccess ||
+        pool_alloc((void **)&d_bad, sizeof(int), s) != cudaSuccess ||
+        pool_alloc(&d_tmp, exclusive_scan_scratch_bytes(V + 1), s) != cudaSuccess)
         return fail(MK_ERR_NO_MEMORY);
     cudaMemsetAsync(d_bad, 0, sizeof(int), s);
     k_fill_buckets<<<grid_for(V, 256), 256, 0, s>>>(d_b, V, buckets ? buckets : 1, d_bucket_per_vertex, d_bad);
@@ -835,14 +833,13 @@ mk_status mk_set_create(uint32_t V, uint64_t edge_capacity_hint, uint32_t bucket
     g->v.H = (uint32_t)H;
     g->v.P = (uint32_t)P;
     g->v.pool_words = (uint32_t)(P / 32);
-    uint2 *vinfo = nullptr;
-    if ((st = set_alloc(g, (void **)&vinfo, (size_t)V * 8)) != MK_OK ||
-        (st = set_alloc(g, (void **)&g->v.slabs, (H + P) * 128)) != MK_OK ||
-        (st = set_alloc(g, (void **)&g->v.bitmap, (size_t)g->v.pool_words * 4)) != MK_OK ||
-        (st = set_alloc(g, (void **)&g->v.owner, (H + P) * 4)) != MK_OK ||
-        (st = set_alloc(g, (void **)&g->v.st, sizeof(DevState))) != MK_OK)
+    if ((st = set_alloc(g, (void **)&g->v.vinfo, (size_t)V * 8, s)) != MK_OK ||
+        (st = set_alloc(g, (void **)&g->v.slabs, (H + P) * 128, s)) != MK_OK ||
+        (st = set_alloc(g, (void **)&g->v.bitmap, (size_t)g->v.pool_words * 4, s)) != MK_OK ||
+        (st = set_alloc(g, (void **)&g->v.owner, (H + P) * 4, s)) != MK_OK ||
+        (st = set_alloc(g, (void **)&g->v.st, sizeof(DevState), s)) != MK_OK)
         return fail(st);
-    g->v.vinfo = vinfo;
+    uint2 *vinfo = (uint2 *)g->v.vinfo;
     if (cudaMallocHost((void **)&g->h_pinned, 64) != cudaSuccess)
         return fail(MK_ERR_NO_MEMORY);
     cudaMemsetAsync(g->v.st, 0, sizeof(DevState), s);
@@ -852,10 +849,10 @@ mk_status mk_set_create(uint32_t V, uint64_t edge_capacity_hint, uint32_t bucket
     k_init_bitmap<<<grid_for(g->v.pool_words, 256), 256, 0, s>>>(g->v.bitmap, g->v.pool_words, (uint32_t)P);
     if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess)
         return fail(MK_ERR_CUDA);
-    cudaFree(d_b);
-    cudaFree(d_off);
-    cudaFree(d_tmp);
-    cudaFree(d_bad);
+    pool_free(d_b, s);
+    pool_free(d_off, s);
+    pool_free(d_tmp, s);
+    pool_free(d_bad, s);
     *out = g;
     return MK_OK;
 }
@@ -903,9 +900,9 @@ mk_status mk_set_bfs(mk_set_graph *g, uint32_t source, uint32_t *d_dist, uint32_
     // levels go out in groups; the host reads the frontier size once a group
     constexpr uint32_t kGroup = 6;
     uint32_t *front[2] = {nullptr, nullptr}, *cnt = nullptr;
-    MK_CUDA(cudaMallocAsync((void **)&front[0], H * 4, s));
-    MK_CUDA(cudaMallocAsync((void **)&front[1], H * 4, s));
-    MK_CUDA(cudaMallocAsync((void **)&cnt, 16, s));
+    MK_CUDA(pool_alloc((void **)&front[0], H * 4, s));
+    MK_CUDA(pool_alloc((void **)&front[1], H * 4, s));
+    MK_CUDA(pool_alloc((void **)&cnt, 16, s));
     k_set_bfs_init<<<grid_for(V, 256), 256, 0, s>>>(g->v, d_dist, d_parent, source, front[0], cnt);
     const uint32_t grid = (uint32_t)num_sms() * 8;
     mk_status st = MK_OK;
@@ -941,7 +938,7 @@ mk_status mk_set_wcc(mk_set_graph *g, uint32_t *d_label, void *stream)
     // failure flag in one block
     const size_t words = (size_t)V + ((size_t)V + 31) / 32 + 2;
     uint32_t *p = nullptr;
-    MK_CUDA(cudaMallocAsync((void **)&p, words * 4, s));
+    MK_CUDA(pool_alloc((void **)&p, words * 4, s));
     uint32_t *bits = p + V, *ctr = p + words - 2;
     int launches = 0;
     cudaError_t e = cudaMemsetAsync(ctr, 0, 8, s);
@@ -958,7 +955,7 @@ mk_status mk_set_stats(mk_set_graph *g, uint64_t *h_lists, uint64_t *h_slabs_in_
         return MK_ERR_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)stream;
     unsigned long long *d = nullptr;
-    MK_CUDA(cudaMallocAsync((void **)&d, 8, s));
+    MK_CUDA(pool_alloc((void **)&d, 8, s));
     k_set_pool_used<<<1, 1, 0, s>>>(g->v.st, d);
     unsigned long long used = 0;
     const cudaError_t e1 = cudaMemcpyAsync(&used, d, 8, cudaMemcpyDeviceToHost, s);

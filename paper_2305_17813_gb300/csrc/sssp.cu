@@ -1406,7 +1406,7 @@ __global__ void __launch_bounds__(kRoundsMaxThreads, 1) k_rounds_multi(MultiArgs
 
 namespace {
 
-mk_status get_consumer(mk_graph *g, int kind, uint32_t source, Consumer **out)
+mk_status get_consumer(mk_graph *g, int kind, uint32_t source, cudaStream_t s, Consumer **out)
 {
     auto key = std::make_pair(kind, source);
     auto it = g->consumers.find(key);
@@ -1418,31 +1418,31 @@ mk_status get_consumer(mk_graph *g, int kind, uint32_t source, Consumer **out)
     c->kind = kind;
     c->source = source;
     const size_t V = g->v.V, H = g->v.H;
-    mk_status st = device_alloc(g, (void **)&c->D, V * 8);
+    mk_status st = device_alloc(g, (void **)&c->D, V * 8, s);
     if (st == MK_OK)
-        st = device_alloc(g, (void **)&c->front[0], H * 8);
+        st = device_alloc(g, (void **)&c->front[0], H * 8, s);
     if (st == MK_OK)
-        st = device_alloc(g, (void **)&c->front[1], H * 8);
+        st = device_alloc(g, (void **)&c->front[1], H * 8, s);
     // frontier slots hold <kNil, ...> until written, so a slot read before
     // it is written names no list
-    if (st == MK_OK && (cudaMemset(c->front[0], 0xFF, H * 8) != cudaSuccess ||
-                        cudaMemset(c->front[1], 0xFF, H * 8) != cudaSuccess))
+    if (st == MK_OK && (cudaMemsetAsync(c->front[0], 0xFF, H * 8, s) != cudaSuccess ||
+                        cudaMemsetAsync(c->front[1], 0xFF, H * 8, s) != cudaSuccess))
         st = MK_ERR_CUDA;
     if (st == MK_OK)
-        st = device_alloc(g, (void **)&c->stamp, V * 4);
+        st = device_alloc(g, (void **)&c->stamp, V * 4, s);
     if (st == MK_OK)
-        st = device_alloc(g, (void **)&c->inv, (V + 31) / 32 * 4);
+        st = device_alloc(g, (void **)&c->inv, (V + 31) / 32 * 4, s);
     if (st == MK_OK)
-        st = device_alloc(g, (void **)&c->counters, kConsumerWords * 4);
-    if (st == MK_OK && (cudaMemset(c->stamp, 0, V * 4) != cudaSuccess || cudaMemset(c->counters, 0, kConsumerWords * 4) != cudaSuccess))
+        st = device_alloc(g, (void **)&c->counters, kConsumerWords * 4, s);
+    if (st == MK_OK && (cudaMemsetAsync(c->stamp, 0, V * 4, s) != cudaSuccess || cudaMemsetAsync(c->counters, 0, kConsumerWords * 4, s) != cudaSuccess))
         st = MK_ERR_CUDA;
     if (st != MK_OK) {
-        device_free(g, c->D, V * 8);
-        device_free(g, c->front[0], H * 8);
-        device_free(g, c->front[1], H * 8);
-        device_free(g, c->stamp, V * 4);
-        device_free(g, c->inv, (V + 31) / 32 * 4);
-        device_free(g, c->counters, kConsumerWords * 4);
+        device_free(g, c->D, V * 8, s);
+        device_free(g, c->front[0], H * 8, s);
+        device_free(g, c->front[1], H * 8, s);
+        device_free(g, c->stamp, V * 4, s);
+        device_free(g, c->inv, (V + 31) / 32 * 4, s);
+        device_free(g, c->counters, kConsumerWords * 4, s);
         delete c;
         return st;
     }
@@ -1526,7 +1526,7 @@ mk_status run_sssp(mk_graph *g, int kind, uint32_t source, uint32_t *d_dist, uin
     if (!g || source >= g->v.V)
         return MK_ERR_INVALID_ARG;
     Consumer *c = nullptr;
-    MK_TRY(get_consumer(g, kind, source, &c));
+    MK_TRY(get_consumer(g, kind, source, s, &c));
     const uint32_t V = g->v.V, H = g->v.H;
     RoundArgs a{};
     a.g = g->v;
@@ -1549,17 +1549,17 @@ mk_status run_sssp(mk_graph *g, int kind, uint32_t source, uint32_t *d_dist, uin
     // call (the host-driven fallback runs plain rounds)
     a.delta = kind == kSssp && !g->dbg_host_rounds ? (incremental ? g->sssp_delta_incr : g->sssp_delta_static) : 0;
     if (a.delta && !c->fstamp) {
-        mk_status st = device_alloc(g, (void **)&c->far[0], (size_t)V * 4);
+        mk_status st = device_alloc(g, (void **)&c->far[0], (size_t)V * 4, s);
         if (st == MK_OK)
-            st = device_alloc(g, (void **)&c->far[1], (size_t)V * 4);
+            st = device_alloc(g, (void **)&c->far[1], (size_t)V * 4, s);
         if (st == MK_OK)
-            st = device_alloc(g, (void **)&c->fstamp, (size_t)V * 4);
+            st = device_alloc(g, (void **)&c->fstamp, (size_t)V * 4, s);
         if (st == MK_OK && cudaMemsetAsync(c->fstamp, 0, (size_t)V * 4, s) != cudaSuccess)
             st = MK_ERR_CUDA;
         if (st != MK_OK) {
-            device_free(g, c->far[0], (size_t)V * 4);
-            device_free(g, c->far[1], (size_t)V * 4);
-            device_free(g, c->fstamp, (size_t)V * 4);
+            device_free(g, c->far[0], (size_t)V * 4, s);
+            device_free(g, c->far[1], (size_t)V * 4, s);
+            device_free(g, c->fstamp, (size_t)V * 4, s);
             c->far[0] = c->far[1] = c->fstamp = nullptr;
             return st;
         }
@@ -1642,7 +1642,7 @@ mk_status run_multi(mk_graph *g, const mk_algo_req *reqs, uint32_t n, cudaStream
     const uint32_t V = g->v.V, H = g->v.H;
     for (uint32_t j = 0; j < n; ++j) {
         const int kind = reqs[j].kind == MK_REQ_BFS ? kBfs : kSssp;
-        MK_TRY(get_consumer(g, kind, reqs[j].source, &cs[j]));
+        MK_TRY(get_consumer(g, kind, reqs[j].source, s, &cs[j]));
         Consumer *c = cs[j];
         RoundArgs &a = m.c[j];
         a.g = g->v;
@@ -1753,7 +1753,7 @@ namespace mk {
 mk_status time_static_bfs(mk_graph *g, uint32_t source, cudaStream_t s, float *ms)
 {
     Consumer *c = nullptr;
-    MK_TRY(get_consumer(g, kBfs, source, &c));
+    MK_TRY(get_consumer(g, kBfs, source, s, &c));
     c->epoch = ~0ull;
     cudaEvent_t a, b;
     MK_CUDA(cudaEventCreate(&a));

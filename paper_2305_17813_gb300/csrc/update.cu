@@ -998,13 +998,13 @@ mk_status insert_impl(mk_graph *g, const uint32_t *d_src, const uint32_t *d_dst,
     if (g->ilog_ok && current && need > g->ilog_cap) {
         const uint64_t cap = std::max<uint64_t>(need, g->ilog_cap * 2);
         uint4 *nl = nullptr;
-        if (device_alloc(g, (void **)&nl, cap * 16) != MK_OK) {
+        if (device_alloc(g, (void **)&nl, cap * 16, s) != MK_OK) {
             g->ilog_ok = false; // the prologues walk the updated lists instead
         } else {
             if (g->d_ilog) {
                 MK_CUDA(cudaMemcpyAsync(nl, g->d_ilog, g->ilog_bound * 16, cudaMemcpyDeviceToDevice, s));
                 MK_CUDA(cudaStreamSynchronize(s));
-                device_free(g, g->d_ilog, g->ilog_cap * 16);
+                device_free(g, g->d_ilog, g->ilog_cap * 16, s);
             }
             g->d_ilog = nl;
             g->ilog_cap = cap;
@@ -1052,11 +1052,11 @@ mk_status delete_impl(mk_graph *g, const uint32_t *d_src, const uint32_t *d_dst,
     if (need > g->dlog_cap) {
         const uint64_t cap = std::max<uint64_t>(need, g->dlog_cap * 2);
         unsigned long long *nl = nullptr;
-        MK_TRY(device_alloc(g, (void **)&nl, cap * 8));
+        MK_TRY(device_alloc(g, (void **)&nl, cap * 8, s));
         if (g->d_dlog) {
             MK_CUDA(cudaMemcpyAsync(nl, g->d_dlog, g->dlog_bound * 8, cudaMemcpyDeviceToDevice, s));
             MK_CUDA(cudaStreamSynchronize(s));
-            device_free(g, g->d_dlog, g->dlog_cap * 8);
+            device_free(g, g->d_dlog, g->dlog_cap * 8, s);
         }
         g->d_dlog = nl;
         g->dlog_cap = cap;
@@ -1151,10 +1151,10 @@ mk_status mk_update_multi(mk_graph *g, const mk_update_req *h_reqs, uint32_t nre
     uint32_t *d_m = nullptr;
     uint8_t *d_mf = nullptr;
     if (max_total) {
-        MK_CUDA(cudaMallocAsync((void **)&d_blk, block_bytes, s));
+        MK_CUDA(pool_alloc((void **)&d_blk, block_bytes, s));
         MK_CUDA(cudaMemcpyAsync(d_blk, img.data(), block_bytes, cudaMemcpyHostToDevice, s));
-        MK_CUDA(cudaMallocAsync((void **)&d_m, max_total * 12, s));
-        MK_CUDA(cudaMallocAsync((void **)&d_mf, max_total, s));
+        MK_CUDA(pool_alloc((void **)&d_m, max_total * 12, s));
+        MK_CUDA(pool_alloc((void **)&d_mf, max_total, s));
     }
     mk_status st = MK_OK;
     size_t pre = 0;

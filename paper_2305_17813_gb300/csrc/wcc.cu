@@ -487,15 +487,15 @@ extern "C" mk_status mk_incr_wcc(mk_graph *g, uint32_t *d_label, void *stream)
     if (it == g->consumers.end()) {
         c = new Consumer;
         c->kind = kWcc;
-        mk_status st = device_alloc(g, (void **)&c->uf, (size_t)V * 4);
+        mk_status st = device_alloc(g, (void **)&c->uf, (size_t)V * 4, s);
         if (st == MK_OK)
-            st = device_alloc(g, (void **)&c->inv, ((size_t)V + 31) / 32 * 4);
+            st = device_alloc(g, (void **)&c->inv, ((size_t)V + 31) / 32 * 4, s);
         if (st == MK_OK)
-            st = device_alloc(g, (void **)&c->counters, kConsumerWords * 4);
+            st = device_alloc(g, (void **)&c->counters, kConsumerWords * 4, s);
         if (st != MK_OK) {
-            device_free(g, c->uf, (size_t)V * 4);
-            device_free(g, c->inv, ((size_t)V + 31) / 32 * 4);
-            device_free(g, c->counters, kConsumerWords * 4);
+            device_free(g, c->uf, (size_t)V * 4, s);
+            device_free(g, c->inv, ((size_t)V + 31) / 32 * 4, s);
+            device_free(g, c->counters, kConsumerWords * 4, s);
             delete c;
             return st;
         }

@@ -282,3 +282,55 @@ def test_large_vertex_count_offsets(cuda_lib):
     absent_bm, _ = g.query(s, ((d.astype(np.uint64) + 2) % V).astype(np.uint32))
     assert mk.to_numpy_u32(absent_bm)[0] == 0
     assert g.last_error() == mk.MK_OK
+
+
+def test_pool_memory_is_bounded_and_given_back(cuda_lib):
+    """What a destroyed graph held is kept for the next one up to 2 GiB, and
+    given back by trim; graphs made and destroyed on two threads and streams
+    at once do not disturb one another."""
+    import threading
+
+    import torch
+
+    mk = _mk()
+
+    def free():
+        torch.cuda.synchronize()
+        return torch.cuda.mem_get_info()[0]
+
+    mk.trim()
+    before = free()
+    big = mk.Graph(1 << 16, edge_capacity_hint=1 << 20, pool_slabs=24 << 20)  # 3 GiB of slabs
+    assert before - free() >= 3 << 30
+    big.close()
+    assert before - free() <= (2 << 30) + (64 << 20)
+    mk.trim()
+    assert before - free() <= 64 << 20
+
+    errors = []
+
+    def work(seed):
+        try:
+            rng = np.random.default_rng(seed)
+            with torch.cuda.stream(torch.cuda.Stream()):
+                for _ in range(20):
+                    V = int(rng.integers(100, 5000))
+                    n = int(rng.integers(1000, 50000))
+                    s, d = (rng.integers(0, V, n).astype(np.uint32) for _ in range(2))
+                    w = rng.integers(1, 9, n).astype(np.uint32)
+                    g, o = mk.Graph(V, edge_capacity_hint=n, buckets=2), oracle.OracleGraph(V)
+                    f = g.insert(s, d, w)
+                    lab, (dist, _) = g.wcc(), g.sssp(0)
+                    assert np.array_equal(f.cpu().numpy(), o.insert(s, d, w))
+                    assert np.array_equal(mk.to_numpy_u32(lab), o.wcc())
+                    assert np.array_equal(mk.to_numpy_u32(dist), o.sssp(0)[0])
+                    g.close()
+        except BaseException as e:  # noqa: BLE001
+            errors.append(e)
+
+    threads = [threading.Thread(target=work, args=(k,)) for k in range(2)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors[0]
