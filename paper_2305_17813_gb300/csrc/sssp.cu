@@ -41,22 +41,27 @@ constexpr uint32_t kBarrierSpins = 1u << 24;
 
 // consumer counter words (kConsumerWords)
 enum {
-    kCnt0 = 0,        // three rotating pairs <frontier size, blocks that have ended the round that filled it>
-    kOverflow = 6,
-    kInvTotal = 7,    // nonzero once this call invalidated a vertex
-    kClearWords = 8,  // words [0, 8) are cleared at the start of every call
-    kSoloR = 8,       // round index reached by a solo phase of block 0, and the frontier size there (9)
-    kRoundsDone = 10,
-    kRid = 11,        // last round stamp used (kept across calls)
-    kPhase = 12,      // Near-Far: last far-pile phase stamp used (kept across calls)
-    kBar = 13,        // grid barrier: arrivals of the launch so far
-    kFarCnt0 = 14,    // Near-Far ordering: sizes of the two far piles (14, 15),
-    kFarMin0 = 16,    // the smallest distance pushed to each (16, 17)
-    kThresh = 18      // and the smallest source distance of the first frontier
+    kCnt0 = 0,        // size of the first frontier
+    kOverflow = 1,
+    kCnt = 2,         // three rotating pairs <frontier size, blocks that have ended the round that filled it>
+    kInvTotal = 8,    // nonzero once this call invalidated a vertex
+    kBar = 9,         // grid barrier: arrivals of the launch so far
+    kFarCnt0 = 10,    // Near-Far ordering: sizes of the two far piles (10, 11),
+    kClearWords = 12, // words [0, 12) are cleared at the start of every call
+    kFarMin0 = 12,    // the smallest distance pushed to each pile (12, 13)
+    kThresh = 14,     // and the smallest source distance of the first frontier: set to INF by ordered calls
+    kSoloR = 16,      // round index reached by a solo phase of block 0, and the frontier size there (17)
+    kRoundsDone = 18,
+    kRid = 19,        // last round stamp used (kept across calls)
+    kPhase = 20       // Near-Far: last far-pile phase stamp used (kept across calls)
 };
 
-// The count of frontier r (the pair's first word).
-__device__ __host__ __forceinline__ uint32_t *count_of(uint32_t *ctr, uint32_t r) { return ctr + kCnt0 + 2 * (r % 3); }
+// The count of frontier r (a pair's first word but for the first frontier's,
+// which nothing changes while the rounds run).
+__device__ __host__ __forceinline__ uint32_t *count_of(uint32_t *ctr, uint32_t r)
+{
+    return r ? ctr + kCnt + 2 * (r % 3) : ctr + kCnt0;
+}
 
 // A frontier of at most kSoloLists lists is processed by block 0 alone, with
 // block-level barriers between rounds, for at most kSoloRounds rounds in a
@@ -509,7 +514,7 @@ __device__ __forceinline__ void far_split(const RoundArgs &a, const uint32_t *pi
 } // namespace
 
 // All rounds of one phase in one cooperative launch.  The phase input is
-// front[0] with its size in ctr[kCnt0]; ctr[kCnt0 + 1] must be zero.  Large
+// front[0] with its size in ctr[kCnt0]; the rotating pairs must be zero.  Large
 // frontiers are processed by the whole grid, one grid barrier per round.
 // While the frontier stays small, block 0 runs the rounds alone (its warps
 // striding over the frontier, its frontier sizes in shared memory,
@@ -842,76 +847,71 @@ __global__ void k_inv_walk(RoundArgs a)
 // which stays fixed during the pass, so every such edge is relaxed even after
 // another in-neighbour has already given its target a finite distance; does
 // nothing if nothing was invalidated.  A streaming scan over the whole slab
-// array (scan_slab_chunks: 32-slab chunks, of which only the slabs whose
-// source has a finite distance are staged in shared memory by bulk copies;
-// the owners' tree nodes are gathered two chunks ahead); each kept slab is
-// relaxed by one lane.  Only
-// distances change here (64-bit atomic minima whose results are not needed);
-// the improved targets are enqueued by k_enqueue_invalid.
-__global__ void __launch_bounds__(kScanWarps * 32) k_relax_into_invalid_slabs(RoundArgs a)
+// array: a warp takes 32 consecutive slabs, reads their owners and the owners'
+// tree nodes (two and one chunk ahead), and then the slabs whose source has a
+// finite distance, eight lanes a slab, 16 bytes a lane.  Few edges lead to an
+// invalidated vertex, so what bounds the pass is the reading and the tests:
+// kBits 1 keeps the bitmap in shared memory, where a test is a word out of
+// 32 banks instead of a line of L1 for each of a warp's keys; 2 reads it from
+// memory where it does not fit.  Only distances change here (64-bit atomic
+// minima whose results are not needed); the improved targets are enqueued by
+// k_enqueue_invalid.  R-MAT scale 20: 122 us with bulk copies into shared
+// memory, a lane a slab and the bitmap in L1, 82 us so (scale 17: 24 -> 18 us).
+constexpr uint32_t kInvThreads = 1024;
+
+template <int kBits>
+__global__ void __launch_bounds__(kInvThreads, 1) k_relax_into_invalid_slabs(RoundArgs a)
 {
-    __shared__ ScanSmem sm;
+    extern __shared__ uint32_t s_inv[];
     const GView &g = a.g;
     if (__ldg(a.ctr + kInvTotal) == 0) // set by the kernels before this one
         return;
-    const uint32_t lane = lane_id();
+    if (kBits == 1) {
+        for (uint32_t i = threadIdx.x; i < (g.V + 31) / 32; i += kInvThreads)
+            s_inv[i] = __ldg(&a.inv[i]);
+        __syncthreads();
+    }
+    auto invalid = [&](uint32_t v) -> uint32_t {
+        return ((kBits == 1 ? s_inv[v >> 5] : __ldg(&a.inv[v >> 5])) >> (v & 31u)) & 1u;
+    };
+    const uint32_t lane = lane_id(), gr = lane >> 3, sub = lane & 7u;
+    const uint64_t total = (uint64_t)g.H + g.P, stride = (((uint64_t)gridDim.x * kInvThreads) >> 5) * 32;
+    auto owner_of = [&](uint64_t c) { return c + lane < total ? __ldcg(&g.owner[c + lane]) : kNil; };
+    auto dist_of = [&](uint32_t own) { return own != kNil ? node_dist(__ldcg(&a.D[own])) : kInf32; };
     // per-lane tallies, summed over the warp once at the end
     uint32_t slabs = 0, edges = 0, owners = 0, targets = 0;
-    const bool ok = scan_slab_chunks(
-        g, sm,
-        [&](uint32_t own) {
-            owners += own != kNil;
-            return own != kNil ? node_dist(__ldcg(&a.D[own])) : kInf32;
-        },
-        [](uint32_t dx) { return dx != kInf32; }, // slabs of unreached or invalidated sources are not read
-        [&](const uint4 *buf, const uint8_t *comp, uint32_t n, uint32_t own_l, uint32_t dx_l) {
-            // lane j takes the chunk's j-th slab in use whole: first the
-            // bitmap words of all its 15 destinations (loads in flight
-            // together), keeping the keys in registers and the live pairs
-            // as bits of a mask; then the bit tests, reading a weight from
-            // shared memory only for a relaxed edge.  The slab's 16-byte
-            // parts are read in a lane-rotated order, so the eight lanes of
-            // each shared-memory phase hit distinct banks.
-            const bool active = lane < n; // every kept slab's source has a finite distance
-            const uint32_t it = active ? comp[lane] : 0u;
-            const uint32_t own = __shfl_sync(kFull, own_l, it);
-            const uint32_t dx = __shfl_sync(kFull, dx_l, it);
-            slabs += active;
-            if (!__any_sync(kFull, active))
-                return;
-            const uint32_t *mine = reinterpret_cast<const uint32_t *>(buf + (active ? lane : 0) * 8);
-            uint32_t key[16], word[16];
-            uint32_t live = 0; // bit k: pair k of the rotated order is a live edge
+    uint64_t c = ((blockIdx.x * (uint64_t)kInvThreads + threadIdx.x) >> 5) * 32;
+    uint32_t own = owner_of(c), own1 = owner_of(c + stride), dx = dist_of(own);
+    for (; c < total; c += stride) {
+        const uint32_t live = __ballot_sync(kFull, dx != kInf32); // slabs of unreached or invalidated sources are not read
+        uint4 part[8];
+        const uint4 *at = reinterpret_cast<const uint4 *>(slab_ptr(g, (uint32_t)c + gr)) + sub;
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                const uint32_t qq = (q + lane) & 7u;
-                const uint4 v = reinterpret_cast<const uint4 *>(mine)[qq];
-                const bool l0 = active && v.x < kTombKey, l1 = active && qq != 7u && v.z < kTombKey;
-                key[2 * q] = v.x;
-                key[2 * q + 1] = v.z;
-                live |= (l0 ? 1u : 0u) << (2 * q) | (l1 ? 1u : 0u) << (2 * q + 1);
-                word[2 * q] = l0 ? __ldg(&a.inv[v.x >> 5]) : 0u; // the bitmap is fixed during the pass
-                word[2 * q + 1] = l1 ? __ldg(&a.inv[v.z >> 5]) : 0u;
-            }
-            uint32_t hit = 0; // bit k: pair k's destination is invalidated
+        for (uint32_t j = 0; j < 8; ++j)
+            part[j] = (live >> (4 * j + gr)) & 1u ? __ldcg(at + j * 32) : make_uint4(kEmptyKey, 0u, kEmptyKey, 0u);
+        const uint32_t own2 = owner_of(c + 2 * stride), dx1 = dist_of(own1);
+        owners += own != kNil;
+        slabs += dx != kInf32;
 #pragma unroll
-            for (int k = 0; k < 16; ++k)
-                hit |= ((word[k] >> (key[k] & 31u)) & 1u) << k;
-            hit &= live;
-            edges += __popc(live);
-            targets += __popc(hit);
-            while (hit) {
-                const int k = __ffs(hit) - 1;
-                hit &= hit - 1;
-                // pair k sits in part (k/2 + lane) % 8, word 2 * (k & 1), weight next to it
-                const uint32_t at = (((uint32_t)(k >> 1) + lane) & 7u) * 4 + 2 * (k & 1);
-                const unsigned long long nd = (unsigned long long)dx + (a.unit ? 1u : mine[at + 1]);
-                if (nd < kInf32)
-                    atomicMin(&a.D[mine[at]], (nd << 32) | own);
-            }
-        });
-    if (!ok)
-        set_status(g.st, kErrTimeout);
+        for (uint32_t j = 0; j < 8; ++j) {
+            const bool k0 = part[j].x < kTombKey, k1 = sub != 7u && part[j].z < kTombKey;
+            edges += (k0 ? 1u : 0u) + (k1 ? 1u : 0u);
+            const uint32_t h0 = k0 ? invalid(part[j].x) : 0u, h1 = k1 ? invalid(part[j].z) : 0u;
+            if (!__any_sync(kFull, h0 | h1))
+                continue;
+            const uint32_t from = __shfl_sync(kFull, own, 4 * j + gr), d = __shfl_sync(kFull, dx, 4 * j + gr);
+            targets += h0 + h1;
+            const unsigned long long n0 = (unsigned long long)d + (a.unit ? 1u : part[j].y);
+            const unsigned long long n1 = (unsigned long long)d + (a.unit ? 1u : part[j].w);
+            if (h0 && n0 < kInf32)
+                atomicMin(&a.D[part[j].x], (n0 << 32) | from);
+            if (h1 && n1 < kInf32)
+                atomicMin(&a.D[part[j].z], (n1 << 32) | from);
+        }
+        own = own1;
+        own1 = own2;
+        dx = dx1;
+    }
     count_add(g.st, kCtrScanOwners, __reduce_add_sync(kFull, owners));
     count_add(g.st, kCtrScanSlabs, __reduce_add_sync(kFull, slabs));
     count_add(g.st, kCtrScanEdges, __reduce_add_sync(kFull, edges));
@@ -1235,8 +1235,9 @@ __global__ void __launch_bounds__(256, 5) k_relax_updated_multi(MultiArgs m)
 }
 
 // The decremental relax-into-invalid scan (k_relax_into_invalid_slabs) for
-// every state at once: a slab is staged when its source has a finite
-// distance in any state that invalidated something, and its live pairs are
+// every state at once (scan_slab_chunks: 32-slab chunks, of which only the
+// slabs kept are staged in shared memory by bulk copies): a slab is staged
+// when its source has a finite distance in any state that invalidated something, and its live pairs are
 // then tested against each such state's invalidation bitmap.
 __global__ void __launch_bounds__(kScanWarps * 32) k_relax_into_invalid_multi(MultiArgs m)
 {
@@ -1484,7 +1485,7 @@ namespace {
 
 // Runs every round of one phase and the call's epilogue (round stamp,
 // overflow check, a.dist / a.parent written from D).  Input: front[0], size
-// in ctr[kCnt0], ctr[kCnt0 + 1] zero.
+// in ctr[kCnt0], the rotating pairs zero.
 mk_status run_phase(mk_graph *g, RoundArgs a, const char *name, cudaStream_t s)
 {
     const int grid = rounds_grid(g->tune.rounds_blocks_per_sm);
@@ -1568,12 +1569,8 @@ mk_status run_sssp(mk_graph *g, int kind, uint32_t source, uint32_t *d_dist, uin
     a.far[1] = c->far[1];
     a.fstamp = c->fstamp;
     MK_CUDA(cudaMemsetAsync(c->counters, 0, kClearWords * 4, s));
-    MK_CUDA(cudaMemsetAsync(c->counters + kBar, 0, 4, s));
-    if (a.delta) {
-        // empty far piles, their minima and the first frontier's minimum at INF
-        MK_CUDA(cudaMemsetAsync(c->counters + kFarCnt0, 0, 8, s));
+    if (a.delta) // the piles' minima and the first frontier's at INF
         MK_CUDA(cudaMemsetAsync(c->counters + kFarMin0, 0xFF, 12, s));
-    }
     if (!incremental) {
         MK_TRY(timed(g, "sssp_init", s, 1, [&]() {
             k_sssp_init<<<grid_for(V, 256), 256, 0, s>>>(c->D, V, source, c->front[0], c->counters + kCnt0,
@@ -1595,8 +1592,16 @@ mk_status run_sssp(mk_graph *g, int kind, uint32_t source, uint32_t *d_dist, uin
                 return cudaSuccess;
             }));
             MK_TRY(timed(g, "sssp_relax_into_invalid", s, 1, [&]() {
-                static const uint32_t grid = resident_grid(k_relax_into_invalid_slabs, kScanWarps * 32);
-                k_relax_into_invalid_slabs<<<grid, kScanWarps * 32, 0, s>>>(a);
+                const size_t bytes = ((size_t)V + 31) / 32 * 4;
+                if (bytes > 200u << 10) {
+                    k_relax_into_invalid_slabs<2><<<num_sms(), kInvThreads, 0, s>>>(a);
+                    return cudaSuccess;
+                }
+                auto k = k_relax_into_invalid_slabs<1>;
+                const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+                if (e != cudaSuccess)
+                    return e;
+                k<<<num_sms(), kInvThreads, bytes, s>>>(a);
                 return cudaSuccess;
             }));
             MK_TRY(timed(g, "sssp_enqueue_invalid", s, 1, [&]() {
@@ -1662,7 +1667,6 @@ mk_status run_multi(mk_graph *g, const mk_algo_req *reqs, uint32_t n, cudaStream
         a.parent = reqs[j].d_parent;
         incr[j] = c->epoch == g->epoch;
         MK_CUDA(cudaMemsetAsync(c->counters, 0, kClearWords * 4, s));
-        MK_CUDA(cudaMemsetAsync(c->counters + kBar, 0, 4, s));
     }
     // the states that recompute statically start from their sources
     for (uint32_t j = 0; j < n; ++j)

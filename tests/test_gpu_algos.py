@@ -275,3 +275,30 @@ def test_static_components(cuda_lib, store, V, shape):
     assert np.array_equal(mk.to_numpy_u32(g.wcc()), o.wcc())
     assert g.last_error() == mk.MK_OK
     g.close()
+
+
+@pytest.mark.parametrize("V", [33, 1638400, 1638401])  # the last with the bitmap in shared memory; the first without
+def test_decremental_bitmap_limits(cuda_lib, V):
+    """Distances after deletes that invalidate much of the tree, the last
+    vertex included, with the invalidated set on each side of the scan."""
+    mk = _mk()
+    rng = np.random.default_rng(V)
+    n = min(3 * V, 60000)
+    name = np.unique(np.append(rng.integers(0, V, 20000), V - 1)).astype(np.uint32)  # the vertices in use
+    s, d = rng.choice(name, n), rng.choice(name, n)
+    s[:8], d[:8] = name[0], name[-8:]
+    w = rng.integers(1, 100, n).astype(np.uint32)
+    g, o = mk.Graph(V, edge_capacity_hint=2 * n, buckets=1), oracle.OracleGraph(V)
+    g.insert(s, d, w)
+    o.insert(s, d, w)
+    src = int(name[0])
+    for k in range(3):
+        check_algos(g, o, [src], wcc=False)
+        g.commit()
+        cut = rng.permutation(n)[: n // 8]
+        cut[:4] = range(4)  # tree edges of the root
+        g.delete(s[cut], d[cut])
+        o.delete(s[cut], d[cut])
+    check_algos(g, o, [src], wcc=False)
+    assert g.last_error() == mk.MK_OK
+    g.close()
