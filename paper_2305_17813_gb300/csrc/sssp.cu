@@ -41,11 +41,10 @@ constexpr uint32_t kBarrierSpins = 1u << 24;
 
 // consumer counter words (kConsumerWords)
 enum {
-    kCnt0 = 0,        // size of the first frontier
-    kOverflow = 1,
-    kCnt = 2,         // three rotating pairs <frontier size, blocks that have ended the round that filled it>
-    kInvTotal = 8,    // nonzero once this call invalidated a vertex
-    kBar = 9,         // grid barrier: arrivals of the launch so far
+    kCnt0 = 0,        // three rotating pairs <frontier size, blocks that have ended the round that filled it>
+    kOverflow = 6,
+    kInvTotal = 7,    // nonzero once this call invalidated a vertex
+    kBar = 8,         // grid barrier: arrivals of the launch so far
     kFarCnt0 = 10,    // Near-Far ordering: sizes of the two far piles (10, 11),
     kClearWords = 12, // words [0, 12) are cleared at the start of every call
     kFarMin0 = 12,    // the smallest distance pushed to each pile (12, 13)
@@ -56,12 +55,8 @@ enum {
     kPhase = 20       // Near-Far: last far-pile phase stamp used (kept across calls)
 };
 
-// The count of frontier r (a pair's first word but for the first frontier's,
-// which nothing changes while the rounds run).
-__device__ __host__ __forceinline__ uint32_t *count_of(uint32_t *ctr, uint32_t r)
-{
-    return r ? ctr + kCnt + 2 * (r % 3) : ctr + kCnt0;
-}
+// The count of frontier r (the pair's first word).
+__device__ __host__ __forceinline__ uint32_t *count_of(uint32_t *ctr, uint32_t r) { return ctr + kCnt0 + 2 * (r % 3); }
 
 // A frontier of at most kSoloLists lists is processed by block 0 alone, with
 // block-level barriers between rounds, for at most kSoloRounds rounds in a
