@@ -23,16 +23,7 @@ mk_status time_static_bfs(mk_graph *g, uint32_t source, cudaStream_t s, float *m
 
 namespace {
 
-int multi_grid(int block)
-{
-    static int sms = 0;
-    if (!sms) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    }
-    return sms * std::max(1, 2048 / block);
-}
+int multi_grid(int block) { return num_sms() * std::max(1, kQueryThreads / block); }
 
 // Device layout of one group of requests: requests, chunk prefix (nreq + 1)
 // and {total chunks, nreq}.

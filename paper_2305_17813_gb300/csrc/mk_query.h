@@ -15,6 +15,9 @@ struct QueryReq {
     uint32_t *w;
 };
 
+// threads of the query kernels that an SM holds at once (their registers)
+constexpr int kQueryThreads = 1024;
+
 cudaError_t launch_query(mk_graph *g, int group, int block, const uint32_t *src, const uint32_t *dst, uint64_t n,
                          uint32_t *bitmap, uint32_t *w, cudaStream_t s);
 cudaError_t launch_query_multi(mk_graph *g, int group, int block, int grid, const QueryReq *reqs,

@@ -334,3 +334,33 @@ def test_pool_memory_is_bounded_and_given_back(cuda_lib):
     for t in threads:
         t.join()
     assert not errors, errors[0]
+
+
+@pytest.mark.parametrize("group", [4, 8, 16, 32])
+@pytest.mark.parametrize("block", [128, 512])
+def test_query_forms(cuda_lib, group, block):
+    """Lookups of one lane to several chunks a warp, in chains of one to
+    hundreds of slabs with deleted pairs in them, every pair of a slab."""
+    mk = _mk()
+    rng = np.random.default_rng(group)
+    V, n = 3000, 40000
+    s = np.where(rng.random(n) < 0.3, 7, rng.integers(0, V, n)).astype(np.uint32)
+    d = rng.integers(0, V, n).astype(np.uint32)
+    w = rng.integers(0, 1 << 20, n).astype(np.uint32)
+    g, o = mk.Graph(V, edge_capacity_hint=2 * n, buckets=1), oracle.OracleGraph(V)
+    g.set_tuning(group, block)
+    g.insert(s, d, w)
+    o.insert(s, d, w)
+    cut = rng.permutation(n)[: n // 5]
+    g.delete(s[cut], d[cut])
+    o.delete(s[cut], d[cut])
+    for m in (1, 31, 32, 33, 40000, 400003):
+        at = rng.integers(0, n, m)
+        qs, qd = s[at], np.where(rng.random(m) < 0.5, d[at], rng.integers(0, V, m)).astype(np.uint32)
+        bm, wt = g.query(qs, qd)
+        obm, ow = o.query(qs, qd)
+        assert np.array_equal(mk.to_numpy_u32(bm), obm) and np.array_equal(mk.to_numpy_u32(wt), ow), m
+        only, none = g.query(qs, qd, weights=False)
+        assert none is None and np.array_equal(mk.to_numpy_u32(only), obm), m
+    assert g.last_error() == mk.MK_OK
+    g.close()
