@@ -43,12 +43,27 @@ struct Weights {
     float w1[kIn * kHid], b1[kHid], w2[kHid * kHid], b2[kHid], w3[kHid], b3, pad[3];
 };
 
+__device__ __forceinline__ float4 ld4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
+__device__ __forceinline__ void st4(float *p, float a, float b, float c, float d)
+{
+    *reinterpret_cast<float4 *>(p) = make_float4(a, b, c, d);
+}
+
+// The tile position of a thread's r-th sample and c-th column: samples
+// 4 * ty + 64 * q + 0..3, columns tx + 8 * c.  The rows of W1, W2 and of W2
+// transposed are kept in shared memory in the order in which the threads read
+// them (place_of), so that a quarter warp's 16-byte accesses cover all banks,
+// the reads of a weight row and the writes of a tile alike (with columns
+// 4 * tx + 32 * h + 0..3 the writes met four at a bank).
+__device__ __forceinline__ int column_of(int tx, int c) { return tx + 8 * c; }
+__device__ __forceinline__ int place_of(int col) { return 4 * (col & 7) + 32 * (col >> 5) + ((col >> 3) & 3); }
+
 __device__ __forceinline__ void load_weights(Weights &s, const float *P)
 {
     for (int i = threadIdx.x; i < kIn * kHid; i += kThreads)
-        s.w1[i] = bf16r(P[kW1 + i]);
+        s.w1[i / kHid * kHid + place_of(i % kHid)] = bf16r(P[kW1 + i]);
     for (int i = threadIdx.x; i < kHid * kHid; i += kThreads)
-        s.w2[i] = bf16r(P[kW2 + i]);
+        s.w2[i / kHid * kHid + place_of(i % kHid)] = bf16r(P[kW2 + i]);
     for (int i = threadIdx.x; i < kHid; i += kThreads) {
         s.b1[i] = bf16r(P[kB1 + i]);
         s.b2[i] = bf16r(P[kB2 + i]);
@@ -58,27 +73,15 @@ __device__ __forceinline__ void load_weights(Weights &s, const float *P)
         s.b3 = bf16r(P[kB3]);
 }
 
-__device__ __forceinline__ float4 ld4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
-__device__ __forceinline__ void st4(float *p, float a, float b, float c, float d)
-{
-    *reinterpret_cast<float4 *>(p) = make_float4(a, b, c, d);
-}
-
-// The tile position of a thread's r-th sample and c-th column: samples
-// 4 * ty + 64 * q + 0..3, columns 4 * tx + 32 * h + 0..3, so that a quarter
-// warp's 16-byte loads cover consecutive banks.
-__device__ __forceinline__ int sample_of(int ty, int r) { return 4 * ty + 64 * (r >> 2) + (r & 3); }
-__device__ __forceinline__ int column_of(int tx, int c) { return 4 * tx + 32 * (c >> 2) + (c & 3); }
-
 // acc[r][c] += sum over k of A[k][sample r] * W[k][column c], k ascending,
 // one fused multiply-add each.  A thread holds 4Q samples x 8 columns and
 // reads Q + 2 16-byte words for 32Q multiply-adds: one thread a sample read
 // two words for each (shared memory 96 % busy, the fp32 pipe 38 %).
-template <int Q, int LD>
+template <int Q, int LD, int K>
 __device__ __forceinline__ void tile_product(const float *A, const float *W, int tx, int ty, float (&acc)[4 * Q][8])
 {
 #pragma unroll 4
-    for (int k = 0; k < kHid; ++k) {
+    for (int k = 0; k < K; ++k) {
         float a[4 * Q], w[8];
 #pragma unroll
         for (int q = 0; q < Q; ++q) {
@@ -98,50 +101,19 @@ __device__ __forceinline__ void tile_product(const float *A, const float *W, int
     }
 }
 
-// First layer of the tile's samples t, t + 128, ... into H1 (ReLU applied);
-// xs[q] are the thread's samples' inputs.
-template <int N, int LD>
-__device__ __forceinline__ void first_layer(const Weights &s, const float (&xs)[N][kIn], float *H1)
-{
-#pragma unroll 2
-    for (int j = 0; j < kHid; j += 4) {
-        const float4 b = ld4(s.b1 + j);
-        float a[N][4];
-#pragma unroll
-        for (int n = 0; n < N; ++n)
-            a[n][0] = b.x, a[n][1] = b.y, a[n][2] = b.z, a[n][3] = b.w;
-#pragma unroll
-        for (int i = 0; i < kIn; ++i) {
-            const float4 w = ld4(s.w1 + i * kHid + j);
-#pragma unroll
-            for (int n = 0; n < N; ++n) {
-                a[n][0] = fmaf(xs[n][i], w.x, a[n][0]);
-                a[n][1] = fmaf(xs[n][i], w.y, a[n][1]);
-                a[n][2] = fmaf(xs[n][i], w.z, a[n][2]);
-                a[n][3] = fmaf(xs[n][i], w.w, a[n][3]);
-            }
-        }
-#pragma unroll
-        for (int n = 0; n < N; ++n)
-#pragma unroll
-            for (int c = 0; c < 4; ++c)
-                H1[(j + c) * LD + threadIdx.x + n * kThreads] = fmaxf(a[n][c], 0.f);
-    }
-}
-
-// Second layer of the tile: H2 = ReLU(H1 W2 + b2), written over or beside H1
-// (the caller's barriers order it).
-template <int Q, int LD>
-__device__ __forceinline__ void second_layer(const Weights &s, const float *H1, int tx, int ty, float (&acc)[4 * Q][8])
+// A layer of the tile: ReLU(A W + bias), into registers.
+template <int Q, int LD, int K>
+__device__ __forceinline__ void relu_layer(const float *A, const float *W, const float *bias, int tx, int ty,
+                                           float (&acc)[4 * Q][8])
 {
 #pragma unroll
     for (int c = 0; c < 8; ++c) {
-        const float b = s.b2[column_of(tx, c)];
+        const float b = bias[column_of(tx, c)];
 #pragma unroll
         for (int r = 0; r < 4 * Q; ++r)
             acc[r][c] = b;
     }
-    tile_product<Q, LD>(H1, s.w2, tx, ty, acc);
+    tile_product<Q, LD, K>(A, W, tx, ty, acc);
 #pragma unroll
     for (int r = 0; r < 4 * Q; ++r)
 #pragma unroll
@@ -165,22 +137,50 @@ template <int LD>
 __device__ __forceinline__ float output_of(const Weights &s, const float *H2, int t)
 {
     float y = s.b3;
-#pragma unroll 8
-    for (int j = 0; j < kHid; ++j)
-        y = fmaf(H2[j * LD + t], s.w3[j], y);
+#pragma unroll 4
+    for (int j = 0; j < kHid; j += 4) {
+        const float4 w = ld4(s.w3 + j);
+        y = fmaf(H2[j * LD + t], w.x, y);
+        y = fmaf(H2[(j + 1) * LD + t], w.y, y);
+        y = fmaf(H2[(j + 2) * LD + t], w.z, y);
+        y = fmaf(H2[(j + 3) * LD + t], w.w, y);
+    }
     return y;
 }
 
+// Inputs of samples base + t, base + t + 128, ...; 16 bytes at a time if the
+// array's address allows.
 template <int N>
 __device__ __forceinline__ void load_inputs(const float *__restrict__ X, uint64_t base, uint64_t n, float (&xs)[N][kIn])
 {
+    const bool wide = (reinterpret_cast<uintptr_t>(X) & 15) == 0;
 #pragma unroll
     for (int k = 0; k < N; ++k) {
         const uint64_t i = base + threadIdx.x + k * kThreads;
+        if (wide) {
+#pragma unroll
+            for (int f = 0; f < kIn; f += 4) {
+                float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (i < n)
+                    v = __ldg(reinterpret_cast<const float4 *>(X + i * kIn + f));
+                xs[k][f] = v.x, xs[k][f + 1] = v.y, xs[k][f + 2] = v.z, xs[k][f + 3] = v.w;
+            }
+        } else {
+#pragma unroll
+            for (int f = 0; f < kIn; ++f)
+                xs[k][f] = i < n ? __ldg(X + i * kIn + f) : 0.f;
+        }
+    }
+}
+
+template <int N, int LD>
+__device__ __forceinline__ void store_inputs(float *x, const float (&xs)[N][kIn])
+{
+#pragma unroll
+    for (int k = 0; k < N; ++k)
 #pragma unroll
         for (int f = 0; f < kIn; ++f)
-            xs[k][f] = i < n ? __ldg(X + i * kIn + f) : 0.f;
-    }
+            x[f * LD + threadIdx.x + k * kThreads] = xs[k][f];
 }
 
 // Forward pass: 256 samples a tile, 16 samples x 8 columns a thread.
@@ -188,27 +188,39 @@ constexpr int kFwdTile = 256, kFwdLd = kFwdTile + 4;
 
 struct FwdSmem {
     Weights w;
-    float h[kHid * kFwdLd]; // H1, then H2
+    float x[kIn * kFwdLd], h[kHid * kFwdLd]; // h: H1, then H2
 };
 
-// 4.2 M samples: 3.88 -> 0.83 ms (47 TFLOP/s).
+// The fp32 pipe sets the pace (549 us of it for 4.2 M samples at 2.06 GHz)
+// once shared memory does not: both layers are tile products (the first by a
+// thread a sample read a weight for each two multiply-adds), and no access
+// meets another at a bank.  4.2 M samples: 3.88 -> 0.72 ms (55 TFLOP/s; 0.83
+// with the first layer by samples and the conflicts; 0.84 with 128-sample
+// tiles, four blocks an SM, so it is not the warps; 0.73 with packed pairs of
+// multiply-adds).
 __global__ void __launch_bounds__(kThreads, 2) k_mlp_forward(const float *P, const float *X, uint64_t n, float *Y)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     FwdSmem &s = *reinterpret_cast<FwdSmem *>(smem_raw);
     const int tx = threadIdx.x & 7, ty = threadIdx.x >> 3;
+    const uint64_t stride = (uint64_t)gridDim.x * kFwdTile;
+    uint64_t base = (uint64_t)blockIdx.x * kFwdTile;
     load_weights(s.w, P);
-    __syncthreads();
-    for (uint64_t base = (uint64_t)blockIdx.x * kFwdTile; base < n; base += (uint64_t)gridDim.x * kFwdTile) {
+    float xs[2][kIn]; // the next tile's inputs, read while a tile is computed
+    load_inputs<2>(X, base, n, xs);
+    for (; base < n; base += stride) {
+        store_inputs<2, kFwdLd>(s.x, xs);
+        __syncthreads(); // and the tile before has been read
+        load_inputs<2>(X, base + stride, n, xs);
         {
-            float xs[2][kIn];
-            load_inputs<2>(X, base, n, xs);
-            first_layer<2, kFwdLd>(s.w, xs, s.h);
+            float acc[16][8];
+            relu_layer<4, kFwdLd, kIn>(s.x, s.w.w1, s.w.b1, tx, ty, acc);
+            store_tile<4, kFwdLd>(s.h, tx, ty, acc);
         }
         __syncthreads();
         {
             float acc[16][8];
-            second_layer<4, kFwdLd>(s.w, s.h, tx, ty, acc);
+            relu_layer<4, kFwdLd, kHid>(s.h, s.w.w2, s.w.b2, tx, ty, acc);
             __syncthreads(); // every thread has read H1
             store_tile<4, kFwdLd>(s.h, tx, ty, acc);
         }
@@ -220,7 +232,6 @@ __global__ void __launch_bounds__(kThreads, 2) k_mlp_forward(const float *P, con
             if (i < n)
                 Y[i] = y;
         }
-        __syncthreads(); // H2 is read; the next tile writes H1 over it
     }
 }
 
@@ -264,7 +275,7 @@ __device__ __forceinline__ float row_dot(const float *A, const float *B)
 // floats, zeroed by the caller); the sum of squared errors into *sse.  Each
 // block keeps its gradient in registers over its tiles (32 entries of W2 a
 // thread, its 4 entries of W1, its bias entries) and adds it once, one atomic
-// a parameter.  262,144 samples: 718 -> 213 us.
+// a parameter.  262,144 samples: 718 -> 190 us.
 __global__ void __launch_bounds__(kThreads, 2) k_mlp_backward(const float *P, const float *X, const float *T,
                                                               uint64_t n, float inv_n, float *G, double *sse)
 {
@@ -274,7 +285,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_mlp_backward(const float *P, co
     load_weights(s.w, P);
     __syncthreads();
     for (int i = t; i < kHid * kHid; i += kThreads)
-        s.w2t[(i % kHid) * kHid + i / kHid] = s.w.w2[i];
+        s.w2t[(i % kHid) * kHid + place_of(i / kHid)] = s.w.w2[i / kHid * kHid + place_of(i % kHid)];
     // W2 entries of the thread: rows k = tx + 8 * a (a < 8), columns j = ty + 16 * b (b < 4)
     float gw2[8][4] = {}, gw1[4] = {}, gvec[2] = {0.f, 0.f}, gb3 = 0.f;
     double my_sse = 0.0;
@@ -284,14 +295,14 @@ __global__ void __launch_bounds__(kThreads, 2) k_mlp_backward(const float *P, co
         {
             float xs[1][kIn];
             load_inputs<1>(X, base, n, xs);
-#pragma unroll
-            for (int f = 0; f < kIn; ++f)
-                s.x[f * kLd + t] = xs[0][f];
-            first_layer<1, kLd>(s.w, xs, s.h1);
+            store_inputs<1, kLd>(s.x, xs);
         }
         __syncthreads();
         float acc[8][8];
-        second_layer<2, kLd>(s.w, s.h1, tx, ty, acc);
+        relu_layer<2, kLd, kIn>(s.x, s.w.w1, s.w.b1, tx, ty, acc);
+        store_tile<2, kLd>(s.h1, tx, ty, acc);
+        __syncthreads();
+        relu_layer<2, kLd, kHid>(s.h1, s.w.w2, s.w.b2, tx, ty, acc);
         store_tile<2, kLd>(s.h2, tx, ty, acc);
         __syncthreads();
         const float y = output_of<kLd>(s.w, s.h2, t);
@@ -349,7 +360,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_mlp_backward(const float *P, co
 #pragma unroll
             for (int c = 0; c < 8; ++c)
                 acc[r][c] = 0.f;
-        tile_product<2, kLd>(s.h2, s.w2t, tx, ty, acc);
+        tile_product<2, kLd, kHid>(s.h2, s.w2t, tx, ty, acc);
         __syncthreads(); // H1 has been read for gW2
 #pragma unroll
         for (int c = 0; c < 8; ++c)

@@ -181,3 +181,29 @@ def test_learned_sizing_shortens_chains_with_identical_results(cuda_lib):
     assert res["learned"]["query_slabs_per_query"] < res["rule"]["query_slabs_per_query"], res
     assert res["learned"]["chain_max"] <= res["rule"]["chain_max"], res
     assert res["train_losses"][-1] < res["train_losses"][0]
+
+
+@pytest.mark.parametrize("n", [1, 255, 257, 80001])  # the last: several tiles a block
+def test_forward_tiles_and_alignment(cuda_lib, n):
+    """Part of a tile, several tiles a block, and inputs that start 4 bytes
+    off a 16-byte boundary (the same values, so the same results)."""
+    torch, mk, sizing = _mods()
+    m = sizing.SizingModel(seed=4)
+    rng = np.random.default_rng(n)
+    P = rng.normal(0, 0.2, omlp.NPARAMS).astype(np.float32)
+    m.set_params(P)
+    X = rng.normal(0, 1, (n, 8)).astype(np.float32)
+    Xd = torch.from_numpy(X).cuda()
+    off = torch.empty(8 * n + 1, device="cuda")[1:].view(n, 8)
+    off.copy_(Xd)
+    assert Xd.data_ptr() % 16 == 0 and off.data_ptr() % 16 == 4
+    y = m.forward(Xd)
+    y_ref = omlp.forward(P, X)
+    assert np.allclose(y.cpu().numpy().astype(np.float64), y_ref, rtol=1e-5, atol=1e-5 * (1 + np.abs(y_ref).max()))
+    assert torch.equal(m.forward(off), y)
+    T = torch.from_numpy(rng.normal(0, 1, n).astype(np.float32)).cuda()
+    g_ref, sse_ref = omlp.gradient(P, X, T.cpu().numpy())
+    for x in (Xd, off):
+        G, sse = m.gradient(x, T)
+        assert np.allclose(G.cpu().numpy().astype(np.float64), g_ref, rtol=1e-4, atol=1e-5 * np.abs(g_ref).max())
+        assert np.isclose(float(sse.item()), sse_ref, rtol=1e-5)
