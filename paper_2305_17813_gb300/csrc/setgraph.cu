@@ -17,6 +17,7 @@
 // labels) run statically: BFS level by level over a frontier of lists, WCC
 // as the map store's static pass (wcc.cu).
 #include "mk_host.h"
+#include "walk.cuh"
 #include "uf.cuh"
 
 #include <algorithm>
@@ -545,39 +546,58 @@ __global__ void __launch_bounds__(256) k_set_query(GView g, const uint32_t *__re
     count_add(g.st, kCtrQuerySlabs, loads);
 }
 
-// One BFS level over a frontier of lists, one list per 4-lane group (eight
-// lists per warp in flight, so a hub's buckets spread over many groups);
-// each lane tests the eight keys of its 32 bytes of a slab at once.  A
-// destination still unreached gets level + 1 with a CAS and its lists join
-// the next frontier: one atomicAdd a warp per slab step for all the new
-// vertices of its eight slabs.  The parents come out of the same pass: an
-// edge read into a vertex of the next level is tight, so an atomicMin of
-// the list's source (its head slab's owner) leaves the smallest one.  The frontier sizes live on the device in
-// three rotating counters (this level reads cnt[L % 3], appends to
-// cnt[(L + 1) % 3] and clears cnt[(L + 2) % 3], the input of the level
-// before), so several levels go out without the host.
-__global__ void __launch_bounds__(256) k_set_bfs_level(GView g, const uint32_t *__restrict__ front, uint32_t *next,
+// One BFS level over a frontier of <list, source>, one list per 4-lane group
+// (eight lists per warp in flight, so a hub's buckets spread over many
+// groups, and the next eight being read); each lane tests the eight keys of
+// its 32 bytes of a slab at once.  A destination still unreached gets level +
+// 1 with a CAS and its lists join the next frontier through the warp's
+// staging buffer.  The parents come out of the same pass: an edge read into a
+// vertex of the next level is tight, so an atomicMin of the list's source
+// leaves the smallest one.  The frontier sizes live on the device in three
+// rotating counters (this level reads cnt[L % 3], appends to cnt[(L + 1) % 3]
+// and clears cnt[(L + 2) % 3], the input of the level before), so several
+// levels go out without the host.  What bounds a large level is the chain of
+// a list (distances, CAS, bucket ranges), at 100 G gathers/s: R-MAT scale 19,
+// 8 M edges, 156 us a search, 165 with an append to the frontier a slab step
+// (a read of the parent before its atomicMin made it 174).
+__global__ void __launch_bounds__(256, 4) k_set_bfs_level(GView g, const uint2 *__restrict__ front, uint2 *next,
                                                        uint32_t *cnt, uint32_t *dist, uint32_t *parent,
                                                        uint32_t level, uint32_t max_hops)
 {
+    __shared__ FrontierSmem<8> bq;
     const uint32_t lane = lane_id(), s4 = lane & 3u, gbase = lane & ~3u;
     const uint32_t n = __ldcg(&cnt[level % 3]);
     uint32_t *next_count = &cnt[(level + 1) % 3];
+    int *overflow = (int *)&cnt[3]; // a vertex is queued once, so its lists fit
     if (blockIdx.x == 0 && threadIdx.x == 0)
         cnt[(level + 2) % 3] = 0;
+    if ((blockIdx.x * (uint64_t)blockDim.x) >> 2 >= n)
+        return;
+    frontier_init(bq);
     const uint64_t groups = ((uint64_t)gridDim.x * blockDim.x) >> 2;
     const uint64_t g0 = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 2;
     unsigned long long loads = 0;
+    auto entry = [&](uint64_t k) { return k < n ? __ldcg(&front[k]) : make_uint2(kNil, 0u); };
+    auto load = [&](uint32_t slab, uint4 &lo, uint4 &hi) {
+        lo = hi = make_uint4(kFull, kFull, kFull, kFull);
+        if (slab != kNil)
+            set_group_load(g, slab, lo, hi);
+    };
+    // the group's next list is read while the current one is worked on
+    uint2 e = entry(g0), ne = entry(g0 + groups);
+    uint4 lo, hi;
+    load(e.x, lo, hi);
     // the warp's eight groups move together: `wb` is its first group's index
     for (uint64_t wb = g0 & ~7ull; wb < n; wb += groups) {
-        const uint64_t k = wb + (g0 & 7u);
-        uint32_t slab = k < n ? __ldcg(&front[k]) : kNil;
+        const uint2 nne = entry(wb + (g0 & 7u) + 2 * groups);
+        uint4 nlo, nhi;
+        load(ne.x, nlo, nhi);
+        uint32_t slab = e.x;
+        const uint32_t u = e.y; // the list's source, at this level
         bool active = slab != kNil;
-        const uint32_t u = active ? __ldg(&g.owner[slab]) : 0u; // the list's source, at this level
         for (uint32_t hop = 0; __any_sync(kFull, active); ++hop) {
-            uint4 lo = make_uint4(kFull, kFull, kFull, kFull), hi = lo;
-            if (active)
-                set_group_load(g, slab, lo, hi);
+            if (hop)
+                load(active ? slab : kNil, lo, hi);
             loads += __popc(__ballot_sync(kFull, active && s4 == 0));
             const uint32_t wv[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
             uint32_t cur[8];
@@ -587,11 +607,12 @@ __global__ void __launch_bounds__(256) k_set_bfs_level(GView g, const uint32_t *
                 key[q] = active && s4 * 8 + q < kSetKeys && wv[q] < kTombKey;
                 cur[q] = key[q] ? __ldcg(&dist[wv[q]]) : 0u;
             }
-            uint32_t grab = 0;
+            bool grab[8], any = false;
 #pragma unroll
-            for (int q = 0; q < 8; ++q)
-                if (key[q] && cur[q] == kNil && atomicCAS(&dist[wv[q]], kNil, level + 1) == kNil)
-                    grab |= 1u << q;
+            for (int q = 0; q < 8; ++q) {
+                grab[q] = key[q] && cur[q] == kNil && atomicCAS(&dist[wv[q]], kNil, level + 1) == kNil;
+                any = any || grab[q];
+            }
             // every edge into a vertex of the next level is tight: the
             // smallest such source is the parent (dist only moves from
             // unreached to level + 1 during this launch, so a destination
@@ -601,55 +622,12 @@ __global__ void __launch_bounds__(256) k_set_bfs_level(GView g, const uint32_t *
                 if (key[q] && (cur[q] == kNil || cur[q] == level + 1))
                     atomicMin(&parent[wv[q]], u);
             const uint32_t nxt = __shfl_sync(kFull, hi.w, gbase + 3);
-            if (__any_sync(kFull, grab != 0)) {
+            if (__any_sync(kFull, any)) {
                 uint2 vi[8];
-                uint32_t c = 0;
 #pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    vi[q] = (grab >> q) & 1u ? __ldg(&g.vinfo[wv[q]]) : make_uint2(0, 0);
-                    c += vi[q].y;
-                }
-                // exclusive scan of the lanes' list counts, one reservation
-                uint32_t incl = c;
-#pragma unroll
-                for (uint32_t o = 1; o < 32; o <<= 1) {
-                    const uint32_t t = __shfl_up_sync(kFull, incl, o);
-                    if (lane >= o)
-                        incl += t;
-                }
-                const uint32_t total = __shfl_sync(kFull, incl, 31);
-                uint32_t wbase = 0;
-                if (lane == 0)
-                    wbase = atomicAdd(next_count, total);
-                uint32_t off[8];
-                uint32_t o = __shfl_sync(kFull, wbase, 0) + incl - c;
-                bool big = false;
-#pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    off[q] = o;
-                    if (vi[q].y <= 8) {
-                        for (uint32_t b = 0; b < vi[q].y; ++b)
-                            next[o + b] = vi[q].x + b;
-                    } else {
-                        big = true;
-                    }
-                    o += vi[q].y;
-                }
-                // vertices with many lists: written by the whole warp
-                uint32_t bigs = __ballot_sync(kFull, big);
-                while (bigs) {
-                    const uint32_t j = __ffs(bigs) - 1;
-                    bigs &= bigs - 1;
-#pragma unroll
-                    for (int q = 0; q < 8; ++q) {
-                        const uint32_t nj = __shfl_sync(kFull, vi[q].y, j);
-                        const uint32_t fj = __shfl_sync(kFull, vi[q].x, j);
-                        const uint32_t oj = __shfl_sync(kFull, off[q], j);
-                        if (nj > 8)
-                            for (uint32_t b = lane; b < nj; b += 32)
-                                next[oj + b] = fj + b;
-                    }
-                }
+                for (int q = 0; q < 8; ++q)
+                    vi[q] = grab[q] ? __ldg(&g.vinfo[wv[q]]) : make_uint2(0, 0);
+                enqueue_lists<8>(bq, wv, grab, vi, next, next_count, g.H, overflow);
             }
             if (active) {
                 if (nxt == kNil || hop + 1 >= max_hops)
@@ -658,12 +636,17 @@ __global__ void __launch_bounds__(256) k_set_bfs_level(GView g, const uint32_t *
                     slab = nxt;
             }
         }
+        e = ne;
+        ne = nne;
+        lo = nlo;
+        hi = nhi;
     }
+    frontier_flush(bq, next, next_count, g.H, overflow);
     count_add(g.st, kCtrRelaxSlabs, loads);
 }
 
 // dist / parent start values; the first frontier is the source's lists.
-__global__ void k_set_bfs_init(GView g, uint32_t *dist, uint32_t *parent, uint32_t source, uint32_t *front,
+__global__ void k_set_bfs_init(GView g, uint32_t *dist, uint32_t *parent, uint32_t source, uint2 *front,
                                uint32_t *cnt)
 {
     const uint32_t v = blockIdx.x * blockDim.x + threadIdx.x;
@@ -673,10 +656,10 @@ __global__ void k_set_bfs_init(GView g, uint32_t *dist, uint32_t *parent, uint32
         parent[v] = v == source ? source : kNil;
     }
     for (uint32_t i = v; i < vi.y; i += gridDim.x * blockDim.x)
-        front[i] = vi.x + i;
+        front[i] = make_uint2(vi.x + i, source);
     if (v == 0) {
         cnt[0] = vi.y;
-        cnt[1] = cnt[2] = 0;
+        cnt[1] = cnt[2] = cnt[3] = 0;
     }
 }
 
@@ -899,9 +882,10 @@ mk_status mk_set_bfs(mk_set_graph *g, uint32_t source, uint32_t *d_dist, uint32_
     const uint64_t H = g->v.H;
     // levels go out in groups; the host reads the frontier size once a group
     constexpr uint32_t kGroup = 6;
-    uint32_t *front[2] = {nullptr, nullptr}, *cnt = nullptr;
-    MK_CUDA(pool_alloc((void **)&front[0], H * 4, s));
-    MK_CUDA(pool_alloc((void **)&front[1], H * 4, s));
+    uint2 *front[2] = {nullptr, nullptr};
+    uint32_t *cnt = nullptr;
+    MK_CUDA(pool_alloc((void **)&front[0], H * 8, s));
+    MK_CUDA(pool_alloc((void **)&front[1], H * 8, s));
     MK_CUDA(pool_alloc((void **)&cnt, 16, s));
     k_set_bfs_init<<<grid_for(V, 256), 256, 0, s>>>(g->v, d_dist, d_parent, source, front[0], cnt);
     const uint32_t grid = (uint32_t)num_sms() * 8;
