@@ -136,10 +136,11 @@ __device__ __forceinline__ void far_put(const RoundArgs &a, const NearFar &nf, u
 }
 
 // Appends the lane's vertices y[k] with push[k] (distances d[k]) to the far
-// pile, each once per phase.  Must be called by the full warp.
+// pile, each once per phase: st[k] is the pile stamp that the caller exchanged
+// for the phase's.  Must be called by the full warp.
 template <int N>
 __device__ __forceinline__ void far_push(const RoundArgs &a, const NearFar &nf, FarSmem &sm, const uint32_t (&y)[N],
-                                         const bool (&push)[N], const uint32_t (&d)[N])
+                                         const bool (&push)[N], const uint32_t (&d)[N], const uint32_t (&stamps)[N])
 {
     const uint32_t lane = lane_id(), w = threadIdx.x >> 5;
     bool any = false;
@@ -151,7 +152,7 @@ __device__ __forceinline__ void far_push(const RoundArgs &a, const NearFar &nf, 
     uint32_t st[N], c = 0, dm = kInf32;
 #pragma unroll
     for (int k = 0; k < N; ++k)
-        st[k] = push[k] ? atomicExch(&a.fstamp[y[k]], nf.phase) : nf.phase;
+        st[k] = push[k] ? stamps[k] : nf.phase;
 #pragma unroll
     for (int k = 0; k < N; ++k)
         if (st[k] != nf.phase) {
@@ -196,35 +197,39 @@ __device__ __forceinline__ void far_push(const RoundArgs &a, const NearFar &nf, 
     __syncwarp();
 }
 
-// Copies the block's staged vertices to the pile.  Called by every thread of
-// the block, which the caller synchronises before more are staged.
-__device__ __forceinline__ void far_flush(const RoundArgs &a, const NearFar &nf, FarSmem &sm)
+// Reserves the staged vertices' places in the pile: by one warp, between two
+// barriers of the block (beside the frontier's reservation, so that a round
+// waits for one of them only).
+__device__ __forceinline__ void far_reserve(const NearFar &nf, FarSmem &sm)
 {
     constexpr uint32_t kWarps = kRoundsMaxThreads / 32;
-    const uint32_t lane = lane_id(), w = threadIdx.x >> 5;
-    __syncthreads();
-    if (w == 0) {
-        const uint32_t h = lane < kWarps ? sm.held[lane] : 0u;
-        uint32_t incl = h;
+    const uint32_t lane = lane_id();
+    const uint32_t h = lane < kWarps ? sm.held[lane] : 0u;
+    uint32_t incl = h;
 #pragma unroll
-        for (uint32_t o = 1; o < 32; o <<= 1) {
-            const uint32_t t = __shfl_up_sync(kFull, incl, o);
-            if (lane >= o)
-                incl += t;
-        }
-        uint32_t base = 0;
-        if (lane == 31) {
-            if (incl)
-                base = atomicAdd(nf.count, incl);
-            if (sm.dmin != kInf32)
-                atomicMin(nf.dmin, sm.dmin);
-            sm.dmin = kInf32;
-        }
-        base = __shfl_sync(kFull, base, 31);
-        if (lane < kWarps)
-            sm.at[lane] = base + incl - h;
+    for (uint32_t o = 1; o < 32; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(kFull, incl, o);
+        if (lane >= o)
+            incl += t;
     }
-    __syncthreads();
+    uint32_t base = 0;
+    if (lane == 31) {
+        if (sm.dmin != kInf32)
+            atomicMin(nf.dmin, sm.dmin);
+        sm.dmin = kInf32;
+        if (incl)
+            base = atomicAdd(nf.count, incl);
+    }
+    base = __shfl_sync(kFull, base, 31);
+    if (lane < kWarps)
+        sm.at[lane] = base + incl - h;
+}
+
+// Then copies them, each warp its own; the caller synchronises the block
+// before more are staged.
+__device__ __forceinline__ void far_copy(const RoundArgs &a, const NearFar &nf, FarSmem &sm)
+{
+    const uint32_t lane = lane_id(), w = threadIdx.x >> 5;
     const uint32_t held = sm.held[w], at = sm.at[w];
     for (uint32_t t = lane; t < held; t += 32)
         far_put(a, nf, at + t, sm.buf[w][t]);
@@ -290,15 +295,12 @@ __device__ __forceinline__ void relax_edges4(const RoundArgs &a, uint32_t x, uin
     }
     if (!__any_sync(kFull, any))
         return;
-    if (kNF) {
-        // improvements at or beyond the split distance wait in the far pile
-        bool fp[4];
+    // improvements at or beyond the split distance wait in the far pile
+    bool fp[4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            fp[k] = up[k] && nd[k] >= nf->T;
-            up[k] = up[k] && !fp[k];
-        }
-        far_push<4>(a, *nf, *fs, y, fp, nd);
+    for (int k = 0; k < 4; ++k) {
+        fp[k] = kNF && up[k] && nd[k] >= nf->T;
+        up[k] = up[k] && !fp[k];
     }
     uint2 vi[4];
     uint32_t st[4];
@@ -306,11 +308,13 @@ __device__ __forceinline__ void relax_edges4(const RoundArgs &a, uint32_t x, uin
     for (int k = 0; k < 4; ++k) {
         vi[k] = make_uint2(0, 0);
         st[k] = round;
-        if (up[k]) {
+        if (up[k])
             vi[k] = a.g.vinfo[y[k]];
-            st[k] = atomicExch(&a.stamp[y[k]], round);
-        }
+        if (up[k] || (kNF && fp[k])) // one exchange, of the stamp that counts
+            st[k] = atomicExch(kNF && fp[k] ? &a.fstamp[y[k]] : &a.stamp[y[k]], kNF && fp[k] ? nf->phase : round);
     }
+    if (kNF)
+        far_push<4>(a, *nf, *fs, y, fp, nd, st);
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         up[k] = up[k] && st[k] != round;
@@ -390,9 +394,12 @@ __device__ __forceinline__ void round_step(const RoundArgs &a, uint32_t *cnt, ui
 {
     const uint32_t in = r & 1;
     relax_body<kNF>(a, a.front[in], n, a.front[in ^ 1], cnt, rid + 2 + r, warp0, nwarps, bq, nf, fs);
-    frontier_flush(bq, a.front[in ^ 1], cnt, a.cap, (int *)(a.ctr + kOverflow));
+    frontier_flush(bq, a.front[in ^ 1], cnt, a.cap, (int *)(a.ctr + kOverflow), [&]() {
+        if (kNF)
+            far_reserve(*nf, *fs);
+    });
     if (kNF)
-        far_flush(a, *nf, *fs);
+        far_copy(a, *nf, *fs);
 }
 
 __device__ __forceinline__ void fence_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
@@ -490,20 +497,21 @@ __device__ __forceinline__ void far_split(const RoundArgs &a, const uint32_t *pi
         bool near = valid && dy < T2;
         uint2 vi = make_uint2(0, 0);
         uint32_t st = stampv;
-        if (near) {
+        const bool far = valid && dy >= T2;
+        if (near)
             vi = a.g.vinfo[y];
-            st = atomicExch(&a.stamp[y], stampv);
-        }
+        if (valid)
+            st = atomicExch(far ? &a.fstamp[y] : &a.stamp[y], far ? next.phase : stampv);
         const uint32_t ys[1] = {y};
         const bool ups[1] = {near && st != stampv};
         const uint2 vis[1] = {vi};
         enqueue_lists<1>(bq, ys, ups, vis, out, cnt, a.cap, overflow);
-        const bool fars[1] = {valid && dy >= T2};
-        const uint32_t ds[1] = {dy};
-        far_push<1>(a, next, fs, ys, fars, ds);
+        const bool fars[1] = {far};
+        const uint32_t ds[1] = {dy}, sts[1] = {st};
+        far_push<1>(a, next, fs, ys, fars, ds, sts);
     }
-    frontier_flush(bq, out, cnt, a.cap, overflow);
-    far_flush(a, next, fs);
+    frontier_flush(bq, out, cnt, a.cap, overflow, [&]() { far_reserve(next, fs); });
+    far_copy(a, next, fs);
 }
 
 } // namespace

@@ -103,10 +103,12 @@ __device__ __forceinline__ void enqueue_lists(FrontierSmem<kWarps> &sm, const ui
 
 // Copies the block's staged entries to the global frontier and empties the
 // staging area.  Called by every thread of the block; the caller synchronises
-// the block before the entries or the staging area are used again.
-template <uint32_t kWarps>
+// the block before the entries or the staging area are used again.  `beside`
+// is called by the block's second warp while the first one waits for its
+// places: another reservation of the round.
+template <uint32_t kWarps, typename F>
 __device__ __forceinline__ void frontier_flush(FrontierSmem<kWarps> &sm, uint2 *out, uint32_t *count, uint32_t cap,
-                                               int *overflow)
+                                               int *overflow, F &&beside)
 {
     const uint32_t lane = lane_id(), w = threadIdx.x >> 5;
     __syncthreads();
@@ -125,6 +127,8 @@ __device__ __forceinline__ void frontier_flush(FrontierSmem<kWarps> &sm, uint2 *
         base = __shfl_sync(kFull, base, 31);
         if (lane < kWarps)
             sm.at[lane] = base + incl - h;
+    } else if (w == 1) {
+        beside();
     }
     __syncthreads();
     const uint32_t held = sm.held[w], at = sm.at[w];
@@ -137,6 +141,13 @@ __device__ __forceinline__ void frontier_flush(FrontierSmem<kWarps> &sm, uint2 *
     __syncwarp();
     if (lane == 0)
         sm.held[w] = 0;
+}
+
+template <uint32_t kWarps>
+__device__ __forceinline__ void frontier_flush(FrontierSmem<kWarps> &sm, uint2 *out, uint32_t *count, uint32_t cap,
+                                               int *overflow)
+{
+    frontier_flush(sm, out, count, cap, overflow, []() {});
 }
 
 } // namespace mk
