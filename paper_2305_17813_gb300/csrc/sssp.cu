@@ -254,7 +254,7 @@ template <bool kNF = false, uint32_t kWarps>
 __device__ __forceinline__ void relax_edges4(const RoundArgs &a, uint32_t x, uint32_t dx, const uint32_t (&y)[4],
                                              const uint32_t (&w)[4], const bool (&live)[4], uint32_t round,
                                              FrontierSmem<kWarps> &bq, uint2 *Fn, uint32_t *cnt, int *overflow,
-                                             unsigned long long &edges, unsigned long long &improved,
+                                             uint32_t &edges, uint32_t &improved,
                                              const NearFar *nf = nullptr, FarSmem *fs = nullptr,
                                              bool direct = false)
 {
@@ -338,17 +338,17 @@ __device__ __forceinline__ unsigned long long warp_sum(unsigned long long v)
 // (the entry two steps ahead) while the current list is relaxed.
 template <bool kNF = false, uint32_t kWarps>
 __device__ __forceinline__ void relax_body(const RoundArgs &a, const uint2 *F, uint32_t n, uint2 *Fn, uint32_t *cnt,
-                                           uint32_t round, uint64_t warp0, uint64_t nwarps, FrontierSmem<kWarps> &bq,
+                                           uint32_t round, uint32_t warp0, uint32_t nwarps, FrontierSmem<kWarps> &bq,
                                            const NearFar *nf = nullptr, FarSmem *fs = nullptr)
 {
     const GView &g = a.g;
     const bool direct = n <= kDirectLists;
     const uint32_t s4 = lane_id() & 3u, g4 = lane_id() >> 2;
     int *overflow = (int *)(a.ctr + kOverflow);
-    unsigned long long lists = 0, slabs = 0, edges = 0, improved = 0;
-    const uint64_t gs = nwarps * 8; // groups in the grid
+    uint32_t lists = 0, slabs = 0, edges = 0, improved = 0;
+    const uint32_t gs = nwarps * 8; // groups in the grid (indexes stay below H + 2 gs, far from 2^32)
     const uint2 none = make_uint2(kNil, 0);
-    uint64_t i = warp0 * 8 + g4;
+    uint32_t i = warp0 * 8 + g4;
     // pipeline: entry e with its distance dx and head slab (lo, hi) (this
     // step), entry ne (next step)
     uint2 e = i < n ? __ldcg(&F[i]) : none;
@@ -356,7 +356,7 @@ __device__ __forceinline__ void relax_body(const RoundArgs &a, const uint2 *F, u
     uint32_t dx = e.x != kNil ? node_dist(__ldcg(&a.D[e.y])) : kInf32;
     uint4 lo, hi;
     group4_load(g, e.x, lo, hi);
-    for (uint64_t base = warp0 * 8; base < n; base += gs, i += gs) {
+    for (uint32_t base = warp0 * 8; base < n; base += gs, i += gs) {
         const uint2 nne = i + 2 * gs < n ? __ldcg(&F[i + 2 * gs]) : none;
         const uint32_t ndx = ne.x != kNil ? node_dist(__ldcg(&a.D[ne.y])) : kInf32;
         uint4 nlo, nhi;
@@ -1019,7 +1019,7 @@ __global__ void __launch_bounds__(256, 5) k_relax_updated(RoundArgs a)
     frontier_init(bq);
     const uint32_t round = __ldg(a.ctr + kRid) + 1;
     int *overflow = (int *)(a.ctr + kOverflow);
-    unsigned long long lists = 0, slabs = 0, edges = 0, improved = 0;
+    uint32_t lists = 0, slabs = 0, edges = 0, improved = 0;
     uint64_t i = warp0 * 8 + g4;
     uint32_t L = i < n ? g.ulog[i] : kNil;
     uint32_t nL = i + gs < n ? g.ulog[i + gs] : kNil;
@@ -1190,7 +1190,7 @@ __global__ void __launch_bounds__(256, 5) k_relax_updated_multi(MultiArgs m)
 #pragma unroll
     for (uint32_t j = 0; j < kMaxMulti; ++j)
         round[j] = j < m.k ? __ldg(m.c[j].ctr + kRid) + 1 : 0u;
-    unsigned long long lists = 0, slabs = 0, edges = 0, improved = 0;
+    uint32_t lists = 0, slabs = 0, edges = 0, improved = 0;
     uint64_t i = warp0 * 8 + g4;
     uint32_t L = i < n ? g.ulog[i] : kNil;
     uint32_t nL = i + gs < n ? g.ulog[i + gs] : kNil;
