@@ -131,25 +131,27 @@ mk_status mk_trim(void);
  * Evaluation", insertion: an edge is stored at the end of its slab list only
  * if it is not already present): an edge already in the graph keeps its
  * weight.  Within the batch the first occurrence of a repeated (src, dst)
- * is the one stored (a hash set of the batch's pairs keeps each pair's
- * first position).  Each tile of 256 edges is sorted and grouped by slab
- * list (source and bucket) in shared memory; one warp handles the edges of
- * one slab list, walks the whole chain once with 128-byte slab loads, claims
- * free pairs with 64-bit atomicCAS and links pool slabs taken from the
- * bitmap allocator.
+ * is the one stored.  The batch is grouped by slab list (source and bucket);
+ * four lanes then apply a list's edges together: they find the repeats among
+ * them, walk the chain once, fill the tail's free pairs with plain stores and
+ * link pool slabs taken from the bitmap allocator.  A list with more than 32
+ * edges in the batch goes through whole warps instead, which claim free pairs
+ * with 64-bit atomicCAS.
  * d_inserted (n bytes, nullable): 1 where edge i was stored by this call.
  * If the pool runs out, the status becomes MK_ERR_POOL_EXHAUSTED and the
  * batch is applied partially: exactly the edges flagged 1 were stored.
- * Marks the touched slab lists as updated for the UpdateIterator and records
- * each stored edge <src, dst, weight> in the epoch's inserted-edge log (grown
- * on demand like the staging buffers). */
+ * Marks the touched slab lists as updated for the UpdateIterator and, while an
+ * algorithm state of the graph has followed the epoch so far, records each
+ * stored edge <src, dst, weight> in the epoch's inserted-edge log (grown on
+ * demand like the staging buffers). */
 mk_status mk_insert_batch(mk_graph *g, const uint32_t *d_src, const uint32_t *d_dst, const uint32_t *d_w,
                           uint64_t n, uint8_t *d_inserted, void *stream);
 
 /* mk_insert_batch without any allocation.  The paper has no counterpart:
  * this is a service of this library.  mk_insert_batch grows its staging
- * buffers with cudaMalloc the first time it sees a larger batch (after a
- * cudaStreamSynchronize and cudaFree of the old ones); a caller that must
+ * buffers from the library's memory pool the first time it sees a larger
+ * batch (after a cudaStreamSynchronize and the release of the old ones), and
+ * the pool may have to map device memory for them; a caller that must
  * not synchronise or allocate at that point -- a serving loop between
  * requests, or a process whose device memory is owned by another allocator
  * or fixed at start-up -- uses this entry point instead.  Results and flags
@@ -170,7 +172,7 @@ mk_status mk_insert_batch(mk_graph *g, const uint32_t *d_src, const uint32_t *d_
  *    that must start empty (the hash set) on its stream.  Two calls whose work
  *    overlaps on the GPU (different streams, or different graphs at the same
  *    time) race on it: order them on one stream or with events.
- *  - Calls no cudaMalloc, cudaFree or allocating library routine. */
+ *  - Calls nothing that allocates or frees device memory. */
 #define MK_NOALLOC_MAX_BATCH 65536u
 mk_status mk_insert_batch_noalloc(mk_graph *g, const uint32_t *d_src, const uint32_t *d_dst, const uint32_t *d_w,
                                   uint64_t n, uint8_t *d_inserted, void *stream);
@@ -187,9 +189,9 @@ mk_status mk_delete_batch(mk_graph *g, const uint32_t *d_src, const uint32_t *d_
 /* Looks up n edges (paper, Sec. "Experimental Evaluation", query: hash to one
  * bucket, walk its chain).  d_bitmap (ceil(n/32) words, required): bit i%32 of
  * word i/32 is 1 iff edge i is present.  d_w (n words, nullable): the stored
- * weight, or 0 when absent.  Queries are independent and unsorted; one
- * group of 4 or 8 lanes (the tuned shape) with 16-byte loads walks one
- * query's chain. */
+ * weight, or 0 when absent.  Queries are independent and unsorted; a warp
+ * answers 32 of them and reads their head slabs at once, each by one group of
+ * lanes (the tuned shape), then the next slabs of the chains that go on. */
 mk_status mk_query_batch(mk_graph *g, const uint32_t *d_src, const uint32_t *d_dst, uint64_t n,
                          uint32_t *d_bitmap, uint32_t *d_w, void *stream);
 
@@ -244,7 +246,8 @@ typedef struct mk_update_req {
  * directly.  So a stream of many small requests costs a few launches per run
  * instead of per request (the paper applies one batch per launch).  The
  * descriptors are copied to the device before the call returns; the staging
- * arrays are stream-ordered allocations (cudaMallocAsync) freed on `stream`.
+ * arrays are stream-ordered allocations from the library's pool, freed on
+ * `stream`.
  * MK_ERR_INVALID_ARG (nothing enqueued) for an unknown kind or a null
  * src/dst with n > 0. */
 mk_status mk_update_multi(mk_graph *g, const mk_update_req *h_reqs, uint32_t nreq, void *stream);
@@ -400,7 +403,9 @@ mk_status mk_incr_multi(mk_graph *g, const mk_algo_req *h_reqs, uint32_t n, void
 /* Weakly connected components (paper, Sec. "Incremental WCC"): union-find with
  * Union-Async hooking of the larger root under the smaller and full path
  * compression.  The first call, and any call whose epoch holds deletions
- * (the paper has no decremental WCC), runs the static pass over every edge;
+ * (the paper has no decremental WCC), runs the static pass: a few edges a
+ * vertex are united first, the tree that most of a sample of vertices are in
+ * is found, and the scan of every edge unites those that leave it;
  * otherwise only the edges inserted since the last commit are united, read
  * from the epoch's inserted-edge log (or found with the UpdateIterator when
  * an insert of the epoch could not log).  d_label (V words): the smallest vertex id of each
@@ -418,12 +423,16 @@ mk_status mk_incr_wcc(mk_graph *g, uint32_t *d_label, void *stream);
  * ranks start at 1 / V (static); with warm_start != 0 they start from
  * d_pr's contents (the ranks before the last batch: the incremental and
  * decremental cases); on return d_pr holds the ranks.  Ranks are kept as
- * 64-bit fixed-point values (scale 2^48) and the contributions are pushed
- * along out-edges with integer atomics, so the result does not depend on the
- * order of the atomics; each super-step's rounding is below 2^-48 per term.
+ * 64-bit fixed-point values (scale 2^48) and the contributions are summed as
+ * integers, so the result does not depend on their order; each super-step's
+ * rounding is below 2^-48 per term.  A call of several super-steps first
+ * writes the edges out in order of their destinations' ranges (about 4 bytes
+ * an edge; where that memory cannot be had, the contributions are pushed along
+ * the slab lists at every super-step).
  * damping in (0, 1), eps > 0, max_iter >= 1.  *h_iters / *h_delta
  * (nullable, host): super-steps run and the last L1 delta.  Synchronises
- * `stream` once per super-step (the host reads the delta); work arrays are
+ * `stream` once per four super-steps at most (the host reads the deltas; a
+ * super-step after the last one changes nothing); work arrays are
  * stream-ordered allocations freed before the call returns. */
 mk_status mk_pagerank(mk_graph *g, float *d_pr, int warm_start, float damping, float eps, uint32_t max_iter,
                       uint32_t *h_iters, float *h_delta, void *stream);
@@ -433,16 +442,18 @@ mk_status mk_pagerank(mk_graph *g, float *d_pr, int warm_start, float damping, f
  * mk_tc_count is the paper's Count kernel: *d_total (device, one uint64)
  * += sum over the n edges (d_src[i], d_dst[i]) of |N_g1(src) ∩ N_g2(dst)|
  * (the walk goes over the side with fewer buckets; the sum is the same).
- * g1 and g2 must have the same V.  The edges are handed to the warps one
- * at a time from an 8-byte stream-ordered counter allocated for the call. */
+ * g1 and g2 must have the same V.  The edges are handed to the warps from an
+ * 8-byte stream-ordered counter allocated for the call. */
 mk_status mk_tc_count(mk_graph *g1, mk_graph *g2, const uint32_t *d_src, const uint32_t *d_dst, uint64_t n,
                       unsigned long long *d_total, void *stream);
 
 /* Static count into *h_triangles (host): every triangle once, on its two
  * lower-ranked vertices' edge, the vertices ranked by (bucket count, id);
  * equal to Count(g, g, every live edge) / 6 on a graph that meets the
- * conditions above (which this count does not check).  Synchronises
- * `stream`. */
+ * conditions above (which this count does not check).  Each vertex's
+ * higher-ranked neighbours are copied out first (stream-ordered work arrays
+ * of 28 bytes a vertex and 4 an edge, freed on `stream`; where they cannot
+ * be had, the slab lists themselves are intersected).  Synchronises `stream`. */
 mk_status mk_tc_static(mk_graph *g, uint64_t *h_triangles, void *stream);
 
 /* Change in the triangle count after a batch (paper, Algorithms "Triangle
@@ -483,20 +494,20 @@ mk_status mk_set_create(uint32_t V, uint64_t edge_capacity_hint, uint32_t bucket
 mk_status mk_set_destroy(mk_set_graph *g);
 /* Insert / delete / query n edges as mk_insert_batch / mk_delete_batch /
  * mk_query_batch do (no weights; flags and bitmap nullable / required
- * alike).  A warp walks eight chains at once, one per 4-lane group (32
- * bytes of the slab a lane). */
+ * alike).  Batches are grouped by slab list as there; a warp walks eight
+ * chains at once, one per 4-lane group (32 bytes of the slab a lane). */
 mk_status mk_set_insert_batch(mk_set_graph *g, const uint32_t *d_src, const uint32_t *d_dst, uint64_t n,
                               uint8_t *d_inserted, void *stream);
 mk_status mk_set_delete_batch(mk_set_graph *g, const uint32_t *d_src, const uint32_t *d_dst, uint64_t n,
                               uint8_t *d_deleted, void *stream);
 mk_status mk_set_query_batch(mk_set_graph *g, const uint32_t *d_src, const uint32_t *d_dst, uint64_t n,
                              uint32_t *d_bitmap, void *stream);
-/* Static BFS from `source`, level by level over a frontier of lists (one
- * warp a list; frontier sizes kept on the device, levels launched six at a
+/* Static BFS from `source`, level by level over a frontier of lists (four
+ * lanes a list; frontier sizes kept on the device, levels launched six at a
  * time, the host reading the frontier size once per six levels): d_dist =
  * hop counts (MK_NONE unreachable), d_parent = the smallest-id u with a live
  * edge u -> v and dist(u) + 1 = dist(v) (the source its own parent).
- * Synchronises `stream`; allocates two frontiers of `lists` words each from
+ * Synchronises `stream`; allocates two frontiers of 8 bytes a list each from
  * the stream-ordered pool. */
 mk_status mk_set_bfs(mk_set_graph *g, uint32_t source, uint32_t *d_dist, uint32_t *d_parent, void *stream);
 /* Static WCC: d_label = the smallest vertex id of each vertex's component. */
@@ -653,10 +664,12 @@ mk_status mk_l2_window(mk_graph *g, int region, void *stream, mk_l2_info *out);
  * runs the rounds with the host-driven fallback (one launch per round, the
  * host reading each frontier size) that is otherwise used only when the
  * cooperative launch is refused; 0 restores the kernel.  Results are the
- * same either way.  After mk_last_error has returned an error status, every
+ * same either way.  knob MK_DEBUG_NO_SCRATCH: value 1 counts triangles as on
+ * a device without room for the work arrays of mk_tc_static; 0 restores them.
+ * After mk_last_error has returned an error status, every
  * incremental algorithm state of the graph recomputes statically at its
  * next call. */
-enum { MK_DEBUG_BARRIER_SPINS = 1, MK_DEBUG_HOST_ROUNDS = 2 };
+enum { MK_DEBUG_BARRIER_SPINS = 1, MK_DEBUG_HOST_ROUNDS = 2, MK_DEBUG_NO_SCRATCH = 3 };
 mk_status mk_debug_set(mk_graph *g, int knob, uint64_t value);
 
 /* Library version string. */

@@ -533,6 +533,51 @@ __device__ __forceinline__ unsigned long long tc_rank(uint32_t buckets, uint32_t
     return ((unsigned long long)buckets << 32) | x;
 }
 
+// The static count without any copy of the neighbours, for a device that has
+// no room for it: a warp takes a slab of u, and for each v there that ranks
+// above u looks the keys of u's lists that rank above v up in v's.
+__global__ void __launch_bounds__(256) k_tc_walk(GView g, uint32_t max_hops, unsigned long long *total)
+{
+    __shared__ uint32_t s_keys[8][kPairs + 1];
+    const uint32_t lane = lane_id();
+    uint32_t *keys = s_keys[threadIdx.x >> 5];
+    const uint64_t slabs = (uint64_t)g.H + g.P, nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
+    unsigned long long count = 0;
+    for (uint64_t c = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5; c < slabs; c += nwarps) {
+        const uint32_t u = __ldcg(&g.owner[c]);
+        if (u == kNil)
+            continue;
+        auto above = [&](uint32_t x, unsigned long long rank) {
+            return is_key_lane(lane) && x < kTombKey && tc_rank(__ldg(&g.vinfo[x]).y, x) > rank;
+        };
+        const uint2 vu = __ldg(&g.vinfo[u]);
+        const uint32_t x = __ldcg(slab_ptr(g, (uint32_t)c) + lane);
+        for (uint32_t todo = __ballot_sync(kFull, above(x, tc_rank(vu.y, u))); todo; todo &= todo - 1) {
+            const uint32_t v = __shfl_sync(kFull, x, __ffs(todo) - 1);
+            const uint2 vv = __ldg(&g.vinfo[v]);
+            for (uint32_t b = 0; b < vu.y; ++b) {
+                uint32_t slab = vu.x + b;
+                for (uint32_t hop = 0; slab != kNil && hop < max_hops; ++hop) {
+                    const uint32_t w = __ldcg(slab_ptr(g, slab) + lane);
+                    const bool key = above(w, tc_rank(vv.y, v));
+                    const uint32_t m = __ballot_sync(kFull, key);
+                    if (key)
+                        keys[__popc(m & lanemask_lt())] = w;
+                    __syncwarp();
+                    if (m)
+                        count += count_neighbours(g, vv, keys, __popc(m), max_hops);
+                    __syncwarp();
+                    slab = __shfl_sync(kFull, w, kNextLane);
+                }
+            }
+        }
+    }
+    for (int o = 16; o; o >>= 1)
+        count += __shfl_xor_sync(kFull, count, o);
+    if (lane == 0 && count)
+        atomicAdd(total, count);
+}
+
 } // namespace
 
 // Static count, each triangle once: with the vertices ranked by tc_rank, a
@@ -820,6 +865,25 @@ __global__ void __launch_bounds__(1024) k_tc_large(TcArrays t, uint32_t vbits)
 
 // ---------------------------------------------------------------- host side
 
+static mk_status tc_walk(mk_graph *g, uint64_t *h_triangles, cudaStream_t s)
+{
+    unsigned long long *d = nullptr;
+    MK_CUDA(pool_alloc((void **)&d, 8, s));
+    unsigned long long total = 0;
+    mk_status st = cudaMemsetAsync(d, 0, 8, s) == cudaSuccess ? MK_OK : MK_ERR_CUDA;
+    if (st == MK_OK)
+        st = timed(g, "tc_static", s, 1, [&]() {
+            k_tc_walk<<<resident_grid(k_tc_walk, 256), 256, 0, s>>>(g->v, g->v.P + 2, d);
+            return cudaSuccess;
+        });
+    if (st == MK_OK && (cudaMemcpyAsync(&total, d, 8, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+                        cudaStreamSynchronize(s) != cudaSuccess))
+        st = MK_ERR_CUDA;
+    cudaFreeAsync(d, s);
+    *h_triangles = total;
+    return st;
+}
+
 extern "C" {
 
 mk_status mk_pagerank(mk_graph *g, float *d_pr, int warm_start, float damping, float eps, uint32_t max_iter,
@@ -1001,7 +1065,8 @@ mk_status mk_tc_static(mk_graph *g, uint64_t *h_triangles, void *stream)
     // are, read back first) in another
     unsigned char *block = nullptr;
     const size_t bytes = V * (16 + 4 + 4 + 4) + kTcWords * 8;
-    MK_CUDA(pool_alloc((void **)&block, bytes, s));
+    if (g->dbg_no_scratch || pool_alloc((void **)&block, bytes, s) != cudaSuccess)
+        return tc_walk(g, h_triangles, s);
     TcArrays t{};
     t.list = (ulonglong2 *)block;
     t.ctr = (unsigned long long *)(t.list + V);
@@ -1027,7 +1092,11 @@ mk_status mk_tc_static(mk_graph *g, uint64_t *h_triangles, void *stream)
     if (st == MK_OK)
         cuda(cudaStreamSynchronize(s));
     if (st == MK_OK && total) {
-        if (cuda(pool_alloc((void **)&t.adj, total * 4, s)))
+        if (pool_alloc((void **)&t.adj, total * 4, s) != cudaSuccess) {
+            cudaFreeAsync(block, s);
+            return tc_walk(g, h_triangles, s);
+        }
+        if (st == MK_OK)
             st = timed(g, "tc_static", s, 3, [&]() {
                 k_tc_orient<true><<<slab_grid, kTcThreads, 0, s>>>(g->v, t);
                 // a bitmap of up to 128 KB (2^20 vertices), with blocks large

@@ -693,6 +693,9 @@ mk_status mk_debug_set(mk_graph *g, int knob, uint64_t value)
     case MK_DEBUG_HOST_ROUNDS:
         g->dbg_host_rounds = value != 0;
         return MK_OK;
+    case MK_DEBUG_NO_SCRATCH:
+        g->dbg_no_scratch = value != 0;
+        return MK_OK;
     default:
         return MK_ERR_INVALID_ARG;
     }

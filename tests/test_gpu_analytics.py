@@ -206,3 +206,34 @@ def test_pagerank_binned_and_pushed(cuda_lib, V):
     assert i3 == i9 and d3 == d9
     assert g.last_error() == mk.MK_OK
     g.close()
+
+
+@pytest.mark.parametrize("buckets", [1, 3])
+def test_triangles_without_work_arrays(cuda_lib, buckets):
+    """The count over the slab lists themselves, used where the neighbours'
+    copy does not fit: vertices with one slab and with chains, deleted pairs."""
+    from paper_2305_17813_gb300._native import MK_DEBUG_NO_SCRATCH
+
+    mk = _mk()
+    rng = np.random.default_rng(buckets)
+    V = 400
+    i, j = np.triu_indices(40, 1)
+    a = np.concatenate([i, np.zeros(V - 1, np.int64), rng.integers(0, V, 4000)])
+    b = np.concatenate([j, np.arange(1, V), rng.integers(0, V, 4000)])
+    pairs = np.unique(np.sort(np.stack([a, b], 1), 1), axis=0)
+    pairs = pairs[pairs[:, 0] != pairs[:, 1]]
+    s, d = _undirected(*pairs.T.astype(np.uint32))
+    o = oracle.OracleGraph(V)
+    g = mk.Graph(V, edge_capacity_hint=2 * len(s), buckets=buckets)
+    o.insert(s, d, np.ones(len(s), np.uint32))
+    g.insert(s, d)
+    cut = _undirected(*pairs[rng.permutation(len(pairs))[:300]].T.astype(np.uint32))
+    o.delete(*cut)
+    g.delete(*cut)
+    g.commit()
+    mk.check(mk.load().mk_debug_set(g.handle, MK_DEBUG_NO_SCRATCH, 1), "mk_debug_set")
+    assert g.triangles() == o.triangles()
+    mk.check(mk.load().mk_debug_set(g.handle, MK_DEBUG_NO_SCRATCH, 0), "mk_debug_set")
+    assert g.triangles() == o.triangles()
+    assert g.last_error() == mk.MK_OK
+    g.close()
