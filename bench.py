@@ -219,9 +219,15 @@ def algorithmic_bytes(family, ctr, n_per_launch, launches):
     if family == "query":
         return launches * n_per_launch * (8 + 32 + 0.125) + 128 * ctr["query_slabs"]
     if family == "insert":
+        # the entry and its weight (12 B), a sector of its list's range, one of
+        # the logs; a slab is read, or written when new
         return launches * n_per_launch * (12 + 32 + 32) + 128 * (ctr["insert_slabs"] + ctr["insert_new_slabs"])
     if family == "delete":
         return launches * n_per_launch * (8 + 32 + 32) + 128 * ctr["delete_slabs"]
+    if family == "stage_group":
+        # per edge: the edge (12 B), its index sector, a counter, its list and
+        # rank written and read (10 B), destination, range sector and entry
+        return launches * n_per_launch * (12 + 32 + 16 + 10 + 4 + 32 + 8)
     if family == "sssp_rounds":
         # rounds, then the tree nodes unpacked into the caller's dist/parent
         return (ctr["relax_lists"] * (4 + 4 + 8) + 128 * ctr["relax_slabs"] + 16 * ctr["relax_edges"]
@@ -237,7 +243,8 @@ def algorithmic_bytes(family, ctr, n_per_launch, launches):
                 + ctr["seed_improved"] * (8 + 4 + 8) + ctr.get("seed_log", 0) * (16 + 8))
     if family == "sssp_invalidate_walk":
         return ctr["walk_vertices"] * 8 + ctr["invalidated"] * 8
-    if family == "wcc_hook_all":
+    if family in ("wcc_static", "wcc_hook_all"):
+        # the slabs with edges outside the sampled tree, two finds a united edge
         return 128 * ctr["wcc_slabs"] + 16 * ctr["wcc_edges"]
     if family == "wcc_hook_updated":
         # walk of the updated lists, or the inserted-edge log (16 B an entry)
@@ -250,21 +257,21 @@ def algorithmic_bytes(family, ctr, n_per_launch, launches):
 # (full workload, one pass), and
 # the SHA-256 of the kernel sources (csrc/) it was taken with.  A figure is
 # reported only while those sources are unchanged; otherwise traffic is null.
-NCU_TRAFFIC_SOURCES_SHA = "23cc176d5d3307aa6d343140c981b5fca75866b242cd4298c6962f3e813fb31d"
+NCU_TRAFFIC_SOURCES_SHA = "03eaba235dbef8b921bc13205e888fa5968969413daccf39fe52d52d51b9a135"
 NCU_TRAFFIC = {
-"sssp_rounds": 49676000,
-    "sssp_relax_into_invalid": 280899072,
-    "sssp_enqueue_invalid": 11004224,
-    "sssp_relax_updated": 26472768,
-    "sssp_invalidate_walk": 8524864,
-    "sssp_invalidate": 13739456,
-    "wcc_hook_all": 350455296,
-    "wcc_hook_updated": 19096192,
-    "insert": 255002240,
-    "delete": 198414976,
-    "query": 130889088,
-    "stage_dedup": 40148544,
-    "update_slab_pointers": 60540224,
+    "sssp_rounds": 44158496,
+    "sssp_relax_into_invalid": 280970240,
+    "sssp_enqueue_invalid": 11001792,
+    "sssp_relax_updated": 26405248,
+    "sssp_invalidate_walk": 8524544,
+    "sssp_invalidate": 13740416,
+    "wcc_static": 542555104,
+    "wcc_hook_updated": 20227200,
+    "insert": 194368768,
+    "delete": 164786432,
+    "query": 130626304,
+    "stage_group": 75261696,
+    "update_slab_pointers": 60560192,
 }
 
 
@@ -659,7 +666,7 @@ def o_e_share(kernels):
     """Share of the summed kernel time taken by the passes over every edge
     (the decremental relax-into-invalid scan and the static WCC pass), which
     do not shrink with the batch."""
-    return round(sum(kernels[k]["share"] for k in ("sssp_relax_into_invalid", "wcc_hook_all", "wcc_init")
+    return round(sum(kernels[k]["share"] for k in ("sssp_relax_into_invalid", "wcc_static")
                      if k in kernels), 4)
 
 
@@ -1412,13 +1419,11 @@ def run_analytics(args):
     ms_warm, (_, it_warm, _) = timed_ms(lambda: g.pagerank(pr, eps=1e-7, max_iter=100))
     ms_cold, (_, it_cold, _) = timed_ms(lambda: g.pagerank(eps=1e-7, max_iter=100))
     n_step, t_step = prof.get("pr_step", (0, 0.0))
-    slabs_in_use = int(st["chain_slabs"])
     E, V = int(st["live_edges"]), G.V
-    # per super-step: every slab in use read once (128 B) with its owner
-    # (4 B), one 8-byte contribution gather and one 8-byte atomic add per
-    # edge, and the per-vertex passes (rank, degree, contribution and
-    # accumulator reads and writes: 44 B per vertex)
-    step_bytes = 132 * slabs_in_use + 16 * E + 44 * V
+    # per super-step: every edge read from its bin (4 B) with one 8-byte
+    # contribution gather, and the per-vertex passes (sums written, read and
+    # cleared, rank read and written, degree, contribution: 64 B per vertex)
+    step_bytes = 12 * E + 64 * V
     peak, _ = measured_peak()
     gbs = step_bytes * n_step / (t_step / 1e3) / 1e9 if t_step else None
     out["pagerank"] = {

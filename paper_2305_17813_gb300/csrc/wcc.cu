@@ -147,13 +147,12 @@ __global__ void __launch_bounds__(256) k_uf_hook_log(DevState *st, const uint4 *
 // edge by edge is what the pass cost: two finds each, ending in the same few
 // roots, and hooks that lose to one another there (168-194 us on an R-MAT
 // graph of scale 18 whose slabs are read in 12).  So the pass first builds a
-// forest from a sample -- the pairs in the first 32 bytes of every vertex's
-// first slab, at most 4 (8 keys of the set layout): every vertex points to its
-// smallest sampled neighbour below it, the trees are compressed, the roots
-// that sampled edges connect are hooked with plain atomic minima, and the
-// trees are compressed again.  The tree that holds most of 1,024 sampled
-// vertices is the giant one; a bitmap names its vertices.  The scan over all
-// slabs then tests both ends of an edge in the bitmap, which it keeps in
+// forest from a sample -- the first four or so keys of every vertex's first
+// list (sample_of): every vertex points to its smallest sampled neighbour
+// below it, the trees are compressed, the roots that sampled edges connect
+// are hooked with plain atomic minima, and the trees are compressed again.
+// The tree that holds most of 1,024 sampled vertices is the giant one; a
+// bitmap names its vertices.  The scan over all slabs then tests both ends of an edge in the bitmap, which it keeps in
 // shared memory where it fits, and only slabs with an edge that is not inside
 // the giant tree unite anything.  Kernel boundaries in between also drop the
 // parents that the SMs' L1 caches still hold from before the hooks.
@@ -178,17 +177,37 @@ __device__ __forceinline__ void keys_of(const uint4 &q, uint32_t (&e)[kSet ? 4 :
     }
 }
 
-// The sampled neighbours of v: keys of the first 32 bytes of its first slab
-// (kNil where there is none; the next index is past them).
-template <bool kSet>
-__device__ __forceinline__ void sample_of(const GView &g, uint32_t v, uint32_t (&d)[8])
+// The sampled neighbours of v: f(d) for 32 bytes of its first list at a time
+// (d: their keys, kNil where there is none) until four keys were found or the
+// list ends.  A new list has them in its first 32 bytes; one that has seen
+// deletions starts with tombstones, and a sample of those alone would leave
+// the vertex out of its tree and all its edges to the scan (20 batches of
+// 2^20 inserts and deletes on R-MAT scale 20: 343 us for the scan instead of
+// 110).
+template <bool kSet, typename F>
+__device__ __forceinline__ void sample_of(const GView &g, uint32_t v, F &&f)
 {
-    const uint4 *p = reinterpret_cast<const uint4 *>(slab_ptr(g, __ldg(&g.vinfo[v]).x));
-    const uint4 a = __ldcg(p), b = __ldcg(p + 1);
-    const uint32_t w[8] = {a.x, kSet ? a.y : kNil, a.z, kSet ? a.w : kNil, b.x, kSet ? b.y : kNil, b.z, kSet ? b.w : kNil};
+    constexpr uint32_t kParts = 32, kEnough = 4; // 8 slabs at most
+    uint32_t slab = __ldg(&g.vinfo[v]).x, found = 0;
+    for (uint32_t part = 0; part < kParts && found < kEnough; ++part) {
+        const uint32_t in = part & 3u;
+        const uint4 *p = reinterpret_cast<const uint4 *>(slab_ptr(g, slab)) + 2 * in;
+        const uint4 a = __ldcg(p), b = __ldcg(p + 1);
+        uint32_t d[8] = {a.x, kSet ? a.y : kNil, a.z, kSet ? a.w : kNil,
+                         b.x, kSet ? b.y : kNil, b.z, kSet && in != 3u ? b.w : kNil};
+        bool end = false; // keys fill in order: a free one ends the list
 #pragma unroll
-    for (int k = 0; k < 8; ++k)
-        d[k] = w[k] < kTombKey ? w[k] : kNil;
+        for (int k = 0; k < 8; ++k) {
+            end = end || d[k] == kEmptyKey;
+            d[k] = d[k] < kTombKey ? d[k] : kNil;
+            found += d[k] != kNil;
+        }
+        f(d);
+        if (in == 3u)
+            slab = b.w;
+        if (end || slab == kNil)
+            break;
+    }
 }
 
 } // namespace
@@ -199,11 +218,12 @@ __global__ void __launch_bounds__(256) k_cc_sample(GView g, uint32_t *p)
     const uint32_t v = blockIdx.x * blockDim.x + threadIdx.x;
     if (v >= g.V)
         return;
-    uint32_t d[8], m = v;
-    sample_of<kSet>(g, v, d);
+    uint32_t m = v;
+    sample_of<kSet>(g, v, [&](const uint32_t(&d)[8]) {
 #pragma unroll
-    for (int k = 0; k < 8; ++k)
-        m = min(m, d[k]);
+        for (int k = 0; k < 8; ++k)
+            m = min(m, d[k]);
+    });
     p[v] = m;
 }
 
@@ -219,18 +239,19 @@ __global__ void __launch_bounds__(256) k_cc_link(GView g, uint32_t *p)
     if (at >= g.V)
         return;
     const uint32_t v = (uint32_t)at;
-    uint32_t d[8], r[8];
-    sample_of<kSet>(g, v, d);
     const uint32_t rv = __ldcg(&p[v]);
+    sample_of<kSet>(g, v, [&](const uint32_t(&d)[8]) {
+        uint32_t r[8];
 #pragma unroll
-    for (int k = 0; k < 8; ++k)
-        r[k] = d[k] != kNil ? __ldcg(&p[d[k]]) : rv;
+        for (int k = 0; k < 8; ++k)
+            r[k] = d[k] != kNil ? __ldcg(&p[d[k]]) : rv;
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-        const uint32_t hi = max(r[k], rv), lo = min(r[k], rv);
-        if (hi != lo && __ldcg(&p[hi]) > lo)
-            atomicMin(&p[hi], lo);
-    }
+        for (int k = 0; k < 8; ++k) {
+            const uint32_t hi = max(r[k], rv), lo = min(r[k], rv);
+            if (hi != lo && __ldcg(&p[hi]) > lo)
+                atomicMin(&p[hi], lo);
+        }
+    });
 }
 
 // p[v] = v's root for every vertex, and into label where that is given.  Ends

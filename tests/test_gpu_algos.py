@@ -302,3 +302,33 @@ def test_decremental_bitmap_limits(cuda_lib, V):
     check_algos(g, o, [src], wcc=False)
     assert g.last_error() == mk.MK_OK
     g.close()
+
+
+@pytest.mark.parametrize("store", ["map", "set"])
+@pytest.mark.parametrize("degree", [3, 40, 400])  # less than a slab; a few; more than the sample reads
+def test_static_components_after_churn(cuda_lib, store, degree):
+    """Static components of lists that begin with deleted pairs: the oldest
+    edges of every vertex gone, new ones behind them."""
+    mk = _mk()
+    V = 12000
+    rng = np.random.default_rng(degree)
+    src = np.arange(V, dtype=np.uint32)
+    old = np.stack([(src + 1 + k) % V for k in range(degree)]).astype(np.uint32)
+    new = np.stack([(src + 1 + 3 * V // 4) % V, rng.permutation(V)]).astype(np.uint32)
+    o = oracle.OracleGraph(V)
+    g = (mk.Graph if store == "map" else mk.SetGraph)(V, edge_capacity_hint=(degree + 4) * V, buckets=1)
+    s = np.tile(src, degree)
+
+    def insert(a, b):
+        o.insert(a, b, np.ones(len(a), np.uint32))
+        g.insert(a, b, np.ones(len(a), np.uint32)) if store == "map" else g.insert(a, b)
+
+    insert(s, old.ravel())
+    o.delete(s, old.ravel())
+    g.delete(s, old.ravel())
+    assert np.array_equal(mk.to_numpy_u32(g.wcc()), o.wcc())  # every vertex by itself
+    insert(src[: V // 3], new[0][: V // 3])
+    insert(src[::2], new[1][::2])
+    assert np.array_equal(mk.to_numpy_u32(g.wcc()), o.wcc())
+    assert g.last_error() == mk.MK_OK
+    g.close()
