@@ -96,17 +96,28 @@ __global__ void __launch_bounds__(kBlock) k_group_count(GView g, const uint32_t 
 
 // Ranges of the entry array, one atomic a block on the cursor, so that the
 // ranges follow the order of the lists up to the order of the blocks.  The
-// range of a list with more than `most` edges starts as a free hash set.
+// range of a list with more than `most` edges starts as a free hash set.  Four
+// lists a thread: a block waits for its chain (list, count, scan, cursor), so
+// there are as few blocks as fill the chip once (2^20 edges: 12 us, 26 with
+// one list a thread).
 __global__ void __launch_bounds__(kBlock) k_group_place(const uint32_t *__restrict__ alist, uint32_t H, uint2 *slot,
                                                         uint2 *ent, uint32_t most, uint32_t *ctr)
 {
     __shared__ uint32_t s_warp[kBlock / 32], s_base;
     const uint32_t n = alist ? __ldcg(&ctr[kGroupActive]) : H;
-    for (uint64_t b = blockIdx.x * (uint64_t)kBlock; b < n; b += (uint64_t)gridDim.x * kBlock) {
-        const uint64_t k = b + threadIdx.x;
-        const uint32_t L = k < n ? (alist ? alist[k] : (uint32_t)k) : kNil;
-        const uint32_t c = L != kNil ? slot[L].x : 0;
-        uint32_t incl = c;
+    for (uint64_t b = blockIdx.x * (uint64_t)(kBlock * kPer); b < n; b += (uint64_t)gridDim.x * (kBlock * kPer)) {
+        const uint64_t k0 = b + (uint64_t)threadIdx.x * kPer;
+        uint32_t L[kPer], c[kPer], sum = 0;
+#pragma unroll
+        for (uint32_t j = 0; j < kPer; ++j)
+            L[j] = k0 + j < n ? (alist ? alist[k0 + j] : (uint32_t)(k0 + j)) : kNil;
+#pragma unroll
+        for (uint32_t j = 0; j < kPer; ++j)
+            c[j] = L[j] != kNil ? slot[L[j]].x : 0;
+#pragma unroll
+        for (uint32_t j = 0; j < kPer; ++j)
+            sum += c[j];
+        uint32_t incl = sum;
 #pragma unroll
         for (uint32_t o = 1; o < 32; o <<= 1) {
             const uint32_t t = __shfl_up_sync(kFull, incl, o);
@@ -126,14 +137,18 @@ __global__ void __launch_bounds__(kBlock) k_group_place(const uint32_t *__restri
             s_base = t ? atomicAdd(&ctr[kGroupCursor], t) : 0u;
         }
         __syncthreads();
-        const uint32_t off = s_base + s_warp[threadIdx.x >> 5] + incl - c;
-        if (c)
-            slot[L].y = off;
-        for (uint32_t big = __ballot_sync(kFull, c > most); big; big &= big - 1) {
-            const uint32_t l = __ffs(big) - 1;
-            const uint32_t o = __shfl_sync(kFull, off, l), m = __shfl_sync(kFull, c, l);
-            for (uint32_t e = lane_id(); e < m; e += 32)
-                ent[o + e] = make_uint2(kNil, kNil);
+        uint32_t off = s_base + s_warp[threadIdx.x >> 5] + incl - sum;
+#pragma unroll
+        for (uint32_t j = 0; j < kPer; ++j) {
+            if (c[j])
+                slot[L[j]].y = off;
+            for (uint32_t big = __ballot_sync(kFull, c[j] > most); big; big &= big - 1) {
+                const uint32_t l = __ffs(big) - 1;
+                const uint32_t o = __shfl_sync(kFull, off, l), m = __shfl_sync(kFull, c[j], l);
+                for (uint32_t e = lane_id(); e < m; e += 32)
+                    ent[o + e] = make_uint2(kNil, kNil);
+            }
+            off += c[j];
         }
         __syncthreads(); // s_warp and s_base are written again
     }
@@ -247,8 +262,8 @@ cudaError_t group_batch(const GView &g, GroupScratch &gs, const uint32_t *src, c
     const uint32_t grid = grid_for((n + kPer - 1) / kPer, kBlock);
     k_group_count<<<grid, kBlock, 0, s>>>(g, src, dst, w, n, gs.slot, gs.lst, gs.rank, alist, gs.ctr);
     const uint64_t lists = dense ? g.H : n;
-    k_group_place<<<std::min<uint32_t>(grid_for(lists, kBlock), num_sms() * 64), kBlock, 0, s>>>(alist, g.H, gs.slot,
-                                                                                             gs.ent, most, gs.ctr);
+    k_group_place<<<std::min<uint32_t>(grid_for((lists + kPer - 1) / kPer, kBlock), num_sms() * 16), kBlock, 0, s>>>(
+        alist, g.H, gs.slot, gs.ent, most, gs.ctr);
     // One pass for each 64 MB of entries: the range of lists a pass writes
     // stays in L2, where its 8-byte stores run at 190 G/s; over an array
     // beyond L2 they run at 33 G/s.
