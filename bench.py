@@ -257,21 +257,21 @@ def algorithmic_bytes(family, ctr, n_per_launch, launches):
 # (full workload, one pass), and
 # the SHA-256 of the kernel sources (csrc/) it was taken with.  A figure is
 # reported only while those sources are unchanged; otherwise traffic is null.
-NCU_TRAFFIC_SOURCES_SHA = "03eaba235dbef8b921bc13205e888fa5968969413daccf39fe52d52d51b9a135"
+NCU_TRAFFIC_SOURCES_SHA = "f8d84621f0936ef372b1df8fa062c10102627fb5e0ab804d0ab655f205cf5c03"
 NCU_TRAFFIC = {
-    "sssp_rounds": 44158496,
-    "sssp_relax_into_invalid": 280970240,
-    "sssp_enqueue_invalid": 11001792,
-    "sssp_relax_updated": 26405248,
-    "sssp_invalidate_walk": 8524544,
-    "sssp_invalidate": 13740416,
-    "wcc_static": 542555104,
-    "wcc_hook_updated": 20227200,
-    "insert": 194368768,
-    "delete": 164786432,
-    "query": 130626304,
-    "stage_group": 75261696,
-    "update_slab_pointers": 60560192,
+    "sssp_rounds": 44152736,
+    "sssp_relax_into_invalid": 280935488,
+    "sssp_enqueue_invalid": 11005184,
+    "sssp_relax_updated": 26406208,
+    "sssp_invalidate_walk": 8530176,
+    "sssp_invalidate": 13738688,
+    "wcc_static": 542275040,
+    "wcc_hook_updated": 20227072,
+    "insert": 194249088,
+    "delete": 164794368,
+    "query": 130748416,
+    "stage_group": 75260992,
+    "update_slab_pointers": 60571456,
 }
 
 
