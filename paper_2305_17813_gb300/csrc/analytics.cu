@@ -981,7 +981,9 @@ mk_status mk_pagerank(mk_graph *g, float *d_pr, int warm_start, float damping, f
     const size_t sums = (size_t)8 << shift;
     const void *pull = packed ? (const void *)k_pr_pull<uint32_t> : (const void *)k_pr_pull<uint2>;
     int per = 1;
-    if (st == MK_OK && binned && cuda(cudaFuncSetAttribute(pull, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sums)))
+    // (the limit for the largest bins, whatever this call's are: the attribute is
+    // the function's, and another thread may be about to launch it)
+    if (st == MK_OK && binned && cuda(cudaFuncSetAttribute(pull, cudaFuncAttributeMaxDynamicSharedMemorySize, 8 << 14)))
         cuda(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, pull, 512, sums));
     const uint32_t pull_grid = (uint32_t)std::min<uint64_t>((uint64_t)num_sms() * std::max(per, 1), bins + edges_n / kChunk);
     // 4 * kPushHalves slabs per warp step
@@ -1105,12 +1107,15 @@ mk_status mk_tc_static(mk_graph *g, uint64_t *h_triangles, void *stream)
                 while (vbits < 32 && (1ull << vbits) < V)
                     ++vbits;
                 const size_t map = (1ull << vbits) / 8;
-                const bool use_map = map <= 128u << 10;
-                const size_t smem = use_map ? map : sizeof(uint32_t) << kTcBlockBits;
+                constexpr size_t kMapMax = 128u << 10, kSets = sizeof(uint32_t) << kTcBlockBits;
+                const bool use_map = map <= kMapMax;
+                const size_t smem = use_map ? map : kSets;
                 const int threads = smem <= 24u << 10 ? 256 : smem <= 48u << 10 ? 512 : 1024;
                 const void *k = use_map ? (const void *)k_tc_large<true> : (const void *)k_tc_large<false>;
                 int per = 0;
-                cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                // (not `smem`: another thread may be about to launch the same kernel)
+                cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                     (int)(use_map ? kMapMax : kSets));
                 if (e == cudaSuccess)
                     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, threads, smem);
                 if (e != cudaSuccess)

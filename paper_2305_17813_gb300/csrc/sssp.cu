@@ -1596,12 +1596,14 @@ mk_status run_sssp(mk_graph *g, int kind, uint32_t source, uint32_t *d_dist, uin
             }));
             MK_TRY(timed(g, "sssp_relax_into_invalid", s, 1, [&]() {
                 const size_t bytes = ((size_t)V + 31) / 32 * 4;
-                if (bytes > 200u << 10) {
+                constexpr size_t kMost = 200u << 10;
+                if (bytes > kMost) {
                     k_relax_into_invalid_slabs<2><<<num_sms(), kInvThreads, 0, s>>>(a);
                     return cudaSuccess;
                 }
                 auto k = k_relax_into_invalid_slabs<1>;
-                const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+                // (not `bytes`: another thread may be about to launch it for a larger graph)
+                const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMost);
                 if (e != cudaSuccess)
                     return e;
                 k<<<num_sms(), kInvThreads, bytes, s>>>(a);

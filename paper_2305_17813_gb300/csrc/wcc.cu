@@ -473,7 +473,8 @@ static cudaError_t launch_static(const GView &g, uint32_t *p, uint32_t *label, u
         k_cc_bits<<<vgrid, 256, 0, s>>>(p, g.V, giant, bits);
         if (bytes <= kCcBitBytes) {
             auto k = k_cc_scan<kSet, 1>;
-            cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+            // (not `bytes`: another thread may be about to launch it for a larger graph)
+            cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCcBitBytes);
             if (e != cudaSuccess)
                 return e;
             k<<<num_sms(), kScanThreads, bytes, s>>>(g, p, bits, giant, failed);

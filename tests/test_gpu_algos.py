@@ -332,3 +332,58 @@ def test_static_components_after_churn(cuda_lib, store, degree):
     assert np.array_equal(mk.to_numpy_u32(g.wcc()), o.wcc())
     assert g.last_error() == mk.MK_OK
     g.close()
+
+
+def test_two_sizes_from_two_threads(cuda_lib):
+    """Graphs of very different size worked on by two host threads, each on a
+    stream of its own: kernels that size their shared memory by the graph."""
+    import threading
+
+    import torch
+
+    mk = _mk()
+
+    def build(V, n, seed):
+        rng = np.random.default_rng(seed)
+        s, d = rng.integers(0, V, n).astype(np.uint32), rng.integers(0, V, n).astype(np.uint32)
+        o = oracle.OracleGraph(V)
+        o.insert(s, d, np.ones(n, np.uint32))
+        g = mk.Graph(V, edge_capacity_hint=2 * n, buckets=1)
+        g.insert(s, d, np.ones(n, np.uint32))
+        dist, _ = g.sssp(int(s[0]))
+        g.commit()
+        g.delete(s[: n // 8], d[: n // 8])
+        o.delete(s[: n // 8], d[: n // 8])
+        return g, int(s[0]), o
+
+    work = [build(20000, 60000, 1), build(900000, 500000, 2)]
+    torch.cuda.synchronize()
+    out = [None, None]
+
+    def run(k):
+        g, src, _ = work[k]
+        st = torch.cuda.Stream()
+        with torch.cuda.stream(st):
+            d, p = g.sssp(src)
+            for _ in range(20):
+                lab = g.wcc()
+                st.synchronize()
+            r = g.pagerank(max_iter=8)[0]
+            st.synchronize()
+        out[k] = d, p, lab, r
+
+    threads = [threading.Thread(target=run, args=(k,)) for k in range(2)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    for k in range(2):
+        g, src, o = work[k]
+        assert out[k] is not None
+        d, p, lab, r = out[k]
+        od, op = o.sssp(src)
+        assert np.array_equal(mk.to_numpy_u32(d), od) and np.array_equal(mk.to_numpy_u32(p), op)
+        assert np.array_equal(mk.to_numpy_u32(lab), o.wcc())
+        assert abs(float(r.sum().item()) - 1.0) < 1e-3
+        assert g.last_error() == mk.MK_OK
+        g.close()
