@@ -67,8 +67,13 @@ __device__ __host__ __forceinline__ uint32_t *count_of(uint32_t *ctr, uint32_t r
 constexpr uint32_t kSoloLists = 192;
 constexpr uint32_t kSoloRounds = 4096;
 // A frontier of at most kDirectLists lists issues the atomic minima without
-// reading the nodes first.
-constexpr uint32_t kDirectLists = 16384;
+// reading the nodes first: a round trip less, and such rounds are made of round
+// trips.  So does one of up to kDirectMost lists that is not much smaller than
+// the one before: where each list goes on improving about another (a road
+// grid: 3.78 -> 3.35 ms of rounds a pass), few of the minima are in vain; a
+// frontier that shrinks is running out of improvements (R-MAT scale 20:
+// everything up to 2^18 lists direct cost 9 % of the rounds).
+constexpr uint32_t kDirectLists = 16384, kDirectMost = 1u << 18;
 // Near-Far ordering: the far pile is split into the frontier whenever the
 // frontier holds fewer lists than this (a smaller frontier costs a round
 // about as much as a larger one).
@@ -338,11 +343,10 @@ __device__ __forceinline__ unsigned long long warp_sum(unsigned long long v)
 // (the entry two steps ahead) while the current list is relaxed.
 template <bool kNF = false, uint32_t kWarps>
 __device__ __forceinline__ void relax_body(const RoundArgs &a, const uint2 *F, uint32_t n, uint2 *Fn, uint32_t *cnt,
-                                           uint32_t round, uint32_t warp0, uint32_t nwarps, FrontierSmem<kWarps> &bq,
+                                           uint32_t round, uint32_t warp0, uint32_t nwarps, bool direct, FrontierSmem<kWarps> &bq,
                                            const NearFar *nf = nullptr, FarSmem *fs = nullptr)
 {
     const GView &g = a.g;
-    const bool direct = n <= kDirectLists;
     const uint32_t s4 = lane_id() & 3u, g4 = lane_id() >> 2;
     int *overflow = (int *)(a.ctr + kOverflow);
     uint32_t lists = 0, slabs = 0, edges = 0, improved = 0;
@@ -389,11 +393,11 @@ __device__ __forceinline__ void relax_body(const RoundArgs &a, const uint2 *F, u
 // staged entries are flushed at the end.
 template <bool kNF = false, uint32_t kWarps>
 __device__ __forceinline__ void round_step(const RoundArgs &a, uint32_t *cnt, uint32_t r, uint32_t n, uint64_t warp0,
-                                           uint64_t nwarps, uint32_t rid, FrontierSmem<kWarps> &bq,
+                                           uint64_t nwarps, uint32_t rid, bool direct, FrontierSmem<kWarps> &bq,
                                            const NearFar *nf = nullptr, FarSmem *fs = nullptr)
 {
     const uint32_t in = r & 1;
-    relax_body<kNF>(a, a.front[in], n, a.front[in ^ 1], cnt, rid + 2 + r, warp0, nwarps, bq, nf, fs);
+    relax_body<kNF>(a, a.front[in], n, a.front[in ^ 1], cnt, rid + 2 + r, warp0, nwarps, direct, bq, nf, fs);
     frontier_flush(bq, a.front[in ^ 1], cnt, a.cap, (int *)(a.ctr + kOverflow), [&]() {
         if (kNF)
             far_reserve(*nf, *fs);
@@ -556,6 +560,7 @@ __global__ void __launch_bounds__(kRoundsMaxThreads, 1) k_rounds(RoundArgs a)
     const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
     const uint32_t rid = __ldg(a.ctr + kRid);
     uint32_t r = 0, bars = 0, passed = 0;
+    uint32_t before = 0; // lists of the last round of the whole grid, none after other steps
     bool ok = true;
     // a frontier never holds more than `cap` entries; a larger count
     // (entries dropped on overflow, reported below) is read as cap
@@ -644,7 +649,9 @@ __global__ void __launch_bounds__(kRoundsMaxThreads, 1) k_rounds(RoundArgs a)
             // that of frontier r + 2
             if (blockIdx.x == 0 && threadIdx.x == 0)
                 *reinterpret_cast<unsigned long long *>(count_of(a.ctr, r + 2)) = 0;
-            round_step<kNF>(a, count_of(a.ctr, r + 1), r, n, warp0, nwarps, rid, bq, &nf, fs);
+            const bool direct = n <= kDirectLists || (n <= kDirectMost && before && n >= before - before / 4);
+            before = n;
+            round_step<kNF>(a, count_of(a.ctr, r + 1), r, n, warp0, nwarps, rid, direct, bq, &nf, fs);
             ++bars;
             ++r;
             ok = round_barrier(a.ctr, r, a.barrier_spins, &n);
@@ -664,7 +671,7 @@ __global__ void __launch_bounds__(kRoundsMaxThreads, 1) k_rounds(RoundArgs a)
             __syncthreads();
             uint32_t steps = 0;
             do {
-                round_step<kNF>(a, &solo_cnt[(r + 1) % 3], r, n, bw0, bnw, rid, bq, &nf, fs);
+                round_step<kNF>(a, &solo_cnt[(r + 1) % 3], r, n, bw0, bnw, rid, true, bq, &nf, fs);
                 __syncthreads();
                 ++r;
                 ++steps;
@@ -692,6 +699,7 @@ __global__ void __launch_bounds__(kRoundsMaxThreads, 1) k_rounds(RoundArgs a)
         __syncthreads();
         r = s_word;
         n = s_fc;
+        before = 0;
         __syncthreads(); // every thread has read them before thread 0 rewrites them
     }
     // The phase is over: every block left the loop at the same round, after
@@ -734,7 +742,7 @@ __global__ void __launch_bounds__(256) k_round_once(RoundArgs a, uint32_t r, uin
         *count_of(a.ctr, r + 2) = 0;
         a.ctr[kRoundsDone] = r + 1;
     }
-    round_step(a, count_of(a.ctr, r + 1), r, n, warp0, nwarps, __ldg(a.ctr + kRid), bq);
+    round_step(a, count_of(a.ctr, r + 1), r, n, warp0, nwarps, __ldg(a.ctr + kRid), n <= kDirectLists, bq);
 }
 
 __global__ void k_sssp_init(unsigned long long *D, uint32_t V, uint32_t source, uint2 *front, uint32_t *count,
@@ -1369,7 +1377,8 @@ __global__ void __launch_bounds__(kRoundsMaxThreads, 1) k_rounds_multi(MultiArgs
             const RoundArgs &a = m.c[j];
             const uint32_t in = r & 1;
             uint32_t *cnt = count_of(a.ctr, r + 1);
-            relax_body(a, a.front[in], n, a.front[in ^ 1], cnt, __ldg(a.ctr + kRid) + 2 + r, warp0, nwarps, bqs[j]);
+            relax_body(a, a.front[in], n, a.front[in ^ 1], cnt, __ldg(a.ctr + kRid) + 2 + r, warp0, nwarps,
+                       n <= kDirectLists, bqs[j]);
             frontier_flush(bqs[j], a.front[in ^ 1], cnt, a.cap, (int *)(a.ctr + kOverflow));
         }
         ++bars;

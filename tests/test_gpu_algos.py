@@ -387,3 +387,34 @@ def test_two_sizes_from_two_threads(cuda_lib):
         assert abs(float(r.sum().item()) - 1.0) < 1e-3
         assert g.last_error() == mk.MK_OK
         g.close()
+
+
+@pytest.mark.parametrize("width", [16384, 16385, 262144, 262145])
+def test_frontiers_of_constant_width(cuda_lib, width):
+    """Layers of equal width, so that the frontier keeps its size (and, after
+    deletes in one layer, does not), on each side of the sizes at which a
+    round issues its minima without reading the nodes."""
+    mk = _mk()
+    rng = np.random.default_rng(width)
+    layers = 4
+    V = layers * width + 1
+    at = 1 + np.arange(width)
+    s, d = [np.zeros(width, np.int64)], [at]
+    for k in range(layers - 1):
+        for _ in range(2):
+            s.append(k * width + at)
+            d.append((k + 1) * width + rng.permutation(at))
+    s, d = np.concatenate(s).astype(np.uint32), np.concatenate(d).astype(np.uint32)
+    w = rng.integers(1, 50, len(s)).astype(np.uint32)
+    nb = np.ones(V, np.uint32)
+    nb[0] = 1 + width // 15
+    g, o = mk.Graph(V, edge_capacity_hint=2 * len(s), buckets=mk.to_device_u32(nb)), oracle.OracleGraph(V)
+    g.insert(s, d, w)
+    o.insert(s, d, w)
+    check_algos(g, o, [0], wcc=False)
+    g.commit()
+    cut = slice(width, width + width // 2)
+    g.delete(s[cut], d[cut])
+    o.delete(s[cut], d[cut])
+    check_algos(g, o, [0], wcc=False)
+    g.close()
