@@ -257,21 +257,21 @@ def algorithmic_bytes(family, ctr, n_per_launch, launches):
 # (full workload, one pass), and
 # the SHA-256 of the kernel sources (csrc/) it was taken with.  A figure is
 # reported only while those sources are unchanged; otherwise traffic is null.
-NCU_TRAFFIC_SOURCES_SHA = "f8d84621f0936ef372b1df8fa062c10102627fb5e0ab804d0ab655f205cf5c03"
+NCU_TRAFFIC_SOURCES_SHA = "479f7834c9db531231d2565df3ae36c74fdf4a02c1ced3f54b5b75803610245d"
 NCU_TRAFFIC = {
-    "sssp_rounds": 44152736,
-    "sssp_relax_into_invalid": 280935488,
-    "sssp_enqueue_invalid": 11005184,
-    "sssp_relax_updated": 26406208,
-    "sssp_invalidate_walk": 8530176,
-    "sssp_invalidate": 13738688,
-    "wcc_static": 542275040,
-    "wcc_hook_updated": 20227072,
-    "insert": 194249088,
-    "delete": 164794368,
-    "query": 130748416,
-    "stage_group": 75260992,
-    "update_slab_pointers": 60571456,
+    "sssp_rounds": 44279264,
+    "sssp_relax_into_invalid": 281529984,
+    "sssp_enqueue_invalid": 11016768,
+    "sssp_relax_updated": 26401408,
+    "sssp_invalidate_walk": 8524864,
+    "sssp_invalidate": 13740800,
+    "wcc_static": 542356480,
+    "wcc_hook_updated": 20228608,
+    "insert": 194113408,
+    "delete": 165060224,
+    "query": 130645376,
+    "stage_group": 75269888,
+    "update_slab_pointers": 60586432,
 }
 
 
