@@ -340,13 +340,15 @@ __device__ __forceinline__ unsigned long long warp_sum(unsigned long long v)
 // one list at a time (group index + k * groups in the grid; eight lists per
 // warp in flight), so a round's lists are spread over all warps; each
 // group's entry, source distance and head slab are loaded one step ahead
-// (the entry two steps ahead) while the current list is relaxed.
+// (the entry two steps ahead) while the current list is relaxed.  A frontier
+// of at most `most` lists issues its minima directly (relax_edges4).
 template <bool kNF = false, uint32_t kWarps>
 __device__ __forceinline__ void relax_body(const RoundArgs &a, const uint2 *F, uint32_t n, uint2 *Fn, uint32_t *cnt,
-                                           uint32_t round, uint32_t warp0, uint32_t nwarps, bool direct, FrontierSmem<kWarps> &bq,
+                                           uint32_t round, uint32_t warp0, uint32_t nwarps, uint32_t most, FrontierSmem<kWarps> &bq,
                                            const NearFar *nf = nullptr, FarSmem *fs = nullptr)
 {
     const GView &g = a.g;
+    const bool direct = n <= most;
     const uint32_t s4 = lane_id() & 3u, g4 = lane_id() >> 2;
     int *overflow = (int *)(a.ctr + kOverflow);
     uint32_t lists = 0, slabs = 0, edges = 0, improved = 0;
@@ -393,11 +395,11 @@ __device__ __forceinline__ void relax_body(const RoundArgs &a, const uint2 *F, u
 // staged entries are flushed at the end.
 template <bool kNF = false, uint32_t kWarps>
 __device__ __forceinline__ void round_step(const RoundArgs &a, uint32_t *cnt, uint32_t r, uint32_t n, uint64_t warp0,
-                                           uint64_t nwarps, uint32_t rid, bool direct, FrontierSmem<kWarps> &bq,
+                                           uint64_t nwarps, uint32_t rid, uint32_t most, FrontierSmem<kWarps> &bq,
                                            const NearFar *nf = nullptr, FarSmem *fs = nullptr)
 {
     const uint32_t in = r & 1;
-    relax_body<kNF>(a, a.front[in], n, a.front[in ^ 1], cnt, rid + 2 + r, warp0, nwarps, direct, bq, nf, fs);
+    relax_body<kNF>(a, a.front[in], n, a.front[in ^ 1], cnt, rid + 2 + r, warp0, nwarps, most, bq, nf, fs);
     frontier_flush(bq, a.front[in ^ 1], cnt, a.cap, (int *)(a.ctr + kOverflow), [&]() {
         if (kNF)
             far_reserve(*nf, *fs);
@@ -649,9 +651,9 @@ __global__ void __launch_bounds__(kRoundsMaxThreads, 1) k_rounds(RoundArgs a)
             // that of frontier r + 2
             if (blockIdx.x == 0 && threadIdx.x == 0)
                 *reinterpret_cast<unsigned long long *>(count_of(a.ctr, r + 2)) = 0;
-            const bool direct = n <= kDirectLists || (n <= kDirectMost && before && n >= before - before / 4);
+            const uint32_t most = before && n >= before - before / 4 ? kDirectMost : kDirectLists;
             before = n;
-            round_step<kNF>(a, count_of(a.ctr, r + 1), r, n, warp0, nwarps, rid, direct, bq, &nf, fs);
+            round_step<kNF>(a, count_of(a.ctr, r + 1), r, n, warp0, nwarps, rid, most, bq, &nf, fs);
             ++bars;
             ++r;
             ok = round_barrier(a.ctr, r, a.barrier_spins, &n);
@@ -671,7 +673,7 @@ __global__ void __launch_bounds__(kRoundsMaxThreads, 1) k_rounds(RoundArgs a)
             __syncthreads();
             uint32_t steps = 0;
             do {
-                round_step<kNF>(a, &solo_cnt[(r + 1) % 3], r, n, bw0, bnw, rid, true, bq, &nf, fs);
+                round_step<kNF>(a, &solo_cnt[(r + 1) % 3], r, n, bw0, bnw, rid, kDirectLists, bq, &nf, fs);
                 __syncthreads();
                 ++r;
                 ++steps;
@@ -742,7 +744,7 @@ __global__ void __launch_bounds__(256) k_round_once(RoundArgs a, uint32_t r, uin
         *count_of(a.ctr, r + 2) = 0;
         a.ctr[kRoundsDone] = r + 1;
     }
-    round_step(a, count_of(a.ctr, r + 1), r, n, warp0, nwarps, __ldg(a.ctr + kRid), n <= kDirectLists, bq);
+    round_step(a, count_of(a.ctr, r + 1), r, n, warp0, nwarps, __ldg(a.ctr + kRid), kDirectLists, bq);
 }
 
 __global__ void k_sssp_init(unsigned long long *D, uint32_t V, uint32_t source, uint2 *front, uint32_t *count,
@@ -1378,7 +1380,7 @@ __global__ void __launch_bounds__(kRoundsMaxThreads, 1) k_rounds_multi(MultiArgs
             const uint32_t in = r & 1;
             uint32_t *cnt = count_of(a.ctr, r + 1);
             relax_body(a, a.front[in], n, a.front[in ^ 1], cnt, __ldg(a.ctr + kRid) + 2 + r, warp0, nwarps,
-                       n <= kDirectLists, bqs[j]);
+                       kDirectLists, bqs[j]);
             frontier_flush(bqs[j], a.front[in ^ 1], cnt, a.cap, (int *)(a.ctr + kOverflow));
         }
         ++bars;
