@@ -257,21 +257,21 @@ def algorithmic_bytes(family, ctr, n_per_launch, launches):
 # (full workload, one pass), and
 # the SHA-256 of the kernel sources (csrc/) it was taken with.  A figure is
 # reported only while those sources are unchanged; otherwise traffic is null.
-NCU_TRAFFIC_SOURCES_SHA = "479f7834c9db531231d2565df3ae36c74fdf4a02c1ced3f54b5b75803610245d"
+NCU_TRAFFIC_SOURCES_SHA = "c2340c15631bb49b009251658d640214bd580a64a671f3b024b078e5df4000ba"
 NCU_TRAFFIC = {
-    "sssp_rounds": 44279264,
-    "sssp_relax_into_invalid": 281529984,
-    "sssp_enqueue_invalid": 11016768,
-    "sssp_relax_updated": 26401408,
-    "sssp_invalidate_walk": 8524864,
-    "sssp_invalidate": 13740800,
-    "wcc_static": 542356480,
-    "wcc_hook_updated": 20228608,
-    "insert": 194113408,
-    "delete": 165060224,
-    "query": 130645376,
-    "stage_group": 75269888,
-    "update_slab_pointers": 60586432,
+    "sssp_rounds": 44265088,
+    "sssp_relax_into_invalid": 281357376,
+    "sssp_enqueue_invalid": 11010688,
+    "sssp_relax_updated": 26409152,
+    "sssp_invalidate_walk": 8526464,
+    "sssp_invalidate": 13741056,
+    "wcc_static": 542402464,
+    "wcc_hook_updated": 20226816,
+    "insert": 194252416,
+    "delete": 164788608,
+    "query": 130846464,
+    "stage_group": 75266176,
+    "update_slab_pointers": 60586112,
 }
 
 
