@@ -66,8 +66,8 @@ struct Vec<8> {
     }
 };
 
-// A lane's query: its destination and its source's buckets, none (vi.y 0)
-// where there is no query.
+// A lane's query: its destination and its source's buckets; none (vi.y 0, and
+// kNil, which no key word holds) where there is no query or a rejected one.
 struct Lookup {
     uint32_t d;
     uint2 vi;
@@ -75,10 +75,10 @@ struct Lookup {
 
 __device__ __forceinline__ Lookup look_up(const GView &g, uint32_t s, uint32_t d, bool live)
 {
-    Lookup q{d, make_uint2(0u, 0u)};
+    Lookup q{kNil, make_uint2(0u, 0u)};
     const bool bad = live && (s >= g.V || d >= g.V);
     if (live && !bad)
-        q.vi = __ldg(&g.vinfo[s]);
+        q = {d, __ldg(&g.vinfo[s])};
     if (__any_sync(kFull, bad) && lane_id() == 0)
         set_status(g.st, kErrInvalid);
     return q;
@@ -117,7 +117,7 @@ __device__ __forceinline__ void query_chunk(const GView &g, const Lookup &q, boo
         uint32_t w[kSteps][W], note[kAcc];
 #pragma unroll
         for (uint32_t k = 0; k < kSteps; ++k) {
-            // a query that is answered reads slab 0 along with the others of its step
+            // a query that is answered, or none, reads slab 0 along with the others of its step
             const uint32_t at = __shfl_sync(kFull, slab, k * kGroups + gi);
             if (!skip(k))
                 Vec<W>::load(slab_ptr(g, at != kNil ? at : 0u) + sub * W, w[k]);
@@ -132,7 +132,11 @@ __device__ __forceinline__ void query_chunk(const GView &g, const Lookup &q, boo
             const uint32_t d = __shfl_sync(kFull, q.d, k * kGroups + gi);
 #pragma unroll
             for (uint32_t j = 0; j < W; j += 2)
-                if (w[k][j] == d) // keys are unique in a list: at most one pair adds to a step's bits
+                // At most one pair adds to a step's four bits: a list holds a
+                // vertex once, and d is a vertex or kNil.  (The key of a free
+                // or deleted pair as d would match many, and their sum carry
+                // into the bits of another query.)
+                if (w[k][j] == d)
                     note[k / 8] += code[j / 2] << (4 * (k % 8));
         }
         uint32_t mine = 0;

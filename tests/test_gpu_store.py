@@ -364,3 +364,38 @@ def test_query_forms(cuda_lib, group, block):
         assert none is None and np.array_equal(mk.to_numpy_u32(only), obm), m
     assert g.last_error() == mk.MK_OK
     g.close()
+
+
+@pytest.mark.parametrize("group", [4, 8, 16, 32])
+def test_rejected_lookups_leave_the_others_answers_alone(cuda_lib, group):
+    """A destination that is the key of free or of deleted pairs (list 0 has
+    both), or no vertex, among a warp's lookups: the status is set, and the
+    other 31 answers are the oracle's."""
+    mk = _mk()
+    V = 100
+    deg = 10 + np.arange(40) % 13  # list 0: ten pairs of its slab, three of them deleted below
+    s = np.repeat(np.arange(40), deg).astype(np.uint32)
+    k = np.concatenate([np.arange(n) for n in deg])
+    d = ((s * 7 + k * 3) % V).astype(np.uint32)
+    w = (np.arange(len(s)) + 1).astype(np.uint32)
+    g, o = mk.Graph(V, edge_capacity_hint=4000, buckets=1), oracle.OracleGraph(V)
+    g.set_tuning(group, 256)
+    cut = np.flatnonzero(k % 4 == 1)
+    for x in (g, o):
+        x.insert(s, d, w)
+        x.delete(s[cut], d[cut])
+    at = np.cumsum(deg)[:32] - 1 - np.arange(32) % 7
+    qs, qd = s[at], np.where(np.arange(32) % 3 == 0, (d[at] + 1) % V, d[at]).astype(np.uint32)
+    obm, ow = o.query(qs, qd)
+    for pos in (0, 5, 17, 31):
+        for bad_s, bad_d in ((0, 0xFFFFFFFE), (0, 0xFFFFFFFD), (0, V), (V, 0xFFFFFFFE), (V, 3)):
+            xs, xd = qs.copy(), qd.copy()
+            xs[pos], xd[pos] = bad_s, bad_d
+            want, want_w = int(obm[0]) & ~(1 << pos), ow.copy()
+            want_w[pos] = 0
+            for ask in (g.query, lambda a, b: g.query_multi([(a, b)])[0]):
+                bm, wt = ask(xs, xd)
+                assert g.last_error() == mk.MK_ERR_INVALID_ARG
+                assert int(mk.to_numpy_u32(bm)[0]) == want, (pos, bad_s, bad_d)
+                assert np.array_equal(mk.to_numpy_u32(wt), want_w), (pos, bad_s, bad_d)
+    g.close()
