@@ -48,11 +48,13 @@ enum {
     kFarCnt0 = 10,    // Near-Far ordering: sizes of the two far piles (10, 11),
     kClearWords = 12, // words [0, 12) are cleared at the start of every call
     kFarMin0 = 12,    // the smallest distance pushed to each pile (12, 13)
-    kThresh = 14,     // and the smallest source distance of the first frontier: set to INF by ordered calls
-    kSoloR = 16,      // round index reached by a solo phase of block 0, and the frontier size there (17)
-    kRoundsDone = 18,
-    kRid = 19,        // last round stamp used (kept across calls)
-    kPhase = 20       // Near-Far: last far-pile phase stamp used (kept across calls)
+    kThresh = 14,     // the smallest source distance of the first frontier,
+    kFarFirst0 = 15,  // and the round from which each pile is known to hold something (15, 16):
+    kOrderWords = 5,  // words [12, 17) are set to INF by ordered calls
+    kSoloR = 17,      // round index reached by a solo phase of block 0, and the frontier size there (18)
+    kRoundsDone = 19,
+    kRid = 20,        // last round stamp used (kept across calls)
+    kPhase = 21       // Near-Far: last far-pile phase stamp used (kept across calls)
 };
 
 // The count of frontier r (the pair's first word).
@@ -123,7 +125,18 @@ struct NearFar {
     uint32_t *pile = nullptr; // the pile this phase appends to
     uint32_t *count = nullptr;
     uint32_t *dmin = nullptr; // smallest distance pushed to it
+    // Smallest r such that a step before round r pushed to it.  Whether a pile
+    // is split or a round run decides which barrier a block waits at next, so
+    // every block has to decide alike; a block that runs round r ahead of the
+    // others raises the pile's count, but can only set r + 1 here.
+    uint32_t *first = nullptr;
 };
+
+// The pile of index k.
+__device__ __forceinline__ NearFar far_pile(const RoundArgs &a, uint32_t k, uint32_t T, uint32_t phase)
+{
+    return {T, phase, a.far[k], a.ctr + kFarCnt0 + k, a.ctr + kFarMin0 + k, a.ctr + kFarFirst0 + k};
+}
 
 // A block's staging area for the far pile, as FrontierSmem for the frontier.
 struct FarSmem {
@@ -204,8 +217,8 @@ __device__ __forceinline__ void far_push(const RoundArgs &a, const NearFar &nf, 
 
 // Reserves the staged vertices' places in the pile: by one warp, between two
 // barriers of the block (beside the frontier's reservation, so that a round
-// waits for one of them only).
-__device__ __forceinline__ void far_reserve(const NearFar &nf, FarSmem &sm)
+// waits for one of them only).  `round`: the first round after this step.
+__device__ __forceinline__ void far_reserve(const NearFar &nf, FarSmem &sm, uint32_t round)
 {
     constexpr uint32_t kWarps = kRoundsMaxThreads / 32;
     const uint32_t lane = lane_id();
@@ -219,8 +232,10 @@ __device__ __forceinline__ void far_reserve(const NearFar &nf, FarSmem &sm)
     }
     uint32_t base = 0;
     if (lane == 31) {
-        if (sm.dmin != kInf32)
+        if (sm.dmin != kInf32) { // something was pushed, staged still or not
             atomicMin(nf.dmin, sm.dmin);
+            atomicMin(nf.first, round);
+        }
         sm.dmin = kInf32;
         if (incl)
             base = atomicAdd(nf.count, incl);
@@ -402,7 +417,7 @@ __device__ __forceinline__ void round_step(const RoundArgs &a, uint32_t *cnt, ui
     relax_body<kNF>(a, a.front[in], n, a.front[in ^ 1], cnt, rid + 2 + r, warp0, nwarps, most, bq, nf, fs);
     frontier_flush(bq, a.front[in ^ 1], cnt, a.cap, (int *)(a.ctr + kOverflow), [&]() {
         if (kNF)
-            far_reserve(*nf, *fs);
+            far_reserve(*nf, *fs, r + 1);
     });
     if (kNF)
         far_copy(a, *nf, *fs);
@@ -516,7 +531,7 @@ __device__ __forceinline__ void far_split(const RoundArgs &a, const uint32_t *pi
         const uint32_t ds[1] = {dy}, sts[1] = {st};
         far_push<1>(a, next, fs, ys, fars, ds, sts);
     }
-    frontier_flush(bq, out, cnt, a.cap, overflow, [&]() { far_reserve(next, fs); });
+    frontier_flush(bq, out, cnt, a.cap, overflow, [&]() { far_reserve(next, fs, r); });
     far_copy(a, next, fs);
 }
 
@@ -546,7 +561,7 @@ __global__ void __launch_bounds__(kRoundsMaxThreads, 1) k_rounds(RoundArgs a)
     __shared__ uint32_t solo_cnt[3];
     __shared__ FrontierSmem<kRoundsMaxThreads / 32> bq;
     __shared__ FarSmem fs[1];
-    __shared__ uint32_t s_word, s_fc, s_fm;
+    __shared__ uint32_t s_word, s_fc, s_fm, s_first;
     if (threadIdx.x == 0)
         s_word = ld_volatile(count_of(a.ctr, 0));
     if (kNF) {
@@ -583,25 +598,23 @@ __global__ void __launch_bounds__(kRoundsMaxThreads, 1) k_rounds(RoundArgs a)
         ++bars;
         ok = grid_barrier(a.ctr + kBar, passed, a.barrier_spins);
         const uint32_t t0 = ld_volatile(a.ctr + kThresh);
-        nf.T = t0 >= kInf32 - a.delta ? kInf32 : t0 + a.delta;
-        nf.phase = phase0;
-        nf.pile = a.far[0];
-        nf.count = a.ctr + kFarCnt0;
-        nf.dmin = a.ctr + kFarMin0;
+        nf = far_pile(a, 0, t0 >= kInf32 - a.delta ? kInf32 : t0 + a.delta, phase0);
     }
     while (ok && r < a.max_rounds) {
         if (kNF && n < kNearMin) {
-            // one read of the pile's size per block
+            // one read of the pile's words per block; its size and smallest
+            // distance are final where `first` says that it is split
             if (threadIdx.x == 0) {
+                s_first = ld_volatile(a.ctr + kFarFirst0 + cur);
                 s_fc = ld_volatile(a.ctr + kFarCnt0 + cur);
                 s_fm = ld_volatile(a.ctr + kFarMin0 + cur);
             }
             __syncthreads();
             const uint32_t fc = min(s_fc, a.g.V), fm = s_fm;
-            if (fc != 0) {
+            if (s_first <= r) {
                 // the near frontier is small: move the far pile's vertices
                 // below the next split distance into it, once every block
-                // has read the sizes above; the distance grows with each
+                // has read the words above; the distance grows with each
                 // split in a row
                 ++bars;
                 if (!grid_barrier(a.ctr + kBar, passed, a.barrier_spins)) {
@@ -610,12 +623,9 @@ __global__ void __launch_bounds__(kRoundsMaxThreads, 1) k_rounds(RoundArgs a)
                 }
                 const uint32_t base = max(nf.T, fm);
                 const uint64_t width = (uint64_t)a.delta << min(burst, 16u);
-                NearFar next;
-                next.T = (uint64_t)base + width >= kInf32 ? kInf32 : (uint32_t)(base + width);
-                next.phase = phase0 + ++splits;
-                next.pile = a.far[cur ^ 1];
-                next.count = a.ctr + kFarCnt0 + (cur ^ 1);
-                next.dmin = a.ctr + kFarMin0 + (cur ^ 1);
+                ++splits;
+                const NearFar next = far_pile(a, cur ^ 1, (uint64_t)base + width >= kInf32 ? kInf32 : (uint32_t)(base + width),
+                                              phase0 + splits);
                 far_split(a, nf.pile, fc, next, next.T, r, rid, warp0, nwarps, bq, fs[0]);
                 ++bars;
                 if (!grid_barrier(a.ctr + kBar, passed, a.barrier_spins)) {
@@ -628,6 +638,7 @@ __global__ void __launch_bounds__(kRoundsMaxThreads, 1) k_rounds(RoundArgs a)
                     if (blockIdx.x == 0) {
                         a.ctr[kFarCnt0 + cur] = 0;
                         a.ctr[kFarMin0 + cur] = kInf32;
+                        a.ctr[kFarFirst0 + cur] = kInf32;
                     }
                     s_word = ld_volatile(count_of(a.ctr, r));
                 }
@@ -1585,8 +1596,8 @@ mk_status run_sssp(mk_graph *g, int kind, uint32_t source, uint32_t *d_dist, uin
     a.far[1] = c->far[1];
     a.fstamp = c->fstamp;
     MK_CUDA(cudaMemsetAsync(c->counters, 0, kClearWords * 4, s));
-    if (a.delta) // the piles' minima and the first frontier's at INF
-        MK_CUDA(cudaMemsetAsync(c->counters + kFarMin0, 0xFF, 12, s));
+    if (a.delta) // the piles' minima and first rounds, and the first frontier's minimum, at INF
+        MK_CUDA(cudaMemsetAsync(c->counters + kFarMin0, 0xFF, kOrderWords * 4, s));
     if (!incremental) {
         MK_TRY(timed(g, "sssp_init", s, 1, [&]() {
             k_sssp_init<<<grid_for(V, 256), 256, 0, s>>>(c->D, V, source, c->front[0], c->counters + kCnt0,

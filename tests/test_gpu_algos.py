@@ -418,3 +418,43 @@ def test_frontiers_of_constant_width(cuda_lib, width):
     o.delete(s[cut], d[cut])
     check_algos(g, o, [0], wcc=False)
     g.close()
+
+
+@pytest.mark.parametrize("width", [193, 700, 2047, 2048])
+@pytest.mark.parametrize("delta", [3, 60, 100000])
+def test_ordered_rounds_while_the_pile_fills_and_empties(cuda_lib, width, delta):
+    """Ordered rounds of the whole grid whose frontier is below the size at
+    which the far pile is split: most of them meet an empty pile, and a few
+    heavy edges fill it in the very round that the blocks decide about.  All
+    have to take the same way, call after call."""
+    mk = _mk()
+    rng = np.random.default_rng(width + delta)
+    layers = 40
+    V = layers * width + 1
+    at = 1 + np.arange(width)
+    s, d = [np.zeros(width, np.int64)], [at]
+    for k in range(layers - 1):
+        for _ in range(2):
+            s.append(k * width + at)
+            d.append((k + 1) * width + rng.permutation(at))
+    s, d = np.concatenate(s).astype(np.uint32), np.concatenate(d).astype(np.uint32)
+    w = np.where(rng.random(len(s)) < 0.01, rng.integers(200, 5000, len(s)), rng.integers(1, 6, len(s))).astype(np.uint32)
+    nb = np.ones(V, np.uint32)
+    nb[0] = 1 + width // 15
+    g, o = mk.Graph(V, edge_capacity_hint=4 * len(s), buckets=mk.to_device_u32(nb)), oracle.OracleGraph(V)
+    g.set_sssp_delta(delta, delta)
+    g.insert(s, d, w)
+    o.insert(s, d, w)
+    for _ in range(6):
+        check_algos(g, o, [0], wcc=False)
+        assert g.last_error() == mk.MK_OK
+        g.commit()
+        cut = rng.permutation(len(s))[: len(s) // 20]
+        g.delete(s[cut], d[cut])
+        o.delete(s[cut], d[cut])
+        check_algos(g, o, [0], wcc=False)
+        assert g.last_error() == mk.MK_OK
+        g.insert(s[cut], d[cut], w[cut])
+        o.insert(s[cut], d[cut], w[cut])
+        g.commit()  # an epoch that the state has not followed: from scratch next
+    g.close()
