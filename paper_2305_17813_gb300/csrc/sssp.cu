@@ -57,8 +57,12 @@ enum {
     kPhase = 21       // Near-Far: last far-pile phase stamp used (kept across calls)
 };
 
-// The count of frontier r (the pair's first word).
-__device__ __host__ __forceinline__ uint32_t *count_of(uint32_t *ctr, uint32_t r) { return ctr + kCnt0 + 2 * (r % 3); }
+// The pair of frontier r, always accessed as one word: its size below 2^32,
+// the blocks above.
+__device__ __host__ __forceinline__ unsigned long long *count_of(uint32_t *ctr, uint32_t r)
+{
+    return reinterpret_cast<unsigned long long *>(ctr + kCnt0) + r % 3;
+}
 
 // A frontier of at most kSoloLists lists is processed by block 0 alone, with
 // block-level barriers between rounds, for at most kSoloRounds rounds in a
@@ -84,7 +88,11 @@ constexpr uint32_t kNearMin = 2048;
 __device__ __forceinline__ uint32_t node_dist(unsigned long long d) { return (uint32_t)(d >> 32); }
 __device__ __forceinline__ uint32_t node_parent(unsigned long long d) { return (uint32_t)d; }
 
-__device__ __forceinline__ uint32_t ld_volatile(const uint32_t *p) { return *(volatile const uint32_t *)p; }
+template <typename T>
+__device__ __forceinline__ uint32_t ld_volatile(const T *p)
+{
+    return (uint32_t)*(volatile const T *)p;
+}
 
 } // namespace
 
@@ -270,10 +278,10 @@ __device__ __forceinline__ void far_copy(const RoundArgs &a, const NearFar &nf, 
 // depends on its distance alone.  `direct` leaves the read of the nodes out
 // and issues every minimum: one round trip less, more atomics, for the rounds
 // whose time is their round trips.  Must be called by the full warp.
-template <bool kNF = false, uint32_t kWarps>
+template <bool kNF = false, uint32_t kWarps, typename C>
 __device__ __forceinline__ void relax_edges4(const RoundArgs &a, uint32_t x, uint32_t dx, const uint32_t (&y)[4],
                                              const uint32_t (&w)[4], const bool (&live)[4], uint32_t round,
-                                             FrontierSmem<kWarps> &bq, uint2 *Fn, uint32_t *cnt, int *overflow,
+                                             FrontierSmem<kWarps> &bq, uint2 *Fn, C *cnt, int *overflow,
                                              uint32_t &edges, uint32_t &improved,
                                              const NearFar *nf = nullptr, FarSmem *fs = nullptr,
                                              bool direct = false)
@@ -357,8 +365,8 @@ __device__ __forceinline__ unsigned long long warp_sum(unsigned long long v)
 // group's entry, source distance and head slab are loaded one step ahead
 // (the entry two steps ahead) while the current list is relaxed.  A frontier
 // of at most `most` lists issues its minima directly (relax_edges4).
-template <bool kNF = false, uint32_t kWarps>
-__device__ __forceinline__ void relax_body(const RoundArgs &a, const uint2 *F, uint32_t n, uint2 *Fn, uint32_t *cnt,
+template <bool kNF = false, uint32_t kWarps, typename C>
+__device__ __forceinline__ void relax_body(const RoundArgs &a, const uint2 *F, uint32_t n, uint2 *Fn, C *cnt,
                                            uint32_t round, uint32_t warp0, uint32_t nwarps, uint32_t most, FrontierSmem<kWarps> &bq,
                                            const NearFar *nf = nullptr, FarSmem *fs = nullptr)
 {
@@ -408,8 +416,8 @@ __device__ __forceinline__ void relax_body(const RoundArgs &a, const uint2 *F, u
 // appends to frontier r + 1, whose size is counted in *cnt (a global counter
 // or, in a solo phase, block 0's own).  Called by whole blocks: the block's
 // staged entries are flushed at the end.
-template <bool kNF = false, uint32_t kWarps>
-__device__ __forceinline__ void round_step(const RoundArgs &a, uint32_t *cnt, uint32_t r, uint32_t n, uint64_t warp0,
+template <bool kNF = false, uint32_t kWarps, typename C>
+__device__ __forceinline__ void round_step(const RoundArgs &a, C *cnt, uint32_t r, uint32_t n, uint64_t warp0,
                                            uint64_t nwarps, uint32_t rid, uint32_t most, FrontierSmem<kWarps> &bq,
                                            const NearFar *nf = nullptr, FarSmem *fs = nullptr)
 {
@@ -442,7 +450,7 @@ __device__ __forceinline__ bool round_barrier(uint32_t *ctr, uint32_t r, uint32_
     __shared__ uint32_t s_n, s_ok;
     __syncthreads();
     if (threadIdx.x == 0) {
-        unsigned long long *pair = reinterpret_cast<unsigned long long *>(count_of(ctr, r));
+        unsigned long long *pair = count_of(ctr, r);
         fence_gpu();
         atomicAdd(pair, 1ull << 32);
         uint32_t ok = 1, spins = 0;
@@ -504,7 +512,7 @@ __device__ __forceinline__ void far_split(const RoundArgs &a, const uint32_t *pi
                                           FrontierSmem<kRoundsMaxThreads / 32> &bq, FarSmem &fs)
 {
     uint2 *out = a.front[r & 1];
-    uint32_t *cnt = count_of(a.ctr, r);
+    unsigned long long *cnt = count_of(a.ctr, r);
     const uint32_t stampv = rid + 1 + r;
     int *overflow = (int *)(a.ctr + kOverflow);
     for (uint64_t wb = warp0 * 32; wb < fc; wb += nwarps * 32) {
@@ -661,7 +669,7 @@ __global__ void __launch_bounds__(kRoundsMaxThreads, 1) k_rounds(RoundArgs a)
             // the pair of frontier r - 1, which every block has left, is
             // that of frontier r + 2
             if (blockIdx.x == 0 && threadIdx.x == 0)
-                *reinterpret_cast<unsigned long long *>(count_of(a.ctr, r + 2)) = 0;
+                *count_of(a.ctr, r + 2) = 0;
             const uint32_t most = before && n >= before - before / 4 ? kDirectMost : kDirectLists;
             before = n;
             round_step<kNF>(a, count_of(a.ctr, r + 1), r, n, warp0, nwarps, rid, most, bq, &nf, fs);
@@ -696,7 +704,7 @@ __global__ void __launch_bounds__(kRoundsMaxThreads, 1) k_rounds(RoundArgs a)
             if (threadIdx.x == 0) {
                 *count_of(a.ctr, r) = n;
                 for (uint32_t k = 1; k < 3; ++k)
-                    *reinterpret_cast<unsigned long long *>(count_of(a.ctr, r + k)) = 0;
+                    *count_of(a.ctr, r + k) = 0;
                 a.ctr[kSoloR] = r;
                 a.ctr[kSoloR + 1] = n;
             }
@@ -1389,7 +1397,7 @@ __global__ void __launch_bounds__(kRoundsMaxThreads, 1) k_rounds_multi(MultiArgs
                 continue;
             const RoundArgs &a = m.c[j];
             const uint32_t in = r & 1;
-            uint32_t *cnt = count_of(a.ctr, r + 1);
+            unsigned long long *cnt = count_of(a.ctr, r + 1);
             relax_body(a, a.front[in], n, a.front[in ^ 1], cnt, __ldg(a.ctr + kRid) + 2 + r, warp0, nwarps,
                        kDirectLists, bqs[j]);
             frontier_flush(bqs[j], a.front[in ^ 1], cnt, a.cap, (int *)(a.ctr + kOverflow));

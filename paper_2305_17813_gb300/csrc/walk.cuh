@@ -34,10 +34,12 @@ __device__ __forceinline__ void frontier_init(FrontierSmem<kWarps> &sm)
 // and at most one reservation for all of them (one for each vertex with many
 // buckets made the round after a hub wait for 25 of them in a row).  Must be
 // called by the full warp; sets
-// *overflow for an entry that would not fit in `cap`.
-template <int N, uint32_t kWarps>
+// *overflow for an entry that would not fit in `cap`.  The count is a 32-bit
+// word, or the low half of a 64-bit one: every access to a word that blocks
+// race on has the word's own width.
+template <int N, uint32_t kWarps, typename C>
 __device__ __forceinline__ void enqueue_lists(FrontierSmem<kWarps> &sm, const uint32_t (&y)[N], const bool (&up)[N],
-                                              const uint2 (&vi)[N], uint2 *out, uint32_t *count, uint32_t cap,
+                                              const uint2 (&vi)[N], uint2 *out, C *count, uint32_t cap,
                                               int *overflow)
 {
     constexpr uint32_t kSmall = 8;
@@ -69,7 +71,7 @@ __device__ __forceinline__ void enqueue_lists(FrontierSmem<kWarps> &sm, const ui
     uint32_t base = 0;
     if (!fits) {
         if (lane == 0)
-            base = atomicAdd(count, held + total);
+            base = (uint32_t)atomicAdd(count, (C)(held + total));
         base = __shfl_sync(kFull, base, 0);
         for (uint32_t t = lane; t < held; t += 32)
             put(base + t, sm.buf[w][t]);
@@ -106,8 +108,8 @@ __device__ __forceinline__ void enqueue_lists(FrontierSmem<kWarps> &sm, const ui
 // the block before the entries or the staging area are used again.  `beside`
 // is called by the block's second warp while the first one waits for its
 // places: another reservation of the round.
-template <uint32_t kWarps, typename F>
-__device__ __forceinline__ void frontier_flush(FrontierSmem<kWarps> &sm, uint2 *out, uint32_t *count, uint32_t cap,
+template <uint32_t kWarps, typename C, typename F>
+__device__ __forceinline__ void frontier_flush(FrontierSmem<kWarps> &sm, uint2 *out, C *count, uint32_t cap,
                                                int *overflow, F &&beside)
 {
     const uint32_t lane = lane_id(), w = threadIdx.x >> 5;
@@ -123,7 +125,7 @@ __device__ __forceinline__ void frontier_flush(FrontierSmem<kWarps> &sm, uint2 *
         }
         uint32_t base = 0;
         if (lane == 31 && incl)
-            base = atomicAdd(count, incl);
+            base = (uint32_t)atomicAdd(count, (C)incl);
         base = __shfl_sync(kFull, base, 31);
         if (lane < kWarps)
             sm.at[lane] = base + incl - h;
@@ -143,8 +145,8 @@ __device__ __forceinline__ void frontier_flush(FrontierSmem<kWarps> &sm, uint2 *
         sm.held[w] = 0;
 }
 
-template <uint32_t kWarps>
-__device__ __forceinline__ void frontier_flush(FrontierSmem<kWarps> &sm, uint2 *out, uint32_t *count, uint32_t cap,
+template <uint32_t kWarps, typename C>
+__device__ __forceinline__ void frontier_flush(FrontierSmem<kWarps> &sm, uint2 *out, C *count, uint32_t cap,
                                                int *overflow)
 {
     frontier_flush(sm, out, count, cap, overflow, []() {});
