@@ -27,7 +27,7 @@ mk_status device_alloc(mk_graph *g, void **p, size_t bytes, cudaStream_t s)
 void device_free(mk_graph *g, void *p, size_t bytes, cudaStream_t s)
 {
     if (p) {
-        pool_free(p, s);
+        pool_free_kept(p, bytes, s);
         if (g)
             g->bytes -= bytes;
     }
@@ -414,15 +414,15 @@ mk_status mk_graph_create_ex(const mk_config *cfg, void *stream, mk_graph **out)
     if (st == MK_OK)
         st = device_alloc(nullptr, (void **)&d_bad, sizeof(int), s);
     if (st != MK_OK) {
-        device_free(nullptr, d_b, 0, s);
-        device_free(nullptr, d_off, 0, s);
-        device_free(nullptr, d_bad, 0, s);
+        device_free(nullptr, d_b, (size_t)V * 4, s);
+        device_free(nullptr, d_off, (size_t)V * 8, s);
+        device_free(nullptr, d_bad, sizeof(int), s);
         return fail(st);
     }
     auto cleanup_tmp = [&]() {
-        device_free(nullptr, d_b, 0, s);
-        device_free(nullptr, d_off, 0, s);
-        device_free(nullptr, d_bad, 0, s);
+        device_free(nullptr, d_b, (size_t)V * 4, s);
+        device_free(nullptr, d_off, (size_t)V * 8, s);
+        device_free(nullptr, d_bad, sizeof(int), s);
         d_b = nullptr;
     };
     cudaMemsetAsync(d_bad, 0, sizeof(int), s);
@@ -543,7 +543,7 @@ mk_status mk_graph_destroy(mk_graph *g)
     }
     for (auto e : g->spare_events)
         cudaEventDestroy(e);
-    pool_settle();
+    pool_settle(g->bytes); // of the arrays freed above: the others have taken theirs off
     delete g;
     return MK_OK;
 }

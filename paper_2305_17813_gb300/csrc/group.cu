@@ -213,9 +213,11 @@ namespace mk {
 
 void group_release(GroupScratch &gs, uint64_t *bytes, cudaStream_t s)
 {
-    pool_free(gs.ent, s);
-    pool_free(gs.slot, s);
-    *bytes -= (gs.cap ? edge_bytes(gs.cap) : 0) + (gs.slot ? (uint64_t)gs.lists * 8 + kGroupWords * 4 : 0);
+    const uint64_t edges = gs.cap ? edge_bytes(gs.cap) : 0;
+    const uint64_t lists = gs.slot ? (uint64_t)gs.lists * 8 + kGroupWords * 4 : 0;
+    pool_free_kept(gs.ent, edges, s);
+    pool_free_kept(gs.slot, lists, s);
+    *bytes -= edges + lists;
     gs = GroupScratch{};
 }
 
@@ -237,7 +239,7 @@ cudaError_t group_reserve(GroupScratch &gs, uint64_t n, uint32_t H, cudaStream_t
     const uint64_t old = gs.cap, cap = (std::max<uint64_t>({n, 1024, old + old / 2}) + 15) & ~15ull;
     if ((e = cudaStreamSynchronize(s)) != cudaSuccess)
         return e;
-    pool_free(gs.ent, s);
+    pool_free_kept(gs.ent, old ? edge_bytes(old) : 0, s);
     *bytes -= old ? edge_bytes(old) : 0;
     gs.ent = nullptr;
     gs.cap = 0;

@@ -5,6 +5,7 @@
 #include "meerkat.h"
 #include "group.h"
 #include "mk_device.cuh"
+#include "pool.h"
 
 #include <cuda_runtime.h>
 
@@ -189,13 +190,6 @@ inline uint32_t grid_for(uint64_t threads, uint32_t block)
 int rounds_grid(int units);
 int rounds_block(int units);
 int rounds_max_blocks_per_sm();
-// Memory from the library's pool (pool.cu): usable in `s` from this point,
-// anywhere once `s` has reached it.  pool_alloc is for workspaces freed in the
-// same call, pool_alloc_kept for what outlives it (refused in a capture).
-cudaError_t pool_alloc(void **p, size_t bytes, cudaStream_t s);
-cudaError_t pool_alloc_kept(void **p, size_t bytes, cudaStream_t s);
-void pool_free(void *p, cudaStream_t s); // null: nothing
-void pool_settle(); // after a graph's memory has been freed: what the pool keeps follows
 mk_status device_alloc(mk_graph *g, void **p, size_t bytes, cudaStream_t s);
 void device_free(mk_graph *g, void *p, size_t bytes, cudaStream_t s);
 

@@ -8,26 +8,33 @@
 // which came from the default pool and were unmapped at every synchronisation,
 // come from here too.
 //
-// Bounds: the pool gives memory that nothing uses back to the device down to
-// kPoolHold bytes at the next synchronisation (its release threshold counts
-// the memory in use too and follows it), all of it when an allocation fails
+// Bounds: the pool keeps what the library's objects hold (`kept` below; call
+// workspaces do not count) and kPoolHold bytes beside it; what it has beyond
+// that and nothing uses goes back to the device at the next synchronisation, at
+// once when an object is destroyed, and all of it when an allocation fails
 // (which is then tried once more) and on mk_trim.
 // Threads and streams: the CUDA pool serialises its calls itself and hands a
 // block freed in one stream to another only when the free has completed; the
 // table below is behind a mutex.
-#include "mk_host.h"
+#include "meerkat.h"
+#include "pool.h"
 
+#include <algorithm>
 #include <mutex>
 
 namespace {
 
+// Below 1 % of the device, so that another allocator in the process hardly
+// misses it, and enough for a graph of 33 M edges to be destroyed and made again
+// without mapping; a larger one maps the rest anew.
 constexpr uint64_t kPoolHold = 2ull << 30;
-constexpr size_t kFollow = 1 << 20; // allocations that move the threshold
+constexpr size_t kFollow = 1 << 20; // kept allocations that move the threshold
 constexpr int kMaxDevices = 64;
 
 struct DevicePool {
     cudaMemPool_t pool = nullptr;
     unsigned long long ctx = 0; // id of the context the pool belongs to
+    uint64_t kept = 0;          // bytes that outlive the call which allocated them
 };
 std::mutex g_mutex;
 DevicePool g_pools[kMaxDevices];
@@ -51,7 +58,8 @@ unsigned long long context_id()
     return fn && fn(nullptr, &id) == 0 ? id : 0;
 }
 
-cudaError_t device_pool(cudaMemPool_t *out)
+// The current device's entry, its pool made on first use; locks g_mutex.
+cudaError_t device_pool(DevicePool **out, std::unique_lock<std::mutex> &lock)
 {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -64,7 +72,7 @@ cudaError_t device_pool(cudaMemPool_t *out)
         cudaFree(nullptr);
         ctx = context_id();
     }
-    std::lock_guard<std::mutex> lock(g_mutex);
+    lock = std::unique_lock<std::mutex>(g_mutex);
     DevicePool &d = g_pools[dev];
     if (!d.pool || d.ctx != ctx) {
         cudaMemPoolProps props{};
@@ -76,19 +84,32 @@ cudaError_t device_pool(cudaMemPool_t *out)
             return e;
         d.pool = pool;
         d.ctx = ctx;
+        d.kept = 0;
+        uint64_t hold = kPoolHold;
+        cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &hold);
     }
-    *out = d.pool;
+    *out = &d;
     return cudaSuccess;
 }
 
-// The threshold: what is in use and kPoolHold.
-void follow_use(cudaMemPool_t pool)
+// Adds to the kept bytes; with `follow` the pool's threshold goes with them.
+void count_kept(uint64_t add, uint64_t take, bool follow)
 {
-    uint64_t used = 0;
-    if (cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used) != cudaSuccess)
+    DevicePool *d = nullptr;
+    std::unique_lock<std::mutex> lock;
+    if (device_pool(&d, lock) != cudaSuccess)
         return;
-    used += kPoolHold;
-    cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &used);
+    d->kept += add;
+    d->kept -= std::min(d->kept, take);
+    uint64_t most = d->kept + kPoolHold;
+    if (follow)
+        cudaMemPoolSetAttribute(d->pool, cudaMemPoolAttrReleaseThreshold, &most);
+}
+
+bool capturing(cudaStream_t s)
+{
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    return cudaStreamIsCapturing(s, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone;
 }
 
 } // namespace
@@ -99,29 +120,27 @@ cudaError_t pool_alloc(void **p, size_t bytes, cudaStream_t s)
 {
     *p = nullptr;
     cudaMemPool_t pool = nullptr;
-    cudaError_t e = device_pool(&pool);
-    if (e != cudaSuccess)
-        return e;
-    e = cudaMallocFromPoolAsync(p, bytes ? bytes : 1, pool, s);
+    {
+        DevicePool *d = nullptr;
+        std::unique_lock<std::mutex> lock;
+        const cudaError_t e = device_pool(&d, lock);
+        if (e != cudaSuccess)
+            return e;
+        pool = d->pool;
+    }
+    cudaError_t e = cudaMallocFromPoolAsync(p, bytes ? bytes : 1, pool, s);
     if (e == cudaErrorMemoryAllocation) {
         cudaGetLastError();
+        if (!capturing(s)) // a free is over when the host has seen its stream pass it
+            cudaDeviceSynchronize();
         cudaMemPoolTrimTo(pool, 0);
         e = cudaMallocFromPoolAsync(p, bytes ? bytes : 1, pool, s);
     }
     if (e != cudaSuccess) {
         cudaGetLastError();
         *p = nullptr;
-    } else if (bytes >= kFollow) {
-        follow_use(pool);
     }
     return e;
-}
-
-void pool_settle()
-{
-    cudaMemPool_t pool = nullptr;
-    if (device_pool(&pool) == cudaSuccess)
-        follow_use(pool);
 }
 
 cudaError_t pool_alloc_kept(void **p, size_t bytes, cudaStream_t s)
@@ -129,16 +148,35 @@ cudaError_t pool_alloc_kept(void **p, size_t bytes, cudaStream_t s)
     // memory allocated in a capture belongs to its graph
     cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
     *p = nullptr;
-    const cudaError_t e = cudaStreamIsCapturing(s, &st);
+    cudaError_t e = cudaStreamIsCapturing(s, &st);
     if (e != cudaSuccess)
         return e;
-    return st == cudaStreamCaptureStatusNone ? pool_alloc(p, bytes, s) : cudaErrorStreamCaptureUnsupported;
+    if (st != cudaStreamCaptureStatusNone)
+        return cudaErrorStreamCaptureUnsupported;
+    if ((e = pool_alloc(p, bytes, s)) == cudaSuccess)
+        count_kept(bytes, 0, bytes >= kFollow);
+    return e;
 }
 
-void pool_free(void *p, cudaStream_t s)
+cudaError_t pool_free(void *p, cudaStream_t s)
 {
-    if (p)
-        cudaFreeAsync(p, s);
+    return p ? cudaFreeAsync(p, s) : cudaSuccess;
+}
+
+cudaError_t pool_free_kept(void *p, size_t bytes, cudaStream_t s)
+{
+    if (!p)
+        return cudaSuccess;
+    const cudaError_t e = cudaFreeAsync(p, s);
+    if (e == cudaSuccess)
+        count_kept(0, bytes, bytes >= kFollow);
+    return e;
+}
+
+cudaError_t pool_settle(uint64_t bytes)
+{
+    count_kept(0, bytes, true);
+    return cudaSuccess;
 }
 
 } // namespace mk
@@ -146,11 +184,11 @@ void pool_free(void *p, cudaStream_t s)
 extern "C" mk_status mk_trim(void)
 {
     int dev = 0;
-    MK_CUDA(cudaGetDevice(&dev));
-    MK_CUDA(cudaDeviceSynchronize()); // a free is over when the host has seen its stream pass it
+    // a free is over when the host has seen its stream pass it
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess)
+        return MK_ERR_CUDA;
     std::lock_guard<std::mutex> lock(g_mutex);
     if (dev < 0 || dev >= kMaxDevices || !g_pools[dev].pool || g_pools[dev].ctx != context_id())
         return MK_OK;
-    MK_CUDA(cudaMemPoolTrimTo(g_pools[dev].pool, 0));
-    return MK_OK;
+    return cudaMemPoolTrimTo(g_pools[dev].pool, 0) == cudaSuccess ? MK_OK : MK_ERR_CUDA;
 }

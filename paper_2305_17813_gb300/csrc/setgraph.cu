@@ -761,7 +761,7 @@ mk_status mk_set_destroy(mk_set_graph *g)
     group_release(g->group, &g->bytes, nullptr);
     if (g->h_pinned)
         cudaFreeHost(g->h_pinned);
-    pool_settle();
+    pool_settle(g->bytes); // of the arrays freed above
     delete g;
     return MK_OK;
 }
