@@ -112,7 +112,8 @@ mk_status mk_graph_create_ex(const mk_config *cfg, void *stream, mk_graph **out)
 mk_status mk_graph_create(uint32_t V, uint64_t edge_capacity_hint, uint32_t buckets,
                           const uint32_t *d_bucket_per_vertex, void *stream, mk_graph **out);
 
-/* Frees every device buffer of the graph after synchronising the device.
+/* Frees every device buffer of the graph after synchronising its device,
+ * whichever device is current.
  * Device memory comes from a memory pool of the library (one a device, apart
  * from the process's default pool), which keeps up to 2 GiB that nothing uses
  * for the next graph or call; see mk_trim. */

@@ -398,7 +398,10 @@ mk_status mk_graph_create_ex(const mk_config *cfg, void *stream, mk_graph **out)
     *out = nullptr;
     cudaStream_t s = (cudaStream_t)stream;
     const uint32_t V = cfg->V;
+    int device = 0;
+    MK_CUDA(cudaGetDevice(&device));
     mk_graph *g = new mk_graph;
+    g->device = device;
     g->vbits = bits_for(V);
     auto fail = [&](mk_status st) {
         mk_graph_destroy(g);
@@ -518,6 +521,9 @@ mk_status mk_graph_destroy(mk_graph *g)
 {
     if (!g)
         return MK_ERR_INVALID_ARG;
+    // whatever device is current now: the work waited for, the null stream and
+    // the pool below are those of the graph's own
+    const DeviceScope on(g->device);
     cudaDeviceSynchronize();
     for (auto &kv : g->consumers)
         destroy_consumer(g, kv.second);

@@ -68,6 +68,7 @@ struct Tuning {
 } // namespace mk
 
 struct mk_graph {
+    int device = 0;              // the device that was current at its creation
     mk::GView v{};               // device pointers + sizes
     mk::Tuning tune{};
     uint32_t vbits = 1;          // bits of a vertex id in a sort key

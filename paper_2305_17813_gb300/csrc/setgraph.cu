@@ -44,6 +44,7 @@ constexpr uint32_t kSetKeys = 31; // key lanes 0..30, lane 31 = next
 } // namespace
 
 struct mk_set_graph {
+    int device = 0;            // the device that was current at its creation
     GView v{};                 // V, H, P, pool_words, vinfo, slabs, bitmap, owner, st (the rest unused)
     uint64_t bytes = 0;
     GroupScratch group;        // staging of inserts and deletes
@@ -752,6 +753,7 @@ mk_status mk_set_destroy(mk_set_graph *g)
 {
     if (!g)
         return MK_ERR_INVALID_ARG;
+    const DeviceScope on(g->device); // as mk_graph_destroy
     cudaDeviceSynchronize();
     pool_free((void *)g->v.vinfo, nullptr);
     pool_free((void *)g->v.slabs, nullptr);
@@ -773,7 +775,10 @@ mk_status mk_set_create(uint32_t V, uint64_t edge_capacity_hint, uint32_t bucket
         return MK_ERR_INVALID_ARG;
     *out = nullptr;
     cudaStream_t s = (cudaStream_t)stream;
+    int device = 0;
+    MK_CUDA(cudaGetDevice(&device));
     mk_set_graph *g = new mk_set_graph;
+    g->device = device;
     g->v.V = V;
     uint32_t *d_b = nullptr;
     uint64_t *d_off = nullptr;
