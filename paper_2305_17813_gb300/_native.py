@@ -105,7 +105,7 @@ class mk_request(ctypes.Structure):
 
 
 MK_REQ_QUERY, MK_REQ_INSERT, MK_REQ_DELETE, MK_REQ_SSSP, MK_REQ_BFS = 0, 1, 2, 3, 4
-MK_DEBUG_BARRIER_SPINS, MK_DEBUG_HOST_ROUNDS, MK_DEBUG_NO_SCRATCH = 1, 2, 3
+MK_DEBUG_BARRIER_SPINS, MK_DEBUG_HOST_ROUNDS, MK_DEBUG_NO_SCRATCH, MK_DEBUG_PART_EDGES = 1, 2, 3, 4
 MK_L2_NONE, MK_L2_VINFO, MK_L2_HEADS, MK_L2_POOL = 0, 1, 2, 3
 
 
@@ -156,6 +156,7 @@ SIGNATURES = {
     "mk_set_wcc": (_INT, [_P, _P, _P]),
     "mk_set_stats": (_INT, [_P, ctypes.POINTER(_U64), ctypes.POINTER(_U64), ctypes.POINTER(_U64), _P]),
     "mk_set_last_error": (_INT, [_P]),
+    "mk_set_debug_set": (_INT, [_P, _INT, _U64]),
     "mk_set_sssp_delta": (_INT, [_P, _U32, _U32]),
     "mk_pagerank": (_INT, [_P, _P, _INT, ctypes.c_float, ctypes.c_float, _U32, ctypes.POINTER(_U32),
                            ctypes.POINTER(ctypes.c_float), _P]),

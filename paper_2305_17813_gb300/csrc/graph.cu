@@ -702,6 +702,9 @@ mk_status mk_debug_set(mk_graph *g, int knob, uint64_t value)
     case MK_DEBUG_NO_SCRATCH:
         g->dbg_no_scratch = value != 0;
         return MK_OK;
+    case MK_DEBUG_PART_EDGES:
+        g->dbg_part = part_edges(value);
+        return MK_OK;
     default:
         return MK_ERR_INVALID_ARG;
     }

@@ -44,6 +44,7 @@ struct GroupScratch {
 // Most edges of one grouping (indexes into a hash set, two words an edge,
 // have to tell from none).
 constexpr uint64_t kGroupEdges = (1ull << 30) - 1;
+inline uint64_t part_edges(uint64_t debug) { return debug && debug < kGroupEdges ? debug : kGroupEdges; }
 
 // Whether every list is looked at (and the ranges of the entries follow the
 // lists, so that the slabs are streamed in address order), or the lists with

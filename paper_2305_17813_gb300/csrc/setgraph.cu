@@ -48,6 +48,7 @@ struct mk_set_graph {
     GView v{};                 // V, H, P, pool_words, vinfo, slabs, bitmap, owner, st (the rest unused)
     uint64_t bytes = 0;
     GroupScratch group;        // staging of inserts and deletes
+    uint64_t dbg_part = kGroupEdges; // most edges of one grouping (mk_set_debug_set)
     uint32_t *h_pinned = nullptr;
 };
 
@@ -693,7 +694,7 @@ uint32_t set_grid(uint64_t items_per_warp32)
     return std::min<uint32_t>(grid_for(std::max<uint64_t>(items_per_warp32, 1) * 32, 256), num_sms() * 32);
 }
 
-// Inserts or deletes n edges, in parts of at most kGroupEdges (a batch of more
+// Inserts or deletes n edges, in parts of at most dbg_part (a batch of more
 // is checked whole first, so that it is still rejected whole).
 template <bool kInsert>
 mk_status set_apply(mk_set_graph *g, const uint32_t *d_src, const uint32_t *d_dst, uint64_t n, uint8_t *d_flags,
@@ -701,10 +702,10 @@ mk_status set_apply(mk_set_graph *g, const uint32_t *d_src, const uint32_t *d_ds
 {
     if (d_flags)
         MK_CUDA(cudaMemsetAsync(d_flags, 0, n, s));
-    if (n > kGroupEdges)
+    if (n > g->dbg_part)
         k_check_edges<<<grid_for(n, 256), 256, 0, s>>>(d_src, d_dst, nullptr, n, g->v.V, g->v.st);
-    for (uint64_t at = 0; at < n; at += kGroupEdges) {
-        const uint64_t m = std::min(kGroupEdges, n - at);
+    for (uint64_t at = 0; at < n; at += g->dbg_part) {
+        const uint64_t m = std::min(g->dbg_part, n - at);
         const uint32_t *src = d_src + at, *dst = d_dst + at;
         uint8_t *fl = d_flags ? d_flags + at : nullptr;
         GroupView gv{};
@@ -957,6 +958,14 @@ mk_status mk_set_stats(mk_set_graph *g, uint64_t *h_lists, uint64_t *h_slabs_in_
         *h_slabs_in_use = g->v.H + used;
     if (h_device_bytes)
         *h_device_bytes = g->bytes;
+    return MK_OK;
+}
+
+mk_status mk_set_debug_set(mk_set_graph *g, int knob, uint64_t value)
+{
+    if (!g || knob != MK_DEBUG_PART_EDGES)
+        return MK_ERR_INVALID_ARG;
+    g->dbg_part = part_edges(value);
     return MK_OK;
 }
 

@@ -893,11 +893,6 @@ __global__ void __launch_bounds__(256) k_check_edges(const uint32_t *__restrict_
 
 namespace {
 
-// Edges of one grouping; a larger batch is applied in parts, in order (an
-// edge of a later part that repeats one of an earlier part then finds it
-// present, or gone: the same as in one batch).
-constexpr uint64_t kPart = kGroupEdges;
-
 mk_status stage(mk_graph *g, const uint32_t *src, const uint32_t *dst, const uint32_t *w, uint64_t n, cudaStream_t s,
                 GroupView *gv)
 {
@@ -910,10 +905,13 @@ mk_status stage(mk_graph *g, const uint32_t *src, const uint32_t *dst, const uin
     return st;
 }
 
+// A batch of more edges than one grouping takes is applied in parts, in order
+// (an edge of a later part that repeats one of an earlier part then finds it
+// present, or gone: the same as in one batch), and is checked first.
 mk_status check_whole(mk_graph *g, const uint32_t *src, const uint32_t *dst, const uint32_t *w, uint64_t n,
                       cudaStream_t s)
 {
-    if (n <= kPart)
+    if (n <= g->dbg_part)
         return MK_OK;
     return timed(g, "stage_check", s, 1, [&]() {
         k_check_edges<<<grid_for(n, 256), 256, 0, s>>>(src, dst, w, n, g->v.V, g->d_state);
@@ -1023,8 +1021,8 @@ mk_status insert_impl(mk_graph *g, const uint32_t *d_src, const uint32_t *d_dst,
     g->ulog_bound = std::min<uint64_t>(g->v.H, g->ulog_bound + n);
     const uint32_t max_hops = g->v.P + 2;
     MK_TRY(check_whole(g, d_src, d_dst, d_w, n, s));
-    for (uint64_t at = 0; at < n; at += kPart) {
-        const uint64_t m = std::min(kPart, n - at);
+    for (uint64_t at = 0; at < n; at += g->dbg_part) {
+        const uint64_t m = std::min(g->dbg_part, n - at);
         const uint32_t *src = d_src + at, *dst = d_dst + at, *w = d_w ? d_w + at : nullptr;
         uint8_t *fl = d_inserted ? d_inserted + at : nullptr;
         GroupView gv{};
@@ -1070,8 +1068,8 @@ mk_status delete_impl(mk_graph *g, const uint32_t *d_src, const uint32_t *d_dst,
         MK_CUDA(cudaMemsetAsync(d_deleted, 0, n, s));
     const uint32_t max_hops = g->v.P + 2;
     MK_TRY(check_whole(g, d_src, d_dst, nullptr, n, s));
-    for (uint64_t at = 0; at < n; at += kPart) {
-        const uint64_t m = std::min(kPart, n - at);
+    for (uint64_t at = 0; at < n; at += g->dbg_part) {
+        const uint64_t m = std::min(g->dbg_part, n - at);
         const uint32_t *src = d_src + at, *dst = d_dst + at;
         uint8_t *fl = d_deleted ? d_deleted + at : nullptr;
         GroupView gv{};

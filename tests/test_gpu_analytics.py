@@ -237,3 +237,10 @@ def test_triangles_without_work_arrays(cuda_lib, buckets):
     assert g.triangles() == o.triangles()
     assert g.last_error() == mk.MK_OK
     g.close()
+
+
+@pytest.mark.parametrize("V", [1 << 21, (1 << 24) + 5])
+def test_pagerank_at_the_limits_of_its_forms(cuda_lib, V):
+    """2^21 vertices: a source and its place in a bin fill all bits of a word.
+    More than 2^24: the bins' sums no longer fit, calls of any length push."""
+    test_pagerank_binned_and_pushed(cuda_lib, V)

@@ -126,3 +126,53 @@ def test_states_made_between_unlogged_and_logged_inserts(cuda_lib):
     same(0)
     assert g.last_error() == mk.MK_OK
     g.close()
+
+
+@pytest.mark.parametrize("store", ["map", "set"])
+@pytest.mark.parametrize("part", [1, 100, 512])
+def test_batches_in_parts(cuda_lib, store, part):
+    """A batch beyond one grouping is applied in parts: pairs that repeat
+    across parts, lists with many edges, the places of each part's flags and
+    log entries, and an invalid edge of the last part, which rejects all of
+    them."""
+    import paper_2305_17813_gb300 as mk
+    from paper_2305_17813_gb300._native import MK_DEBUG_PART_EDGES
+
+    rng = np.random.default_rng(part)
+    V, n = 300, 513 if part > 1 else 40
+    make = mk.Graph if store == "map" else mk.SetGraph
+    g, o = make(V, edge_capacity_hint=1 << 14, buckets=1), oracle.OracleGraph(V)
+    name = "mk_debug_set" if store == "map" else "mk_set_debug_set"
+    assert getattr(mk.load(), name)(g.handle, MK_DEBUG_PART_EDGES, part) == mk.MK_OK
+
+    def same():
+        if store == "map":
+            assert np.array_equal(mk.to_numpy_u32(g.wcc()), o.wcc())
+            for (a, b), (x, y) in ((g.sssp(0), o.sssp(0)), (g.bfs(3), o.bfs(3))):
+                assert np.array_equal(mk.to_numpy_u32(a), x) and np.array_equal(mk.to_numpy_u32(b), y)
+            for a, b in zip(g.export(), o.export()):
+                assert np.array_equal(mk.to_numpy_u32(a), b)
+
+    for step in range(4):
+        s = (rng.integers(0, V, n) * rng.random(n) ** 4).astype(np.uint32)  # a few vertices with most of the edges
+        d = rng.integers(0, 60, n).astype(np.uint32)
+        w = rng.integers(1, 1000, n).astype(np.uint32)
+        f = g.insert(s, d, w) if store == "map" else g.insert(s, d)
+        assert np.array_equal(f.cpu().numpy(), o.insert(s, d, w))
+        same()
+        if store == "map" and step % 2:
+            g.commit()
+        take = rng.permutation(np.arange(n).repeat(2))[:n]
+        assert np.array_equal(g.delete(s[take], d[take]).cpu().numpy(), o.delete(s[take], d[take]))
+        same()
+        if store == "map":
+            g.commit()
+        assert np.array_equal(mk.to_numpy_u32(g.query(s, d)[0] if store == "map" else g.query(s, d)), o.query(s, d)[0])
+        bad = d.copy()
+        bad[n - 1] = V
+        assert not (g.insert(s, bad, w) if store == "map" else g.insert(s, bad)).any()
+        assert g.last_error() == mk.MK_ERR_INVALID_ARG
+        assert not g.delete(s, bad).any()
+        assert g.last_error() == mk.MK_ERR_INVALID_ARG
+    same()
+    g.close()
