@@ -243,8 +243,12 @@ def algorithmic_bytes(family, ctr, n_per_launch, launches):
                 + ctr["seed_improved"] * (8 + 4 + 8) + ctr.get("seed_log", 0) * (16 + 8))
     if family == "sssp_invalidate_walk":
         return ctr["walk_vertices"] * 8 + ctr["invalidated"] * 8
-    if family in ("wcc_static", "wcc_hook_all"):
-        # the slabs with edges outside the sampled tree, two finds a united edge
+    if family == "wcc_static":
+        # every slab in use, and two finds for each edge that the scan unites
+        # (the others are tested in shared memory)
+        return 128 * ctr["wcc_slabs"] + 16 * ctr.get("wcc_united", 0)
+    if family == "wcc_hook_all":
+        # a pass that unites every edge
         return 128 * ctr["wcc_slabs"] + 16 * ctr["wcc_edges"]
     if family == "wcc_hook_updated":
         # walk of the updated lists, or the inserted-edge log (16 B an entry)

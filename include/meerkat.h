@@ -608,7 +608,7 @@ mk_status mk_list_marker(mk_graph *g, uint32_t v, uint32_t bucket, uint32_t *sla
  * order: query slabs loaded, insert slabs loaded, insert slabs linked,
  * delete slabs loaded; BFS/SSSP rounds: relaxed lists, slabs loaded, live
  * edges relaxed, improved vertices; vertices invalidated by deletions; WCC
- * slabs loaded, WCC edges united, commit slabs loaded; BFS/SSSP prologue
+ * slabs loaded, WCC edges looked at, commit slabs loaded; BFS/SSSP prologue
  * kernels (inserted-edge and invalidated-target seeds): lists, slabs loaded,
  * live edges relaxed, improved vertices; incremental WCC pass: slabs loaded,
  * edges united; BFS/SSSP rounds and grid barriers of the round kernel;
@@ -616,8 +616,8 @@ mk_status mk_list_marker(mk_graph *g, uint32_t v, uint32_t bucket, uint32_t *sla
  * into invalidated vertices, invalidated vertices given a finite distance;
  * vertices visited by the invalidation pass; BFS/SSSP tree nodes written to
  * the caller's dist/parent arrays; inserted-edge log entries read by the
- * incremental BFS/SSSP prologue and by the incremental WCC pass (then
- * reserved words up to 32).
+ * incremental BFS/SSSP prologue and by the incremental WCC pass; edges united
+ * by the static WCC pass (then reserved words up to 32).
  * The BFS/SSSP prologue words above count the inserted-edge prologue only.  Copies up to n
  * (<= 32) values to out (host); reset != 0 zeroes them.  Synchronises
  * `stream`. */

@@ -68,6 +68,7 @@ enum Counter {
     kCtrUnpacked = 26,     // BFS/SSSP tree nodes written to the caller's dist/parent arrays
     kCtrSeedLog = 27,      // inserted-edge log entries read by the incremental prologue
     kCtrWccLog = 28,       // inserted-edge log entries read by the incremental WCC pass
+    kCtrWccUnited = 29,    // edges that the static WCC pass united (its scan looks at all: kCtrWccEdges)
     kNumCounters = 32
 };
 

@@ -376,7 +376,7 @@ __global__ void __launch_bounds__(kScanThreads, 1) k_cc_scan(GView g, uint32_t *
     const uint64_t total = (uint64_t)g.H + g.P;
     const uint64_t stride = (((uint64_t)gridDim.x * kScanThreads) >> 5) * 32;
     uint32_t slabs = 0, edges = 0; // of this warp, of this lane
-    uint32_t held = 0;             // pairs in the warp's buffer
+    uint32_t held = 0, united = 0; // pairs in the warp's buffer, and taken out of it
     bool ok = true;
     uint64_t c = ((blockIdx.x * (uint64_t)kScanThreads + threadIdx.x) >> 5) * 32;
     uint32_t own_next = c + lane < total ? __ldcg(&g.owner[c + lane]) : kNil;
@@ -423,6 +423,7 @@ __global__ void __launch_bounds__(kScanThreads, 1) k_cc_scan(GView g, uint32_t *
                 __syncwarp();
                 while (held >= 64) {
                     held -= 64;
+                    united += 64;
                     ok = unite_pairs(p, &pairs[w][held], 64) && ok;
                 }
             } else {
@@ -444,7 +445,9 @@ __global__ void __launch_bounds__(kScanThreads, 1) k_cc_scan(GView g, uint32_t *
     if (!ok)
         *failed = 1;
     count_add(g.st, kCtrWccSlabs, slabs);
-    count_add(g.st, kCtrWccEdges, __reduce_add_sync(kFull, edges));
+    const uint32_t all = __reduce_add_sync(kFull, edges);
+    count_add(g.st, kCtrWccEdges, all);
+    count_add(g.st, kCtrWccUnited, kBits ? united + held : all);
 }
 
 namespace mk {

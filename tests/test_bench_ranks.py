@@ -119,3 +119,11 @@ def test_bench_arguments_and_workload_names():
     assert bench.parse_args(["--workload", "road"]).road_delta is None
     with pytest.raises(SystemExit):
         bench.parse_args(["--workload", "nonsense"])
+
+
+def test_bytes_of_the_component_scan():
+    """An edge that the scan only looks at moves no find."""
+    import bench
+
+    ctr = {"wcc_slabs": 9, "wcc_edges": 100, "wcc_united": 3}
+    assert bench.algorithmic_bytes("wcc_static", ctr, 1, 1) == 128 * 9 + 16 * 3

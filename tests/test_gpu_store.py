@@ -421,3 +421,24 @@ def test_a_calls_workspaces_do_not_raise_what_is_kept(cuda_lib):
     del pr
     torch.cuda.empty_cache()
     mk.trim()
+
+
+def test_component_counters_tell_edges_united_from_edges_seen(cuda_lib):
+    """A graph of few lists unites every edge.  A larger one is sampled first:
+    where every vertex has vertex 0 among its four neighbours the sampled tree
+    holds all of them, so that no edge is left to unite; all are looked at."""
+    mk = _mk()
+    for V in (500, 20000):
+        v = np.arange(V, dtype=np.uint32)
+        src = np.tile(v, 4)
+        dst = np.concatenate([np.zeros(V, np.uint32)] + [(v + k) % V for k in (1, 2, 3)]).astype(np.uint32)
+        g = mk.Graph(V, edge_capacity_hint=len(src), buckets=1)
+        E = int(g.insert(src, dst).sum())
+        g.commit()
+        g.counters(reset=True)
+        assert not mk.to_numpy_u32(g.wcc()).any()
+        c = g.counters()
+        assert c["wcc_edges"] == E
+        assert c["wcc_united"] == (E if V == 500 else 0)
+        assert g.last_error() == mk.MK_OK
+        g.close()
