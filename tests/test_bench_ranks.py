@@ -127,3 +127,11 @@ def test_bytes_of_the_component_scan():
 
     ctr = {"wcc_slabs": 9, "wcc_edges": 100, "wcc_united": 3}
     assert bench.algorithmic_bytes("wcc_static", ctr, 1, 1) == 128 * 9 + 16 * 3
+
+
+def test_bytes_of_a_pagerank_step():
+    """A super-step reads a word an edge up to 2^21 vertices, two beyond."""
+    import bench
+
+    assert bench.pagerank_step_bytes(10, 1 << 21) == 12 * 10 + 64 * (1 << 21)
+    assert bench.pagerank_step_bytes(10, (1 << 21) + 1) == 16 * 10 + 64 * ((1 << 21) + 1)
