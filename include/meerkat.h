@@ -669,11 +669,14 @@ mk_status mk_l2_window(mk_graph *g, int region, void *stream, mk_l2_info *out);
  * a device without room for the work arrays of mk_tc_static; 0 restores them.
  * knob MK_DEBUG_PART_EDGES: value v >= 1 applies a batch of inserts or deletes
  * in parts of at most v edges, as one of 2^30 edges or more is; 0 restores the
- * default.  mk_set_debug_set takes that knob alone.
+ * default.  knob MK_DEBUG_HASH_EDGES: value v >= 1 groups the batches of more
+ * than v - 1 edges by slab list (deletes; of the set layout inserts too), 0
+ * restores the default limits.  mk_set_debug_set takes these two knobs.
  * After mk_last_error has returned an error status, every
  * incremental algorithm state of the graph recomputes statically at its
  * next call. */
-enum { MK_DEBUG_BARRIER_SPINS = 1, MK_DEBUG_HOST_ROUNDS = 2, MK_DEBUG_NO_SCRATCH = 3, MK_DEBUG_PART_EDGES = 4 };
+enum { MK_DEBUG_BARRIER_SPINS = 1, MK_DEBUG_HOST_ROUNDS = 2, MK_DEBUG_NO_SCRATCH = 3, MK_DEBUG_PART_EDGES = 4,
+       MK_DEBUG_HASH_EDGES = 5 };
 mk_status mk_debug_set(mk_graph *g, int knob, uint64_t value);
 mk_status mk_set_debug_set(mk_set_graph *g, int knob, uint64_t value);
 

@@ -106,6 +106,7 @@ class mk_request(ctypes.Structure):
 
 MK_REQ_QUERY, MK_REQ_INSERT, MK_REQ_DELETE, MK_REQ_SSSP, MK_REQ_BFS = 0, 1, 2, 3, 4
 MK_DEBUG_BARRIER_SPINS, MK_DEBUG_HOST_ROUNDS, MK_DEBUG_NO_SCRATCH, MK_DEBUG_PART_EDGES = 1, 2, 3, 4
+MK_DEBUG_HASH_EDGES = 5
 MK_L2_NONE, MK_L2_VINFO, MK_L2_HEADS, MK_L2_POOL = 0, 1, 2, 3
 
 

@@ -705,6 +705,9 @@ mk_status mk_debug_set(mk_graph *g, int knob, uint64_t value)
     case MK_DEBUG_PART_EDGES:
         g->dbg_part = part_edges(value);
         return MK_OK;
+    case MK_DEBUG_HASH_EDGES:
+        g->dbg_hash = hash_edges(value, kHashDelete);
+        return MK_OK;
     default:
         return MK_ERR_INVALID_ARG;
     }

@@ -24,7 +24,7 @@ struct GroupView {
     uint2 *slot;           // per list <edges of this batch, their offset>; the count is 0 between calls
     const uint2 *ent;
     const uint32_t *lst;
-    const uint32_t *many;
+    const uint32_t *many;  // null: a batch that is not grouped (hash_batch)
     const uint32_t *alist; // lists with edges, or null when every list is to be looked at
     const uint32_t *ctr;
     uint32_t most;
@@ -62,6 +62,39 @@ void group_release(GroupScratch &gs, uint64_t *bytes, cudaStream_t s);
 // batch must set every active list's count back to 0.
 cudaError_t group_batch(const GView &g, GroupScratch &gs, const uint32_t *src, const uint32_t *dst, const uint32_t *w,
                         uint64_t n, uint32_t most, cudaStream_t s, GroupView *gv, int *launches);
+
+// Batches of at most this many edges are not grouped: k_dedup finds their first
+// occurrences in a hash set, and the kernels for lists with many edges take all
+// of them.  Three launches instead of five, and what is left to do for an edge,
+// one search of a chain, gains little from its list's other edges.  us, grouped
+// and so, R-MAT scale 17, of 2^20 edges scale 20 and of 2^22 scale 21:
+//   deletes of 2^4 / 2^12 / 2^16 / 2^18 / 2^20 / 2^22 edges
+//     26 / 36 / 47 / 66 / 148 / 516 and 15 / 25 / 29 / 49 / 123 / 508
+//   set deletes 25 / 32 / 39 / 61 / 133 / 414 and 16 / 27 / 31 / 53 / 123 / 465
+//   set inserts of 2^4 / 2^12 / 2^16 / 2^18 26 / 37 / 48 / 62 and 19 / 33 / 41 / 69
+// Inserts of the map layout, which append in order and log their lists, are
+// faster grouped from 2^8 edges on (33 for 43 us) and alike below.
+constexpr uint64_t kHashDelete = 1ull << 20, kHashSetInsert = 1ull << 16, kHashSetDelete = 1ull << 20;
+inline uint64_t hash_edges(uint64_t debug, uint64_t most) { return debug ? debug - 1 : most; }
+
+// Words of such a batch's hash set: kHashSpread an edge within 16 MB and what
+// the arrays of an earlier batch hold, but at least four (kHashRoom edges are
+// reserved for each).  A warp waits for its longest probe: 2^16 deletes on
+// scale 17 take 53, 39 and 37 us with 2, 4 and 16 words.
+constexpr uint64_t kHashSpread = 16, kHashWords = 1ull << 22, kHashRoom = 2;
+inline uint32_t hash_words(const GroupScratch &gs, uint64_t n)
+{
+    const uint64_t most = kHashWords < 2 * gs.cap ? kHashWords : 2 * gs.cap;
+    const uint64_t words = kHashSpread * n < most ? kHashSpread * n : most;
+    return (uint32_t)(words < 2 * n ? 2 * n : words);
+}
+
+// Validates n edges of such a batch as group_batch does, and fills *gv with
+// their hash set alone: many is null, lst[i] the index of edge i's word among
+// those at ent, kNil for an invalid edge; gs holds kHashRoom * n edges.  log
+// (nullable) gets n words of all-ones (update.cu).
+cudaError_t hash_batch(const GView &g, GroupScratch &gs, const uint32_t *src, const uint32_t *dst, const uint32_t *w,
+                       uint64_t n, unsigned long long *log, cudaStream_t s, GroupView *gv, int *launches);
 
 // Hash of a destination among the 2c words of a list's hash set.
 __device__ __forceinline__ uint32_t group_hash(uint32_t d, uint32_t words)

@@ -22,8 +22,8 @@ using namespace mk;
 
 // Kernels of update.cu, launched here unchanged.
 __global__ void k_dedup(const uint32_t *__restrict__ src, const uint32_t *__restrict__ dst,
-                        const uint32_t *__restrict__ w, uint64_t n, uint32_t V, uint32_t *tpos, uint32_t mask,
-                        uint32_t *__restrict__ slot, DevState *st);
+                        const uint32_t *__restrict__ w, uint64_t n, uint32_t V, uint32_t *tpos, uint32_t words,
+                        uint32_t *__restrict__ slot, DevState *st, unsigned long long *log);
 __global__ void __launch_bounds__(256, 6) k_insert(GView g, const uint32_t *__restrict__ src,
                                                    const uint32_t *__restrict__ dst, const uint32_t *__restrict__ w_in,
                                                    uint64_t n, const uint32_t *__restrict__ tpos,
@@ -37,7 +37,7 @@ namespace {
 
 constexpr uint64_t kNoAllocMaxBatch = MK_NOALLOC_MAX_BATCH;
 static_assert(kNoAllocMaxBatch == (1ull << 16), "the scratch layout below is sized for 2^16 edges");
-constexpr uint64_t kTable = 2 * kNoAllocMaxBatch;            // hash-set entries (a power of two)
+constexpr uint64_t kTable = 2 * kNoAllocMaxBatch;            // hash-set entries, at most half of them taken
 constexpr size_t kTposBytes = kTable * 4;
 constexpr size_t kEdgeBytes = kNoAllocMaxBatch * 4;
 constexpr size_t kScratchBytes = kTposBytes + 2 * kEdgeBytes; // 1 MiB
@@ -145,8 +145,8 @@ extern "C" mk_status mk_insert_batch_noalloc(mk_graph *g, const uint32_t *d_src,
     // launched without the profiling hook (which creates events and grows
     // a host vector): with profiling on, these kernels are counted in the
     // launch total but missing from the per-kernel times
-    k_dedup<<<grid_for(n, 256), 256, 0, s>>>(d_src, d_dst, d_w, n, g->v.V, tpos, (uint32_t)(kTable - 1), slot,
-                                             g->d_state);
+    k_dedup<<<grid_for(n, 256), 256, 0, s>>>(d_src, d_dst, d_w, n, g->v.V, tpos, (uint32_t)kTable, slot,
+                                             g->d_state, nullptr);
     g->ulog_bound = std::min<uint64_t>(g->v.H, g->ulog_bound + n);
     const uint32_t max_hops = g->v.P + 2;
     k_insert<<<grid_for(n, 256), 256, 0, s>>>(g->v, d_src, d_dst, d_w, n, tpos, slot, d_inserted, max_hops, cand, nullptr,

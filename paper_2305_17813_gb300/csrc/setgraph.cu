@@ -48,7 +48,9 @@ struct mk_set_graph {
     GView v{};                 // V, H, P, pool_words, vinfo, slabs, bitmap, owner, st (the rest unused)
     uint64_t bytes = 0;
     GroupScratch group;        // staging of inserts and deletes
-    uint64_t dbg_part = kGroupEdges; // most edges of one grouping (mk_set_debug_set)
+    // most edges of one grouping, of a delete and of an insert that is not
+    // grouped (mk_set_debug_set)
+    uint64_t dbg_part = kGroupEdges, dbg_hash[2] = {kHashSetDelete, kHashSetInsert};
     uint32_t *h_pinned = nullptr;
 };
 
@@ -253,18 +255,19 @@ __device__ __forceinline__ int group_set_delete(const GView &g, bool go, uint32_
 
 } // namespace
 
-// The lists with many edges in the batch (grouping.many), 32 edges a warp:
+// The lists with many edges in the batch (grouping.many), or all of a batch
+// that is not grouped, 32 edges a warp:
 // eight 4-lane groups take the first occurrences among them eight at a time,
 // so eight chains are walked at once.
 template <bool kInsert>
 __global__ void __launch_bounds__(256) k_set_update(GView g, GroupView gv, const uint32_t *__restrict__ src,
-                                                    const uint32_t *__restrict__ dst, uint8_t *__restrict__ flags,
-                                                    uint32_t max_hops)
+                                                    const uint32_t *__restrict__ dst, uint64_t all,
+                                                    uint8_t *__restrict__ flags, uint32_t max_hops)
 {
     const uint32_t lane = lane_id(), gi = lane >> 2;
     const uint64_t warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
-    const uint32_t n = __ldg(&gv.ctr[kGroupMany]);
-    const uint32_t *order = gv.many + __ldg(&gv.ctr[kGroupActive]);
+    const uint32_t n = gv.many ? __ldg(&gv.ctr[kGroupMany]) : (uint32_t)all;
+    const uint32_t *order = gv.many ? gv.many + __ldg(&gv.ctr[kGroupActive]) : nullptr;
     const uint32_t *tpos = reinterpret_cast<const uint32_t *>(gv.ent);
     unsigned long long loads = 0, linked = 0;
     for (uint64_t q0 = ((blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5) * 32; q0 < n; q0 += warps * 32) {
@@ -273,8 +276,9 @@ __global__ void __launch_bounds__(256) k_set_update(GView g, GroupView gv, const
         bool first = false;
         uint32_t i = 0, s = 0, d = 0;
         if (q0 + lane < n) {
-            i = order[q0 + lane];
-            first = __ldcg(&tpos[gv.lst[i] & ~kSlotBit]) == i;
+            i = order ? order[q0 + lane] : (uint32_t)q0 + lane;
+            const uint32_t at = gv.lst[i]; // kNil: an invalid edge, which no grouped list holds
+            first = at != kNil && __ldcg(&tpos[at & ~kSlotBit]) == i;
             s = src[i];
             d = dst[i];
         }
@@ -710,9 +714,15 @@ mk_status set_apply(mk_set_graph *g, const uint32_t *d_src, const uint32_t *d_ds
         uint8_t *fl = d_flags ? d_flags + at : nullptr;
         GroupView gv{};
         int launches = 0;
-        MK_CUDA(group_reserve(g->group, m, g->v.H, s, &g->bytes));
-        MK_CUDA(group_batch(g->v, g->group, src, dst, nullptr, m, kSetGroupMax, s, &gv, &launches));
-        k_set_update<kInsert><<<set_grid((m + 31) / 32), 256, 0, s>>>(g->v, gv, src, dst, fl, g->v.P + 2);
+        const bool hash = m <= g->dbg_hash[kInsert];
+        MK_CUDA(group_reserve(g->group, hash ? kHashRoom * m : m, g->v.H, s, &g->bytes));
+        MK_CUDA(hash ? hash_batch(g->v, g->group, src, dst, nullptr, m, nullptr, s, &gv, &launches)
+                     : group_batch(g->v, g->group, src, dst, nullptr, m, kSetGroupMax, s, &gv, &launches));
+        k_set_update<kInsert><<<set_grid((m + 31) / 32), 256, 0, s>>>(g->v, gv, src, dst, m, fl, g->v.P + 2);
+        if (hash) {
+            MK_CUDA(cudaGetLastError());
+            continue;
+        }
         const uint64_t lists = group_dense(g->v.H, m) ? g->v.H : m;
         const uint32_t grid = (uint32_t)std::min<uint64_t>((lists + kGroupLists - 1) / kGroupLists,
                                                            (uint64_t)num_sms() * (kInsert ? 4 : 5));
@@ -963,9 +973,14 @@ mk_status mk_set_stats(mk_set_graph *g, uint64_t *h_lists, uint64_t *h_slabs_in_
 
 mk_status mk_set_debug_set(mk_set_graph *g, int knob, uint64_t value)
 {
-    if (!g || knob != MK_DEBUG_PART_EDGES)
+    if (!g || (knob != MK_DEBUG_PART_EDGES && knob != MK_DEBUG_HASH_EDGES))
         return MK_ERR_INVALID_ARG;
-    g->dbg_part = part_edges(value);
+    if (knob == MK_DEBUG_PART_EDGES) {
+        g->dbg_part = part_edges(value);
+    } else {
+        g->dbg_hash[0] = hash_edges(value, kHashSetDelete);
+        g->dbg_hash[1] = hash_edges(value, kHashSetInsert);
+    }
     return MK_OK;
 }
 

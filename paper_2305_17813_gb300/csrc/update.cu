@@ -8,7 +8,8 @@
 // with plain stores.
 //
 // A list with more than kGroupMax edges in the batch (one bucket for a hub,
-// mostly) is applied by k_insert / k_delete instead, as is every list of the
+// mostly) is applied by k_insert / k_delete instead, as is every list of a
+// delete of up to kHashDelete edges, which is not grouped, and of the
 // allocation-free insert (noalloc.cu): the first occurrences come from a hash
 // set of pairs as batch positions (k_dedup, or the set that the grouping
 // keeps in the list's range), the edges are taken in tiles of 256 sorted by
@@ -50,21 +51,24 @@ __device__ __forceinline__ unsigned long long mix64(unsigned long long x)
 // with the batch's pair at the stored position; on a match it lowers the
 // entry to its own position if that is smaller (atomicMin), so every entry
 // ends with the smallest position of its pair.  slot[i] names the entry.
-// Invalid edges get slot kNil and set the invalid-argument status.
+// Invalid edges get slot kNil and set the invalid-argument status.  log
+// (nullable) is filled with all-ones, beside the round trips of the set.
 __global__ void k_dedup(const uint32_t *__restrict__ src, const uint32_t *__restrict__ dst,
-                        const uint32_t *__restrict__ w, uint64_t n, uint32_t V, uint32_t *tpos, uint32_t mask,
-                        uint32_t *__restrict__ slot, DevState *st)
+                        const uint32_t *__restrict__ w, uint64_t n, uint32_t V, uint32_t *tpos, uint32_t words,
+                        uint32_t *__restrict__ slot, DevState *st, unsigned long long *log)
 {
     const uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
     bool bad = false;
     if (i < n) {
+        if (log)
+            log[i] = ~0ull;
         const uint32_t s = src[i], d = dst[i];
         bad = s >= V || d >= V || (w && w[i] == 0);
         uint32_t at = kNil;
         if (!bad) {
             const unsigned long long key = ((unsigned long long)s << 32) | d;
-            uint32_t h = (uint32_t)mix64(key) & mask;
-            for (uint32_t probe = 0; probe <= mask; ++probe) {
+            uint32_t h = (uint32_t)(((unsigned long long)(uint32_t)mix64(key) * words) >> 32);
+            for (uint32_t probe = 0; probe < words; ++probe) {
                 const uint32_t j = atomicCAS(&tpos[h], kNil, (uint32_t)i);
                 if (j == kNil || (src[j] == s && dst[j] == d)) {
                     if (j != kNil && j > (uint32_t)i)
@@ -72,7 +76,7 @@ __global__ void k_dedup(const uint32_t *__restrict__ src, const uint32_t *__rest
                     at = h;
                     break;
                 }
-                h = (h + 1) & mask;
+                h = h + 1 == words ? 0 : h + 1;
             }
         }
         slot[i] = at;
@@ -546,22 +550,26 @@ __global__ void __launch_bounds__(256) k_log_updated(GView g, const uint32_t *__
     block_enqueue(g.ulog, &g.st->ulog_count, g.H, L, L != kNil, s2); // a list is logged once per epoch: fits
 }
 
-// Tiles of 256 of the batch positions in `order`, one warp per 32 sorted
-// edges: find each destination in its list's chain, the pair with TOMBSTONE, stop as soon as every destination of the group is
-// found or the chain ends; removed edges go to the change log.
+// Tiles of 256 of the batch positions in `order`, or without it of all n, one
+// warp per 32 sorted edges: finds each destination in its list's chain,
+// overwrites the pair with TOMBSTONE and stops as soon as every destination of
+// the group is found or the chain ends.  Removed edges go to the change log: to
+// a place of their list's range of it (lists), or to their own.
 __global__ void __launch_bounds__(256, 8) k_delete(GView g, const uint32_t *__restrict__ src,
-                                                   const uint32_t *__restrict__ dst,
+                                                   const uint32_t *__restrict__ dst, uint64_t n,
                                                    const uint32_t *__restrict__ tpos, const uint32_t *__restrict__ slot,
                                                    uint8_t *__restrict__ flags, uint32_t max_hops,
                                                    const uint32_t *order, const uint32_t *group_ctr, uint2 *lists,
                                                    unsigned long long *dlog)
 {
     __shared__ unsigned long long keys[256];
-    const uint64_t m = __ldg(&group_ctr[kGroupMany]);
-    order += __ldg(&group_ctr[kGroupActive]);
+    const uint64_t m = order ? __ldg(&group_ctr[kGroupMany]) : n;
+    if (order)
+        order += __ldg(&group_ctr[kGroupActive]);
     for (uint64_t tile = blockIdx.x; tile * 256 < m; tile += gridDim.x) {
         const uint32_t lane = lane_id();
         LaneEdge e = stage_tile(g, src, dst, m, tpos, slot, flags, keys, tile, order);
+        const bool staged = e.first;
         if (status_hint(g.st) != 0)
             e.first = false;
         const uint32_t gi = lane >> 2, s4 = lane & 3u;
@@ -616,8 +624,8 @@ __global__ void __launch_bounds__(256, 8) k_delete(GView g, const uint32_t *__re
             }
         }
         if (removed)
-            dlog[atomicAdd(&lists[e.list].y, 1u)] = ((unsigned long long)e.src << 32) | e.dst;
-        if (e.first && flags)
+            dlog[order ? atomicAdd(&lists[e.list].y, 1u) : e.idx] = ((unsigned long long)e.src << 32) | e.dst;
+        if (staged && flags)
             flags[e.idx] = removed ? 1 : 0;
         count_add(g.st, kCtrDeleteSlabs, loads);
     }
@@ -877,6 +885,24 @@ __global__ void __launch_bounds__(256, 6) k_apply_delete(GView g, GroupView gv, 
     count_add(g.st, kCtrDeleteSlabs, loads);
 }
 
+namespace mk {
+
+cudaError_t hash_batch(const GView &g, GroupScratch &gs, const uint32_t *src, const uint32_t *dst, const uint32_t *w,
+                       uint64_t n, unsigned long long *log, cudaStream_t s, GroupView *gv, int *launches)
+{
+    const uint32_t words = hash_words(gs, n);
+    const cudaError_t e = cudaMemsetAsync(gs.ent, 0xFF, (size_t)words * 4, s); // the hash set starts free
+    if (e != cudaSuccess)
+        return e;
+    k_dedup<<<grid_for(n, 256), 256, 0, s>>>(src, dst, w, n, g.V, (uint32_t *)gs.ent, words, gs.lst, g.st,
+                                         log);
+    *launches += 1;
+    *gv = {gs.slot, gs.ent, gs.lst, nullptr, nullptr, gs.ctr, 0};
+    return cudaGetLastError();
+}
+
+} // namespace mk
+
 // Validates edges beyond what one grouping takes, so that a batch applied in
 // parts is still rejected whole.
 __global__ void __launch_bounds__(256) k_check_edges(const uint32_t *__restrict__ src, const uint32_t *__restrict__ dst,
@@ -900,6 +926,19 @@ mk_status stage(mk_graph *g, const uint32_t *src, const uint32_t *dst, const uin
     MK_CUDA(group_reserve(g->group, n, g->v.H, s, &g->bytes));
     const mk_status st = timed(g, "stage_group", s, 0, [&]() {
         return group_batch(g->v, g->group, src, dst, w, n, kGroupMax, s, gv, &launches);
+    });
+    g->launches += (uint64_t)launches;
+    return st;
+}
+
+// A batch that is not grouped (hash_batch).
+mk_status stage_hash(mk_graph *g, const uint32_t *src, const uint32_t *dst, uint64_t n, unsigned long long *log,
+                     cudaStream_t s, GroupView *gv)
+{
+    int launches = 0;
+    MK_CUDA(group_reserve(g->group, kHashRoom * n, g->v.H, s, &g->bytes));
+    const mk_status st = timed(g, "stage_dedup", s, 0, [&]() {
+        return hash_batch(g->v, g->group, src, dst, nullptr, n, log, s, gv, &launches);
     });
     g->launches += (uint64_t)launches;
     return st;
@@ -1059,25 +1098,33 @@ mk_status delete_impl(mk_graph *g, const uint32_t *d_src, const uint32_t *d_dst,
         g->d_dlog = nl;
         g->dlog_cap = cap;
     }
-    // places where nothing is removed stay all-ones
-    unsigned long long *dlog = g->d_dlog + g->dlog_bound;
-    MK_CUDA(cudaMemsetAsync(dlog, 0xFF, n * 8, s));
-    g->dlog_bound = need;
     g->epoch_has_deletes = true;
-    if (d_deleted)
-        MK_CUDA(cudaMemsetAsync(d_deleted, 0, n, s));
     const uint32_t max_hops = g->v.P + 2;
     MK_TRY(check_whole(g, d_src, d_dst, nullptr, n, s));
     for (uint64_t at = 0; at < n; at += g->dbg_part) {
         const uint64_t m = std::min(g->dbg_part, n - at);
         const uint32_t *src = d_src + at, *dst = d_dst + at;
         uint8_t *fl = d_deleted ? d_deleted + at : nullptr;
+        // this part of the log: places where nothing is removed stay all-ones
+        // (and it counts from when that is on its way, should the call fail)
+        unsigned long long *dlog = g->d_dlog + g->dlog_bound;
+        const bool hash = m <= g->dbg_hash;
         GroupView gv{};
-        MK_TRY(stage(g, src, dst, nullptr, m, s, &gv));
-        MK_TRY(timed(g, "delete", s, 2, [&]() {
+        if (hash) {
+            MK_TRY(stage_hash(g, src, dst, m, dlog, s, &gv));
+        } else {
+            MK_CUDA(cudaMemsetAsync(dlog, 0xFF, m * 8, s));
+            if (fl)
+                MK_CUDA(cudaMemsetAsync(fl, 0, m, s));
+        }
+        g->dlog_bound += m;
+        if (!hash)
+            MK_TRY(stage(g, src, dst, nullptr, m, s, &gv));
+        MK_TRY(timed(g, "delete", s, hash ? 1 : 2, [&]() {
             k_delete<<<std::min<uint32_t>(grid_for(m, 256), num_sms() * 8), 256, 0, s>>>(
-                g->v, src, dst, (const uint32_t *)gv.ent, gv.lst, fl, max_hops, gv.many, gv.ctr, gv.slot, dlog + at);
-            k_apply_delete<<<apply_grid(m, g->v.H, 6), 256, 0, s>>>(g->v, gv, fl, dlog + at, max_hops);
+                g->v, src, dst, m, (const uint32_t *)gv.ent, gv.lst, fl, max_hops, gv.many, gv.ctr, gv.slot, dlog);
+            if (!hash)
+                k_apply_delete<<<apply_grid(m, g->v.H, 6), 256, 0, s>>>(g->v, gv, fl, dlog, max_hops);
             return cudaSuccess;
         }));
     }

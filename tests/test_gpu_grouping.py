@@ -176,3 +176,59 @@ def test_batches_in_parts(cuda_lib, store, part):
         assert g.last_error() == mk.MK_ERR_INVALID_ARG
     same()
     g.close()
+
+
+@pytest.mark.parametrize("store", ["map", "set"])
+@pytest.mark.parametrize("limit", [1, 1 << 30])  # every batch grouped; none of those that need not be
+@pytest.mark.parametrize("V", [300, 5000])
+def test_batches_grouped_and_not(cuda_lib, store, limit, V):
+    """Deletes, and the set layout's inserts, grouped by list or by their hash
+    set alone: one edge up to several tiles, a hub's lists, repeats, pairs that
+    are absent or gone, invalid edges (the flags of a rejected batch are all
+    zero), and trees that follow the deletes."""
+    import torch
+
+    import paper_2305_17813_gb300 as mk
+    from paper_2305_17813_gb300._native import MK_DEBUG_HASH_EDGES
+
+    rng = np.random.default_rng(V)
+    make = mk.Graph if store == "map" else mk.SetGraph
+    g, o = make(V, edge_capacity_hint=1 << 15, buckets=2), oracle.OracleGraph(V)
+    name = "mk_debug_set" if store == "map" else "mk_set_debug_set"
+    assert getattr(mk.load(), name)(g.handle, MK_DEBUG_HASH_EDGES, limit) == mk.MK_OK
+    live = [np.zeros(0, np.uint32)] * 2
+    for n in (1, 2, 255, 256, 257, 1000, 4099):
+        s = (rng.integers(0, V, n) * rng.random(n) ** 3).astype(np.uint32)
+        d = rng.integers(0, V, n).astype(np.uint32)
+        again = rng.integers(0, n, n // 4)
+        s, d = np.concatenate([s, s[again]]), np.concatenate([d, d[again]])
+        w = rng.integers(1, 1000, len(s)).astype(np.uint32)
+        f = g.insert(s, d, w) if store == "map" else g.insert(s, d)
+        assert np.array_equal(f.cpu().numpy(), o.insert(s, d, w))
+        live = [np.concatenate(x) for x in zip(live, (s, d))]
+        if store == "map":
+            g.sssp(0), g.bfs(0)
+            g.commit()
+        at = rng.integers(0, len(live[0]), n)
+        s, d = live[0][at], live[1][at]
+        s[: n // 8] = rng.integers(0, V, n // 8)
+        bad = s.copy()
+        bad[n // 2] = V
+        flags = torch.full((n,), 7, dtype=torch.uint8, device="cuda")
+        call = mk.load().mk_delete_batch if store == "map" else mk.load().mk_set_delete_batch
+        bs, bd = mk.to_device_u32(bad), mk.to_device_u32(d)
+        assert call(g.handle, bs.data_ptr(), bd.data_ptr(), n, flags.data_ptr(), None) == mk.MK_OK
+        assert g.last_error() == mk.MK_ERR_INVALID_ARG and not flags.any()
+        if store == "map":
+            g.sssp(0), g.bfs(0)  # current again, so that they follow the delete
+        assert np.array_equal(g.delete(s, d).cpu().numpy(), o.delete(s, d))
+        if store == "map":
+            for (a, b), (x, y) in ((g.sssp(0), o.sssp(0)), (g.bfs(0), o.bfs(0))):
+                assert np.array_equal(mk.to_numpy_u32(a), x) and np.array_equal(mk.to_numpy_u32(b), y)
+            g.commit()
+            for a, b in zip(g.export(), o.export()):
+                assert np.array_equal(mk.to_numpy_u32(a), b)
+        q = g.query(*live)
+        assert np.array_equal(mk.to_numpy_u32(q[0] if store == "map" else q), o.query(*live)[0])
+    assert g.last_error() == mk.MK_OK
+    g.close()
