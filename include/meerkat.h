@@ -670,8 +670,8 @@ mk_status mk_l2_window(mk_graph *g, int region, void *stream, mk_l2_info *out);
  * knob MK_DEBUG_PART_EDGES: value v >= 1 applies a batch of inserts or deletes
  * in parts of at most v edges, as one of 2^30 edges or more is; 0 restores the
  * default.  knob MK_DEBUG_HASH_EDGES: value v >= 1 groups the batches of more
- * than v - 1 edges by slab list (deletes; of the set layout inserts too), 0
- * restores the default limits.  mk_set_debug_set takes these two knobs.
+ * than v - 1 edges by slab list, 0 restores the default limits.
+ * mk_set_debug_set takes these two knobs.
  * After mk_last_error has returned an error status, every
  * incremental algorithm state of the graph recomputes statically at its
  * next call. */

@@ -706,7 +706,8 @@ mk_status mk_debug_set(mk_graph *g, int knob, uint64_t value)
         g->dbg_part = part_edges(value);
         return MK_OK;
     case MK_DEBUG_HASH_EDGES:
-        g->dbg_hash = hash_edges(value, kHashDelete);
+        g->dbg_hash[0] = hash_edges(value, kHashDelete);
+        g->dbg_hash[1] = hash_edges(value, kHashInsert);
         return MK_OK;
     default:
         return MK_ERR_INVALID_ARG;

@@ -72,9 +72,9 @@ cudaError_t group_batch(const GView &g, GroupScratch &gs, const uint32_t *src, c
 //     26 / 36 / 47 / 66 / 148 / 516 and 15 / 25 / 29 / 49 / 123 / 508
 //   set deletes 25 / 32 / 39 / 61 / 133 / 414 and 16 / 27 / 31 / 53 / 123 / 465
 //   set inserts of 2^4 / 2^12 / 2^16 / 2^18 26 / 37 / 48 / 62 and 19 / 33 / 41 / 69
-// Inserts of the map layout, which append in order and log their lists, are
-// faster grouped from 2^8 edges on (33 for 43 us) and alike below.
-constexpr uint64_t kHashDelete = 1ull << 20, kHashSetInsert = 1ull << 16, kHashSetDelete = 1ull << 20;
+//   inserts of 1 / 16 / 32 / 2^8 27 / 27 / 28 / 29 and 17 / 21 / 30 / 35: those
+//     fill their lists' tails in order, which the other form does one by one
+constexpr uint64_t kHashDelete = 1ull << 20, kHashInsert = 16, kHashSetInsert = 1ull << 16, kHashSetDelete = 1ull << 20;
 inline uint64_t hash_edges(uint64_t debug, uint64_t most) { return debug ? debug - 1 : most; }
 
 // Words of such a batch's hash set: kHashSpread an edge within 16 MB and what

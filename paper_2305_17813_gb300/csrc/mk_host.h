@@ -92,9 +92,10 @@ struct mk_graph {
     // test hooks (mk_debug_set): grid-barrier poll limit of the round kernel
     // (~0 = the default), the host-driven round loop instead of the
     // cooperative kernel, the static triangle count without its copy of the
-    // neighbours, the most edges of one grouping, and of a delete that
-    // is not grouped
-    uint64_t dbg_barrier_spins = ~0ull, dbg_part = mk::kGroupEdges, dbg_hash = mk::kHashDelete;
+    // neighbours, the most edges of one grouping, and of a delete and an
+    // insert that are not grouped
+    uint64_t dbg_barrier_spins = ~0ull, dbg_part = mk::kGroupEdges;
+    uint64_t dbg_hash[2] = {mk::kHashDelete, mk::kHashInsert};
     bool dbg_host_rounds = false, dbg_no_scratch = false;
     // Near-Far bucket widths of the SSSP rounds, static and incremental
     // calls (mk_set_sssp_delta; 0 = off)

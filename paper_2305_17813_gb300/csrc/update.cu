@@ -9,8 +9,8 @@
 //
 // A list with more than kGroupMax edges in the batch (one bucket for a hub,
 // mostly) is applied by k_insert / k_delete instead, as is every list of a
-// delete of up to kHashDelete edges, which is not grouped, and of the
-// allocation-free insert (noalloc.cu): the first occurrences come from a hash
+// batch that is not grouped (hash_batch: most deletes, the smallest inserts)
+// and of the allocation-free insert (noalloc.cu): the first occurrences come from a hash
 // set of pairs as batch positions (k_dedup, or the set that the grouping
 // keeps in the list's range), the edges are taken in tiles of 256 sorted by
 // list in shared memory, and one warp owns 32 consecutive sorted edges.  An
@@ -533,8 +533,8 @@ __global__ void __launch_bounds__(256, 6) k_insert(GView g, const uint32_t *__re
         }
         if (e.first && flags)
             flags[e.idx] = done;
-        if (ilog && done) // a place of the list's range of the entries, one an edge
-            ilog[atomicAdd(&lists[e.list].y, 1u)] = make_uint4(e.src, e.dst, w, 0u);
+        if (ilog && done) // a place of the list's range of the entries, one an edge, or its own
+            ilog[order ? atomicAdd(&lists[e.list].y, 1u) : e.idx] = make_uint4(e.src, e.dst, w, 0u);
         count_add(g.st, kCtrInsertSlabs, loads);
         count_add(g.st, kCtrInsertNewSlabs, linked);
     }
@@ -932,13 +932,13 @@ mk_status stage(mk_graph *g, const uint32_t *src, const uint32_t *dst, const uin
 }
 
 // A batch that is not grouped (hash_batch).
-mk_status stage_hash(mk_graph *g, const uint32_t *src, const uint32_t *dst, uint64_t n, unsigned long long *log,
-                     cudaStream_t s, GroupView *gv)
+mk_status stage_hash(mk_graph *g, const uint32_t *src, const uint32_t *dst, const uint32_t *w, uint64_t n,
+                     unsigned long long *log, cudaStream_t s, GroupView *gv)
 {
     int launches = 0;
     MK_CUDA(group_reserve(g->group, kHashRoom * n, g->v.H, s, &g->bytes));
     const mk_status st = timed(g, "stage_dedup", s, 0, [&]() {
-        return hash_batch(g->v, g->group, src, dst, nullptr, n, log, s, gv, &launches);
+        return hash_batch(g->v, g->group, src, dst, w, n, log, s, gv, &launches);
     });
     g->launches += (uint64_t)launches;
     return st;
@@ -1064,14 +1064,16 @@ mk_status insert_impl(mk_graph *g, const uint32_t *d_src, const uint32_t *d_dst,
         const uint64_t m = std::min(g->dbg_part, n - at);
         const uint32_t *src = d_src + at, *dst = d_dst + at, *w = d_w ? d_w + at : nullptr;
         uint8_t *fl = d_inserted ? d_inserted + at : nullptr;
+        const bool hash = m <= g->dbg_hash[1];
         GroupView gv{};
-        MK_TRY(stage(g, src, dst, w, m, s, &gv));
-        MK_TRY(timed(g, "insert", s, 2, [&]() {
+        MK_TRY(hash ? stage_hash(g, src, dst, w, m, nullptr, s, &gv) : stage(g, src, dst, w, m, s, &gv));
+        MK_TRY(timed(g, "insert", s, hash ? 1 : 2, [&]() {
             k_insert<<<std::min<uint32_t>(grid_for(m, 256), num_sms() * 6), 256, 0, s>>>(
                 g->v, src, dst, w, m, (const uint32_t *)gv.ent, gv.lst, fl, max_hops, nullptr, gv.many,
                 gv.ctr, gv.slot, ilog ? ilog + at : nullptr);
-            k_apply_insert<<<apply_grid(m, g->v.H, 5), 256, 0, s>>>(g->v, gv, w, fl, max_hops,
-                                                                   ilog ? ilog + at : nullptr);
+            if (!hash)
+                k_apply_insert<<<apply_grid(m, g->v.H, 5), 256, 0, s>>>(g->v, gv, w, fl, max_hops,
+                                                                       ilog ? ilog + at : nullptr);
             return cudaSuccess;
         }));
     }
@@ -1108,10 +1110,10 @@ mk_status delete_impl(mk_graph *g, const uint32_t *d_src, const uint32_t *d_dst,
         // this part of the log: places where nothing is removed stay all-ones
         // (and it counts from when that is on its way, should the call fail)
         unsigned long long *dlog = g->d_dlog + g->dlog_bound;
-        const bool hash = m <= g->dbg_hash;
+        const bool hash = m <= g->dbg_hash[0];
         GroupView gv{};
         if (hash) {
-            MK_TRY(stage_hash(g, src, dst, m, dlog, s, &gv));
+            MK_TRY(stage_hash(g, src, dst, nullptr, m, dlog, s, &gv));
         } else {
             MK_CUDA(cudaMemsetAsync(dlog, 0xFF, m * 8, s));
             if (fl)

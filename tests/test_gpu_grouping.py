@@ -182,10 +182,10 @@ def test_batches_in_parts(cuda_lib, store, part):
 @pytest.mark.parametrize("limit", [1, 1 << 30])  # every batch grouped; none of those that need not be
 @pytest.mark.parametrize("V", [300, 5000])
 def test_batches_grouped_and_not(cuda_lib, store, limit, V):
-    """Deletes, and the set layout's inserts, grouped by list or by their hash
-    set alone: one edge up to several tiles, a hub's lists, repeats, pairs that
-    are absent or gone, invalid edges (the flags of a rejected batch are all
-    zero), and trees that follow the deletes."""
+    """Batches grouped by list or by their hash set alone: one edge up to
+    several tiles, a hub's lists, repeats, pairs that are absent or gone,
+    invalid edges (the flags of a rejected batch are all zero), and trees that
+    follow the inserts and the deletes."""
     import torch
 
     import paper_2305_17813_gb300 as mk
@@ -197,6 +197,12 @@ def test_batches_grouped_and_not(cuda_lib, store, limit, V):
     name = "mk_debug_set" if store == "map" else "mk_set_debug_set"
     assert getattr(mk.load(), name)(g.handle, MK_DEBUG_HASH_EDGES, limit) == mk.MK_OK
     live = [np.zeros(0, np.uint32)] * 2
+
+    def same():
+        for (a, b), (x, y) in ((g.sssp(0), o.sssp(0)), (g.bfs(0), o.bfs(0))):
+            assert np.array_equal(mk.to_numpy_u32(a), x) and np.array_equal(mk.to_numpy_u32(b), y)
+        assert np.array_equal(mk.to_numpy_u32(g.wcc()), o.wcc())
+
     for n in (1, 2, 255, 256, 257, 1000, 4099):
         s = (rng.integers(0, V, n) * rng.random(n) ** 3).astype(np.uint32)
         d = rng.integers(0, V, n).astype(np.uint32)
@@ -207,7 +213,7 @@ def test_batches_grouped_and_not(cuda_lib, store, limit, V):
         assert np.array_equal(f.cpu().numpy(), o.insert(s, d, w))
         live = [np.concatenate(x) for x in zip(live, (s, d))]
         if store == "map":
-            g.sssp(0), g.bfs(0)
+            same()
             g.commit()
         at = rng.integers(0, len(live[0]), n)
         s, d = live[0][at], live[1][at]
@@ -220,11 +226,10 @@ def test_batches_grouped_and_not(cuda_lib, store, limit, V):
         assert call(g.handle, bs.data_ptr(), bd.data_ptr(), n, flags.data_ptr(), None) == mk.MK_OK
         assert g.last_error() == mk.MK_ERR_INVALID_ARG and not flags.any()
         if store == "map":
-            g.sssp(0), g.bfs(0)  # current again, so that they follow the delete
+            same()  # from scratch, and current again, so that they follow the delete
         assert np.array_equal(g.delete(s, d).cpu().numpy(), o.delete(s, d))
         if store == "map":
-            for (a, b), (x, y) in ((g.sssp(0), o.sssp(0)), (g.bfs(0), o.bfs(0))):
-                assert np.array_equal(mk.to_numpy_u32(a), x) and np.array_equal(mk.to_numpy_u32(b), y)
+            same()
             g.commit()
             for a, b in zip(g.export(), o.export()):
                 assert np.array_equal(mk.to_numpy_u32(a), b)
