@@ -136,8 +136,8 @@ mk_status mk_trim(void);
  * four lanes then apply a list's edges together: they find the repeats among
  * them, walk the chain once, fill the tail's free pairs with plain stores and
  * link pool slabs taken from the bitmap allocator.  A list with more than 32
- * edges in the batch goes through whole warps instead, which claim free pairs
- * with 64-bit atomicCAS.
+ * edges in the batch, and a batch of at most 16 edges, goes through whole warps
+ * instead, which claim free pairs with 64-bit atomicCAS.
  * d_inserted (n bytes, nullable): 1 where edge i was stored by this call.
  * If the pool runs out, the status becomes MK_ERR_POOL_EXHAUSTED and the
  * batch is applied partially: exactly the edges flagged 1 were stored.
@@ -181,8 +181,9 @@ mk_status mk_insert_batch_noalloc(mk_graph *g, const uint32_t *d_src, const uint
 /* Deletes n edges: a present edge's pair becomes TOMBSTONE (never reused;
  * paper, Sec. "Experimental Evaluation", deletion), an absent edge is a
  * no-op; the first occurrence of a repeated pair is the one that deletes.
- * Staged like mk_insert_batch.  d_deleted (n bytes, nullable):
- * 1 where edge i was removed by this call.  Removed edges enter the graph's
+ * A batch of more than 2^20 edges is grouped as mk_insert_batch does; the
+ * repeats of a smaller one are found in a hash set of its pairs.  d_deleted (n
+ * bytes, nullable): 1 where edge i was removed by this call.  Removed edges enter the graph's
  * change log for the decremental algorithms. */
 mk_status mk_delete_batch(mk_graph *g, const uint32_t *d_src, const uint32_t *d_dst, uint64_t n,
                           uint8_t *d_deleted, void *stream);
@@ -495,8 +496,9 @@ mk_status mk_set_create(uint32_t V, uint64_t edge_capacity_hint, uint32_t bucket
 mk_status mk_set_destroy(mk_set_graph *g);
 /* Insert / delete / query n edges as mk_insert_batch / mk_delete_batch /
  * mk_query_batch do (no weights; flags and bitmap nullable / required
- * alike).  Batches are grouped by slab list as there; a warp walks eight
- * chains at once, one per 4-lane group (32 bytes of the slab a lane). */
+ * alike).  Inserts of more than 2^16 edges and deletes of more than 2^20 are
+ * grouped by slab list as there; a warp walks eight chains at once, one per
+ * 4-lane group (32 bytes of the slab a lane). */
 mk_status mk_set_insert_batch(mk_set_graph *g, const uint32_t *d_src, const uint32_t *d_dst, uint64_t n,
                               uint8_t *d_inserted, void *stream);
 mk_status mk_set_delete_batch(mk_set_graph *g, const uint32_t *d_src, const uint32_t *d_dst, uint64_t n,

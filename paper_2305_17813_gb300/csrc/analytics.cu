@@ -8,7 +8,10 @@
 // stores in-edges; this store keeps out-edges.  A call first copies its live
 // edges out of the slabs into bins by destination, so that each super-step
 // reads them in order and adds u's contribution PR[u] / out[u] up in shared
-// memory for every edge u -> v of a bin.  Graphs and calls for which the copy
+// memory for every edge u -> v of a bin (the idea of propagation blocking:
+// Beamer, Asanovic and Patterson, "Reducing Pagerank Communication via
+// Propagation Blocking", IPDPS 2017; here the edges are binned, once a call, not
+// the contributions of each step).  Graphs and calls for which the copy
 // does not pay (more than 2^24 vertices, fewer than four super-steps, no
 // memory for it) push along the slabs instead, in address order.  Ranks,
 // contributions and sums are 64-bit fixed-point numbers (value * 2^48) added

@@ -4,10 +4,11 @@
 // owns it: repeats of a pair are found among the list's few edges, a chain is
 // walked once for all of them, and free pairs are filled with plain stores.
 //
-// What this replaces, and why: a hash set of the whole batch's pairs (one
-// random atomic an edge into a table far larger than L2, 33 G/s against
+// What large batches took before, and why: a hash set of the whole batch's pairs
+// (one random atomic an edge into a table far larger than L2, 33 G/s against
 // 128 G/s for the counters here, which stay in L2), a sort of each tile of
-// 256 edges, and one chain walk and one 64-bit CAS an edge.
+// 256 edges, and one chain walk and one 64-bit CAS an edge.  Smaller ones, whose
+// table stays in L2, still do (hash_batch).
 #include "group.h"
 #include "mk_host.h"
 
@@ -236,7 +237,8 @@ cudaError_t group_reserve(GroupScratch &gs, uint64_t n, uint32_t H, cudaStream_t
     }
     if (n <= gs.cap)
         return cudaSuccess;
-    const uint64_t old = gs.cap, cap = (std::max<uint64_t>({n, 1024, old + old / 2}) + 15) & ~15ull;
+    const uint64_t old = gs.cap, want = n <= kHashDelete ? kHashRoom * n : n;
+    const uint64_t cap = (std::max<uint64_t>({want, 1024, old + old / 2}) + 15) & ~15ull;
     if ((e = cudaStreamSynchronize(s)) != cudaSuccess)
         return e;
     pool_free_kept(gs.ent, old ? edge_bytes(old) : 0, s);

@@ -78,9 +78,11 @@ constexpr uint64_t kHashDelete = 1ull << 20, kHashInsert = 16, kHashSetInsert = 
 inline uint64_t hash_edges(uint64_t debug, uint64_t most) { return debug ? debug - 1 : most; }
 
 // Words of such a batch's hash set: kHashSpread an edge within 16 MB and what
-// the arrays of an earlier batch hold, but at least four (kHashRoom edges are
-// reserved for each).  A warp waits for its longest probe: 2^16 deletes on
-// scale 17 take 53, 39 and 37 us with 2, 4 and 16 words.
+// the arrays hold, at least two.  (Arrays that are grown for a batch of this
+// size get room for kHashRoom times its edges; they are never grown for the
+// spread alone, so that a batch that fits neither allocates nor waits.)  A warp
+// waits for its longest probe: 2^16 deletes on scale 17 take 53, 39 and 37 us
+// with 2, 4 and 16 words.
 constexpr uint64_t kHashSpread = 16, kHashWords = 1ull << 22, kHashRoom = 2;
 inline uint32_t hash_words(const GroupScratch &gs, uint64_t n)
 {
@@ -91,7 +93,7 @@ inline uint32_t hash_words(const GroupScratch &gs, uint64_t n)
 
 // Validates n edges of such a batch as group_batch does, and fills *gv with
 // their hash set alone: many is null, lst[i] the index of edge i's word among
-// those at ent, kNil for an invalid edge; gs holds kHashRoom * n edges.  log
+// those at ent, kNil for an invalid edge; gs holds n edges or more.  log
 // (nullable) gets n words of all-ones (update.cu).
 cudaError_t hash_batch(const GView &g, GroupScratch &gs, const uint32_t *src, const uint32_t *dst, const uint32_t *w,
                        uint64_t n, unsigned long long *log, cudaStream_t s, GroupView *gv, int *launches);

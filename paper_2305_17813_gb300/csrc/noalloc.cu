@@ -1,17 +1,16 @@
-// mk_insert_batch_noalloc: the batched insert by tiles of update.cu with its staging
-// scratch (the batch's hash set of (src, dst) pairs, each edge's entry and
-// the updated-list nominations) taken from one fixed device array declared
-// in this file instead of buffers grown with cudaMalloc.  The graph itself
-// must already exist; this call allocates nothing, on the device or on the
-// host.
+// mk_insert_batch_noalloc: the batched insert by tiles of update.cu with its
+// staging scratch (the batch's hash set of (src, dst) pairs, each edge's entry
+// and the updated-list nominations) taken from one fixed device array declared
+// in this file instead of buffers grown on demand.  The graph itself must
+// already exist; this call allocates nothing, on the device or on the host.
 //
-// Why: mk_insert_batch grows its staging buffers on demand, and growing them
-// calls cudaStreamSynchronize, cudaFree and cudaMalloc, which stall the
-// device and may fail.  Some callers cannot do that: a serving loop that must
-// never synchronise the device between requests, and a process whose device
-// memory is handed out by another allocator (a framework's caching allocator)
-// or fixed at start-up, where an extra cudaMalloc can fail or break the
-// budget.  They can use this entry point for batches of up to
+// Why: mk_insert_batch grows its staging buffers and its log on demand, which
+// synchronises the stream and takes memory from the library's pool, where that
+// may have to be mapped and may fail.  Some callers cannot do that: a serving
+// loop that must never synchronise the device between requests, and a process
+// whose device memory is handed out by another allocator (a framework's caching
+// allocator) or fixed at start-up, where more device memory can fail or break
+// the budget.  They can use this entry point for batches of up to
 // kNoAllocMaxBatch edges.
 #include "mk_host.h"
 

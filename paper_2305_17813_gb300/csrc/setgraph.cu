@@ -10,7 +10,7 @@
 // counts, overflow slabs claimed from a bitmap pool, EMPTY and TOMBSTONE
 // keys, deleted keys never reused (so free keys exist only in a chain's last
 // slab), set semantics with the first occurrence of a repeated pair applied
-// (a batch is grouped by slab list, as the map store's batches are: group.cu).
+// (a larger batch is grouped by slab list, as the map store's are: group.cu).
 // Inserts, deletes and queries walk eight chains per warp in 4-lane groups,
 // each lane reading 32 bytes of a slab (the whole group one 128-byte slab).
 // BFS (hop counts, with the smallest-id tight parent) and WCC (smallest-id
@@ -715,7 +715,7 @@ mk_status set_apply(mk_set_graph *g, const uint32_t *d_src, const uint32_t *d_ds
         GroupView gv{};
         int launches = 0;
         const bool hash = m <= g->dbg_hash[kInsert];
-        MK_CUDA(group_reserve(g->group, hash ? kHashRoom * m : m, g->v.H, s, &g->bytes));
+        MK_CUDA(group_reserve(g->group, m, g->v.H, s, &g->bytes));
         MK_CUDA(hash ? hash_batch(g->v, g->group, src, dst, nullptr, m, nullptr, s, &gv, &launches)
                      : group_batch(g->v, g->group, src, dst, nullptr, m, kSetGroupMax, s, &gv, &launches));
         k_set_update<kInsert><<<set_grid((m + 31) / 32), 256, 0, s>>>(g->v, gv, src, dst, m, fl, g->v.P + 2);

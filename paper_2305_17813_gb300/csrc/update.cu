@@ -1,6 +1,6 @@
 // Batched edge insert and delete.
 //
-// A batch's edges are first grouped by slab list (group.cu).  One 4-lane
+// A larger batch's edges are first grouped by slab list (group.cu).  One 4-lane
 // group then applies all of a list's edges (k_apply_insert, k_apply_delete;
 // eight lists a warp): it finds the first occurrence of every repeated pair
 // among them, walks the chain once with 16-byte slab loads, and, as nothing
@@ -10,9 +10,9 @@
 // A list with more than kGroupMax edges in the batch (one bucket for a hub,
 // mostly) is applied by k_insert / k_delete instead, as is every list of a
 // batch that is not grouped (hash_batch: most deletes, the smallest inserts)
-// and of the allocation-free insert (noalloc.cu): the first occurrences come from a hash
-// set of pairs as batch positions (k_dedup, or the set that the grouping
-// keeps in the list's range), the edges are taken in tiles of 256 sorted by
+// and of the allocation-free insert (noalloc.cu): the first occurrences come
+// from a hash set of pairs as batch positions (k_dedup, or the set that the
+// grouping keeps in the list's range), the edges are taken in tiles of 256 sorted by
 // list in shared memory, and one warp owns 32 consecutive sorted edges.  An
 // edge whose list has no other edge in the warp is handled by one 4-lane
 // group, eight at a time; the lists with several edges in the warp are
@@ -345,8 +345,8 @@ __device__ __forceinline__ void nominate(const GView &g, uint32_t *cand, uint32_
 // Tiles of 256 edges, one warp per 32 sorted edges; see the file comment.
 // With order (nullable), only the *many batch positions in it are looked at.
 // Without cand the updated lists go to the epoch's log here, and with ilog
-// the stored edges to theirs (lists: the grouping's ranges; see
-// k_apply_insert).
+// the stored edges to theirs (lists: the grouping's ranges, see
+// k_apply_insert; without order each edge's own place).
 __global__ void __launch_bounds__(256, 6) k_insert(GView g, const uint32_t *__restrict__ src,
                                                    const uint32_t *__restrict__ dst, const uint32_t *__restrict__ w_in,
                                                    uint64_t n, const uint32_t *__restrict__ tpos,
@@ -936,7 +936,7 @@ mk_status stage_hash(mk_graph *g, const uint32_t *src, const uint32_t *dst, cons
                      unsigned long long *log, cudaStream_t s, GroupView *gv)
 {
     int launches = 0;
-    MK_CUDA(group_reserve(g->group, kHashRoom * n, g->v.H, s, &g->bytes));
+    MK_CUDA(group_reserve(g->group, n, g->v.H, s, &g->bytes));
     const mk_status st = timed(g, "stage_dedup", s, 0, [&]() {
         return hash_batch(g->v, g->group, src, dst, w, n, log, s, gv, &launches);
     });

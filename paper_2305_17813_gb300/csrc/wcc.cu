@@ -156,6 +156,10 @@ __global__ void __launch_bounds__(256) k_uf_hook_log(DevState *st, const uint4 *
 // shared memory where it fits, and only slabs with an edge that is not inside
 // the giant tree unite anything.  Kernel boundaries in between also drop the
 // parents that the SMs' L1 caches still hold from before the hooks.
+// (The order of things -- sampled neighbours, link, compress, most frequent tree,
+// then what lies outside it -- is Afforest's: Sutton, Ben-Nun and Barak,
+// "Optimizing Parallel Graph Connectivity Computation via Subgraph Sampling",
+// IPDPS 2018.)
 // Sampled hooks may lose a link (a minimum replaces a root's earlier one):
 // the forest stays one of connected vertices with parents below their
 // children, and the scan looks at every edge again.

@@ -237,3 +237,21 @@ def test_batches_grouped_and_not(cuda_lib, store, limit, V):
         assert np.array_equal(mk.to_numpy_u32(q[0] if store == "map" else q), o.query(*live)[0])
     assert g.last_error() == mk.MK_OK
     g.close()
+
+
+@pytest.mark.parametrize("n", [50, 5000, 300000])
+def test_a_delete_as_large_as_an_insert_grows_nothing(cuda_lib, n):
+    """The arrays that an insert grew hold a delete of as many edges, so that it
+    neither allocates nor waits for its stream (the set store: it keeps no
+    logs beside them)."""
+    import paper_2305_17813_gb300 as mk
+
+    rng = np.random.default_rng(n)
+    g = mk.SetGraph(1 << 14, edge_capacity_hint=n, buckets=1)
+    s, d = (rng.integers(0, 1 << 14, n).astype(np.uint32) for _ in range(2))
+    stored = g.insert(s, d)
+    held = g.stats()["device_bytes"]
+    assert np.array_equal(g.delete(s, d).cpu().numpy(), stored.cpu().numpy())
+    assert g.stats()["device_bytes"] == held
+    assert g.last_error() == mk.MK_OK
+    g.close()
