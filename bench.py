@@ -223,6 +223,8 @@ def algorithmic_bytes(family, ctr, n_per_launch, launches):
         # the logs; a slab is read, or written when new
         return launches * n_per_launch * (12 + 32 + 32) + 128 * (ctr["insert_slabs"] + ctr["insert_new_slabs"])
     if family == "delete":
+        # the edge, a sector of its bucket range (or of its list's), one of the
+        # hash set (or of the log)
         return launches * n_per_launch * (8 + 32 + 32) + 128 * ctr["delete_slabs"]
     if family == "stage_group":
         # per edge: the edge (12 B), its index sector, a counter, its list and
@@ -270,21 +272,22 @@ def pagerank_step_bytes(E, V):
 # (full workload, one pass), and
 # the SHA-256 of the kernel sources (csrc/) it was taken with.  A figure is
 # reported only while those sources are unchanged; otherwise traffic is null.
-NCU_TRAFFIC_SOURCES_SHA = "c2340c15631bb49b009251658d640214bd580a64a671f3b024b078e5df4000ba"
+NCU_TRAFFIC_SOURCES_SHA = "104c5fa90181dc58dd1cf6c799c2e7417fe0dde2cf9d74e215406a94d843d2df"
 NCU_TRAFFIC = {
-    "sssp_rounds": 44265088,
-    "sssp_relax_into_invalid": 281357376,
-    "sssp_enqueue_invalid": 11010688,
-    "sssp_relax_updated": 26409152,
-    "sssp_invalidate_walk": 8526464,
-    "sssp_invalidate": 13741056,
-    "wcc_static": 542402464,
-    "wcc_hook_updated": 20226816,
-    "insert": 194252416,
-    "delete": 164788608,
-    "query": 130846464,
-    "stage_group": 75266176,
-    "update_slab_pointers": 60586112,
+    "sssp_rounds": 43972640,
+    "sssp_relax_into_invalid": 281252864,
+    "sssp_enqueue_invalid": 11012736,
+    "sssp_relax_updated": 26405568,
+    "sssp_invalidate_walk": 8526016,
+    "sssp_invalidate": 13739648,
+    "wcc_static": 542307200,
+    "wcc_hook_updated": 20226944,
+    "insert": 194361984,
+    "delete": 176866560,
+    "query": 130544384,
+    "stage_group": 77223552,
+    "stage_dedup": 24781568,
+    "update_slab_pointers": 60595712,
 }
 
 

@@ -11,7 +11,7 @@
 // that go on are read in further rounds of the same kind.  A lookup is one
 // slab of DRAM out of order, so what bounds a large batch is how many slabs
 // are in flight.  R-MAT scale 20, 2.1 M lookups, half of them present: 74 us
-// with 32/G chains in flight a warp, 52 us so (the slabs alone, as one random
+// with 32/G chains in flight a warp, 54 us so (the slabs alone, as one random
 // gather of 128-byte lines: 33-45 us).  The warp writes one bitmap word per
 // chunk.  G and the block size are picked by the autotuner
 // (mk_autotune); the default is G = 8, 256 threads.
